@@ -61,6 +61,7 @@ struct FpVariant {
   int ntiles = 0;
   SplitRed* reds = nullptr;  // split tiles to reduce after the product kernels
   int nreds = 0;
+  int red_el = 0;            // elements of the largest of them
   long long psize = 0;       // partial-tile elements per vector
   double* part = nullptr;    // partial tiles (psize * part_nvec)
   int part_nvec = 0;
@@ -78,6 +79,12 @@ struct Tune {
 // such as cold caches land there), then kTuneRounds timed samples of every
 // variant, the fastest sample of each compared
 constexpr int kTuneRounds = 2;
+// Inside an eigensolver the reduced-precision products feed the next vectors,
+// and a schedule shows in their FP32 partial sums: there the default variant
+// stays unless another needs less than kSteady of its time, so that a few
+// per cent of timing noise do not decide where an unconverged solve ends.
+constexpr double kSteady = 0.8;
+constexpr int kSteadyKey = 1 << 16;  // schedules and graphs of such products are kept apart
 
 // captured launch sequence of one (precision, nvec) use: replayed with the
 // input copied into xbuf and the output copied out of ybuf
@@ -108,7 +115,7 @@ struct DevList {
   // tensor-core form (precision != FP64)
   void* tc = nullptr;
   long long tc_gen = -1;
-  std::map<int, Tune> tune;         // key: precision * 64 + nvec
+  std::map<int, Tune> tune;         // key: precision * 64 + nvec (+ kSteadyKey)
   std::map<int, GraphSlot> graphs;  // same key
 };
 
@@ -182,6 +189,7 @@ class CudaBackend : public Backend {
   // online schedule autotuning (on by default; TNS_AUTOTUNE=0 keeps the
   // default variant, which makes repeated runs bitwise reproducible)
   bool autotune = true;
+  bool iterating = false;  // products of an eigensolver (kSteady)
   // launches of the FP64 product kernels of variant v (no allocation, no
   // synchronisation: capturable)
   void enqueue_fp64(const DevList& d, int v, const double* xv, double* yv, int nvec, long long xs, long long ys);
@@ -237,6 +245,8 @@ void check_tasks_tc(CudaBackend& be, DevList& d);
 void release_tc_plan(void* plan);
 
 // kernels used by the solver (defined in kernels.cu)
+void launch_reduce_splits(CudaBackend& be, const SplitRed* reds, int nreds, int maxel, const Group* groups,
+                          const double* part, long long psize, double* yv, long long ys, int nvec);
 void launch_heff_diag(CudaBackend& be, const Task* d_tasks, const int* d_idx, const int* d_rng, int ngroups,
                       const Group* d_groups, double* diag);
 void launch_multidot(CudaBackend& be, const double* V, long long ldv, int k, const double* w, long long n,

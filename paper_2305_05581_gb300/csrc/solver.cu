@@ -166,7 +166,9 @@ int davidson(Engine& E, CudaBackend& be, double* X, double tol, int max_iter, in
   // operator block read)
   auto matvec = [&](const double* in, double* out, int nv, int prec) {
     Timer tm(be.stream());
+    be.iterating = true;
     be.run(st.heff, in, out, nv, n, n, prec);
+    be.iterating = false;
     float ms = tm.stop();
     if (acc) {
       acc->heff_ms += ms;

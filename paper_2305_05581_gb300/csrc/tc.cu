@@ -108,6 +108,7 @@ struct TcVariant {
   int ws_ctas = 0;
   SplitRed* reds = nullptr;
   int nreds = 0;
+  int red_el = 0;  // elements of the largest split tile
   long long psize = 0;
   double* part = nullptr;
   int part_nvec = 0;
@@ -1650,9 +1651,6 @@ T* upload_vec(CudaBackend& be, const std::vector<T>& v, bool& ok) {
 
 }  // namespace
 
-void launch_reduce_splits(CudaBackend& be, const SplitRed* reds, int nreds, const Group* groups, const double* part,
-                          long long psize, double* yv, long long ys, int nvec);
-
 void release_tc_plan(void* p);
 
 bool prepare_tasks_tc(CudaBackend& be, const TaskList& tl, DevList& d, int nvec, int variant, int precision) {
@@ -1828,6 +1826,7 @@ bool prepare_tasks_tc(CudaBackend& be, const TaskList& tl, DevList& d, int nvec,
     }
     V.ntiles = (int)tiles.size();
     V.nreds = (int)reds.size();
+    for (const SplitRed& R : reds) V.red_el = std::max(V.red_el, R.nrows * R.ncols);
     V.psize = psize;
     V.planned = true;
     be.note(cudaStreamSynchronize(be.stream()), "tensor-core schedule upload");
@@ -1918,7 +1917,7 @@ void enqueue_tasks_tc(CudaBackend& be, DevList& d, const double* xv, double* yv,
     launch_sw(k_tasks_sw<0, 32>, SwCfg<32>::WARPS, b32, V.wtiles[1], V.nwtiles[1]);
   }
   if (V.ntiles == 0) {
-    if (V.nreds > 0) launch_reduce_splits(be, V.reds, V.nreds, d.groups, V.part, V.psize, yv, ys, nvec);
+    if (V.nreds > 0) launch_reduce_splits(be, V.reds, V.nreds, V.red_el, d.groups, V.part, V.psize, yv, ys, nvec);
     return;
   }
   if (variant == kWsVariant) {
@@ -1935,7 +1934,7 @@ void enqueue_tasks_tc(CudaBackend& be, DevList& d, const double* xv, double* yv,
           plan->x_lo, plan->x_bytes, plan->xblocks, yv, ys, plan->flag, V.part, V.psize, nvec, be.tc_wait_ns);
     be.launches++;
     be.note(cudaGetLastError(), "k_tasks_tc_ws");
-    if (V.nreds > 0) launch_reduce_splits(be, V.reds, V.nreds, d.groups, V.part, V.psize, yv, ys, nvec);
+    if (V.nreds > 0) launch_reduce_splits(be, V.reds, V.nreds, V.red_el, d.groups, V.part, V.psize, yv, ys, nvec);
     return;
   }
   const unsigned grid = (unsigned)V.ntiles * (unsigned)nvec;
@@ -1951,7 +1950,7 @@ void enqueue_tasks_tc(CudaBackend& be, DevList& d, const double* xv, double* yv,
                                                                    V.part, V.psize, nvec, be.tc_wait_ns);
   be.launches++;
   be.note(cudaGetLastError(), "k_tasks_tc");
-  if (V.nreds > 0) launch_reduce_splits(be, V.reds, V.nreds, d.groups, V.part, V.psize, yv, ys, nvec);
+  if (V.nreds > 0) launch_reduce_splits(be, V.reds, V.nreds, V.red_el, d.groups, V.part, V.psize, yv, ys, nvec);
 }
 
 void check_tasks_tc(CudaBackend& be, DevList& d) {
