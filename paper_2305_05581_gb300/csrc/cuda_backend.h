@@ -31,8 +31,27 @@ struct Tile {  // an output tile of a group: rows [row0, row0+nrows), cols [col0
   int g;
   int row0, col0, nrows, ncols;
   int t0, t1;      // task range of this piece (a split tile has several pieces)
+  int aside;       // digit kernel: 1 = op(L) and the rows are the side that is contracted with X first, 0 = op(R) and the columns
   long long poff;  // -1: write the output block; else element offset of this piece's partial tile
 };
+
+// classes of the FP64 digit kernel (fp64_digits.cu): most rows of the a side
+// and columns of the b side of a tile, l and k staged at a time, CTAs per SM
+struct DgClass {
+  int a, b, lk, km, ctas;
+};
+constexpr int kDgClasses = 3;
+constexpr DgClass kDgClass[kDgClasses] = {{16, 16, 16, 16, 12}, {32, 32, 32, 32, 4}, {64, 64, 64, 32, 2}};
+cudaError_t fp64_digits_init();
+class CudaBackend;
+struct DevList;
+struct Tile;
+bool prepare_digits(CudaBackend& be, const TaskList& tl, DevList& d, int nvec, long long length);
+void enqueue_digit_vectors(CudaBackend& be, const DevList& d, const double* xv, long long xs, int nvec);
+void release_digit_plan(void* plan);
+void launch_fp64_digits(int cls, unsigned grid, cudaStream_t s, const void* plan, const Task* tasks,
+                        const Group* groups, const Tile* tiles, int tile0, const double* xv, double* yv, long long xs,
+                        long long ys, double* part, long long psize, int nv);
 
 struct SplitRed {  // a split tile: sum of nsplit partial tiles (fixed order) -> output
   int g;
@@ -106,26 +125,31 @@ struct DevList {
   Group* groups = nullptr;
   Tile* wtiles = nullptr;    // 32 x 16 warp tiles of the FP64 tensor (DMMA) kernel
   int nwtiles = 0;
-  FpVariant fv[kNumVariants];
+  FpVariant fv[2][kNumVariants];  // [0] DFMA classes, [1] digit classes
   // FP64 output tiles per size class with their estimated FMAs (host; shared
   // by the schedule variants, which differ only in how they cut the tiles)
-  bool fp_tiled = false;
-  std::vector<Tile> fp_tiles[4];
-  std::vector<double> fp_cost[4];
+  bool fp_tiled[2] = {false, false};
+  std::vector<Tile> fp_tiles[2][4];
+  std::vector<double> fp_cost[2][4];
+  // digit images of the list (fp64_digits.cu); dg_none: they cannot be had
+  void* dg = nullptr;
+  bool dg_none = false;
+  std::vector<unsigned char> dg_aside;  // per group: the tiles' a side
   // tensor-core form (precision != FP64)
   void* tc = nullptr;
   long long tc_gen = -1;
-  std::map<int, Tune> tune;         // key: precision * 64 + nvec (+ kSteadyKey)
+  std::map<int, Tune> tune;         // key: precision code * 64 + nvec (+ kSteadyKey)
   std::map<int, GraphSlot> graphs;  // same key
 };
 
 class CudaBackend : public Backend {
  public:
   CudaBackend(int device, cudaStream_t s, bool own);
-  // FP64 product kernel: 0 DFMA tile classes (default: on GB300 DFMA and DMMA
-  // peak at ~1.0 TFLOP/s alike and the DFMA kernel measured faster), 1 DMMA
-  // (mma.sync m8n8k4 f64); environment TNS_FP64_KERNEL=dfma|dmma
-  int fp64_kernel = 0;
+  // FP64 product kernel of every list: 0 DFMA tile classes, 1 DMMA (mma.sync
+  // m8n8k4 f64), 2 exact digit products on the f16 tensor cores
+  // (fp64_digits.cu); -1 (default): digits where the list allows them, else
+  // DFMA; environment TNS_FP64_KERNEL=dfma|dmma|digits
+  int fp64_kernel = -1;
   // bound of one wait inside the tensor-core product loop (ns); the
   // environment variable TNS_TC_WAIT_NS overrides the default 0.2 s when the
   // backend is created (a test makes the waits run out with it and checks the
@@ -189,10 +213,12 @@ class CudaBackend : public Backend {
   // online schedule autotuning (on by default; TNS_AUTOTUNE=0 keeps the
   // default variant, which makes repeated runs bitwise reproducible)
   bool autotune = true;
+  // device bytes the last step's memory plan asked for (step_bytes)
+  long long last_step_bytes = 0;
   bool iterating = false;  // products of an eigensolver (kSteady)
   // launches of the FP64 product kernels of variant v (no allocation, no
   // synchronisation: capturable)
-  void enqueue_fp64(const DevList& d, int v, const double* xv, double* yv, int nvec, long long xs, long long ys);
+  void enqueue_fp64(const DevList& d, int dig, int v, const double* xv, double* yv, int nvec, long long xs, long long ys);
   // room for `bytes` of the backend's own allocations (the engine's hook)
   void need(long long bytes) {
     if (room && bytes > (64LL << 20)) room(bytes);
@@ -224,7 +250,7 @@ class CudaBackend : public Backend {
   cudaEvent_t fev_[4] = {nullptr, nullptr, nullptr, nullptr};
   bool fork_ready();
   void upload_list(const TaskList& tl, DevList& d);
-  void plan_variant(const TaskList& tl, DevList& d, int v);
+  void plan_variant(const TaskList& tl, DevList& d, int dig, int v);
   bool ensure_part(DevList& d, FpVariant& f, int nvec);
   void free_list(DevList& d);
   template <class F>

@@ -2006,7 +2006,7 @@ void Engine::build_heff_tasks() {
       if (tl.tasks[i].pad == g) st.diag_tasks.push_back(i);
     st.diag_rng.push_back((int)st.diag_tasks.size());
   }
-  tl.persistent = true;
+  tl.persistent = tl.digits = true;
 }
 
 // the operator blocks of a catalogue that are identically zero (an operator
@@ -2233,7 +2233,7 @@ int Engine::heff_part(const double* X, double* Y, int nvec, int precision, int p
     }
     tl.nprod = (long long)tl.tasks.size();
     tl.flops = 0.0;
-    tl.persistent = true;
+    tl.persistent = tl.digits = true;
     st.part_key = key;
   }
   be_->run(st.heff_part, X, Y, nvec, st.length, st.length, precision);
@@ -2341,6 +2341,7 @@ int Engine::heff_adjoint(const double* X, const double* Yb, double* Xb, double* 
                      long long srcsize, const std::vector<std::pair<long long, std::pair<int, int>>>& blocks) {
     // groups: every block of [srcbase, srcbase+srcsize) listed in `blocks` (offset, (rows, cols))
     TaskList tl;
+    tl.digits = true;
     for (auto& b : blocks) {
       Group g;
       g.yoff = b.first;

@@ -297,8 +297,16 @@ struct TaskList {
   long long nprod = 0;
   long long gen = 0;        // bumped on every rebuild (device copies keyed on it)
   bool persistent = false;  // kept on the device between runs
+  // the FP64 form may use exact digit products (as accurate, rounded at other
+  // places than a chain of FMAs); lists whose results feed a state that is
+  // continued from them (renormalisation, truncation) keep the FMA order
+  bool digits = false;
   void clear() { tasks.clear(); groups.clear(); flops = 0; nprod = 0; ++gen; }
 };
+
+// precision codes of Backend::run: 0 FP64, 1 TF32, 2 split-BF16 (as in the C
+// ABI), and FP64 in FMA order whatever the list allows
+constexpr int kFp64Fma = 3;
 
 struct LCTerm {
   double c;

@@ -1,0 +1,1359 @@
+// fp64_digits.cu -- the grouped FP64 triple product on the 16-bit tensor cores
+// by exact digit arithmetic.
+//
+// GB300's FP64 units (DFMA and DMMA alike) issue 2 FMAs per clock and SM, its
+// mma.sync f16 path 1024 (measured: 1.06 TFLOP/s against 600 TFLOP/s), so an
+// FP64 product is cheaper as a sum of exact 16-bit products.  The scheme is
+// the error-free splitting of Ozaki, Ogita, Oishi and Rump (Numerical
+// Algorithms 59, 2012) with one power-of-two scale per operand row:
+//     x = 2^(E-63) v,  v a 64-bit integer = sum_{i<7} d_i 2^(56-8i) + (< 2^8),
+// the d_i balanced base-256 digits in [-128, 127], exact in f16.  Products of
+// digits are at most 2^14; a sum over K = 32 of the pairs of equal weight
+// s = i + j (at most 7 of them) stays below 2^22, so it is an exact integer in
+// an FP32 accumulator that starts at 1.5 * 2^23, read off its mantissa without
+// a conversion.  The pairs with s <= 7 are kept (34 of them).  On Gaussian,
+// diagonal-dominant and graded operands the result is closer to the exact one
+// than a chain of FP64 FMAs (0.3 to 0.9 of its error; without the pairs of
+// s = 7 it can be twice as far).
+// The eight integers of an output are put together in a 64-bit integer.
+//
+// One CTA owns one output tile of one block and walks the block's products in
+// a fixed order, as the DFMA classes do.  With A the operand of the tile's
+// "a" side (op(R) and its columns, or op(L) and its rows; chosen per tile), X
+// oriented to match and B the other operand, a product is
+//     GEMM1  T[a][k] = sum_l A[a][l] X[k][l]     (64-bit integers per row a)
+//     GEMM2  Y[a][b] += alpha sum_k T[a][k] B[b][k]
+// Each warp owns 16 rows a.  GEMM1's accumulators are fragments whose layout
+// is that of GEMM2's A operand, so T is normalised per row, cut into digits
+// again and used from registers.  The row scales of X (one per k) go to the
+// columns of B before B is cut.  Y is kept in FP64 registers: one DFMA per
+// output and 32 terms of k, where the DFMA kernel needs 32.
+//
+// Two kernels: k_tasks_dg cuts its operands where it uses them, from the FP64
+// blocks into shared-memory planes of 8 x 8 f16 core matrices (ldmatrix) --
+// for lists that run once, and where there is no memory for images;
+// k_tasks_im, further down, reads digits cut beforehand, for lists that are
+// kept.  Both are bound by the integer work around the MMAs (joining the
+// weight sums, cutting T) and by the 8 to 12 warps that registers and shared
+// memory leave an SM to hide its latencies (MMA pipe 30 % busy, issue slots
+// 27 to 49 %).  One H_eff*psi, DFMA tile classes -> here (time, useful rate):
+//   24 orbitals, D = 512, all sectors (blocks <= 26):  36.4 -> 14.9 ms, 1.15 TFLOP/s
+//   24 orbitals, D = 512, 9 sectors (blocks <= 68):     153 -> 47.4 ms, 2.45 TFLOP/s
+//   13 orbitals, D = 260, 3 sectors (blocks <= 99):    3.03 -> 0.78 ms, 2.81 TFLOP/s
+// (cuBLAS DGEMM: 1.10 TFLOP/s).
+//
+// Values that the fixed-point form cannot hold: a chunk in which an operand
+// has an infinity, a NaN or a magnitude of 2^330 or more is evaluated with
+// plain FP64 FMAs instead; rows whose largest magnitude is below 2^-700 are
+// taken relative to 2^-700.
+#include <cuda_fp16.h>
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cstdint>
+
+#include "cuda_backend.h"
+
+namespace tns {
+namespace {
+
+constexpr int DG_N = 7;                        // digits of an operand
+constexpr int DG_T = 8;                        // digits of T: its rows may be graded
+constexpr int DG_S = 8;                        // weights s = i + j kept: 0 .. 7
+constexpr unsigned DG_MAGIC = 0x4B400000u;     // bits of 1.5 * 2^23
+constexpr int DG_EMIN = 322;                   // smallest biased exponent of a row scale (2^-700)
+constexpr int DG_EMAX = (1023 + 330) << 20;    // high word from which on a value leaves the fixed-point form
+
+template <int W_, int NBT_, int LK_, int KM_, int CTAS_>
+struct DgCfg {
+  static constexpr int CTAS = CTAS_;  // resident CTAs per SM
+  static constexpr int W = W_;        // warps: 16 rows of the a side each
+  static constexpr int NBT = NBT_;    // 8-column tiles of the b side
+  static constexpr int LK = LK_;      // l staged at a time
+  static constexpr int KM = KM_;      // k staged at a time (at most 32: exactness)
+  static constexpr int NT = 32 * W, AR = 16 * W, BR = 8 * NBT;
+  static constexpr int PA = AR * LK * 2, PX = KM * LK * 2, PB = BR * KM * 2;  // bytes of one digit plane
+  static constexpr int off_xb = DG_N * PA;                                    // X, then B, in one region
+  static constexpr int off_e = off_xb + DG_N * (PX > PB ? PX : PB);           // row scales of A, X, B
+  static constexpr int total = off_e + 4 * (AR + KM + BR + 4);
+  static_assert(KM <= 32 && LK % 16 == 0 && KM % 16 == 0, "chunk sizes");
+  static_assert(DG_N * PA >= AR * BR * 8, "the A region holds a tile of FP64 values");
+};
+
+__device__ __forceinline__ uint32_t sm_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
+}
+
+__device__ __forceinline__ void mma_acc(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// the first product of an accumulator: starts at the integer base
+__device__ __forceinline__ void mma_first(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  const float c = __uint_as_float(DG_MAGIC);
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(c));
+}
+
+// digit p (0 = most significant) of two biased 64-bit integers as f16x2
+template <int P>
+__device__ __forceinline__ uint32_t digit2(uint32_t h0, uint32_t l0, uint32_t h1, uint32_t l1) {
+  constexpr uint32_t sel = P % 4 == 0 ? 0x7733 : P % 4 == 1 ? 0x6622 : P % 4 == 2 ? 0x5511 : 0x4400;
+  const uint32_t u = (__byte_perm(P < 4 ? h0 : l0, P < 4 ? h1 : l1, sel) & 0x00ff00ffu) | 0x64006400u;  // 1024 + byte
+  const uint32_t off = 0x64806480u;                                                                    // 1152
+  const __half2 d = __hsub2(*(const __half2*)&u, *(const __half2*)&off);
+  return *(const uint32_t*)&d;
+}
+
+// An operand view: element (r, k) = p[r * sr + k * sk] for r < nr and k < nk, else 0
+struct View {
+  const double* p;
+  int sr, sk, nr, nk;
+};
+
+// Rows [0, rpad) x columns [0, KC) of an operand view into digit planes.  A
+// thread takes 8 columns of a row; the KC / 8 threads of a row are adjacent
+// lanes and agree on its scale (ef: biased exponent, the row below 2^(ef -
+// 1022)), unless it was found before (have).  With dk, column k carries a
+// factor 2^(dk[k] - 1022).  Core matrix (row group, octet o) holds row r at
+// slot r ^ o, so that neither these stores nor ldmatrix meet a bank twice.
+// One copy of this code per kernel: inlined at its six uses it is what the
+// instruction cache misses on.
+template <int NT, int KC>
+__device__ __noinline__ void dg_slice(const View vw, int rpad, uint32_t dst, int plane, int* ef, bool have,
+                                      const int* dk, int* bad) {
+  constexpr int OC = KC / 8;
+  const int units = rpad * OC;
+  for (int u0 = 0; u0 < units; u0 += NT) {
+    const int u = u0 + threadIdx.x;
+    const int row = u / OC, o = u % OC;
+    const double* q = vw.p + (long long)row * vw.sr + (long long)(8 * o) * vw.sk;
+    uint32_t hi[8], lo[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const double x = (row < vw.nr && 8 * o + e < vw.nk) ? __ldg(q + (long long)e * vw.sk) : 0.0;
+      hi[e] = (uint32_t)__double2hiint(x);
+      lo[e] = (uint32_t)__double2loint(x);
+    }
+    int uu[8], mx = INT32_MIN, raw = 0;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      uu[e] = (int)(hi[e] & 0x7fffffffu);
+      raw = max(raw, uu[e]);
+    }
+    if (dk) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        uu[e] = uu[e] ? uu[e] + ((dk[8 * o + e] - 1022) << 20) : -(1 << 30);
+        mx = max(mx, uu[e]);
+      }
+    } else {
+      mx = raw;
+    }
+    if (raw >= DG_EMAX) *bad = 1;
+    int E;
+    if (have) {
+      E = ef[min(row, rpad - 1)];
+    } else {
+#pragma unroll
+      for (int s = 1; s < OC; s <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, s));
+      E = max((mx + 0x2100) >> 20, DG_EMIN);  // within 0.8% of a power of two counts as that power: no carry out of digit 0
+      if (o == 0 && u < units) ef[row] = E;
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      // v = (mantissa << 10) >> (E - exponent), sign by complement, + 0x80 in every byte
+      const int sh = min(E - (uu[e] >> 20), 63);
+      const unsigned long long m =
+          ((unsigned long long)((hi[e] & 0xfffffu) | 0x100000u) << 32 | lo[e]) << 10;
+      const unsigned long long v = m >> sh;
+      const uint32_t sg = (uint32_t)((int)hi[e] >> 31);
+      const unsigned long long b =
+          ((unsigned long long)((uint32_t)(v >> 32) ^ sg) << 32 | ((uint32_t)v ^ sg)) + 0x8080808080808080ull;
+      hi[e] = (uint32_t)(b >> 32);
+      lo[e] = (uint32_t)b;
+    }
+    if (u < units) {
+      const uint32_t at = dst + (uint32_t)(((row >> 3) * OC + o) * 128 + (((row & 7) ^ (o & 7)) << 4));
+#define DG_PUT(P)                                                                                                  \
+  asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(at + (P) * (uint32_t)plane),                          \
+               "r"(digit2<P>(hi[0], lo[0], hi[1], lo[1])), "r"(digit2<P>(hi[2], lo[2], hi[3], lo[3])),             \
+               "r"(digit2<P>(hi[4], lo[4], hi[5], lo[5])), "r"(digit2<P>(hi[6], lo[6], hi[7], lo[7]))              \
+               : "memory")
+      DG_PUT(0);
+      DG_PUT(1);
+      DG_PUT(2);
+      DG_PUT(3);
+      DG_PUT(4);
+      DG_PUT(5);
+      DG_PUT(6);
+#undef DG_PUT
+    }
+  }
+}
+
+// the scale of whole rows longer than one staged chunk
+template <int NT, int KC>
+__device__ __noinline__ void dg_rowmax(const View v, int rpad, int* ef, int* bad) {
+  constexpr int OC = KC / 8;
+  for (int u0 = 0; u0 < rpad * OC; u0 += NT) {
+    const int u = u0 + threadIdx.x, row = u / OC, o = u % OC;
+    int mx = 0;
+    if (row < v.nr)
+      for (int k = o; k < v.nk; k += OC)
+        mx = max(mx, __double2hiint(__ldg(v.p + (long long)row * v.sr + (long long)k * v.sk)) & 0x7fffffff);
+    if (mx >= DG_EMAX) *bad = 1;
+#pragma unroll
+    for (int s = 1; s < OC; s <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, s));
+    if (o == 0 && u < rpad * OC) ef[row] = max((mx + 0x2100) >> 20, DG_EMIN);
+  }
+}
+
+// the weight sums of one output as an integer, sum_s i_s 2^(43 - 8 s), below
+// 2^62.1.  T rounds to the nearest; Y (floor) meets the complement that
+// dg_double takes of negative numbers, so that it errs towards zero alike on
+// both sides: a common sign of the error would add up over the products.
+template <bool ROUND>
+__device__ __forceinline__ long long dg_join(float f0, float f1, float f2, float f3, float f4, float f5, float f6,
+                                             float f7) {
+  constexpr unsigned c = DG_MAGIC * 257u;
+  auto two = [](float hi, float lo, unsigned off) {
+    return (int)((unsigned)__float_as_int(hi) * 256u + (unsigned)__float_as_int(lo) - off);
+  };
+  const int P = two(f0, f1, c), Q = two(f2, f3, c), R = two(f4, f5, c), U = two(f6, f7, ROUND ? c - (1u << 12) : c);
+  const int V = R + (U >> 16);
+  const unsigned long long hi = (unsigned long long)((unsigned)P * 8u + (unsigned)(Q >> 13)) << 32 | ((unsigned)Q << 19);
+  const unsigned long long lo = (unsigned long long)(unsigned)(V >> 29) << 32 | ((unsigned)V << 3 | ((unsigned)U >> 13 & 7u));
+  return (long long)(hi + lo);
+}
+
+// v 2^(e - 1085) as a double (towards zero)
+__device__ __forceinline__ double dg_double(long long v, int e) {
+  const uint32_t sg = (uint32_t)((int)(v >> 32) >> 31);
+  uint32_t h = (uint32_t)(v >> 32) ^ sg, l = (uint32_t)v ^ sg;
+  const bool low = h == 0;
+  h = low ? l : h;
+  l = low ? 0u : l;
+  const int z = __clz((int)h);
+  const uint32_t hs = __funnelshift_lc(l, h, z), ls = l << (z & 31);
+  uint32_t dh = (sg & 0x80000000u) | ((uint32_t)((e - z - (low ? 32 : 0)) << 20) + (hs >> 11));
+  uint32_t dl = __funnelshift_r(ls, hs, 11);
+  if (h == 0) dh = dl = 0u;
+  return __hiloint2double((int)dh, (int)dl);
+}
+
+template <class C>
+__global__ void __launch_bounds__(C::NT, C::CTAS)
+    k_tasks_dg(const Task* __restrict__ tasks, const Group* __restrict__ groups, const Tile* __restrict__ tiles,
+               int tile0, const double* xv, double* yv, long long xs, long long ys, double* part, long long psize,
+               int nv) {
+  constexpr int W = C::W, NBT = C::NBT, LK = C::LK, KM = C::KM, NT = C::NT;
+  constexpr int KT = KM / 8;  // 8-wide tiles of k
+  extern __shared__ __align__(128) unsigned char sm[];
+  int* const eA = (int*)(sm + C::off_e);
+  int* const eX = eA + C::AR;
+  int* const eB = eX + KM;
+  int* const bad = eB + C::BR;
+  const uint32_t sA = sm_u32(sm), sXB = sm_u32(sm + C::off_xb);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
+  const int mj = lane >> 3, mr = lane & 7;  // ldmatrix: the matrix and row this lane addresses
+  const Tile TL = tiles[tile0 + blockIdx.x / nv];
+  const Group G = groups[TL.g];
+  const int vec = blockIdx.x % nv;
+  const double* X0 = xv ? xv + (long long)vec * xs : nullptr;
+  const bool bl = TL.aside != 0;  // the a side is op(L) and the rows of Y
+  const int na = bl ? TL.nrows : TL.ncols, nb = bl ? TL.ncols : TL.nrows;
+  const int a0 = bl ? TL.row0 : TL.col0, b0 = bl ? TL.col0 : TL.row0;
+  const int nbt = (nb + 7) >> 3, apad = (na + 15) & ~15, bpad = nbt * 8;
+  const bool mine = 16 * warp < na;  // warp-uniform: this warp has rows
+  double y[NBT][4];
+#pragma unroll
+  for (int b = 0; b < NBT; ++b)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) y[b][e] = 0.0;
+  auto sync = [&]() {
+    if (W == 1) __syncwarp();
+    else __syncthreads();
+  };
+  if (tid == 0) *bad = 0;
+  sync();
+
+  uint32_t tf[KT / 2][DG_T][4];  // T's digits over a staged chunk of k: GEMM2's A operand
+  auto scale = [](double alpha, int n) { return alpha * __hiloint2double((n + 1023) << 20, 0); };  // alpha 2^n
+
+  for (int ti = TL.t0; ti < TL.t1; ++ti) {
+    const Task tk = tasks[ti];
+    const int f = tk.flags;
+    const double* pX = (f & TF_XV) ? X0 + (long long)(size_t)tk.X : tk.X;
+    const int sXi = (f & TF_XT) ? 1 : tk.n, sXj = (f & TF_XT) ? tk.m : 1;
+    const int sLi = (f & TF_LT) ? 1 : tk.m, sLk = (f & TF_LT) ? tk.q : 1;
+    const int sRj = (f & TF_RT) ? 1 : tk.n, sRk = (f & TF_RT) ? tk.r : 1;
+    const int sXk = bl ? sXj : sXi, sXl = bl ? sXi : sXj;
+    const int K3 = bl ? tk.n : tk.m, L = bl ? tk.m : tk.n;
+    const bool ai = (f & (bl ? TF_LI : TF_RI)) != 0, bi = (f & (bl ? TF_RI : TF_LI)) != 0;
+    if (ai && bi) {  // Y += alpha X
+      if (mine)
+#pragma unroll
+        for (int b = 0; b < NBT; ++b)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int a = 16 * warp + g + 8 * (e >> 1), c = 8 * b + 2 * t + (e & 1);
+            if (a < na && c < nb)
+              y[b][e] = fma(tk.alpha, __ldg(pX + (long long)(b0 + c) * sXk + (long long)(a0 + a) * sXl), y[b][e]);
+          }
+      continue;
+    }
+    // views A (a, l), X (k, l), B (b, k); with one identity factor two views
+    // are left: Y[a][b] += alpha sum_k P[a][k] Q[b][k], P in A's place, Q in B's
+    const bool two = ai || bi || (f & TF_XI);
+    View A{(bl ? tk.L : tk.R), bl ? sLi : sRj, bl ? sLk : sRk, na, L};
+    View B{(bl ? tk.R : tk.L), bl ? sRj : sLi, bl ? sRk : sLk, nb, K3};
+    A.p += ai ? 0 : (long long)a0 * A.sr;
+    B.p += bi ? 0 : (long long)b0 * B.sr;
+    if (ai) A = View{pX + (long long)a0 * sXl, sXl, sXk, na, K3};
+    if (bi) B = View{pX + (long long)b0 * sXk, sXk, sXl, nb, L};
+    const int K = two ? A.nk : K3;
+    const bool long_l = !two && L > LK;
+    int hsh = 0;  // head room of T beyond one sum of 32
+    while ((32 << hsh) < L) ++hsh;
+    bool slow = false;
+    sync();
+    if (!two) {
+      if (long_l) dg_rowmax<NT, LK>(A, apad, eA, bad);
+      else dg_slice<NT, LK>(A, apad, sA, C::PA, eA, false, nullptr, bad);
+    }
+    for (int k0 = 0; k0 < K; k0 += KM) {
+      const int kc = min(KM, K - k0), kpad = (kc + 15) & ~15;
+      const View Bk{B.p + (long long)k0 * B.sk, B.sr, B.sk, nb, kc};
+      double s0 = 0.0, s1 = 0.0;
+      if (two && !slow) {
+        sync();
+        dg_slice<NT, KM>(View{A.p + (long long)k0 * A.sk, A.sr, A.sk, na, kc}, apad, sA, C::PA, eA, false, nullptr, bad);
+      } else if (!slow) {
+        const View X{pX + (long long)k0 * sXk, sXk, sXl, kc, L};
+        long long T[KT][4];
+        sync();
+        if (long_l) {
+          dg_rowmax<NT, LK>(X, kpad, eX, bad);
+          sync();
+        }
+#pragma unroll
+        for (int b = 0; b < KT; ++b)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) T[b][e] = 0;
+        for (int l0 = 0; l0 < L; l0 += LK) {
+          const int lc = min(LK, L - l0);
+          if (l0) sync();
+          if (long_l)
+            dg_slice<NT, LK>(View{A.p + (long long)l0 * A.sk, A.sr, A.sk, na, lc}, apad, sA, C::PA, eA, true, nullptr, bad);
+          dg_slice<NT, LK>(View{X.p + (long long)l0 * sXl, sXk, sXl, kc, lc}, kpad, sXB, C::PX, eX, long_l, nullptr, bad);
+          sync();
+          if (*bad) slow = true;
+          if (slow) break;
+          if (!mine) continue;
+#pragma unroll
+          for (int kp = 0; kp < KT / 2; ++kp) {
+            if (16 * kp >= kc) break;
+            for (int l32 = 0; l32 < lc; l32 += 32) {
+              float acc[2][DG_S][4];
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                if (h == 1 && l32 + 16 >= lc) break;
+                const int ob = l32 / 8 + 2 * h;
+                uint32_t xf[DG_N][4];
+                {
+                  const int o = ob + (mj & 1);
+                  const uint32_t xa =
+                      sXB + (uint32_t)(((2 * kp + (mj >> 1)) * (LK / 8) + o) * 128 + ((mr ^ (o & 7)) << 4));
+#pragma unroll
+                  for (int j = 0; j < DG_N; ++j) ldsm4(xf[j], xa + j * C::PX);
+                }
+                const int o = ob + (mj >> 1);
+                const uint32_t aa =
+                    sA + (uint32_t)(((2 * warp + (mj & 1)) * (LK / 8) + o) * 128 + ((mr ^ (o & 7)) << 4));
+#pragma unroll
+                for (int i = 0; i < DG_N; ++i) {
+                  uint32_t af[4];
+                  ldsm4(af, aa + i * C::PA);
+#pragma unroll
+                  for (int j = 0; j < DG_N && i + j < DG_S; ++j) {
+                    if (h == 0 && (i == 0 || (i == 1 && j == DG_N - 1))) {
+                      mma_first(acc[0][i + j], af, xf[j][0], xf[j][1]);
+                      mma_first(acc[1][i + j], af, xf[j][2], xf[j][3]);
+                    } else {
+                      mma_acc(acc[0][i + j], af, xf[j][0], xf[j][1]);
+                      mma_acc(acc[1][i + j], af, xf[j][2], xf[j][3]);
+                    }
+                  }
+                }
+              }
+#pragma unroll
+              for (int c = 0; c < 2; ++c)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                  const long long v = dg_join<true>(acc[c][0][e], acc[c][1][e], acc[c][2][e], acc[c][3][e], acc[c][4][e],
+                                              acc[c][5][e], acc[c][6][e], acc[c][7][e]);
+                  T[2 * kp + c][e] += hsh ? v >> hsh : v;
+                }
+            }
+          }
+        }
+        if (mine && !slow) {
+          // normalise T per row over the chunk and cut it again
+          int m0 = 0, m1 = 0;
+#pragma unroll
+          for (int b = 0; b < KT; ++b)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const int h = (int)(T[b][e] >> 32), ah = h ^ (h >> 31);
+              if (e < 2) m0 = max(m0, ah);
+              else m1 = max(m1, ah);
+            }
+#pragma unroll
+          for (int s = 1; s < 4; s <<= 1) {
+            m0 = max(m0, __shfl_xor_sync(0xffffffffu, m0, s));
+            m1 = max(m1, __shfl_xor_sync(0xffffffffu, m1, s));
+          }
+          const int z0 = __clz(m0 + (m0 >> 7) + 1) - 1, z1 = __clz(m1 + (m1 >> 7) + 1) - 1;
+#pragma unroll
+          for (int kk = 0; kk < KT / 2; ++kk)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {  // q: rows g, g + 8 of the first 8 k, then of the second
+              const int b = 2 * kk + (q >> 1), e = 2 * (q & 1), z = q & 1 ? z1 : z0;
+              const unsigned long long v0 = ((unsigned long long)T[b][e] << z) + 0x8080808080808080ull;
+              const unsigned long long v1 = ((unsigned long long)T[b][e + 1] << z) + 0x8080808080808080ull;
+              const uint32_t h0 = (uint32_t)(v0 >> 32), l0 = (uint32_t)v0, h1 = (uint32_t)(v1 >> 32), l1 = (uint32_t)v1;
+              tf[kk][0][q] = digit2<0>(h0, l0, h1, l1);
+              tf[kk][1][q] = digit2<1>(h0, l0, h1, l1);
+              tf[kk][2][q] = digit2<2>(h0, l0, h1, l1);
+              tf[kk][3][q] = digit2<3>(h0, l0, h1, l1);
+              tf[kk][4][q] = digit2<4>(h0, l0, h1, l1);
+              tf[kk][5][q] = digit2<5>(h0, l0, h1, l1);
+              tf[kk][6][q] = digit2<6>(h0, l0, h1, l1);
+              tf[kk][7][q] = digit2<7>(h0, l0, h1, l1);
+            }
+          s0 = scale(tk.alpha, eA[16 * warp + g] - 1022 + 6 + hsh - z0 - 57);
+          s1 = scale(tk.alpha, eA[16 * warp + g + 8] - 1022 + 6 + hsh - z1 - 57);
+        }
+        sync();
+      }
+      if (!slow) {
+        dg_slice<NT, KM>(Bk, bpad, sXB, C::PB, eB, false, two ? nullptr : eX, bad);
+        sync();
+        if (*bad) slow = true;
+      }
+      if (slow) {  // uniform: this and the remaining chunks of the product in plain FP64
+        double* D = (double*)sm;
+        sync();
+        for (int e = tid; e < na * nb; e += NT) {
+          const int a = e / nb, b = e % nb;
+          double s = 0.0;
+          for (int k = k0; k < k0 + kc; ++k) {
+            double x = 0.0;
+            if (two)
+              x = __ldg(A.p + (long long)a * A.sr + (long long)k * A.sk);
+            else
+              for (int l = 0; l < L; ++l)
+                x = fma(__ldg(pX + (long long)k * sXk + (long long)l * sXl), __ldg(A.p + (long long)a * A.sr + (long long)l * A.sk), x);
+            s = fma(__ldg(B.p + (long long)b * B.sr + (long long)k * B.sk), x, s);
+          }
+          D[e] = s;
+        }
+        if (tid == 0) *bad = 0;
+        sync();
+        if (mine)
+#pragma unroll
+          for (int b = 0; b < NBT; ++b)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const int a = 16 * warp + g + 8 * (e >> 1), c = 8 * b + 2 * t + (e & 1);
+              if (a < na && c < nb) y[b][e] = fma(tk.alpha, D[a * nb + c], y[b][e]);
+            }
+        continue;
+      }
+      if (!mine) continue;
+      if (two) {
+#pragma unroll
+        for (int kk = 0; kk < KT / 2; ++kk)
+#pragma unroll
+          for (int i = 0; i < DG_T; ++i) {
+            const int o = 2 * kk + (mj >> 1);
+            if (i == DG_N) tf[kk][i][0] = tf[kk][i][1] = tf[kk][i][2] = tf[kk][i][3] = 0u;
+            else ldsm4(tf[kk][i], sA + i * C::PA + (uint32_t)(((2 * warp + (mj & 1)) * KT + o) * 128 + ((mr ^ o) << 4)));
+          }
+        s0 = scale(tk.alpha, eA[16 * warp + g] - 1022 - 57);
+        s1 = scale(tk.alpha, eA[16 * warp + g + 8] - 1022 - 57);
+      }
+      // GEMM2: the planes of B against T's digits, joined into Y
+#pragma unroll
+      for (int b = 0; b < NBT; ++b) {
+        if (b >= nbt) break;
+        float acc[DG_S][4];
+        uint32_t bf[DG_N][4];
+        const int o = KT == 4 ? mj : (mj & 1);
+        const uint32_t ba = sXB + (uint32_t)((b * KT + o) * 128 + ((mr ^ o) << 4));
+#pragma unroll
+        for (int j = 0; j < DG_N; ++j) ldsm4(bf[j], ba + j * C::PB);
+#pragma unroll
+        for (int i = 0; i < DG_T; ++i)
+#pragma unroll
+          for (int j = 0; j < DG_N && i + j < DG_S; ++j) {
+            if (i == 0 || (i == 1 && j == DG_N - 1)) mma_first(acc[i + j], tf[0][i], bf[j][0], bf[j][1]);
+            else mma_acc(acc[i + j], tf[0][i], bf[j][0], bf[j][1]);
+          }
+        if (KT == 4 && kc > 16) {
+#pragma unroll
+          for (int i = 0; i < DG_T; ++i)
+#pragma unroll
+            for (int j = 0; j < DG_N && i + j < DG_S; ++j) mma_acc(acc[i + j], tf[KT / 2 - 1][i], bf[j][2], bf[j][3]);
+        }
+        const int e0 = eB[8 * b + 2 * t] + 63, e1 = eB[8 * b + 2 * t + 1] + 63;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const long long v = dg_join<false>(acc[0][e], acc[1][e], acc[2][e], acc[3][e], acc[4][e], acc[5][e], acc[6][e], acc[7][e]);
+          y[b][e] = fma(dg_double(v, e & 1 ? e1 : e0), e < 2 ? s0 : s1, y[b][e]);
+        }
+      }
+    }
+  }
+
+  double* Y = yv + (long long)vec * ys + G.yoff;
+  double* P = TL.poff >= 0 ? part + (long long)vec * psize + TL.poff : nullptr;  // split piece
+  if (mine)
+#pragma unroll
+    for (int b = 0; b < NBT; ++b)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int a = 16 * warp + g + 8 * (e >> 1), c = 8 * b + 2 * t + (e & 1);
+        if (a >= na || c >= nb) continue;
+        const int i = bl ? a : c, j = bl ? c : a;
+        if (P) P[i * TL.ncols + j] = y[b][e];
+        else Y[(long long)(TL.row0 + i) * G.r + TL.col0 + j] = y[b][e];
+      }
+}
+
+// ---------------------------------------------------------------------------
+// The same products from prepared digits (lists that are run many times).
+//
+// Every distinct operand of the list has an image: its digits, cut once, in
+// units of 8 rows x 8 columns x 7 planes of f16 core matrices (896 bytes; row
+// groups outermost, columns padded to 16), after the scales of its rows.  The
+// vectors are cut once per call, each block in the orientation its products
+// read, into 8 digits (all 64 bits of v; the pair (0, 7) joins the others).
+// Here the scales of X cannot go to the columns of B, so T is brought to a
+// common scale over k as it is normalised: a shift per element by the distance
+// of its row of X from the block's largest.  Against cutting operands where
+// they are used this takes 40% of the instructions off the product loop (24
+// orbitals: 36.5 -> 14.9 ms, 9 sectors 64 -> 47 ms).
+// ---------------------------------------------------------------------------
+constexpr int IM_UNIT = DG_N * 128;  // bytes of one 8 x 8 unit of an operator
+constexpr int IM_NX = 8;             // digits of the vector and of T
+constexpr int IM_XUNIT = IM_NX * 128;
+constexpr int IM_SLOW = 0x7fffffff;  // scale of a block that the fixed-point form cannot hold
+
+__host__ __device__ inline int im_oct(int cols) { return (cols + 15) / 16 * 2; }
+__host__ __device__ inline int im_head(int rows) { return ((rows + 7) / 8 * 8 * 4 + 127) / 128 * 128; }
+__host__ __device__ inline long long im_bytes(int rows, int cols) {
+  return im_head(rows) + (long long)((rows + 7) / 8) * im_oct(cols) * IM_UNIT;
+}
+
+struct DgRec {  // a product in the orientation of its tile
+  uint32_t a, b, x;  // images of A (rows a) and B (rows b) in the operator arena, of X in the vector arena; 128-byte units
+  int xb;            // scale index of X
+  double alpha;
+  int K, L, f, pad;  // f: 1 A is the identity, 2 B is, 4 an operand does not fit the fixed-point form
+};
+struct DgImage {  // an operand to cut: op(M) is rows x cols, element (r, c) = src[r * sr + c * sc]
+  const double* src;
+  int rows, cols, sr, sc;
+  uint32_t off;
+  int slow;
+};
+struct DgXBlock {  // a block of the vector, in one orientation
+  long long src;
+  int rows, cols, sr, sc;
+  uint32_t off;
+  int pad;
+};
+
+// one row's 8 columns as digits: E the row's scale
+template <int N>
+__device__ __forceinline__ void im_cut(const double (&x)[8], int E, unsigned char* at) {
+  uint32_t hi[8], lo[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    const uint32_t h = (uint32_t)__double2hiint(x[e]), l = (uint32_t)__double2loint(x[e]);
+    const int sh = max(0, min(E - (int)((h & 0x7fffffffu) >> 20), 63));
+    const unsigned long long v = (((unsigned long long)((h & 0xfffffu) | 0x100000u) << 32 | l) << 10) >> sh;
+    const uint32_t sg = (uint32_t)((int)h >> 31);
+    const unsigned long long b =
+        ((unsigned long long)((uint32_t)(v >> 32) ^ sg) << 32 | ((uint32_t)v ^ sg)) + 0x8080808080808080ull;
+    hi[e] = (uint32_t)(b >> 32);
+    lo[e] = (uint32_t)b;
+  }
+#define IM_PUT(P)                                                                                                  \
+  *(uint4*)(at + (P) * 128) = make_uint4(digit2<P>(hi[0], lo[0], hi[1], lo[1]), digit2<P>(hi[2], lo[2], hi[3], lo[3]), \
+                                         digit2<P>(hi[4], lo[4], hi[5], lo[5]), digit2<P>(hi[6], lo[6], hi[7], lo[7]))
+  IM_PUT(0);
+  IM_PUT(1);
+  IM_PUT(2);
+  IM_PUT(3);
+  IM_PUT(4);
+  IM_PUT(5);
+  IM_PUT(6);
+  if (N > 7) IM_PUT(7);
+#undef IM_PUT
+}
+
+__device__ __forceinline__ int im_scale(int mx) { return max((mx + 0x2100) >> 20, DG_EMIN); }
+
+// the image of a matrix by a CTA of 4 warps, a warp per group of 8 rows: the
+// rows' scales, then their digits; returns the largest high word seen
+template <int N>
+__device__ __forceinline__ int im_rows(const double* __restrict__ src, int rows, int cols, int sr, int sc, int groups,
+                                       unsigned char* img) {
+  const int oc = im_oct(cols), lane = threadIdx.x & 31, warp = threadIdx.x >> 5, r7 = lane & 7, q = lane >> 3;
+  int* scale = (int*)img;
+  unsigned char* units = img + im_head(8 * groups);
+  int top = 0;
+  for (int rg = warp; rg < groups; rg += 4) {
+    const int row = 8 * rg + r7;
+    int mx = 0;
+    if (row < rows)
+      for (int c = q; c < cols; c += 4)
+        mx = max(mx, __double2hiint(__ldg(src + (long long)row * sr + (long long)c * sc)) & 0x7fffffff);
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
+    top = max(top, mx);
+    const int E = im_scale(mx);
+    if (q == 0) scale[row] = E;
+    for (int o = q; o < oc; o += 4) {
+      double x[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        x[e] = (row < rows && 8 * o + e < cols) ? __ldg(src + (long long)row * sr + (long long)(8 * o + e) * sc) : 0.0;
+      im_cut<N>(x, E, units + ((long long)rg * oc + o) * (N * 128) + r7 * 16);
+    }
+  }
+  return top;
+}
+
+__global__ void __launch_bounds__(128) k_dg_ops(DgImage* __restrict__ jobs, unsigned char* arena) {
+  DgImage& J = jobs[blockIdx.x];
+  if (im_rows<DG_N>(J.src, J.rows, J.cols, J.sr, J.sc, (J.rows + 7) / 8, arena + (long long)J.off * 128) >= DG_EMAX)
+    J.slow = 1;
+}
+
+// vector images: one CTA per block, orientation and vector
+__global__ void __launch_bounds__(128) k_dg_x(const DgXBlock* __restrict__ blocks, int nblk, const double* xv,
+                                              long long xs, unsigned char* arena, long long xbytes, int* scales) {
+  const DgXBlock B = blocks[blockIdx.x];
+  const double* X = xv + (long long)blockIdx.y * xs + B.src;
+  unsigned char* img = arena + (long long)blockIdx.y * xbytes + (long long)B.off * 128;
+  const int n = B.rows * B.cols;
+  __shared__ int red[4];
+  int mx = 0;
+  for (int e = threadIdx.x; e < n; e += 128) mx = max(mx, __double2hiint(X[e]) & 0x7fffffff);
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
+  __syncthreads();
+  mx = max(max(red[0], red[1]), max(red[2], red[3]));
+  if (threadIdx.x == 0) scales[(long long)blockIdx.y * nblk + blockIdx.x] = mx >= DG_EMAX ? IM_SLOW : im_scale(mx);
+  im_rows<IM_NX>(X, B.rows, B.cols, B.sr, B.sc, (B.rows + 15) / 16 * 2, img);  // GEMM1 takes X in pairs of row groups
+}
+
+// ---- planning on the device: distinct operands by a hash table of (address,
+// stored transposed), image offsets by atomic addition (their order does not
+// matter), then one record per product ---------------------------------------
+struct DgPlanState {
+  unsigned long long units;  // 128-byte units of the operator arena used so far
+  unsigned long long xunits;
+  int njobs, nx, fail, pad;
+};
+
+__device__ __forceinline__ unsigned im_hash(unsigned long long k) {
+  k ^= k >> 33;
+  k *= 0xff51afd7ed558ccdull;
+  k ^= k >> 33;
+  return (unsigned)k;
+}
+
+__device__ __forceinline__ unsigned long long im_key(const Task& t, int side) {
+  return (unsigned long long)(uintptr_t)(side ? t.R : t.L) | ((t.flags & (side ? TF_RT : TF_LT)) ? 1ull : 0ull);
+}
+
+constexpr int IM_PROBES = 64;
+
+__global__ void k_dg_find(const Task* __restrict__ tasks, const Group* __restrict__ groups,
+                          const unsigned char* __restrict__ aside, unsigned long long* keys, int* slot_job,
+                          unsigned mask, DgImage* jobs, int max_jobs, int* xtab, unsigned long long xtab_n, DgXBlock* xblocks,
+                          int max_x, DgPlanState* st) {
+  const Group G = groups[blockIdx.x];
+  const int bl = aside[blockIdx.x];
+  for (int ti = G.t0 + threadIdx.x; ti < G.t1; ti += blockDim.x) {
+    const Task t = tasks[ti];
+    if ((t.flags & (TF_XV | TF_XT | TF_XI)) != TF_XV || 2ull * (size_t)t.X >= xtab_n) {  // not a product on the vector
+      st->fail = 1;
+      continue;
+    }
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+      if (t.flags & (side ? TF_RI : TF_LI)) continue;
+      const unsigned long long key = im_key(t, side);
+      unsigned h = im_hash(key) & mask;
+      int p = 0;
+      for (; p < IM_PROBES; ++p, h = (h + 1) & mask) {
+        unsigned long long old = keys[h];
+        if (old == key) break;
+        if (old != 0) continue;
+        old = atomicCAS(&keys[h], 0ull, key);
+        if (old == key) break;
+        if (old != 0) continue;
+        const int j = atomicAdd(&st->njobs, 1);
+        if (j >= max_jobs) {
+          st->fail = 1;
+          break;
+        }
+        DgImage J;
+        J.src = side ? t.R : t.L;
+        J.rows = side ? t.r : t.q;
+        J.cols = side ? t.n : t.m;
+        const bool tr = (t.flags & (side ? TF_RT : TF_LT)) != 0;
+        J.sr = tr ? 1 : J.cols;
+        J.sc = tr ? J.rows : 1;
+        J.off = (uint32_t)atomicAdd(&st->units, (unsigned long long)(im_bytes(J.rows, J.cols) / 128));
+        J.slow = 0;
+        jobs[j] = J;
+        slot_job[h] = j;
+        break;
+      }
+      if (p == IM_PROBES) st->fail = 1;
+    }
+    // the vector block in the orientation (k, l) of this tile; a block that
+    // stands in A's place is needed the other way round
+    const int o = ((t.flags & (bl ? TF_LI : TF_RI)) && !(t.flags & (bl ? TF_RI : TF_LI))) ? 1 - bl : bl;
+    int* slot = xtab + 2 * (long long)(size_t)t.X + o;
+    if (*slot == 0 && atomicCAS(slot, 0, -1) == 0) {
+      const int j = atomicAdd(&st->nx, 1);
+      if (j >= max_x) {
+        st->fail = 1;
+        continue;
+      }
+      DgXBlock B;
+      B.src = (long long)(size_t)t.X;
+      B.rows = o ? t.n : t.m;
+      B.cols = o ? t.m : t.n;
+      B.sr = o ? 1 : t.n;
+      B.sc = o ? t.n : 1;
+      B.off = (uint32_t)atomicAdd(&st->xunits, (unsigned long long)((im_head((B.rows + 15) / 16 * 16) + (B.rows + 15) / 16 * 2 * im_oct(B.cols) * IM_XUNIT) / 128));
+      B.pad = 0;
+      xblocks[j] = B;
+      *slot = j + 1;
+    }
+  }
+}
+
+__global__ void k_dg_records(const Task* __restrict__ tasks, const Group* __restrict__ groups,
+                             const unsigned char* __restrict__ aside, const unsigned long long* __restrict__ keys,
+                             const int* __restrict__ slot_job, unsigned mask, const DgImage* __restrict__ jobs,
+                             const int* __restrict__ xtab, const DgXBlock* __restrict__ xblocks, DgRec* recs,
+                             DgPlanState* st) {
+  const Group G = groups[blockIdx.x];
+  const int bl = aside[blockIdx.x];
+  for (int ti = G.t0 + threadIdx.x; ti < G.t1; ti += blockDim.x) {
+    const Task t = tasks[ti];
+    DgRec r;
+    r.a = r.b = 0;
+    r.f = 0;
+    r.pad = 0;
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+      const bool is_a = (side == 0) == (bl != 0);
+      if (t.flags & (side ? TF_RI : TF_LI)) {
+        r.f |= is_a ? 1 : 2;
+        continue;
+      }
+      const unsigned long long key = im_key(t, side);
+      unsigned h = im_hash(key) & mask;
+      int p = 0;
+      while (p < IM_PROBES && keys[h] != key) {
+        h = (h + 1) & mask;
+        ++p;
+      }
+      if (p == IM_PROBES) {
+        st->fail = 1;
+        continue;
+      }
+      const DgImage J = jobs[slot_job[h]];
+      if (J.rows != (side ? t.r : t.q) || J.cols != (side ? t.n : t.m)) st->fail = 1;
+      if (J.slow) r.f |= 4;
+      (is_a ? r.a : r.b) = J.off;
+    }
+    const int o = (r.f & 3) == 1 ? 1 - bl : bl;
+    r.xb = xtab[2 * (long long)(size_t)t.X + o] - 1;
+    const DgXBlock B = xblocks[r.xb];
+    if (B.rows != (o ? t.n : t.m) || B.cols != (o ? t.m : t.n)) st->fail = 1;
+    r.x = B.off;
+    r.alpha = t.alpha;
+    r.K = bl ? t.n : t.m;
+    r.L = bl ? t.m : t.n;
+    recs[ti] = r;
+  }
+}
+
+template <int W_, int NBT_, int LK_, int KM_, int CTAS_>
+struct ImCfg {
+  static constexpr int W = W_, NBT = NBT_, LK = LK_, KM = KM_, CTAS = CTAS_;
+  static constexpr int NT = 32 * W, AR = 16 * W, BR = 8 * NBT;
+  static constexpr int LO = LK / 8, KO = KM / 8;              // octets staged
+  static constexpr int off_x = (AR / 8) * LO * IM_XUNIT;      // X after A (or the vector in its place) in the first slot
+  static constexpr int off_b = off_x + (KM / 8) * LO * IM_XUNIT;
+  static constexpr int off_y = off_b + NBT * KO * IM_UNIT;    // the tile's sums
+  static constexpr int off_e = off_y + AR * BR * 8;           // row scales of A, B and X
+  static constexpr int total = off_e + 4 * (AR + BR + KM);
+  static_assert(CTAS * (total + 1024) <= 228 * 1024, "resident CTAs");
+  static_assert(KM == LK && off_b >= AR * BR * 8, "chunks; the first slot holds a tile of FP64 values");
+};
+
+__device__ __forceinline__ void cp16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+
+// `rows` runs of n 16-byte pieces, a warp per run.  Out of line: the kernel has
+// ten such copies, and inlined they are a third of the code that its warps
+// fetch again for every product.
+template <int W>
+__device__ __noinline__ void im_copy(uint32_t dst, const unsigned char* src, int n, int rows, int sstride, int dstride) {
+  const int warp = W == 1 ? 0 : threadIdx.x >> 5, lane = threadIdx.x & 31;
+  src += (long long)warp * sstride + lane * 16;
+  dst += (uint32_t)(warp * dstride + lane * 16);
+  for (int r = warp; r < rows; r += W) {
+    for (int i = lane; i < n; i += 32) cp16(dst + (uint32_t)(i - lane) * 16, src + (i - lane) * 16);
+    src += (long long)W * sstride;
+    dst += W * dstride;
+  }
+}
+
+template <class C>
+__global__ void __launch_bounds__(C::NT, C::CTAS)
+    k_tasks_im(const DgRec* __restrict__ recs, const Task* __restrict__ tasks, const Group* __restrict__ groups,
+               const Tile* __restrict__ tiles, int tile0, const unsigned char* __restrict__ ops,
+               const unsigned char* __restrict__ xin, long long xbytes, const int* __restrict__ xscale, int nxb,
+               const double* xv, double* yv, long long xs, long long ys, double* part, long long psize, int nv) {
+  constexpr int W = C::W, NBT = C::NBT, LK = C::LK, KM = C::KM, NT = C::NT, LO = C::LO, KO = C::KO;
+  constexpr int KT = KM / 8;
+  extern __shared__ __align__(128) unsigned char sm[];
+  const uint32_t sA = sm_u32(sm), sX = sm_u32(sm + C::off_x), sB = sm_u32(sm + C::off_b);
+  const int* const eA = (const int*)(sm + C::off_e);
+  const int* const eB = eA + C::AR;
+  const int* const eX = eB + C::BR;
+  const uint32_t sEA = sm_u32(eA), sEB = sm_u32(eB), sEX = sm_u32(eX);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
+  const int mj = lane >> 3, mr16 = (lane & 7) * 16;
+  const Tile TL = tiles[tile0 + blockIdx.x / nv];
+  const Group G = groups[TL.g];
+  const int vec = blockIdx.x % nv;
+  const unsigned char* xi = xin + (long long)vec * xbytes;
+  const int* xsc = xscale + (long long)vec * nxb;
+  const bool bl = TL.aside != 0;
+  const int na = bl ? TL.nrows : TL.ncols, nb = bl ? TL.ncols : TL.nrows;
+  const int a0 = bl ? TL.row0 : TL.col0, b0 = bl ? TL.col0 : TL.row0;
+  const int arows = bl ? G.q : G.r, brows = bl ? G.r : G.q;  // rows of the A and B operands
+  const int nbt = (nb + 7) >> 3, arg = (na + 7) >> 3;
+  const bool mine = 16 * warp < na;
+  // Y sits in shared memory, two 16-byte pairs a lane and 8-column tile: four
+  // accesses to some 200 other instructions, which leaves the loop over the
+  // tiles rolled (unrolled over registers its code missed the instruction
+  // cache) and 8 NBT registers free
+  double2* const Ys = (double2*)(sm + C::off_y) + warp * (NBT * 64) + lane;
+  auto sync = [&]() {
+    if (W == 1) __syncwarp();
+    else __syncthreads();
+  };
+  // alpha 2^n; below 2^-1000 only rows of zeros meet rows of zeros
+  auto scale = [](double alpha, int n) { return alpha * __hiloint2double((max(n, -1000) + 1023) << 20, 0); };
+  // the row groups this CTA never copies (a tile of fewer rows than the slot
+  // has) are read by ldmatrix as absent rows: zero once
+  for (int i = tid; i < C::total / 16; i += NT) ((uint4*)sm)[i] = make_uint4(0, 0, 0, 0);
+  sync();
+
+  // row groups rg0 .. rg0 + nrg, octets from o0 (at most mo) of an image with U-byte units
+  auto rows = [&](uint32_t dst, int doct, const unsigned char* img, int img_rows, int cols, int U, int rg0, int nrg, int o0) {
+    const int oc = im_oct(cols), no = min(doct, oc - o0);
+    im_copy<W>(dst, img + im_head(img_rows) + ((long long)rg0 * oc + o0) * U, no * (U / 16), nrg, oc * U, doct * U);
+  };
+  auto scales = [&](uint32_t dst, const unsigned char* img, int row, int groups) {
+    for (int i = tid; i < 2 * groups; i += NT) cp16(dst + i * 16, img + (row + 4 * i) * 4);
+  };
+  // first-slot copy: A (or what stands in its place) and X for chunk (k0, l0)
+  auto load1 = [&](const DgRec& r, int k0, int l0) {
+    const int f = r.f & 3;
+    if (f == 3) return;
+    const unsigned char* ix = xi + (long long)r.x * 128;
+    const unsigned char* ia = f == 1 ? ix : ops + (long long)r.a * 128;  // f == 1: P[a][k] = X^T, rows a of the vector image
+    rows(sA, LO, ia, f == 1 ? (arows + 15) / 16 * 16 : arows, f == 1 ? r.K : r.L, f == 1 ? IM_XUNIT : IM_UNIT, a0 >> 3, arg,
+         (f ? k0 : l0) >> 3);
+    scales(sEA, ia, a0, arg);
+    if (f == 0) {
+      const int kg = ((min(KM, r.K - k0) + 15) >> 4) * 2;
+      rows(sX, LO, ix, (r.K + 15) / 16 * 16, r.L, IM_XUNIT, k0 >> 3, kg, l0 >> 3);
+      scales(sEX, ix, k0, kg);
+    }
+  };
+  // second-slot copy: B (or the vector block in its place, without its last digit), columns from k0
+  auto load2 = [&](const DgRec& r, int k0) {
+    const bool v = (r.f & 3) == 2;
+    const unsigned char* ib = v ? xi + (long long)r.x * 128 : ops + (long long)r.b * 128;
+    if (v) {
+      const int oc = im_oct(r.L), no = min(KO, oc - (k0 >> 3));
+      const unsigned char* u = ib + im_head((brows + 15) / 16 * 16) + ((long long)(b0 >> 3) * oc + (k0 >> 3)) * IM_XUNIT;
+      for (int g = 0; g < nbt; ++g)
+        im_copy<W>(sB + g * KO * IM_UNIT, u + (long long)g * oc * IM_XUNIT, IM_UNIT / 16, no, IM_XUNIT, IM_UNIT);
+    } else {
+      rows(sB, KO, ib, brows, r.K, IM_UNIT, b0 >> 3, nbt, k0 >> 3);
+    }
+    scales(sEB, ib, b0, nbt);
+  };
+
+  DgRec rec, nxt;
+  if (TL.t0 < TL.t1) {
+    nxt = recs[TL.t0];
+    load1(nxt, 0, 0);
+    cp_commit();
+  }
+  for (int ti = TL.t0; ti < TL.t1; ++ti) {
+    rec = nxt;
+    const int ex = xsc[rec.xb];
+    const bool more = ti + 1 < TL.t1;
+    if (more) nxt = recs[ti + 1];
+    const int f = rec.f & 3;
+    if (f == 3 || (rec.f & 4) || ex == IM_SLOW) {
+      // Y += alpha X, or plain FP64 for what the fixed-point form cannot hold
+      const Task tk = tasks[ti];
+      const double* pX = xv + (long long)vec * xs + (long long)(size_t)tk.X;
+      double* D = (double*)sm;
+      cp_wait();
+      sync();
+      for (int e = tid; e < na * nb; e += NT) {
+        const int a = a0 + e / nb, b = b0 + e % nb, i = bl ? a : b, j = bl ? b : a;
+        double s = 0.0;
+        for (int k = (tk.flags & TF_LI) ? i : 0; k < ((tk.flags & TF_LI) ? i + 1 : tk.m); ++k) {
+          double x = 0.0;
+          if (tk.flags & TF_RI) {
+            x = pX[(long long)k * tk.n + j];
+          } else {
+            for (int l = 0; l < tk.n; ++l)
+              x = fma(pX[(long long)k * tk.n + l], (tk.flags & TF_RT) ? tk.R[(long long)l * tk.r + j] : tk.R[(long long)j * tk.n + l], x);
+          }
+          s = (tk.flags & TF_LI) ? x : fma((tk.flags & TF_LT) ? tk.L[(long long)k * tk.q + i] : tk.L[(long long)i * tk.m + k], x, s);
+        }
+        D[e] = s;
+      }
+      sync();
+      if (mine)
+        for (int b = 0; b < nbt; ++b)
+          for (int h = 0; h < 2; ++h) {
+            const int a = 16 * warp + g + 8 * h, c = 8 * b + 2 * t;
+            double2 v = Ys[(2 * b + h) * 32];
+            if (a < na && c < nb) v.x = fma(rec.alpha, D[a * nb + c], v.x);
+            if (a < na && c + 1 < nb) v.y = fma(rec.alpha, D[a * nb + c + 1], v.y);
+            Ys[(2 * b + h) * 32] = v;
+          }
+      sync();
+      // D lay over the first slot: clear what it held, the images leave absent row groups alone
+      for (int i = tid; i < C::off_b / 16; i += NT) ((uint4*)sm)[i] = make_uint4(0, 0, 0, 0);
+      sync();
+      if (more) load1(nxt, 0, 0);
+      cp_commit();
+      continue;
+    }
+    const int K = f == 2 ? rec.L : rec.K, L = rec.L;
+    int hsh = 0;
+    while ((32 << hsh) < L) ++hsh;
+    for (int k0 = 0; k0 < K; k0 += KM) {
+      const int kc = min(KM, K - k0);
+      uint32_t tf[KT / 2][IM_NX][4];
+      double s0 = 0.0, s1 = 0.0;
+      cp_wait();
+      sync();  // the first slot is in, the second is free
+      load2(rec, k0);
+      cp_commit();
+      if (f == 0) {
+        long long T[KT][4];
+#pragma unroll
+        for (int b = 0; b < KT; ++b)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) T[b][e] = 0;
+        for (int l0 = 0; l0 < L; l0 += LK) {
+          const int lc = min(LK, L - l0);
+          if (l0) {
+            sync();
+            load1(rec, k0, l0);
+            cp_commit();
+            cp_wait();
+            sync();
+          }
+          if (!mine) continue;
+#pragma unroll
+          for (int kp = 0; kp < KT / 2; ++kp) {
+            if (16 * kp >= kc) break;
+            float acc[2][DG_S][4];
+#pragma unroll
+            for (int h = 0; h < LK / 16; ++h) {
+              if (h > 0 && 16 * h >= lc) break;
+              uint32_t xf[IM_NX][4];
+              const uint32_t xa = sX + (uint32_t)(((2 * kp + (mj >> 1)) * LO + 2 * h + (mj & 1)) * IM_XUNIT + mr16);
+#pragma unroll
+              for (int j = 0; j < IM_NX; ++j) ldsm4(xf[j], xa + j * 128);
+              const uint32_t aa = sA + (uint32_t)(((2 * warp + (mj & 1)) * LO + 2 * h + (mj >> 1)) * IM_UNIT + mr16);
+#pragma unroll
+              for (int i = 0; i < DG_N; ++i) {
+                uint32_t af[4];
+                ldsm4(af, aa + i * 128);
+#pragma unroll
+                for (int j = 0; i + j < DG_S; ++j) {
+                  if (h == 0 && i == 0) {
+                    mma_first(acc[0][i + j], af, xf[j][0], xf[j][1]);
+                    mma_first(acc[1][i + j], af, xf[j][2], xf[j][3]);
+                  } else {
+                    mma_acc(acc[0][i + j], af, xf[j][0], xf[j][1]);
+                    mma_acc(acc[1][i + j], af, xf[j][2], xf[j][3]);
+                  }
+                }
+              }
+            }
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                const long long v = dg_join<true>(acc[c][0][e], acc[c][1][e], acc[c][2][e], acc[c][3][e], acc[c][4][e],
+                                            acc[c][5][e], acc[c][6][e], acc[c][7][e]);
+                T[2 * kp + c][e] += hsh ? v >> hsh : v;
+              }
+          }
+        }
+        if (mine) {
+          // normalise T per row over the chunk: row k lies eX[k] below the block's scale ex
+          int m0 = 0, m1 = 0, dx[KT][2];
+#pragma unroll
+          for (int b = 0; b < KT; ++b) {
+#pragma unroll
+            for (int e = 0; e < 2; ++e) dx[b][e] = min(ex - eX[8 * b + 2 * t + e], 63);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const int h = (int)(T[b][e] >> 32), ah = (h ^ (h >> 31)) >> min(dx[b][e & 1], 31);
+              if (e < 2) m0 = max(m0, ah);
+              else m1 = max(m1, ah);
+            }
+          }
+#pragma unroll
+          for (int s = 1; s < 4; s <<= 1) {
+            m0 = max(m0, __shfl_xor_sync(0xffffffffu, m0, s));
+            m1 = max(m1, __shfl_xor_sync(0xffffffffu, m1, s));
+          }
+          const int z0 = __clz(m0 + (m0 >> 7) + 1) - 1, z1 = __clz(m1 + (m1 >> 7) + 1) - 1;
+          auto bias = [](long long v, int s) {  // v 2^s, 0x80 in every byte
+            return (unsigned long long)((long long)((unsigned long long)v << max(s, 0)) >> max(-s, 0)) + 0x8080808080808080ull;
+          };
+#pragma unroll
+          for (int kk = 0; kk < KT / 2; ++kk)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const int b = 2 * kk + (q >> 1), e = 2 * (q & 1), z = q & 1 ? z1 : z0;
+              const unsigned long long v0 = bias(T[b][e], z - dx[b][0]), v1 = bias(T[b][e + 1], z - dx[b][1]);
+              const uint32_t h0 = (uint32_t)(v0 >> 32), l0_ = (uint32_t)v0, h1 = (uint32_t)(v1 >> 32), l1_ = (uint32_t)v1;
+              tf[kk][0][q] = digit2<0>(h0, l0_, h1, l1_);
+              tf[kk][1][q] = digit2<1>(h0, l0_, h1, l1_);
+              tf[kk][2][q] = digit2<2>(h0, l0_, h1, l1_);
+              tf[kk][3][q] = digit2<3>(h0, l0_, h1, l1_);
+              tf[kk][4][q] = digit2<4>(h0, l0_, h1, l1_);
+              tf[kk][5][q] = digit2<5>(h0, l0_, h1, l1_);
+              tf[kk][6][q] = digit2<6>(h0, l0_, h1, l1_);
+              tf[kk][7][q] = digit2<7>(h0, l0_, h1, l1_);
+            }
+          const int base = ex - 1022 - 1022 - 57 + 63 - 57 + hsh;  // scales of X and A, of T's sums, of Y's
+          s0 = scale(rec.alpha, eA[16 * warp + g] + base - z0);
+          s1 = scale(rec.alpha, eA[16 * warp + g + 8] + base - z1);
+        }
+      } else if (mine) {
+#pragma unroll
+        for (int kk = 0; kk < KT / 2; ++kk)
+#pragma unroll
+          for (int i = 0; i < IM_NX; ++i) {
+            const uint32_t at = (uint32_t)(((2 * warp + (mj & 1)) * LO + 2 * kk + (mj >> 1)) * (f == 1 ? IM_XUNIT : IM_UNIT) + i * 128 + mr16);
+            if (i < DG_N || f == 1) ldsm4(tf[kk][i], sA + at);
+            else tf[kk][i][0] = tf[kk][i][1] = tf[kk][i][2] = tf[kk][i][3] = 0u;
+          }
+        s0 = scale(rec.alpha, eA[16 * warp + g] - 1022 - 57);
+        s1 = scale(rec.alpha, eA[16 * warp + g + 8] - 1022 - 57);
+      }
+      cp_wait();
+      sync();  // the second slot is in, the first is free
+      if (k0 + KM < K) load1(rec, k0 + KM, 0);
+      else if (more) load1(nxt, 0, 0);
+      cp_commit();
+      if (!mine) continue;
+#pragma unroll 1
+      for (int b = 0; b < nbt; ++b) {
+        float acc[DG_S][4];
+        uint32_t bf[DG_N][4];
+        const uint32_t ba = sB + (uint32_t)((b * KO + (KT == 4 ? mj : (mj & 1))) * IM_UNIT + mr16);
+#pragma unroll
+        for (int j = 0; j < DG_N; ++j) ldsm4(bf[j], ba + j * 128);
+#pragma unroll
+        for (int i = 0; i < IM_NX; ++i)
+#pragma unroll
+          for (int j = 0; j < DG_N && i + j < DG_S; ++j) {
+            if (i == 0 || (i == 1 && j == DG_N - 1)) mma_first(acc[i + j], tf[0][i], bf[j][0], bf[j][1]);
+            else mma_acc(acc[i + j], tf[0][i], bf[j][0], bf[j][1]);
+          }
+        if (KT == 4 && kc > 16) {
+#pragma unroll
+          for (int i = 0; i < IM_NX; ++i)
+#pragma unroll
+            for (int j = 0; j < DG_N && i + j < DG_S; ++j) mma_acc(acc[i + j], tf[KT / 2 - 1][i], bf[j][2], bf[j][3]);
+        }
+        const int2 eb = *(const int2*)(eB + 8 * b + 2 * t);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          double2 v = Ys[(2 * b + h) * 32];
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            const int e = 2 * h + c;
+            const long long j = dg_join<false>(acc[0][e], acc[1][e], acc[2][e], acc[3][e], acc[4][e], acc[5][e], acc[6][e], acc[7][e]);
+            double& o = c ? v.y : v.x;
+            o = fma(dg_double(j, (c ? eb.y : eb.x) + 63), h ? s1 : s0, o);
+          }
+          Ys[(2 * b + h) * 32] = v;
+        }
+      }
+    }
+  }
+  cp_wait();
+
+  double* Y = yv + (long long)vec * ys + G.yoff;
+  double* P = TL.poff >= 0 ? part + (long long)vec * psize + TL.poff : nullptr;  // split piece
+  if (mine)
+    for (int b = 0; b < nbt; ++b)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int a = 16 * warp + g + 8 * (e >> 1), c = 8 * b + 2 * t + (e & 1);
+        if (a >= na || c >= nb) continue;
+        const double2 v = Ys[(2 * b + (e >> 1)) * 32];
+        const int i = bl ? a : c, j = bl ? c : a;
+        if (P) P[i * TL.ncols + j] = e & 1 ? v.y : v.x;
+        else Y[(long long)(TL.row0 + i) * G.r + TL.col0 + j] = e & 1 ? v.y : v.x;
+      }
+}
+
+// residency: 12 CTAs of one warp (168 registers), 4 of two and 2 of four (shared
+// memory: digits of both operands' chunks and the sums)
+using ImS = ImCfg<1, 2, 16, 16, 12>;
+using ImM = ImCfg<2, 4, 32, 32, 4>;
+using ImL = ImCfg<4, 8, 32, 32, 2>;
+
+using DgS = DgCfg<1, 2, 16, 16, 12>;
+using DgM = DgCfg<2, 4, 32, 32, 4>;
+using DgL = DgCfg<4, 8, 64, 32, 2>;
+static_assert(DgS::CTAS == kDgClass[0].ctas && DgM::CTAS == kDgClass[1].ctas && DgL::CTAS == kDgClass[2].ctas &&
+                  DgS::AR == kDgClass[0].a && DgM::AR == kDgClass[1].a && DgL::AR == kDgClass[2].a &&
+                  DgS::BR == kDgClass[0].b && DgM::BR == kDgClass[1].b && DgL::BR == kDgClass[2].b &&
+                  DgS::LK == kDgClass[0].lk && DgM::LK == kDgClass[1].lk && DgL::LK == kDgClass[2].lk &&
+                  DgS::KM == kDgClass[0].km && DgM::KM == kDgClass[1].km && DgL::KM == kDgClass[2].km,
+              "the classes the host plans with");
+
+template <class C>
+void launch_one(unsigned grid, cudaStream_t s, const Task* tasks, const Group* groups, const Tile* tiles, int tile0,
+                const double* xv, double* yv, long long xs, long long ys, double* part, long long psize, int nv) {
+  k_tasks_dg<C><<<grid, C::NT, C::total, s>>>(tasks, groups, tiles, tile0, xv, yv, xs, ys, part, psize, nv);
+}
+
+
+template <class C>
+void launch_im(unsigned grid, cudaStream_t s, const DgRec* recs, const Task* tasks, const Group* groups,
+               const Tile* tiles, int tile0, const unsigned char* ops, const unsigned char* x, long long xbytes,
+               const int* xscale, int nx, const double* xv, double* yv, long long xs, long long ys, double* part,
+               long long psize, int nv) {
+  k_tasks_im<C><<<grid, C::NT, C::total, s>>>(recs, tasks, groups, tiles, tile0, ops, x, xbytes, xscale, nx, xv, yv, xs,
+                                               ys, part, psize, nv);
+}
+
+struct DgPlan {
+  void* mem = nullptr;  // records, operator images and vector blocks
+  DgRec* recs = nullptr;
+  unsigned char* ops = nullptr;
+  DgXBlock* xblocks = nullptr;
+  int nx = 0;
+  unsigned char* x = nullptr;  // vector images, xbytes a vector, then their blocks' scales
+  long long xbytes = 0;
+  int* xscale = nullptr;  // nx a vector
+  int x_nvec = 0;
+};
+
+template <class T>
+T* carve(unsigned char*& p, long long n) {
+  T* r = (T*)p;
+  p += ((long long)sizeof(T) * n + 255) / 256 * 256;
+  return r;
+}
+
+}  // namespace
+
+void release_digit_plan(void* p) {
+  DgPlan* P = (DgPlan*)p;
+  if (!P) return;
+  if (P->mem) dfree(P->mem);
+  if (P->x) dfree(P->x);
+  delete P;
+}
+
+// The plan of a list that is kept on the device: its images and records, made
+// on the device in three launches.  Images are made only where they leave at
+// least half of the memory that neither the step's own plan nor anything else
+// has a claim to; without them the kernel above cuts its operands itself.
+bool prepare_digits(CudaBackend& be, const TaskList& tl, DevList& d, int nvec, long long length) {
+  if (d.dg_none || !be.ok()) return false;
+  DgPlan* P = (DgPlan*)d.dg;
+  if (P && P->x_nvec >= nvec) return true;
+  const long long avail = std::min(be.mem_limit() - be.mem_used(), be.mem_free()) - be.last_step_bytes;
+  if (!P) {
+    d.dg_none = true;  // until it is made
+    const long long nt = (long long)tl.tasks.size(), ng = (long long)tl.groups.size();
+    if (nt == 0 || ng == 0 || length <= 0) return false;
+    P = new DgPlan();
+    const int max_x = (int)(4 * ng + 4096);
+    bool made = false;
+    // a table of a quarter of the products' count holds the operators of a
+    // long list many times over; a larger one is tried if it does not
+    for (long long want = std::max(nt / 4, 4096LL); !made; want *= 8) {
+      unsigned cap = 4096;
+      while (cap < want && cap < (1u << 30)) cap <<= 1;
+      const int max_jobs = (int)(cap / 2);
+      const long long bytes = 12LL * cap + (long long)sizeof(DgImage) * max_jobs + 8 * length +
+                              (long long)sizeof(DgXBlock) * max_x + ng + 8192;
+      if (bytes + nt * (long long)sizeof(DgRec) > avail / 2) break;
+      // small tables stay for the next list, large ones go back
+      const bool keep = bytes <= (16LL << 20);
+      unsigned char* tmp = nullptr;
+      if (keep) tmp = (unsigned char*)be.scratch(16 << 20, 4);
+      else if (dmalloc(&tmp, bytes) != cudaSuccess) cudaGetLastError();
+      if (!tmp) break;
+      unsigned char* p = tmp;
+      DgPlanState* st = carve<DgPlanState>(p, 1);
+      unsigned long long* keys = carve<unsigned long long>(p, cap);
+      int* xtab = carve<int>(p, 2 * length);
+      const size_t zero = p - tmp;
+      int* slot = carve<int>(p, cap);
+      DgImage* jobs = carve<DgImage>(p, max_jobs);
+      DgXBlock* xb = carve<DgXBlock>(p, max_x);
+      unsigned char* aside = carve<unsigned char>(p, ng);
+      be.note(cudaMemsetAsync(tmp, 0, zero, be.stream()), "digit plan");
+      be.note(cudaMemcpyAsync(aside, d.dg_aside.data(), ng, cudaMemcpyHostToDevice, be.stream()), "digit plan");
+      k_dg_find<<<(unsigned)ng, 128, 0, be.stream()>>>(d.tasks, d.groups, aside, keys, slot, cap - 1, jobs, max_jobs, xtab,
+                                                       2ull * length, xb, max_x, st);
+      be.launches++;
+      be.note(cudaGetLastError(), "k_dg_find");
+      DgPlanState h{};
+      auto state = [&]() {
+        be.note(cudaMemcpyAsync(&h, st, sizeof(h), cudaMemcpyDeviceToHost, be.stream()), "digit plan");
+        be.note(cudaStreamSynchronize(be.stream()), "digit plan");
+        return be.ok() && !h.fail;
+      };
+      bool again = false;
+      if (!state()) {
+        again = be.ok() && want < 4 * nt;
+      } else {
+        const long long total = (long long)h.units * 128 + (long long)sizeof(DgRec) * nt +
+                                (long long)sizeof(DgXBlock) * h.nx + 1024;
+        if (total <= avail / 2 && dmalloc(&P->mem, total) == cudaSuccess) {
+          unsigned char* q = (unsigned char*)P->mem;
+          P->ops = carve<unsigned char>(q, (long long)h.units * 128);
+          P->recs = carve<DgRec>(q, nt);
+          P->xblocks = carve<DgXBlock>(q, h.nx);
+          if (h.njobs > 0) k_dg_ops<<<(unsigned)h.njobs, 128, 0, be.stream()>>>(jobs, P->ops);
+          k_dg_records<<<(unsigned)ng, 128, 0, be.stream()>>>(d.tasks, d.groups, aside, keys, slot, cap - 1, jobs, xtab, xb,
+                                                              P->recs, st);
+          be.launches += 2;
+          be.note(cudaGetLastError(), "digit images");
+          be.note(cudaMemcpyAsync(P->xblocks, xb, sizeof(DgXBlock) * h.nx, cudaMemcpyDeviceToDevice, be.stream()), "digit plan");
+          made = state();
+          P->nx = h.nx;
+          P->xbytes = (long long)h.xunits * 128;
+        } else {
+          cudaGetLastError();
+        }
+      }
+      if (!keep) dfree(tmp);
+      if (!again) break;
+    }
+    if (!made) {
+      release_digit_plan(P);
+      return false;
+    }
+    d.dg = P;
+    d.dg_none = false;
+  }
+  if (P->x) {
+    be.free_graphs(d);  // graphs captured with the smaller images would write through freed pointers
+    cudaStreamSynchronize(be.stream());
+    dfree(P->x);
+  }
+  P->x = nullptr;
+  P->x_nvec = 0;
+  const long long bytes = (P->xbytes + 4LL * P->nx + 512) * nvec;
+  if (bytes > avail / 2 || dmalloc(&P->x, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    d.dg_none = true;
+    return false;
+  }
+  P->xscale = (int*)(P->x + P->xbytes * nvec);
+  P->x_nvec = nvec;
+  return true;
+}
+
+// the vectors' digits, ahead of the product kernels
+void enqueue_digit_vectors(CudaBackend& be, const DevList& d, const double* xv, long long xs, int nvec) {
+  const DgPlan* P = (const DgPlan*)d.dg;
+  if (!P || P->nx == 0) return;
+  k_dg_x<<<dim3(P->nx, nvec), 128, 0, be.stream()>>>(P->xblocks, P->nx, xv, xs, P->x, P->xbytes, P->xscale);
+  be.launches++;
+  be.note(cudaGetLastError(), "k_dg_x");
+}
+
+// more than 48 KB of dynamic shared memory is asked for once, outside any capture
+cudaError_t fp64_digits_init() {
+  auto set = [](const void* f, int bytes) {
+    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  };
+  cudaError_t e = set((const void*)k_tasks_dg<DgL>, DgL::total);
+  if (e == cudaSuccess) e = set((const void*)k_tasks_im<ImM>, ImM::total);
+  if (e == cudaSuccess) e = set((const void*)k_tasks_im<ImL>, ImL::total);
+  return e;
+}
+
+// one class of tiles: from the list's images if it has a plan, else from its operands
+void launch_fp64_digits(int cls, unsigned grid, cudaStream_t s, const void* plan, const Task* tasks,
+                        const Group* groups, const Tile* tiles, int tile0, const double* xv, double* yv, long long xs,
+                        long long ys, double* part, long long psize, int nv) {
+  if (const DgPlan* P = (const DgPlan*)plan) {
+    auto f = cls == 0 ? launch_im<ImS> : cls == 1 ? launch_im<ImM> : launch_im<ImL>;
+    f(grid, s, P->recs, tasks, groups, tiles, tile0, P->ops, P->x, P->xbytes, P->xscale, P->nx, xv, yv, xs, ys, part,
+      psize, nv);
+  } else {
+    auto f = cls == 0 ? launch_one<DgS> : cls == 1 ? launch_one<DgM> : launch_one<DgL>;
+    f(grid, s, tasks, groups, tiles, tile0, xv, yv, xs, ys, part, psize, nv);
+  }
+}
+
+}  // namespace tns

@@ -4,7 +4,8 @@
 //     Y_tile = sum_{tasks of the tile's output block} alpha * op(L) op(X) op(R)^T
 // One CTA owns one output tile (<= 64 x 64) of one output block and walks
 // that block's task list in a fixed order, so every run is bitwise
-// reproducible and no atomics are needed.  The position sum of Eq. (2) (and
+// reproducible and no atomics are needed (the other FP64 path, on the tensor
+// cores, is fp64_digits.cu).  The position sum of Eq. (2) (and
 // the sum over all operator pairs and dot blocks that hit the block) is the
 // K loop of the accumulation, as in Alg. 2 where the sum over i becomes the
 // inner dimension of one GEMM.  Each task is evaluated in the cheaper chain
@@ -941,6 +942,7 @@ CudaBackend::CudaBackend(int device, cudaStream_t s, bool own) : device_(device)
   const char* k = std::getenv("TNS_FP64_KERNEL");
   if (k && std::strcmp(k, "dfma") == 0) fp64_kernel = 0;
   if (k && std::strcmp(k, "dmma") == 0) fp64_kernel = 1;
+  if (k && std::strcmp(k, "digits") == 0) fp64_kernel = 2;
   const char* w = std::getenv("TNS_TC_WAIT_NS");
   if (w && *w) tc_wait_ns = std::strtoull(w, nullptr, 10);
   const char* tv = std::getenv("TNS_TC_VARIANT");
@@ -1030,7 +1032,7 @@ long long CudaBackend::step_bytes(const TaskList& tl, long long psi_length) {
     if (!(t.flags & TF_RI) && seenR.insert((uintptr_t)t.R ^ ((t.flags & TF_RT) ? 1u : 0u)).second) b += pad(t.r, t.n);
   }
   // + split-K partial tiles and scratch
-  return b + psi_length * 8LL * 120 + (1LL << 30);
+  return last_step_bytes = b + psi_length * 8LL * 120 + (1LL << 30);
 }
 
 long long CudaBackend::mem_used() { return dmem(device_).used; }
@@ -1138,12 +1140,14 @@ void CudaBackend::free_list(DevList& d) {
   if (d.tasks) dfree(d.tasks);
   if (d.groups) dfree(d.groups);
   if (d.wtiles) dfree(d.wtiles);
-  for (FpVariant& f : d.fv) {
-    if (f.tiles) dfree(f.tiles);
-    if (f.reds) dfree(f.reds);
-    if (f.part) dfree(f.part);
-  }
+  for (auto& fv : d.fv)
+    for (FpVariant& f : fv) {
+      if (f.tiles) dfree(f.tiles);
+      if (f.reds) dfree(f.reds);
+      if (f.part) dfree(f.part);
+    }
   if (d.tc) release_tc_plan(d.tc);
+  if (d.dg) release_digit_plan(d.dg);
   d = DevList();
 }
 
@@ -1187,6 +1191,7 @@ void CudaBackend::upload_list(const TaskList& tl, DevList& d) {
         t.ncols = std::min(DM_WC, G.r - c0);
         t.t0 = G.t0;
         t.t1 = G.t1;
+        t.aside = 0;
         t.poff = -1;
         wt.push_back(t);
       }
@@ -1216,11 +1221,9 @@ static std::vector<std::pair<int, int>> cut_extent(int len, int mx) {
 // FP64 output tiles of every group: tall or wide, whichever executes fewer
 // FMAs over the group's products (fixed overhead per product and tile
 // included), each tile in the smallest class it fits
-static void fp64_tiles(const TaskList& tl, DevList& d) {
-  for (int c = 0; c < kFpClasses; ++c) {
-    d.fp_tiles[c].clear();
-    d.fp_cost[c].clear();
-  }
+static void dfma_tiles(const TaskList& tl, DevList& d) {
+  std::vector<Tile>* const tiles = d.fp_tiles[0];
+  std::vector<double>* const cost = d.fp_cost[0];
   for (int g = 0; g < (int)tl.groups.size(); ++g) {
     const Group& G = tl.groups[g];
     if (G.q <= 0 || G.r <= 0) continue;
@@ -1248,6 +1251,7 @@ static void fp64_tiles(const TaskList& tl, DevList& d) {
         t.ncols = cc.second;
         t.t0 = G.t0;
         t.t1 = G.t1;
+        t.aside = 0;
         t.poff = -1;
         double w = 0;
         for (int k = G.t0; k < G.t1; ++k) w += (double)tile_fmas(tl.tasks[k], t.nrows, t.ncols, nullptr) + kTaskOverhead;
@@ -1255,19 +1259,117 @@ static void fp64_tiles(const TaskList& tl, DevList& d) {
                       : (t.nrows <= C1_TR && t.ncols <= C1_TC) ? 1
                       : (t.ncols <= C2_TC)                     ? 2
                                                                : 3;
-        d.fp_tiles[c].push_back(t);
-        d.fp_cost[c].push_back(w);
+        tiles[c].push_back(t);
+        cost[c].push_back(w);
       }
   }
-  d.fp_tiled = true;
+  d.fp_tiled[0] = true;
+}
+
+// Estimated time of one product on an a x b tile of a digit-kernel class, in
+// clocks of one SM whose resident CTAs share it: its MMAs (34 digit pairs, 8
+// clocks each on one of four tensor cores), the cutting of T (and, without
+// images, of the operands), the joining of sums into Y, and a fixed part per
+// staged chunk.  Only ratios matter: they decide classes, sides and splits.
+static double dg_cost(int cls, const Task& t, int aside, int a, int b, bool images) {
+  const DgClass& c = kDgClass[cls];
+  const int K = aside ? t.n : t.m, L = aside ? t.m : t.n;
+  auto up = [](int x, int m) { return (double)((x + m - 1) / m * m); };
+  const double ap = up(a, 16), bp = up(b, 8);
+  const double ovh0[kDgClasses] = {300.0, 700.0, 1300.0}, ovh1[kDgClasses] = {150.0, 400.0, 800.0};
+  const double ovh = images ? ovh1[cls] : ovh0[cls], mm = 34.0 * 8.0 / 2048.0, cut = images ? 0.0 : 1.7;
+  const int lk = images ? c.km : c.lk;
+  const bool ai = (t.flags & (aside ? TF_LI : TF_RI)) != 0, bi = (t.flags & (aside ? TF_RI : TF_LI)) != 0;
+  if (ai && bi) return ovh + a * b / 4.0;
+  if (ai || bi || (t.flags & TF_XI)) {
+    const double kk = up(ai ? K : L, 16), ch = std::ceil(kk / c.km);
+    return ovh * ch + 0.25 * (ap * bp * kk * mm + cut * kk * (ap + bp) + 4.0 * ap * bp * ch);
+  }
+  const double kp = up(K, 16), lp = up(L, 16), ch = std::ceil(kp / c.km), lch = std::ceil((double)L / lk);
+  return ovh * ch * (1.0 + 0.5 * (lch - 1)) +
+         0.25 * (mm * ap * kp * (lp + bp) + cut * (kp * lp + bp * kp + ap * lp * (lch > 1 ? ch : 1.0)) +
+                 2.4 * ap * kp * lch + 4.0 * ap * bp * ch);
+}
+
+// cut an extent into near-equal parts of at most mx, at multiples of 8 (the row groups of images)
+static std::vector<std::pair<int, int>> cut8(int len, int mx) {
+  std::vector<std::pair<int, int>> out;
+  for (auto& p : cut_extent((len + 7) / 8, mx / 8)) out.push_back({8 * p.first, std::min(8 * p.second, len - 8 * p.first)});
+  return out;
+}
+
+// digit-kernel tiles of every group: the class and the side that is
+// contracted with X first, whichever costs least over the group's products
+// (summed over their distinct shapes)
+static void dg_tiles(const TaskList& tl, DevList& d) {
+  const bool images = tl.persistent;
+  d.dg_aside.assign(tl.groups.size(), 0);
+  struct Shape {
+    int m, n, f, count;
+    const Task* t;
+  };
+  std::vector<Shape> sh;
+  for (int g = 0; g < (int)tl.groups.size(); ++g) {
+    const Group& G = tl.groups[g];
+    if (G.q <= 0 || G.r <= 0) continue;
+    sh.clear();
+    size_t last = 0;
+    for (int i = G.t0; i < G.t1; ++i) {
+      const Task& t = tl.tasks[i];
+      const int f = t.flags & (TF_LI | TF_RI | TF_XI);
+      auto same = [&](const Shape& s) { return s.m == t.m && s.n == t.n && s.f == f; };
+      if (last >= sh.size() || !same(sh[last])) {
+        for (last = 0; last < sh.size() && !same(sh[last]); ++last) {
+        }
+        if (last == sh.size()) sh.push_back({t.m, t.n, f, 0, &t});
+      }
+      ++sh[last].count;
+    }
+    double best = -1;
+    int pc = 0, pa = 0;
+    for (int c = 0; c < kDgClasses; ++c)
+      for (int s = 0; s < 2; ++s) {
+        const int ea = s ? G.q : G.r, eb = s ? G.r : G.q;
+        const int na = (ea + kDgClass[c].a - 1) / kDgClass[c].a, nb = (eb + kDgClass[c].b - 1) / kDgClass[c].b;
+        double w = 0;
+        for (const Shape& x : sh) w += x.count * dg_cost(c, *x.t, s, (ea + na - 1) / na, (eb + nb - 1) / nb, images);
+        w *= (double)na * nb;
+        if (best < 0 || w < best) {
+          best = w;
+          pc = c;
+          pa = s;
+        }
+      }
+    d.dg_aside[g] = (unsigned char)pa;
+    const auto ra = cut8(pa ? G.q : G.r, kDgClass[pc].a), rb = cut8(pa ? G.r : G.q, kDgClass[pc].b);
+    for (auto& aa : ra)
+      for (auto& bb : rb) {
+        const auto &rr = pa ? aa : bb, &cc = pa ? bb : aa;
+        Tile t;
+        t.g = g;
+        t.row0 = rr.first;
+        t.col0 = cc.first;
+        t.nrows = rr.second;
+        t.ncols = cc.second;
+        t.t0 = G.t0;
+        t.t1 = G.t1;
+        t.aside = pa;
+        t.poff = -1;
+        double w = 0;
+        for (const Shape& x : sh) w += x.count * dg_cost(pc, *x.t, pa, aa.second, bb.second, images);
+        d.fp_tiles[1][pc].push_back(t);
+        d.fp_cost[1][pc].push_back(w);
+      }
+  }
+  d.fp_tiled[1] = true;
 }
 
 // schedule variant v of the FP64 kernels: the tiles of each class, a tile
 // whose task list is long cut into pieces of similar cost (split-K), each
 // written to a partial tile and summed afterwards in piece order, so that
 // every class fills the GPU and no CTA walks a much longer list than the rest
-void CudaBackend::plan_variant(const TaskList& tl, DevList& d, int v) {
-  FpVariant& f = d.fv[v];
+void CudaBackend::plan_variant(const TaskList& tl, DevList& d, int dig, int v) {
+  FpVariant& f = d.fv[dig][v];
   if (f.planned) return;
   // kernel attribute once, outside any stream capture: the wide class needs
   // more than 48 KB of dynamic shared memory
@@ -1276,18 +1378,27 @@ void CudaBackend::plan_variant(const TaskList& tl, DevList& d, int v) {
     note(cudaFuncSetAttribute(k_tasks_fp64<C3_NT, C3_ACC, C3_TR, C3_TC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               fp64_smem(C3_TR, C3_TC)),
          "k_tasks_fp64 shared memory");
+    note(fp64_digits_init(), "k_tasks_dg shared memory");
     attr = true;
   }
-  if (!d.fp_tiled) fp64_tiles(tl, d);
+  const bool digits = dig != 0;
+  if (!d.fp_tiled[dig]) {
+    if (digits) dg_tiles(tl, d);
+    else dfma_tiles(tl, d);
+  }
+  const std::vector<Tile>* const ctiles = d.fp_tiles[dig];
+  const std::vector<double>* const ccost = d.fp_cost[dig];
   double ctot[kFpClasses] = {0, 0, 0, 0};
   for (int c = 0; c < kFpClasses; ++c)
-    for (double w : d.fp_cost[c]) ctot[c] += w;
+    for (double w : ccost[c]) ctot[c] += w;
   // resident CTAs per SM of each class (registers) x SMs x rounds
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device_);
   const double rounds = kRounds[v];
-  const double slots[kFpClasses] = {16.0 * sms * rounds, 4.0 * sms * rounds, 2.0 * sms * rounds,
-                                    2.0 * sms * rounds};
+  const double ctas[kFpClasses] = {digits ? (double)kDgClass[0].ctas : 16.0, digits ? (double)kDgClass[1].ctas : 4.0,
+                                   digits ? (double)kDgClass[2].ctas : 2.0, 2.0};
+  double slots[kFpClasses];
+  for (int c = 0; c < kFpClasses; ++c) slots[c] = ctas[c] * sms * rounds;
   std::vector<Tile> all;
   std::vector<SplitRed> reds;
   long long poff = 0;
@@ -1296,9 +1407,9 @@ void CudaBackend::plan_variant(const TaskList& tl, DevList& d, int v) {
     int count = 0;
     const size_t first = all.size();
     std::vector<double> pcost;  // estimated cost of each piece of this class
-    for (size_t i = 0; i < d.fp_tiles[c].size(); ++i) {
-      const Tile t = d.fp_tiles[c][i];
-      const double tc = d.fp_cost[c][i];
+    for (size_t i = 0; i < ctiles[c].size(); ++i) {
+      const Tile t = ctiles[c][i];
+      const double tc = ccost[c][i];
       const int ntask = t.t1 - t.t0;
       int ns = (int)std::min<double>(ntask, std::ceil(tc / target));
       ns = std::max(1, std::min(ns, 64));
@@ -1312,7 +1423,9 @@ void CudaBackend::plan_variant(const TaskList& tl, DevList& d, int v) {
       std::vector<double> kc(ntask);
       double tot = 0;
       for (int k = t.t0; k < t.t1; ++k)
-        tot += kc[k - t.t0] = (double)tile_fmas(tl.tasks[k], t.nrows, t.ncols, nullptr) + kTaskOverhead;
+        tot += kc[k - t.t0] =
+            digits ? dg_cost(c, tl.tasks[k], t.aside, t.aside ? t.nrows : t.ncols, t.aside ? t.ncols : t.nrows, tl.persistent)
+                   : (double)tile_fmas(tl.tasks[k], t.nrows, t.ncols, nullptr) + kTaskOverhead;
       SplitRed R;
       R.g = t.g;
       R.row0 = t.row0;
@@ -1405,15 +1518,17 @@ void CudaBackend::drop(const TaskList& tl) {
   }
 }
 
-void CudaBackend::enqueue_fp64(const DevList& d, int v, const double* xv, double* yv, int nvec, long long xs,
+void CudaBackend::enqueue_fp64(const DevList& d, int dig, int v, const double* xv, double* yv, int nvec, long long xs,
                                long long ys) {
   if (!ok()) return;
-  const FpVariant& f = d.fv[v];
+  const FpVariant& f = d.fv[dig][v];
   // the classes write disjoint tiles and partial tiles: the costliest class
   // runs on the launching stream and the others on forked streams beside it
   // (they fill its tail), joined before the split reduction
   int order[kFpClasses] = {0, 1, 2, 3};
   std::stable_sort(order, order + kFpClasses, [&](int a, int b) { return f.ccost[a] > f.ccost[b]; });
+  const void* plan = dig && !d.dg_none ? d.dg : nullptr;
+  if (plan) enqueue_digit_vectors(*this, d, xv, xs, nvec);
   const int nact = (f.ncls[0] > 0) + (f.ncls[1] > 0) + (f.ncls[2] > 0) + (f.ncls[3] > 0);
   const bool fork = nact > 1 && fork_ready();
   if (fork) {
@@ -1434,7 +1549,9 @@ void CudaBackend::enqueue_fp64(const DevList& d, int v, const double* xv, double
     cudaStream_t s = stream_;
     if (fork && oi > 0) s = fstream_[side++];
     const int t0 = tbeg[c];
-    if (c == 0)
+    if (dig)
+      launch_fp64_digits(c, grid, s, plan, d.tasks, d.groups, f.tiles, t0, xv, yv, xs, ys, f.part, f.psize, nvec);
+    else if (c == 0)
       k_tasks_fp64<C0_NT, C0_ACC, C0_TR, C0_TC><<<grid, C0_NT, fp64_smem(C0_TR, C0_TC), s>>>(
           d.tasks, d.groups, f.tiles, t0, xv, yv, xs, ys, f.part, f.psize, nvec);
     else if (c == 1)
@@ -1447,7 +1564,7 @@ void CudaBackend::enqueue_fp64(const DevList& d, int v, const double* xv, double
       k_tasks_fp64<C3_NT, C3_ACC, C3_TR, C3_TC><<<grid, C3_NT, fp64_smem(C3_TR, C3_TC), s>>>(
           d.tasks, d.groups, f.tiles, t0, xv, yv, xs, ys, f.part, f.psize, nvec);
     launches++;
-    note(cudaGetLastError(), "k_tasks_fp64");
+    note(cudaGetLastError(), dig ? "k_tasks_dg" : "k_tasks_fp64");
   }
   if (fork) {
     for (int i = 0; i < 3; ++i) {
@@ -1531,6 +1648,11 @@ void CudaBackend::run(const TaskList& tl, const double* xv, double* yv, int nvec
                       int precision) {
   if (!ok()) return;
   if (tl.groups.empty()) return;
+  // the FP64 kernel: the one asked for, else digits where the list and the call allow them
+  const int fk = fp64_kernel >= 0 ? fp64_kernel : (precision == 0 && tl.digits) ? 2 : 0;
+  const int dig = fk == 2 ? 1 : 0;
+  const int code = precision;  // tuned schedules and graphs are kept per code and vector count
+  if (precision == kFp64Fma) precision = 0;
   if (!tl.persistent) {
     // one-off list (rotations, truncation products): default schedule, direct launches
     DevList tmp;
@@ -1540,7 +1662,7 @@ void CudaBackend::run(const TaskList& tl, const double* xv, double* yv, int nvec
         enqueue_tasks_tc(*this, tmp, xv, yv, nvec, xs, ys, precision, 1);
         check_tasks_tc(*this, tmp);
       }
-    } else if (fp64_kernel == 1) {
+    } else if (fk == 1) {
       if (tmp.nwtiles > 0) {
         dim3 grid((tmp.nwtiles + DM_WARPS - 1) / DM_WARPS, nvec);
         k_tasks_dmma<<<grid, 32 * DM_WARPS, 0, stream_>>>(tmp.tasks, tmp.groups, tmp.wtiles, tmp.nwtiles, xv, yv, xs,
@@ -1549,15 +1671,16 @@ void CudaBackend::run(const TaskList& tl, const double* xv, double* yv, int nvec
         note(cudaGetLastError(), "k_tasks_dmma");
       }
     } else {
-      plan_variant(tl, tmp, 1);
-      if (ok() && tmp.tasks && tmp.groups && ensure_part(tmp, tmp.fv[1], nvec)) enqueue_fp64(tmp, 1, xv, yv, nvec, xs, ys);
+      plan_variant(tl, tmp, dig, 1);
+      if (ok() && tmp.tasks && tmp.groups && ensure_part(tmp, tmp.fv[dig][1], nvec))
+        enqueue_fp64(tmp, dig, 1, xv, yv, nvec, xs, ys);
     }
     free_list(tmp);
     return;
   }
   DevList& d = dev(tl);
   if (!ok() || !d.tasks || !d.groups) return;
-  if (precision == 0 && fp64_kernel == 1) {
+  if (precision == 0 && fk == 1) {
     if (d.nwtiles > 0) {
       dim3 grid((d.nwtiles + DM_WARPS - 1) / DM_WARPS, nvec);
       k_tasks_dmma<<<grid, 32 * DM_WARPS, 0, stream_>>>(d.tasks, d.groups, d.wtiles, d.nwtiles, xv, yv, xs, ys);
@@ -1569,7 +1692,7 @@ void CudaBackend::run(const TaskList& tl, const double* xv, double* yv, int nvec
   // online autotuner: after one untimed product, the next products of this
   // (precision, nvec) use run the schedule variants in turn, timed with
   // events; the variant with the fastest sample is kept
-  const int key = (iterating ? kSteadyKey : 0) + precision * 64 + nvec;
+  const int key = (iterating ? kSteadyKey : 0) + code * 64 + nvec;
   Tune& tu = d.tune[key];
   if (!autotune && tu.best < 0) tu.best = 1;
   const int nvar = precision != 0 ? kNumVariants : kFp64Variants;
@@ -1588,14 +1711,15 @@ void CudaBackend::run(const TaskList& tl, const double* xv, double* yv, int nvec
   if (precision != 0) {
     if (!prepare_tasks_tc(*this, tl, d, nvec, v, precision)) return;
   } else {
-    plan_variant(tl, d, v);
-    if (!ok() || !ensure_part(d, d.fv[v], nvec)) return;
+    plan_variant(tl, d, dig, v);
+    if (!ok() || !ensure_part(d, d.fv[dig][v], nvec)) return;
+    if (dig) prepare_digits(*this, tl, d, nvec, xs);
   }
   auto enqueue = [&](const double* x, double* y) {
     if (precision != 0)
       enqueue_tasks_tc(*this, d, x, y, nvec, xs, ys, precision, v);
     else
-      enqueue_fp64(d, v, x, y, nvec, xs, ys);
+      enqueue_fp64(d, dig, v, x, y, nvec, xs, ys);
   };
   if (tuning && !timing) {
     enqueue(xv, yv);

@@ -163,11 +163,13 @@ int davidson(Engine& E, CudaBackend& be, double* X, double tol, int max_iter, in
   };
   const int lowp = precision != 0;
   // nv products in one launch (the block of Davidson vectors shares every
-  // operator block read)
+  // operator block read).  FP64 products keep the FMA order: the iterates are
+  // continued from them, and far from convergence (a preconditioner with poles
+  // inside the spectrum) a rounding at another place ends in another vector
   auto matvec = [&](const double* in, double* out, int nv, int prec) {
     Timer tm(be.stream());
     be.iterating = true;
-    be.run(st.heff, in, out, nv, n, n, prec);
+    be.run(st.heff, in, out, nv, n, n, prec == 0 ? kFp64Fma : prec);
     be.iterating = false;
     float ms = tm.stop();
     if (acc) {
