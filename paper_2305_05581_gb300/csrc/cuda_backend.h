@@ -175,6 +175,7 @@ class CudaBackend : public Backend {
   void upload(double* dst, const double* src, long long n) override;
   void download(double* dst, const double* src, long long n) override;
   void zero(double* p, long long n) override;
+  void copy(double* dst, const double* src, long long n) override;
   void lincomb(const LCList& l) override;
   void run(const TaskList& tl, const double* xv, double* yv, int nvec, long long xs, long long ys,
            int precision) override;

@@ -132,6 +132,7 @@ static QN dq_of(int kind, int i, int j) {
 // engine basics
 // ---------------------------------------------------------------------------
 Engine::~Engine() {
+  drop_adjoint();
   for (auto& c : Lcat_) free_cat(c);
   for (auto& c : Rcat_) free_cat(c);
   free_side(step_.L);
@@ -1602,6 +1603,7 @@ void Engine::rotation_tasks(const Side& S, const Catalogue& src, const Catalogue
 // the two catalogues of step k on the device (a previous step's partial sums
 // and work list are released first, so that they leave room)
 int Engine::ensure_step(int k, std::string& err) {
+  if (!step_.valid || step_.k != k) drop_adjoint();
   if (step_.valid && step_.k != k) {
     be_->forget(step_.heff);
     be_->forget(step_.heff_full);
@@ -2040,6 +2042,7 @@ int Engine::refresh_step(std::string& err) {
 }
 
 int Engine::prepare_step(int k, std::string& err) {
+  drop_adjoint();
   be_->forget(step_.heff);  // the device copy of the previous step's work list
   be_->forget(step_.heff_full);
   be_->forget(step_.heff_part);
@@ -2258,9 +2261,6 @@ int Engine::heff_part(const double* X, double* Y, int nvec, int precision, int p
 // to the catalogue operators of its terms (adjoint of the linear combination).
 // ---------------------------------------------------------------------------
 namespace {
-struct AdjTarget {
-  std::vector<Task> tasks;
-};
 Task adj_task(double a, const double* P, int pf, const double* M, int mf, const double* S, int sf, int q, int m, int n,
               int r) {
   Task t;
@@ -2281,125 +2281,139 @@ int lflags_T(int f) { return (f & TF_LI) ? TF_LI : ((f & TF_LT) ? 0 : TF_LT); }
 int rflags_T(int f) { return (f & TF_RI) ? TF_RI : ((f & TF_RT) ? 0 : TF_RT); }
 }  // namespace
 
-int Engine::heff_adjoint(const double* X, const double* Yb, double* Xb, double* Lb, double* Rb, std::string& err) {
-  if (!step_.valid) {
-    err = "heff_adjoint: call build_env first";
-    return -2;
+void Engine::drop_adjoint() {
+  AdjointPlan& P = adj_;
+  for (TaskList* tl : {&P.xbar, &P.side[0].direct, &P.side[0].partial, &P.side[0].sum, &P.side[1].direct,
+                       &P.side[1].partial, &P.side[1].sum}) {
+    be_->forget(*tl);
+    tl->clear();
   }
+  for (double** p : {&P.x, &P.yb, &P.side[0].G, &P.side[0].M, &P.side[1].G, &P.side[1].M}) {
+    if (*p) be_->release(*p);
+    *p = nullptr;
+  }
+  P.gen = -1;
+  P.have[0] = P.have[1] = P.have[2] = false;
+}
+
+// The work lists of the adjoint for the wanted outputs, on fixed copies of X
+// and Ybar, so that they hold for every call of the step: making them (one
+// product per product of the step and output) takes the host several times
+// as long as running them (13 orbitals, D = 160: 9 of 12 ms).
+int Engine::adjoint_plan(const bool want[3], std::string& err) {
   Step& st = step_;
-  const int k = st.k;
-  Catalogue& Lc = Lcat_[k];
-  Catalogue& Rc = Rcat_[k + 2];
+  AdjointPlan& P = adj_;
   const TaskList& fw = st.heff_full;
-  const long long nL = Lc.size, nR = Rc.size, nML = st.L.size, nMR = st.R.size;
-  // temporaries: direct gradients of catalogue blocks and of materialised blocks
-  double* GL = Lb ? be_->alloc(std::max(nL, 1LL)) : nullptr;
-  double* GR = Rb ? be_->alloc(std::max(nR, 1LL)) : nullptr;
-  double* ML = (Lb && nML) ? be_->alloc(nML) : nullptr;
-  double* MR = (Rb && nMR) ? be_->alloc(nMR) : nullptr;
-  if ((Lb && !GL) || (Rb && !GR) || (Lb && nML && !ML) || (Rb && nMR && !MR)) {
+  if (P.gen != fw.gen) drop_adjoint();
+  P.gen = fw.gen;
+  Catalogue* const cats[2] = {&Lcat_[st.k], &Rcat_[st.k + 2]};
+  Side* const sides[2] = {&st.L, &st.R};
+  auto get = [&](double*& p, long long n) {
+    if (!p) p = be_->alloc(std::max(n, 1LL));
+    return p != nullptr;
+  };
+  bool good = get(P.x, st.length) && get(P.yb, st.length);
+  for (int s = 0; s < 2; ++s)
+    if (want[1 + s]) good = good && get(P.side[s].G, cats[s]->size) && (sides[s]->size == 0 || get(P.side[s].M, sides[s]->size));
+  if (!good) {
     err = "heff_adjoint: device allocation failed";
-    for (double* p : {GL, GR, ML, MR})
-      if (p) be_->release(p);
+    drop_adjoint();
     return -3;
   }
-  // target maps: block pointer -> list of tasks
-  std::map<const double*, std::vector<Task>> tx, tl_, tr_;
+  bool make[3];
+  for (int i = 0; i < 3; ++i) make[i] = want[i] && !P.have[i];
+  if (!make[0] && !make[1] && !make[2]) return 0;
+  // products by the block they contribute to
+  std::unordered_map<const double*, std::vector<Task>> tx, ts[2];
   for (size_t g = 0; g < fw.groups.size(); ++g) {
     const Group& G = fw.groups[g];
-    const double* yb = Yb + G.yoff;
+    const double* yb = P.yb + G.yoff;
     for (int i = G.t0; i < G.t1; ++i) {
       const Task& t = fw.tasks[i];
-      const PsiBlock& xbk = st.psi[t.pad];
-      const double* xblk = X + xbk.off;
+      const double* xblk = P.x + st.psi[t.pad].off;
       const int lf = t.flags & (TF_LI | TF_LT), rf = t.flags & (TF_RI | TF_RT);
       const int q = t.q, m = t.m, n = t.n, r = t.r;
-      if (Xb) {  // Xb (m x n) += a op(L)^T Yb op(R)
-        tx[Xb + xbk.off].push_back(adj_task(t.alpha, t.L, lflags_T(lf), yb, 0, t.R, rflags_T(rf), m, q, r, n));
-      }
-      if (Lb && !(t.flags & TF_LI)) {
+      if (make[0])  // Xb (m x n) += a op(L)^T Yb op(R)
+        tx[xblk].push_back(adj_task(t.alpha, t.L, lflags_T(lf), yb, 0, t.R, rflags_T(rf), m, q, r, n));
+      if (make[1] && !(t.flags & TF_LI)) {
         const int mfR = (t.flags & TF_RI) ? TF_XI : ((t.flags & TF_RT) ? TF_XT : 0);
         if (!(t.flags & TF_LT))  // L (q x m) += a Yb op(R) op(X)^T
-          tl_[t.L].push_back(adj_task(t.alpha, yb, 0, t.R, mfR, xblk, 0, q, r, n, m));
+          ts[0][t.L].push_back(adj_task(t.alpha, yb, 0, t.R, mfR, xblk, 0, q, r, n, m));
         else  // L stored (m x q) += a op(X) op(R)^T Yb^T
-          tl_[t.L].push_back(adj_task(t.alpha, xblk, 0, t.R, (t.flags & TF_RI) ? TF_XI : ((t.flags & TF_RT) ? 0 : TF_XT),
-                                      yb, 0, m, n, r, q));
+          ts[0][t.L].push_back(adj_task(t.alpha, xblk, 0, t.R, (t.flags & TF_RI) ? TF_XI : ((t.flags & TF_RT) ? 0 : TF_XT),
+                                        yb, 0, m, n, r, q));
       }
-      if (Rb && !(t.flags & TF_RI)) {
+      if (make[2] && !(t.flags & TF_RI)) {
         if (!(t.flags & TF_RT))  // R (r x n) += a Yb^T op(L) op(X)
-          tr_[t.R].push_back(adj_task(t.alpha, yb, TF_LT, t.L,
-                                      (t.flags & TF_LI) ? TF_XI : ((t.flags & TF_LT) ? TF_XT : 0), xblk, TF_RT, r, q,
-                                      m, n));
+          ts[1][t.R].push_back(adj_task(t.alpha, yb, TF_LT, t.L,
+                                        (t.flags & TF_LI) ? TF_XI : ((t.flags & TF_LT) ? TF_XT : 0), xblk, TF_RT, r, q,
+                                        m, n));
         else  // R stored (n x r) += a op(X)^T op(L)^T Yb
-          tr_[t.R].push_back(adj_task(t.alpha, xblk, TF_LT, t.L,
-                                      (t.flags & TF_LI) ? TF_XI : ((t.flags & TF_LT) ? 0 : TF_XT), yb, TF_RT, n, m, q,
-                                      r));
+          ts[1][t.R].push_back(adj_task(t.alpha, xblk, TF_LT, t.L,
+                                        (t.flags & TF_LI) ? TF_XI : ((t.flags & TF_LT) ? 0 : TF_XT), yb, TF_RT, n, m, q,
+                                        r));
       }
     }
   }
-  auto run_map = [&](std::map<const double*, std::vector<Task>>& mp, double* outbase, const double* srcbase,
-                     long long srcsize, const std::vector<std::pair<long long, std::pair<int, int>>>& blocks) {
-    // groups: every block of [srcbase, srcbase+srcsize) listed in `blocks` (offset, (rows, cols))
-    TaskList tl;
-    tl.digits = true;
-    for (auto& b : blocks) {
+  // a list with one group per block (offset, rows, cols), overwritten by its products
+  struct Blk {
+    long long off;
+    int rows, cols;
+  };
+  auto list = [](TaskList& tl, const std::vector<Blk>& blocks, auto&& products) {
+    tl.clear();
+    tl.persistent = tl.digits = true;
+    for (const Blk& b : blocks) {
       Group g;
-      g.yoff = b.first;
-      g.q = b.second.first;
-      g.r = b.second.second;
+      g.yoff = b.off;
+      g.q = g.nrows = b.rows;
+      g.r = g.ncols = b.cols;
       g.row0 = g.col0 = 0;
-      g.nrows = g.q;
-      g.ncols = g.r;
       g.t0 = (int)tl.tasks.size();
-      auto it = mp.find(srcbase + b.first);
-      if (it != mp.end())
-        for (auto& t : it->second) tl.tasks.push_back(t);
+      if (const std::vector<Task>* v = products(b.off)) tl.tasks.insert(tl.tasks.end(), v->begin(), v->end());
       g.t1 = (int)tl.tasks.size();
       tl.groups.push_back(g);
     }
-    (void)srcsize;
-    be_->run(tl, nullptr, outbase, 1, 0, 0, 0);
   };
-  auto cat_blocks = [&](const Catalogue& c) {
-    std::vector<std::pair<long long, std::pair<int, int>>> v;
-    for (auto& o : c.ops) {
-      const Layout& L = c.layouts[o.layout];
-      for (size_t b = 0; b < L.in.size(); ++b)
-        v.push_back({o.off + L.off[b], {c.basis.dim[L.out[b]], c.basis.dim[L.in[b]]}});
-    }
-    return v;
+  auto of = [](std::unordered_map<const double*, std::vector<Task>>& mp, const double* base) {
+    return [&mp, base](long long off) -> const std::vector<Task>* {
+      auto it = mp.find(base + off);
+      return it == mp.end() ? nullptr : &it->second;
+    };
   };
-  auto mat_blocks = [&](const Side& s, const Catalogue& c) {
-    std::vector<std::pair<long long, std::pair<int, int>>> v;
-    for (auto& mt : s.mats) {
-      const Layout& L = c.layouts[mt.layout];
-      for (size_t b = 0; b < L.in.size(); ++b)
-        v.push_back({mt.off + L.off[b], {c.basis.dim[L.out[b]], c.basis.dim[L.in[b]]}});
-    }
-    return v;
-  };
-  if (Xb) {
-    std::vector<std::pair<long long, std::pair<int, int>>> v;
-    for (auto& p : st.psi) v.push_back({p.off, {p.m, p.n}});
-    run_map(tx, Xb, Xb, st.length, v);
+  if (make[0]) {
+    std::vector<Blk> v;
+    for (auto& p : st.psi) v.push_back({p.off, p.m, p.n});
+    list(P.xbar, v, of(tx, P.x));
+    P.have[0] = true;
   }
-  // second phase: catalogue gradient = direct part + adjoint of the partial sums
-  auto finish = [&](Side& S, Catalogue& C, double* G, double* M, double* out, std::map<const double*, std::vector<Task>>& mp) {
-    const auto cb = cat_blocks(C);
-    run_map(mp, G, C.d, C.size, cb);
-    if (M) run_map(mp, M, S.d, S.size, mat_blocks(S, C));
-    be_->sync();
-    std::map<long long, std::vector<Task>> add;  // target offset -> tasks
-    for (auto& b : cb)
-      add[b.first].push_back(adj_task(1.0, nullptr, TF_LI, G + b.first, 0, nullptr, TF_RI, b.second.first,
-                                      b.second.first, b.second.second, b.second.second));
+  for (int s = 0; s < 2; ++s) {
+    if (!make[1 + s]) continue;
+    AdjointSide& A = P.side[s];
+    const Catalogue& C = *cats[s];
+    const Side& S = *sides[s];
     const Basis& bs = C.basis;
+    std::vector<Blk> cb, mb;
+    for (auto& o : C.ops) {
+      const Layout& L = C.layouts[o.layout];
+      for (size_t b = 0; b < L.in.size(); ++b) cb.push_back({o.off + L.off[b], bs.dim[L.out[b]], bs.dim[L.in[b]]});
+    }
+    for (auto& mt : S.mats) {
+      const Layout& L = C.layouts[mt.layout];
+      for (size_t b = 0; b < L.in.size(); ++b) mb.push_back({mt.off + L.off[b], bs.dim[L.out[b]], bs.dim[L.in[b]]});
+    }
+    list(A.direct, cb, of(ts[s], C.d));
+    if (A.M) list(A.partial, mb, of(ts[s], S.d));
+    // catalogue gradient = direct part + adjoint of the partial sums
+    std::unordered_map<long long, std::vector<Task>> add;  // target offset -> products
+    for (auto& b : cb)
+      add[b.off].push_back(adj_task(1.0, nullptr, TF_LI, A.G + b.off, 0, nullptr, TF_RI, b.rows, b.rows, b.cols, b.cols));
     for (auto& mt : S.mats) {
       const Expr& x = S.exprs[mt.expr];
       const Layout& L = C.layouts[mt.layout];
       for (size_t b = 0; b < L.in.size(); ++b) {
         const int in = L.in[b], out = L.out[b];
-        const double* mb = M + mt.off + L.off[b];
+        const double* m = A.M + mt.off + L.off[b];
         for (auto& tm : x.t) {
           if (tm.op < 0) continue;
           const double sign = tm.par == 1 ? sgn_n(bs.q[in].n) : tm.par == 2 ? sgn_n(bs.q[out].n) : 1.0;
@@ -2409,34 +2423,52 @@ int Engine::heff_adjoint(const double* X, const double* Yb, double* Xb, double* 
           if (ob < 0) continue;
           if (tm.tr && OL.out[ob] != in) continue;
           if (!tm.tr && OL.out[ob] != out) continue;
-          const long long toff = o.off + OL.off[ob];
           const int tr = bs.dim[OL.out[ob]], tc = bs.dim[OL.in[ob]];
-          add[toff].push_back(adj_task(tm.c * sign, nullptr, TF_LI, mb, tm.tr ? TF_XT : 0, nullptr, TF_RI, tr, tr, tc, tc));
+          add[o.off + OL.off[ob]].push_back(
+              adj_task(tm.c * sign, nullptr, TF_LI, m, tm.tr ? TF_XT : 0, nullptr, TF_RI, tr, tr, tc, tc));
         }
       }
     }
-    TaskList tl;
-    for (auto& b : cb) {
-      Group g;
-      g.yoff = b.first;
-      g.q = b.second.first;
-      g.r = b.second.second;
-      g.row0 = g.col0 = 0;
-      g.nrows = g.q;
-      g.ncols = g.r;
-      g.t0 = (int)tl.tasks.size();
-      for (auto& t : add[b.first]) tl.tasks.push_back(t);
-      g.t1 = (int)tl.tasks.size();
-      tl.groups.push_back(g);
-    }
-    be_->run(tl, nullptr, out, 1, 0, 0, 0);
-  };
-  if (Lb) finish(st.L, Lc, GL, ML, Lb, tl_);
-  if (Rb) finish(st.R, Rc, GR, MR, Rb, tr_);
+    list(A.sum, cb, [&](long long off) -> const std::vector<Task>* { return &add[off]; });
+    A.sum.digits = false;  // sums of blocks
+    P.have[1 + s] = true;
+  }
+  return 0;
+}
+
+int Engine::heff_adjoint(const double* X, const double* Yb, double* Xb, double* Lb, double* Rb, std::string& err) {
+  if (!step_.valid) {
+    err = "heff_adjoint: call build_env first";
+    return -2;
+  }
+  const bool want[3] = {Xb != nullptr, Lb != nullptr, Rb != nullptr};
+  int rc = adjoint_plan(want, err);
+  if (rc) return rc;
+  AdjointPlan& P = adj_;
+  be_->copy(P.x, X, step_.length);
+  be_->copy(P.yb, Yb, step_.length);
+  if (Xb) be_->run(P.xbar, nullptr, Xb, 1, 0, 0, 0);
+  double* const out[2] = {Lb, Rb};
+  for (int s = 0; s < 2; ++s) {
+    if (!out[s]) continue;
+    AdjointSide& A = P.side[s];
+    be_->run(A.direct, nullptr, A.G, 1, 0, 0, 0);
+    if (A.M) be_->run(A.partial, nullptr, A.M, 1, 0, 0, 0);
+    be_->run(A.sum, nullptr, out[s], 1, 0, 0, 0);
+  }
   be_->sync();
-  for (double* p : {GL, GR, ML, MR})
-    if (p) be_->release(p);
   std::string e = be_->error();
+  // the lists and buffers stay for the step's next call where they take little
+  // of the memory that is left, and go back at once otherwise
+  long long bytes = 8 * (2 * step_.length);
+  for (int s = 0; s < 2; ++s) {
+    if (P.side[s].G) bytes += 8 * (s ? Rcat_[step_.k + 2].size : Lcat_[step_.k].size);
+    if (P.side[s].M) bytes += 8 * (s ? step_.R.size : step_.L.size);
+    bytes += (long long)sizeof(Task) * 3 / 2 * (long long)(P.side[s].direct.tasks.size() + P.side[s].partial.tasks.size() + P.side[s].sum.tasks.size());
+  }
+  bytes += (long long)sizeof(Task) * 3 / 2 * (long long)P.xbar.tasks.size();
+  const long long limit = be_->mem_limit();
+  if (!e.empty() || (limit > 0 && bytes * 16 > std::min(limit - be_->mem_used(), be_->mem_free()))) drop_adjoint();
   if (!e.empty()) {
     err = e;
     return -6;

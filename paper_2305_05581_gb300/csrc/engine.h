@@ -333,6 +333,11 @@ struct Backend {
   virtual void upload(double* dst, const double* src, long long n) = 0;
   virtual void download(double* dst, const double* src, long long n) = 0;
   virtual void zero(double* p, long long n) = 0;
+  virtual void copy(double* dst, const double* src, long long n) {  // within backend memory
+    std::vector<double> h((size_t)n);
+    download(h.data(), src, n);
+    upload(dst, h.data(), n);
+  }
   virtual void lincomb(const LCList& l) = 0;
   // run a task list: each group's output (tile) is overwritten with the sum of
   // its tasks.  xv/yv: bases for TF_XV offsets and group yoff.
@@ -426,6 +431,19 @@ struct Step {
   std::vector<int> diag_tasks;  // tasks contributing to the diagonal, in group order
   std::vector<int> diag_rng;    // per group: range [diag_rng[g], diag_rng[g+1]) of diag_tasks
   bool valid = false;
+};
+
+// work lists of heff_adjoint, kept for the step whose full list has this gen
+struct AdjointSide {
+  TaskList direct, partial, sum;  // gradients of the catalogue's and the partial sums' blocks, and their sum
+  double *G = nullptr, *M = nullptr;  // the first two lists' results
+};
+struct AdjointPlan {
+  long long gen = -1;
+  bool have[3] = {false, false, false};  // Xbar, left, right
+  double *x = nullptr, *yb = nullptr;    // copies of X and Ybar that the lists read
+  TaskList xbar;
+  AdjointSide side[2];
 };
 
 // two-site wavefunction layout: blocks (ql, s1, s2, qr) ordered by (ql, s1, s2, qr)
@@ -540,6 +558,9 @@ class Engine {
   std::vector<Catalogue> Lcat_;  // Lcat_[k]: orbitals 0..k-1
   std::vector<Catalogue> Rcat_;  // Rcat_[k]: orbitals k..N-1
   Step step_;
+  AdjointPlan adj_;
+  void drop_adjoint();
+  int adjoint_plan(const bool want[3], std::string& err);
   // catalogue staging: the position of the current work (eviction order is
   // the distance from it: the catalogue needed last leaves first), the
   // catalogues in use (never moved), pinned host memory in use and budget

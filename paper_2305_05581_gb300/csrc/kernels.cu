@@ -1087,6 +1087,10 @@ void CudaBackend::download(double* dst, const double* src, long long n) {
 
 void CudaBackend::zero(double* p, long long n) { note(cudaMemsetAsync(p, 0, (size_t)n * 8, stream_), "zero"); }
 
+void CudaBackend::copy(double* dst, const double* src, long long n) {
+  note(cudaMemcpyAsync(dst, src, (size_t)n * 8, cudaMemcpyDeviceToDevice, stream_), "copy");
+}
+
 void CudaBackend::sync() { note(cudaStreamSynchronize(stream_), "sync"); }
 
 void* CudaBackend::scratch(size_t bytes, int slot) {
@@ -1298,11 +1302,16 @@ static std::vector<std::pair<int, int>> cut8(int len, int mx) {
   return out;
 }
 
+// lists of products on vectors that are kept get digit images
+static bool digit_images(const TaskList& tl) {
+  return tl.persistent && !tl.tasks.empty() && (tl.tasks[0].flags & TF_XV);
+}
+
 // digit-kernel tiles of every group: the class and the side that is
 // contracted with X first, whichever costs least over the group's products
 // (summed over their distinct shapes)
 static void dg_tiles(const TaskList& tl, DevList& d) {
-  const bool images = tl.persistent;
+  const bool images = digit_images(tl);
   d.dg_aside.assign(tl.groups.size(), 0);
   struct Shape {
     int m, n, f, count;
@@ -1424,7 +1433,7 @@ void CudaBackend::plan_variant(const TaskList& tl, DevList& d, int dig, int v) {
       double tot = 0;
       for (int k = t.t0; k < t.t1; ++k)
         tot += kc[k - t.t0] =
-            digits ? dg_cost(c, tl.tasks[k], t.aside, t.aside ? t.nrows : t.ncols, t.aside ? t.ncols : t.nrows, tl.persistent)
+            digits ? dg_cost(c, tl.tasks[k], t.aside, t.aside ? t.nrows : t.ncols, t.aside ? t.ncols : t.nrows, digit_images(tl))
                    : (double)tile_fmas(tl.tasks[k], t.nrows, t.ncols, nullptr) + kTaskOverhead;
       SplitRed R;
       R.g = t.g;
@@ -1586,7 +1595,7 @@ void CudaBackend::launch_graphed(DevList& d, int key, const double* xv, double* 
   GraphSlot& gs = d.graphs[key];
   if (!gs.exec && !gs.failed) need(2LL * (long long)sizeof(double) * nvec * std::max(xs, ys));
   const long long elems = (long long)nvec * xs;
-  if (!use_graphs || gs.failed || xs != ys) {
+  if (!use_graphs || gs.failed || xs != ys || xs == 0) {  // xs == 0: a list on fixed operands
     enqueue(xv, yv);
     return;
   }
@@ -1648,6 +1657,11 @@ void CudaBackend::run(const TaskList& tl, const double* xv, double* yv, int nvec
                       int precision) {
   if (!ok()) return;
   if (tl.groups.empty()) return;
+  if (tl.tasks.empty()) {  // sums of nothing
+    for (int v = 0; v < nvec; ++v)
+      for (const Group& g : tl.groups) zero(yv + (long long)v * ys + g.yoff, (long long)g.q * g.r);
+    return;
+  }
   // the FP64 kernel: the one asked for, else digits where the list and the call allow them
   const int fk = fp64_kernel >= 0 ? fp64_kernel : (precision == 0 && tl.digits) ? 2 : 0;
   const int dig = fk == 2 ? 1 : 0;
@@ -1694,7 +1708,7 @@ void CudaBackend::run(const TaskList& tl, const double* xv, double* yv, int nvec
   // events; the variant with the fastest sample is kept
   const int key = (iterating ? kSteadyKey : 0) + code * 64 + nvec;
   Tune& tu = d.tune[key];
-  if (!autotune && tu.best < 0) tu.best = 1;
+  if ((!autotune || xs == 0) && tu.best < 0) tu.best = 1;  // xs == 0: a list on fixed operands, run now and then
   const int nvar = precision != 0 ? kNumVariants : kFp64Variants;
   if (precision != 0 && forced_tc_variant >= 0) tu.best = forced_tc_variant;
   const auto ckey = std::make_pair(key, d.shape);
@@ -1713,7 +1727,7 @@ void CudaBackend::run(const TaskList& tl, const double* xv, double* yv, int nvec
   } else {
     plan_variant(tl, d, dig, v);
     if (!ok() || !ensure_part(d, d.fv[dig][v], nvec)) return;
-    if (dig) prepare_digits(*this, tl, d, nvec, xs);
+    if (dig && digit_images(tl)) prepare_digits(*this, tl, d, nvec, xs);
   }
   auto enqueue = [&](const double* x, double* y) {
     if (precision != 0)
