@@ -153,9 +153,10 @@ class CudaBackend : public Backend {
   // bound of one wait inside the tensor-core product loop (ns); the
   // environment variable TNS_TC_WAIT_NS overrides the default 0.2 s when the
   // backend is created (a test makes the waits run out with it and checks the
-  // reported error and that the context stays usable; with 0 every warp of
-  // the small-block kernel first waits on a barrier that nothing completes,
-  // since its copies may land before any wait could run out)
+  // reported error and that the context stays usable; with 0 every CTA of the
+  // tile kernel and every warp of the small-block kernel first waits on a
+  // barrier that nothing completes, since its copies may land before any wait
+  // could run out)
   unsigned long long tc_wait_ns = 200000000ull;
   // TNS_TC_VARIANT=v (0..kNumVariants-1) fixes the tensor-core schedule
   // variant instead of tuning it (tests run each kernel this way)

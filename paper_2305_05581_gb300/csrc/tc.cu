@@ -21,11 +21,11 @@
 // pipe stays out of the product loop.
 //
 // One CTA (256 threads) per output tile piece (128 rows x <= 64 columns);
-// thread 0 issues copies and MMAs from the chunk's product metadata, which
-// all threads stage in shared memory one chunk ahead; GEMM2's first copies
-// are issued while the T pass runs; all threads do the T pass and the
-// epilogue.  Steps of 32 X rows and one staging region shared by the two
-// GEMMs keep a CTA at 56 KB of shared memory, three per SM.
+// warp 0 issues copies (its lanes share them out) and MMAs from the chunk's
+// product metadata, which all threads stage in shared memory one chunk ahead;
+// GEMM1's copies run under the previous step's T pass and GEMM2, GEMM2's under
+// GEMM1; all threads do the T pass and the epilogue.  Steps of 32 X rows and
+// an L region of 18 KB keep a CTA at 75 KB of shared memory, three per SM.
 // Every wait is bounded; a timeout sets a flag the host reads, after the CTA
 // has drained (bounded) its own copies and MMAs and released its TMEM.
 #include <cuda_bf16.h>
@@ -330,14 +330,20 @@ struct TcSmem {
   static constexpr int CB2 = TC_M * CH_BYTES;   // one K chunk of B2 (all 128 rows)
   static constexpr int B2 = TC_MC * ES / CH_BYTES * CB2;  // T^T of all products, K = TC_MC
   static constexpr int A2 = TC_M * CH_BYTES;    // L rows, one K chunk (two buffers)
-  // GEMM1's two operand buffers and GEMM2's two L buffers share one region
-  // (they are never live together: GEMM2's copies start once D1 is
-  // complete, GEMM1's once the previous GEMM2's MMAs are done), which keeps
-  // a CTA at 56 KB (split-BF16) so that three fit on an SM
-  static constexpr int G1 = 2 * NS * (A1 + B1), G2 = 2 * NS * A2;
-  static constexpr int R1 = G1 > G2 ? G1 : G2;
-  static constexpr int total = R1 + NS * B2;
+  // GEMM1's two operand buffers and GEMM2's L slices have regions of their own,
+  // so that the next step's GEMM1 chunks are copied while this step's T pass
+  // and GEMM2 run, and the L slices while GEMM1 does.  The L region holds two
+  // slices of 72 rows (split-BF16) or more smaller ones; with it a CTA takes
+  // 74.8 KB, a third of an SM's shared memory.
+  static constexpr int G1 = 2 * NS * (A1 + B1);
+  static constexpr int LR = 18432;
+  // the L region comes first: an MMA reads 128 rows of A, and the rows past a
+  // shorter slice (whose results no one stores) then lie in the regions behind
+  static constexpr int off_g1 = LR, off_b2 = LR + G1;
+  static constexpr int total = off_b2 + NS * B2;
+  static_assert(LR >= NS * A2 && LR + A2 <= total && TC_CTAS * (total + 1024 + 1024) <= 228 * 1024, "regions");
 };
+constexpr int TC_LB = 4;  // L slices in flight, at most
 
 template <int TF32>
 __global__ void __launch_bounds__(TC_NT, TC_CTAS)
@@ -353,14 +359,14 @@ __global__ void __launch_bounds__(TC_NT, TC_CTAS)
   constexpr int EPC = CH_BYTES / ES;              // elements per K chunk
   constexpr uint32_t SBO_FULL = (CH_BYTES / 16) * 128;
   extern __shared__ __align__(128) unsigned char smem[];
-  unsigned char* const sG1 = smem;                    // GEMM1 operand buffers, or
-  unsigned char* const sA2 = smem;                    // GEMM2 L buffers: buffer b, plane p at + (b * NS + p) * S::A2
-  unsigned char* const sB2 = smem + S::R1;            // planes at + p * S::B2
+  unsigned char* const sL = smem;               // L slices
+  unsigned char* const sG1 = smem + S::off_g1;  // GEMM1 operand buffers
+  unsigned char* const sB2 = smem + S::off_b2;  // planes at + p * S::B2
   auto sA1 = [&](int b) { return sG1 + b * S::NS * (S::A1 + S::B1); };          // plane p at + p * S::A1
   auto sB1 = [&](int b) { return sG1 + b * S::NS * (S::A1 + S::B1) + S::NS * S::A1; };  // plane p at + p * S::B1
-  __shared__ uint64_t lbar1[2], mbar1[2], lbar2[2], mbar2[2];
+  __shared__ uint64_t lbar1[2], mbar1[2], lbar2[TC_LB], mbar2[TC_LB], never;
   __shared__ uint32_t tbase;
-  __shared__ int bad;
+  __shared__ volatile int bad;
   // metadata of the products of a chunk (at most TC_M / 16 share one X
   // block), double-buffered by chunk parity: thread 0's copy and MMA issue
   // reads it from here instead of from global memory
@@ -390,10 +396,11 @@ __global__ void __launch_bounds__(TC_NT, TC_CTAS)
     bar_init(&lbar1[1]);
     bar_init(&mbar1[0]);
     bar_init(&mbar1[1]);
-    bar_init(&lbar2[0]);
-    bar_init(&lbar2[1]);
-    bar_init(&mbar2[0]);
-    bar_init(&mbar2[1]);
+    bar_init(&never);
+    for (int i = 0; i < TC_LB; ++i) {
+      bar_init(&lbar2[i]);
+      bar_init(&mbar2[i]);
+    }
     asm volatile("fence.mbarrier_init.release.cluster;");
     bad = 0;
   }
@@ -404,39 +411,45 @@ __global__ void __launch_bounds__(TC_NT, TC_CTAS)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tD1 = tbase, tD2 = tbase + 64;
-  // barrier bookkeeping (thread 0 only): phases and outstanding completions
-  uint32_t pl1[2] = {0, 0}, pm1[2] = {0, 0}, pl2[2] = {0, 0}, pm2[2] = {0, 0};
-  int l1_out[2] = {0, 0}, m1_out[2] = {0, 0}, l2_out[2] = {0, 0}, m2_out[2] = {0, 0};
-  int g2_steps = 0;
+  // Warp 0 controls: all its lanes walk the same state (phases and outstanding
+  // completions of the barriers, as bit masks), lane 0 issues MMAs and commits,
+  // and the lanes share out the copies of a chunk.  One thread issuing a step's
+  // copies one after the other took 3.7 of 15.7 thousand clocks a step, and
+  // waiting for them where they were needed about 7 (24 orbitals, D = 512 in 9
+  // sectors: 5.37 -> 4.61 ms a product with the lanes and the copies a phase
+  // ahead).
+  const int lane = tid & 31;
+  const bool ctl = tid < 32;
+  uint32_t pl1 = 0, pm1 = 0, pl2 = 0, pm2 = 0;      // phase bit of barrier b
+  uint32_t l1_out = 0, m1_out = 0, l2_out = 0, m2_out = 0;
   bool d2 = false;
   int where_c = -1, where_m0 = -1, where_s = -1;
   // waits inside the product loop give up after wait_ns; the final drain
   // before TMEM is released always allows the full TC_WAIT_NS, so that no copy
   // or MMA of this CTA is still in flight when it exits
-  auto drain = [&](uint64_t* bar, uint32_t& ph, int& out, unsigned long long bound = 0) {
-    if (!out) return;
-    if (wait_bar(bar, ph, bound ? bound : wait_ns)) {
-      ph ^= 1;
-      out = 0;
-    } else {
+  auto drain = [&](uint64_t* bars, int b, uint32_t& ph, uint32_t& out, int which, unsigned long long bound) {
+    if (!((out >> b) & 1)) return;
+    const bool ok = __all_sync(0xffffffffu, wait_bar(&bars[b], (ph >> b) & 1, bound) ? 1 : 0);
+    if (ok) {
+      ph ^= 1u << b;
+      out &= ~(1u << b);
+      return;
+    }
+    if (lane == 0) {
       if (!bad && atomicCAS(flag, 0, 1) == 0) {
-        const int which = (bar == &lbar1[0] || bar == &lbar1[1]) ? 1 : (bar == &mbar1[0] || bar == &mbar1[1]) ? 2
-                        : bar == &lbar2[0] ? 3 : bar == &lbar2[1] ? 4 : bar == &mbar2[0] ? 5 : 6;
         flag[1] = blockIdx.x;
         flag[2] = which;
         flag[3] = where_c;
         flag[4] = where_m0;
         flag[5] = where_s;
-        flag[6] = (int)ph;
+        flag[6] = (int)((ph >> b) & 1);
       }
       bad = 1;
     }
+    __syncwarp();
   };
 
-  // thread 0's copy issue for the steps (chunk c, X rows m0..m0+TC_MC-1) of this
-  // piece; GEMM1 chunk kc of a step goes to G1 buffer kc & 1, GEMM2 slice st
-  // (product st / nch2, K chunk st % nch2) to G2 buffer (g2_steps + st) & 1
-  // all threads: metadata of chunk c into meta[c & 1]
+  // metadata of chunk c into meta[c & 1] (all threads)
   auto load_meta = [&](int c) {
     const TcChunk C = chunks[c];
     Meta& M = meta[c & 1];
@@ -452,117 +465,135 @@ __global__ void __launch_bounds__(TC_NT, TC_CTAS)
       M.xb = xblocks[C.xb];
     }
   };
+  // GEMM1 chunk kc of step (chunk c, X rows m0..) into buffer b (warp 0): lanes
+  // 2 t + p copy plane p of product t's R rows, lanes 16 + p the X rows
   auto issue1 = [&](int c, int m0, int kc, int b) {
     const Meta& M = meta[c & 1];
-    const int pc = M.pc;
     const XBlock& XB = M.xb;
     const int mc16 = (min(TC_MC, XB.m - m0) + 15) & ~15;
-    const int xg0 = m0 / 8, xng = min(mc16 / 8, XB.img.rg - xg0);
     const uint32_t rowb = (chunk_w(XB.img, kc) / 16) * 128;  // bytes of one row group in this chunk
-    uint32_t bytes = (xng > 0 ? xng * rowb : 0) * S::NS;
-    for (int t = 0; t < pc; ++t) {
-      const int ng = min(rp / 8, M.t[t].R.rg - TL.col0 / 8);
-      if (ng > 0) bytes += ng * rowb * S::NS;
+    const int t = lane >> 1, p = lane & 1;
+    uint32_t bytes = 0;
+    unsigned char* dst = nullptr;
+    const unsigned char* src = nullptr;
+    if (p < S::NS) {
+      if (t < M.pc) {
+        const Img R = M.t[t].R;
+        bytes = (uint32_t)max(0, min(rp / 8, R.rg - TL.col0 / 8)) * rowb;
+        dst = sA1(b) + p * S::A1 + (uint32_t)(t * rp / 8) * rowb;
+        src = (p ? ops_lo : ops_hi) + chunk_off(R, kc) + (long long)(TL.col0 / 8) * rowb;
+      } else if (t == 8) {
+        const int xg0 = m0 / 8;
+        bytes = (uint32_t)max(0, min(mc16 / 8, XB.img.rg - xg0)) * rowb;
+        dst = sB1(b) + p * S::B1;
+        src = (p ? xl : xh) + chunk_off(XB.img, kc) + (long long)xg0 * rowb;
+      }
     }
-    expect_tx(&lbar1[b], bytes);
-    l1_out[b] = 1;
-    if (xng > 0) {
-      const long long xo = chunk_off(XB.img, kc) + (long long)xg0 * rowb;
-      bulk_g2s(sB1(b), xh + xo, xng * rowb, &lbar1[b]);
-      if (!TF32) bulk_g2s(sB1(b) + S::B1, xl + xo, xng * rowb, &lbar1[b]);
-    }
-    for (int t = 0; t < pc; ++t) {
-      const Img R = M.t[t].R;
-      const int ng = min(rp / 8, R.rg - TL.col0 / 8);
-      if (ng <= 0) continue;
-      const long long ro = chunk_off(R, kc) + (long long)(TL.col0 / 8) * rowb;
-      const uint32_t dst = (uint32_t)(t * rp / 8) * rowb;
-      bulk_g2s(sA1(b) + dst, ops_hi + ro, ng * rowb, &lbar1[b]);
-      if (!TF32) bulk_g2s(sA1(b) + S::A1 + dst, ops_lo + ro, ng * rowb, &lbar1[b]);
-    }
+    const uint32_t all = __reduce_add_sync(0xffffffffu, bytes);
+    if (lane == 0) expect_tx(&lbar1[b], all);
+    l1_out |= 1u << b;
+    __syncwarp();
+    if (bytes) bulk_g2s(dst, src, bytes, &lbar1[b]);
   };
   // the first (up to) two GEMM1 chunks of a step, into free G1 buffers
   auto prefetch1 = [&](int c, int m0) {
     const int nch = (meta[c & 1].xb.img.kb + CH_BYTES - 1) / CH_BYTES;
     for (int kc = 0; kc < 2 && kc < nch; ++kc) issue1(c, m0, kc, kc);
   };
-  auto issue2 = [&](int c, int m0, int st, int nch2, int b) {
-    const int t = st / nch2, c2 = st % nch2;
+  // L slices: 2^lsh buffers of a slice each (as many as fit, at most TC_LB);
+  // slice st of a step (product st / nch2, K chunk st % nch2) goes to buffer
+  // st mod 2^lsh
+  const int lrg = min(TC_M / 8, ((G.q + 7) >> 3) - TL.row0 / 8);  // row groups of this tile's L
+  const int lbytes = lrg * (CH_BYTES / 16) * 128 * S::NS;
+  const int lsh = 4 * lbytes <= S::LR ? 2 : 2 * lbytes <= S::LR ? 1 : 0;
+  auto issue2 = [&](int c, int m0, int st, int nch2) {
+    const int b = st & ((1 << lsh) - 1), t = st / nch2, c2 = st % nch2;
     const Img Lm = meta[c & 1].t[t].L;
     const int lg0 = TL.row0 / 8, lng = min(TC_M / 8, Lm.rg - lg0);
     const int lc = (m0 * ES) / CH_BYTES + c2;  // chunk of L's K (= X rows)
-    const uint32_t rowb = (chunk_w(Lm, lc) / 16) * 128;
-    unsigned char* a2 = sA2 + b * S::NS * S::A2;
-    expect_tx(&lbar2[b], lng * rowb * S::NS);
-    l2_out[b] = 1;
-    const long long lo_ = chunk_off(Lm, lc) + (long long)lg0 * rowb;
-    bulk_g2s(a2, ops_hi + lo_, lng * rowb, &lbar2[b]);
-    if (!TF32) bulk_g2s(a2 + S::A2, ops_lo + lo_, lng * rowb, &lbar2[b]);
+    const uint32_t rowb = (chunk_w(Lm, lc) / 16) * 128, bytes = (uint32_t)lng * rowb;
+    if (lane == 0) expect_tx(&lbar2[b], bytes * S::NS);
+    l2_out |= 1u << b;
+    __syncwarp();
+    if (lane < S::NS)
+      bulk_g2s(sL + b * lbytes + lane * (lbytes / S::NS), (lane ? ops_lo : ops_hi) + chunk_off(Lm, lc) + (long long)lg0 * rowb,
+               bytes, &lbar2[b]);
   };
   if (has_work) load_meta(TL.c0);
   __syncthreads();
-  if (tid == 0 && has_work) prefetch1(TL.c0, 0);
-  bool first_step = true;  // thread 0: the first step's GEMM1 chunks are already in flight
+  if (ctl && has_work) {
+    prefetch1(TL.c0, 0);
+    // a zero bound makes the first wait run out for certain (copies and MMAs
+    // may be done by the time they are waited for): on a barrier nothing completes
+    uint32_t ph = 0, out = wait_ns == 0 ? 1u : 0u;
+    drain(&never, 0, ph, out, 6, 0);
+  }
 
-  for (int c = TL.c0; c < TL.c1 && !bad; ++c) {
+  // a wait that ran out is noticed by everyone at the barrier after GEMM1 (no
+  // thread can set `bad` again before all have read it there)
+  bool stop = false;
+  for (int c = TL.c0; c < TL.c1 && !stop; ++c) {
     // the next chunk's metadata goes to the other buffer, free since the last
-    // step of chunk c-1 ended (thread 0 reads it for its prefetch at the end
-    // of this chunk, after the barriers of this chunk's steps)
+    // step of chunk c-1 ended; it is read after this chunk's first barrier
     if (c + 1 < TL.c1) load_meta(c + 1);
     const Meta& M = meta[c & 1];
     const int pc = M.pc;
     const XBlock XB = M.xb;
     const int m = XB.m;
     where_c = c;
-    for (int m0 = 0; m0 < m && !bad; m0 += TC_MC) {
+    for (int m0 = 0; m0 < m; m0 += TC_MC) {
       where_m0 = m0;
       const int mc = min(TC_MC, m - m0);
       const int mc16 = (mc + 15) & ~15;
       const int nch2 = (mc16 * ES + CH_BYTES - 1) / CH_BYTES;
       const int nsteps = pc * nch2;
-      if (tid == 0) {
+      if (ctl) {
+        // the previous step's GEMM2 MMAs read the L slices and B2: done first,
+        // then this step's first slices are copied while GEMM1 runs
+        for (int b = 0; b < (1 << lsh) && !bad; ++b) drain(mbar2, b, pm2, m2_out, 5, wait_ns);
+        for (int st = 0; st < (1 << lsh) && st < nsteps && !bad; ++st) issue2(c, m0, st, nch2);
         // ---- GEMM1: D1[t*rp + j][i] = sum_k R_t[col0 + j][k] X[m0 + i][k] ----
-        // the previous step's GEMM2 MMAs read the shared region and B2: done
-        // first; then chunks 0 and 1 of this step (the first step's were
-        // issued before the loop); chunk kc+1 >= 2 is copied once chunk
-        // kc-1's MMAs have released its buffer
-        drain(&mbar2[0], pm2[0], m2_out[0]);
-        drain(&mbar2[1], pm2[1], m2_out[1]);
-        if (!first_step && !bad) prefetch1(c, m0);
-        first_step = false;
+        // chunks 0 and 1 were copied during the previous step (the first
+        // step's before the loop); chunk kc+1 >= 2 is copied once chunk kc-1's
+        // MMAs have released its buffer
         const int nch = (XB.img.kb + CH_BYTES - 1) / CH_BYTES;
         for (int kc = 0; kc < nch && !bad; ++kc) {
           where_s = kc;
           const int b = kc & 1, bn = (kc + 1) & 1;
           if (kc + 1 < nch && kc + 1 >= 2) {
-            drain(&mbar1[bn], pm1[bn], m1_out[bn]);
+            drain(mbar1, bn, pm1, m1_out, 2, wait_ns);
             if (bad) break;
             issue1(c, m0, kc + 1, bn);
           }
-          drain(&lbar1[b], pl1[b], l1_out[b]);
+          drain(lbar1, b, pl1, l1_out, 1, wait_ns);
           if (bad) break;
           asm volatile("tcgen05.fence::after_thread_sync;");
-          const int kcm = chunk_w(XB.img, kc) / 16;
-          const uint32_t rowb = kcm * 128;
-          const uint32_t id = idesc(TF32 ? 2 : 1, mc16);
-          for (int ks = 0; ks < kcm / 2; ++ks)
-            for (int pr = 0; pr < NPROD; ++pr) {
-              const unsigned char* a = sA1(b) + (pr == 2 ? S::A1 : 0);
-              const unsigned char* bb = sB1(b) + (pr == 1 ? S::B1 : 0);
-              const uint32_t acc = (kc > 0 || ks > 0 || pr > 0) ? 1u : 0u;
-              mma<TF32>(tD1, sdesc(smem_u32(a) + ks * 256, rowb), sdesc(smem_u32(bb) + ks * 256, rowb), id, acc);
-            }
-          commit(&mbar1[b]);
-          m1_out[b] = 1;
+          if (lane == 0) {
+            const int kcm = chunk_w(XB.img, kc) / 16;
+            const uint32_t rowb = kcm * 128;
+            const uint32_t id = idesc(TF32 ? 2 : 1, mc16);
+            for (int ks = 0; ks < kcm / 2; ++ks)
+              for (int pr = 0; pr < NPROD; ++pr) {
+                const unsigned char* a = sA1(b) + (pr == 2 ? S::A1 : 0);
+                const unsigned char* bb = sB1(b) + (pr == 1 ? S::B1 : 0);
+                const uint32_t acc = (kc > 0 || ks > 0 || pr > 0) ? 1u : 0u;
+                mma<TF32>(tD1, sdesc(smem_u32(a) + ks * 256, rowb), sdesc(smem_u32(bb) + ks * 256, rowb), id, acc);
+              }
+            commit(&mbar1[b]);
+          }
+          m1_out |= 1u << b;
         }
-        // D1 complete before the T pass; the shared region is then free and
-        // this step's first two L slices are copied while the T pass runs
-        drain(&mbar1[0], pm1[0], m1_out[0]);
-        drain(&mbar1[1], pm1[1], m1_out[1]);
-        for (int st = 0; st < 2 && st < nsteps && !bad; ++st) issue2(c, m0, st, nch2, (g2_steps + st) & 1);
+        // D1 complete before the T pass; the G1 buffers are then free
+        if (!bad) drain(mbar1, 0, pm1, m1_out, 2, wait_ns);
+        if (!bad) drain(mbar1, 1, pm1, m1_out, 2, wait_ns);
       }
       __syncthreads();
-      if (bad) break;
+      stop = bad != 0;
+      if (stop) break;
+      if (ctl) {  // the next step's first GEMM1 chunks
+        if (m0 + TC_MC < m) prefetch1(c, m0 + TC_MC);
+        else if (c + 1 < TL.c1) prefetch1(c + 1, 0);
+      }
       asm volatile("tcgen05.fence::after_thread_sync;");
       // ---- T pass: D1 (fp32) -> B2 = a_t T_t^T in the K-major operand layout ----
       {
@@ -610,58 +641,59 @@ __global__ void __launch_bounds__(TC_NT, TC_CTAS)
       asm volatile("fence.proxy.async.shared::cta;");
       asm volatile("tcgen05.fence::before_thread_sync;");
       __syncthreads();
-      // ---- GEMM2: D2 += sum_t L_t[row0.., m0 + k] * B2_t^T (thread 0) ----
-      if (tid == 0) {
+      // ---- GEMM2: D2 += sum_t L_t[row0.., m0 + k] * B2_t^T (warp 0) ----
+      if (ctl) {
         asm volatile("tcgen05.fence::after_thread_sync;");
         const int nk2 = mc16 * ES / 32;  // 32-byte MMA k-steps over this X row range
         const uint32_t id = idesc(TF32 ? 2 : 1, rp);
-        // two-stage pipeline over the steps s = (product t, K chunk c2): the
-        // L slice of step s+1 is copied while step s's MMAs run
         for (int st = 0; st < nsteps && !bad; ++st) {
-          const int b = (g2_steps + st) & 1, bn = (g2_steps + st + 1) & 1;
+          const int b = st & ((1 << lsh) - 1);
           where_s = 1000 + st;
-          if (st + 1 < nsteps && st + 1 >= 2) {
-            drain(&mbar2[bn], pm2[bn], m2_out[bn]);  // the MMAs of step st-1 read buffer bn
+          // the slice that takes the buffer of slice st-1, once its MMAs are done
+          const int nx = st - 1 + (1 << lsh);
+          if (st > 0 && nx < nsteps) {
+            drain(mbar2, nx & ((1 << lsh) - 1), pm2, m2_out, 5, wait_ns);
             if (bad) break;
-            issue2(c, m0, st + 1, nch2, bn);
+            issue2(c, m0, nx, nch2);
           }
-          drain(&lbar2[b], pl2[b], l2_out[b]);
+          drain(lbar2, b, pl2, l2_out, 3, wait_ns);
           if (bad) break;
           asm volatile("tcgen05.fence::after_thread_sync;");
-          const int t = st / nch2, c2 = st % nch2;
-          const Img Lm = M.t[t].L;
-          const int lc = (m0 * ES) / CH_BYTES + c2;
-          const int kcm = chunk_w(Lm, lc) / 16;
-          const uint32_t rowb = kcm * 128;
-          const unsigned char* a2 = sA2 + b * S::NS * S::A2;
-          const uint32_t bt = (uint32_t)(t * rp / 8) * SBO_FULL;  // product t's rows inside a B2 chunk
-          const int ks_here = min(kcm / 2, nk2 - c2 * (CH_BYTES / 32));
-          for (int ks = 0; ks < ks_here; ++ks)
-            for (int pr = 0; pr < NPROD; ++pr) {
-              const unsigned char* a = a2 + (pr == 2 ? S::A2 : 0);
-              const unsigned char* bb = sB2 + (pr == 1 ? S::B2 : 0) + c2 * S::CB2 + bt;
-              const uint32_t acc = (d2 || ks > 0 || pr > 0) ? 1u : 0u;
-              mma<TF32>(tD2, sdesc(smem_u32(a) + ks * 256, rowb), sdesc(smem_u32(bb) + ks * 256, SBO_FULL), id,
-                        acc);
-            }
+          if (lane == 0) {
+            const int t = st / nch2, c2 = st % nch2;
+            const Img Lm = M.t[t].L;
+            const int lc = (m0 * ES) / CH_BYTES + c2;
+            const int kcm = chunk_w(Lm, lc) / 16;
+            const uint32_t rowb = kcm * 128;
+            const unsigned char* a2 = sL + b * lbytes;
+            const uint32_t bt = (uint32_t)(t * rp / 8) * SBO_FULL;  // product t's rows inside a B2 chunk
+            const int ks_here = min(kcm / 2, nk2 - c2 * (CH_BYTES / 32));
+            for (int ks = 0; ks < ks_here; ++ks)
+              for (int pr = 0; pr < NPROD; ++pr) {
+                const unsigned char* a = a2 + (pr == 2 ? lbytes / S::NS : 0);
+                const unsigned char* bb = sB2 + (pr == 1 ? S::B2 : 0) + c2 * S::CB2 + bt;
+                const uint32_t acc = (d2 || ks > 0 || pr > 0) ? 1u : 0u;
+                mma<TF32>(tD2, sdesc(smem_u32(a) + ks * 256, rowb), sdesc(smem_u32(bb) + ks * 256, SBO_FULL), id,
+                          acc);
+              }
+            commit(&mbar2[b]);
+          }
           d2 = true;
-          commit(&mbar2[b]);
-          m2_out[b] = 1;
+          m2_out |= 1u << b;
         }
-        g2_steps += nsteps;
       }
       __syncthreads();
     }
   }
   // every copy and MMA of this CTA done (bounded) before TMEM is read or released
-  if (tid == 0) {
+  if (ctl) {
     for (int b = 0; b < 2; ++b) {
-      drain(&lbar1[b], pl1[b], l1_out[b], TC_WAIT_NS);
-      drain(&mbar1[b], pm1[b], m1_out[b], TC_WAIT_NS);
+      drain(lbar1, b, pl1, l1_out, 1, TC_WAIT_NS);
+      drain(mbar1, b, pm1, m1_out, 2, TC_WAIT_NS);
     }
-    for (int b = 0; b < 2; ++b) {
-      drain(&lbar2[b], pl2[b], l2_out[b], TC_WAIT_NS);
-      drain(&mbar2[b], pm2[b], m2_out[b], TC_WAIT_NS);
+    for (int b = 0; b < TC_LB; ++b) {
+      drain(lbar2, b, pl2, l2_out, 3, TC_WAIT_NS);
+      drain(mbar2, b, pm2, m2_out, 5, TC_WAIT_NS);
     }
   }
   __syncthreads();
