@@ -211,13 +211,16 @@ __device__ __forceinline__ unsigned long long gtimer() {
 // wait for phase `ph`, bounded in time (bound_ns); returns false on timeout
 __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t ph, unsigned long long bound_ns) {
   uint32_t done = 0;
-  const unsigned long long t0 = gtimer();
-  while (!done) {
+  unsigned long long t0 = 0;  // the clock is read only once a wait has to go on: reading it costs as much as a try
+  for (int i = 0; !done; ++i) {
     asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
                  : "=r"(done)
                  : "r"(smem_u32(bar)), "r"(ph)
                  : "memory");
-    if (!done && gtimer() - t0 > bound_ns) break;
+    if (done) break;
+    const unsigned long long t = gtimer();
+    if (i == 0) t0 = t;
+    if (t - t0 > bound_ns || (i > 0 && bound_ns == 0)) break;
   }
   return done != 0;
 }
@@ -411,18 +414,21 @@ __global__ void __launch_bounds__(TC_NT, TC_CTAS)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tD1 = tbase, tD2 = tbase + 64;
-  // Warp 0 controls: all its lanes walk the same state (phases and outstanding
-  // completions of the barriers, as bit masks), lane 0 issues MMAs and commits,
-  // and the lanes share out the copies of a chunk.  One thread issuing a step's
-  // copies one after the other took 3.7 of 15.7 thousand clocks a step, and
-  // waiting for them where they were needed about 7 (24 orbitals, D = 512 in 9
-  // sectors: 5.37 -> 4.61 ms a product with the lanes and the copies a phase
-  // ahead).
-  const int lane = tid & 31;
-  const bool ctl = tid < 32;
+  // Roles, each a warp whose lanes walk the same state (phases and outstanding
+  // completions of the barriers, as bit masks) and whose lane 0 issues: warp 0
+  // the MMAs and GEMM1's chunks beyond the second, warp 1 the L slices, all
+  // warps a share of the next step's first GEMM1 chunks.  A bulk copy or an MMA
+  // takes its thread 60 to 150 clocks to issue (lanes of one warp take turns),
+  // so one thread that issued all of them, and waited for copies where they
+  // were needed, took 15.7 thousand clocks a step (24 orbitals, D = 512 in 9
+  // sectors, 5.37 ms a product; copies a phase ahead, still one warp: 4.61 ms;
+  // the roles split as here: 3.56 ms, and 16 orbitals, D = 256, 4 vectors
+  // 1955 / 1753 / 1283 us, 13 orbitals TF32 148 / 146 / 133 us).
+  const int lane = tid & 31, wid = tid >> 5;
   uint32_t pl1 = 0, pm1 = 0, pl2 = 0, pm2 = 0;      // phase bit of barrier b
   uint32_t l1_out = 0, m1_out = 0, l2_out = 0, m2_out = 0;
   bool d2 = false;
+  bool fail = false;  // one of this warp's own waits ran out (`bad`: anyone's; it can change between two lanes' reads)
   int where_c = -1, where_m0 = -1, where_s = -1;
   // waits inside the product loop give up after wait_ns; the final drain
   // before TMEM is released always allows the full TC_WAIT_NS, so that no copy
@@ -446,6 +452,7 @@ __global__ void __launch_bounds__(TC_NT, TC_CTAS)
       }
       bad = 1;
     }
+    fail = true;
     __syncwarp();
   };
 
@@ -465,40 +472,40 @@ __global__ void __launch_bounds__(TC_NT, TC_CTAS)
       M.xb = xblocks[C.xb];
     }
   };
-  // GEMM1 chunk kc of step (chunk c, X rows m0..) into buffer b (warp 0): lanes
-  // 2 t + p copy plane p of product t's R rows, lanes 16 + p the X rows
-  auto issue1 = [&](int c, int m0, int kc, int b) {
+  // GEMM1 chunks [kc0, kc0 + nk) of step (chunk c, X rows m0..) into buffers kc & 1:
+  // planes of the products' R rows and of the X rows, shared out over `nw` warps
+  const int ng = max(0, min(rp / 8, ((G.r + 7) >> 3) - TL.col0 / 8));  // row groups of R in this tile
+  auto issue1 = [&](int c, int m0, int kc0, int nk, int w, int nw) {
     const Meta& M = meta[c & 1];
     const XBlock& XB = M.xb;
-    const int mc16 = (min(TC_MC, XB.m - m0) + 15) & ~15;
-    const uint32_t rowb = (chunk_w(XB.img, kc) / 16) * 128;  // bytes of one row group in this chunk
-    const int t = lane >> 1, p = lane & 1;
-    uint32_t bytes = 0;
-    unsigned char* dst = nullptr;
-    const unsigned char* src = nullptr;
-    if (p < S::NS) {
-      if (t < M.pc) {
-        const Img R = M.t[t].R;
-        bytes = (uint32_t)max(0, min(rp / 8, R.rg - TL.col0 / 8)) * rowb;
-        dst = sA1(b) + p * S::A1 + (uint32_t)(t * rp / 8) * rowb;
-        src = (p ? ops_lo : ops_hi) + chunk_off(R, kc) + (long long)(TL.col0 / 8) * rowb;
-      } else if (t == 8) {
-        const int xg0 = m0 / 8;
-        bytes = (uint32_t)max(0, min(mc16 / 8, XB.img.rg - xg0)) * rowb;
-        dst = sB1(b) + p * S::B1;
-        src = (p ? xl : xh) + chunk_off(XB.img, kc) + (long long)xg0 * rowb;
+    const int pc = M.pc, mc16 = (min(TC_MC, XB.m - m0) + 15) & ~15;
+    const int xng = max(0, min(mc16 / 8, XB.img.rg - m0 / 8));
+    if (w == 0) {  // a copy that completes before its barrier is armed only counts ahead
+      for (int kc = kc0; kc < kc0 + nk; ++kc) {
+        if (lane == 0) expect_tx(&lbar1[kc & 1], (uint32_t)(pc * ng + xng) * (chunk_w(XB.img, kc) / 16) * 128 * S::NS);
+        l1_out |= 1u << (kc & 1);
       }
     }
-    const uint32_t all = __reduce_add_sync(0xffffffffu, bytes);
-    if (lane == 0) expect_tx(&lbar1[b], all);
-    l1_out |= 1u << b;
-    __syncwarp();
-    if (bytes) bulk_g2s(dst, src, bytes, &lbar1[b]);
+    if (lane == 0)
+      for (int i = w; i < (pc + 1) * nk * S::NS; i += nw) {
+        const int p = i & (S::NS - 1), q = S::NS == 2 ? i >> 1 : i, kc = kc0 + (nk == 2 ? q & 1 : 0), t = nk == 2 ? q >> 1 : q;
+        const int b = kc & 1;
+        const uint32_t rowb = (chunk_w(XB.img, kc) / 16) * 128;  // bytes of one row group in this chunk
+        if (t < pc) {
+          const Img R = M.t[t].R;
+          if (ng > 0)
+            bulk_g2s(sA1(b) + p * S::A1 + (uint32_t)(t * rp / 8) * rowb,
+                     (p ? ops_lo : ops_hi) + chunk_off(R, kc) + (long long)(TL.col0 / 8) * rowb, ng * rowb, &lbar1[b]);
+        } else if (xng > 0) {
+          bulk_g2s(sB1(b) + p * S::B1, (p ? xl : xh) + chunk_off(XB.img, kc) + (long long)(m0 / 8) * rowb, xng * rowb,
+                   &lbar1[b]);
+        }
+      }
   };
-  // the first (up to) two GEMM1 chunks of a step, into free G1 buffers
+  // the first (up to) two GEMM1 chunks of a step, into free G1 buffers (all warps)
   auto prefetch1 = [&](int c, int m0) {
     const int nch = (meta[c & 1].xb.img.kb + CH_BYTES - 1) / CH_BYTES;
-    for (int kc = 0; kc < 2 && kc < nch; ++kc) issue1(c, m0, kc, kc);
+    issue1(c, m0, 0, min(nch, 2), wid, TC_NT / 32);
   };
   // L slices: 2^lsh buffers of a slice each (as many as fit, at most TC_LB);
   // slice st of a step (product st / nch2, K chunk st % nch2) goes to buffer
@@ -512,25 +519,30 @@ __global__ void __launch_bounds__(TC_NT, TC_CTAS)
     const int lg0 = TL.row0 / 8, lng = min(TC_M / 8, Lm.rg - lg0);
     const int lc = (m0 * ES) / CH_BYTES + c2;  // chunk of L's K (= X rows)
     const uint32_t rowb = (chunk_w(Lm, lc) / 16) * 128, bytes = (uint32_t)lng * rowb;
-    if (lane == 0) expect_tx(&lbar2[b], bytes * S::NS);
+    if (lane == 0) {
+      expect_tx(&lbar2[b], bytes * S::NS);
+      for (int p = 0; p < S::NS; ++p)
+        bulk_g2s(sL + b * lbytes + p * (lbytes / S::NS), (p ? ops_lo : ops_hi) + chunk_off(Lm, lc) + (long long)lg0 * rowb,
+                 bytes, &lbar2[b]);
+    }
+    pl2 ^= 1u << b;      // warp 1: the phase of the buffer's latest copy
     l2_out |= 1u << b;
-    __syncwarp();
-    if (lane < S::NS)
-      bulk_g2s(sL + b * lbytes + lane * (lbytes / S::NS), (lane ? ops_lo : ops_hi) + chunk_off(Lm, lc) + (long long)lg0 * rowb,
-               bytes, &lbar2[b]);
+    m2_out |= 1u << b;   // its MMAs are awaited before the buffer is filled again
   };
   if (has_work) load_meta(TL.c0);
   __syncthreads();
-  if (ctl && has_work) {
+  if (has_work) {
     prefetch1(TL.c0, 0);
-    // a zero bound makes the first wait run out for certain (copies and MMAs
-    // may be done by the time they are waited for): on a barrier nothing completes
-    uint32_t ph = 0, out = wait_ns == 0 ? 1u : 0u;
-    drain(&never, 0, ph, out, 6, 0);
+    if (wid == 0) {
+      // a zero bound makes the first wait run out for certain (copies and MMAs
+      // may be done by the time they are waited for): on a barrier nothing completes
+      uint32_t ph = 0, out = wait_ns == 0 ? 1u : 0u;
+      drain(&never, 0, ph, out, 6, 0);
+    }
   }
-
-  // a wait that ran out is noticed by everyone at the barrier after GEMM1 (no
-  // thread can set `bad` again before all have read it there)
+  uint32_t com = 0, used = 0;  // warp 0: parity of the commits to each L buffer, buffers committed to
+  // a wait that ran out is noticed by everyone at the barrier after GEMM1 (the
+  // next wait is behind the T pass's barrier, so all read the same `bad` there)
   bool stop = false;
   for (int c = TL.c0; c < TL.c1 && !stop; ++c) {
     // the next chunk's metadata goes to the other buffer, free since the last
@@ -547,53 +559,55 @@ __global__ void __launch_bounds__(TC_NT, TC_CTAS)
       const int mc16 = (mc + 15) & ~15;
       const int nch2 = (mc16 * ES + CH_BYTES - 1) / CH_BYTES;
       const int nsteps = pc * nch2;
-      if (ctl) {
+      if (wid == 1) {
         // the previous step's GEMM2 MMAs read the L slices and B2: done first,
         // then this step's first slices are copied while GEMM1 runs
-        for (int b = 0; b < (1 << lsh) && !bad; ++b) drain(mbar2, b, pm2, m2_out, 5, wait_ns);
-        for (int st = 0; st < (1 << lsh) && st < nsteps && !bad; ++st) issue2(c, m0, st, nch2);
+        for (int b = 0; b < (1 << lsh) && !fail; ++b) drain(mbar2, b, pm2, m2_out, 5, wait_ns);
+        for (int st = 0; st < (1 << lsh) && st < nsteps && !fail; ++st) issue2(c, m0, st, nch2);
+      }
+      if (wid == 0) {
         // ---- GEMM1: D1[t*rp + j][i] = sum_k R_t[col0 + j][k] X[m0 + i][k] ----
         // chunks 0 and 1 were copied during the previous step (the first
         // step's before the loop); chunk kc+1 >= 2 is copied once chunk kc-1's
         // MMAs have released its buffer
         const int nch = (XB.img.kb + CH_BYTES - 1) / CH_BYTES;
-        for (int kc = 0; kc < nch && !bad; ++kc) {
+        const uint32_t id = idesc(TF32 ? 2 : 1, mc16);
+        for (int kc = 0; kc < nch && !fail; ++kc) {
           where_s = kc;
           const int b = kc & 1, bn = (kc + 1) & 1;
           if (kc + 1 < nch && kc + 1 >= 2) {
             drain(mbar1, bn, pm1, m1_out, 2, wait_ns);
-            if (bad) break;
-            issue1(c, m0, kc + 1, bn);
+            if (fail) break;
+            issue1(c, m0, kc + 1, 1, 0, 1);
           }
           drain(lbar1, b, pl1, l1_out, 1, wait_ns);
-          if (bad) break;
+          if (fail) break;
           asm volatile("tcgen05.fence::after_thread_sync;");
           if (lane == 0) {
             const int kcm = chunk_w(XB.img, kc) / 16;
-            const uint32_t rowb = kcm * 128;
-            const uint32_t id = idesc(TF32 ? 2 : 1, mc16);
-            for (int ks = 0; ks < kcm / 2; ++ks)
-              for (int pr = 0; pr < NPROD; ++pr) {
-                const unsigned char* a = sA1(b) + (pr == 2 ? S::A1 : 0);
-                const unsigned char* bb = sB1(b) + (pr == 1 ? S::B1 : 0);
-                const uint32_t acc = (kc > 0 || ks > 0 || pr > 0) ? 1u : 0u;
-                mma<TF32>(tD1, sdesc(smem_u32(a) + ks * 256, rowb), sdesc(smem_u32(bb) + ks * 256, rowb), id, acc);
-              }
+            const uint64_t da = sdesc(smem_u32(sA1(b)), kcm * 128), db = sdesc(smem_u32(sB1(b)), kcm * 128);
+#pragma unroll
+            for (int ks = 0; ks < CH_BYTES / 32; ++ks) {
+              if (ks >= kcm / 2) break;
+#pragma unroll
+              for (int pr = 0; pr < NPROD; ++pr)  // a descriptor's address counts 16 bytes
+                mma<TF32>(tD1, da + (pr == 2 ? S::A1 / 16 : 0) + ks * 16, db + (pr == 1 ? S::B1 / 16 : 0) + ks * 16, id,
+                          (kc > 0 || ks > 0 || pr > 0) ? 1u : 0u);
+            }
             commit(&mbar1[b]);
           }
           m1_out |= 1u << b;
         }
         // D1 complete before the T pass; the G1 buffers are then free
-        if (!bad) drain(mbar1, 0, pm1, m1_out, 2, wait_ns);
-        if (!bad) drain(mbar1, 1, pm1, m1_out, 2, wait_ns);
+        if (!fail) drain(mbar1, 0, pm1, m1_out, 2, wait_ns);
+        if (!fail) drain(mbar1, 1, pm1, m1_out, 2, wait_ns);
       }
       __syncthreads();
       stop = bad != 0;
       if (stop) break;
-      if (ctl) {  // the next step's first GEMM1 chunks
-        if (m0 + TC_MC < m) prefetch1(c, m0 + TC_MC);
-        else if (c + 1 < TL.c1) prefetch1(c + 1, 0);
-      }
+      // the next step's first GEMM1 chunks
+      if (m0 + TC_MC < m) prefetch1(c, m0 + TC_MC);
+      else if (c + 1 < TL.c1) prefetch1(c + 1, 0);
       asm volatile("tcgen05.fence::after_thread_sync;");
       // ---- T pass: D1 (fp32) -> B2 = a_t T_t^T in the K-major operand layout ----
       {
@@ -642,59 +656,64 @@ __global__ void __launch_bounds__(TC_NT, TC_CTAS)
       asm volatile("tcgen05.fence::before_thread_sync;");
       __syncthreads();
       // ---- GEMM2: D2 += sum_t L_t[row0.., m0 + k] * B2_t^T (warp 0) ----
-      if (ctl) {
+      if (wid == 0) {
         asm volatile("tcgen05.fence::after_thread_sync;");
         const int nk2 = mc16 * ES / 32;  // 32-byte MMA k-steps over this X row range
         const uint32_t id = idesc(TF32 ? 2 : 1, rp);
-        for (int st = 0; st < nsteps && !bad; ++st) {
+        for (int st = 0, t = 0, c2 = 0; st < nsteps && !fail; ++st) {
           const int b = st & ((1 << lsh) - 1);
           where_s = 1000 + st;
-          // the slice that takes the buffer of slice st-1, once its MMAs are done
-          const int nx = st - 1 + (1 << lsh);
-          if (st > 0 && nx < nsteps) {
-            drain(mbar2, nx & ((1 << lsh) - 1), pm2, m2_out, 5, wait_ns);
-            if (bad) break;
-            issue2(c, m0, nx, nch2);
-          }
-          drain(lbar2, b, pl2, l2_out, 3, wait_ns);
-          if (bad) break;
+          uint32_t wait_it = 1u << b;
+          drain(lbar2, b, pl2, wait_it, 3, wait_ns);
+          if (fail) break;
           asm volatile("tcgen05.fence::after_thread_sync;");
           if (lane == 0) {
-            const int t = st / nch2, c2 = st % nch2;
-            const Img Lm = M.t[t].L;
-            const int lc = (m0 * ES) / CH_BYTES + c2;
-            const int kcm = chunk_w(Lm, lc) / 16;
-            const uint32_t rowb = kcm * 128;
-            const unsigned char* a2 = sL + b * lbytes;
+            const int kcm = chunk_w(M.t[t].L, (m0 * ES) / CH_BYTES + c2) / 16;
             const uint32_t bt = (uint32_t)(t * rp / 8) * SBO_FULL;  // product t's rows inside a B2 chunk
             const int ks_here = min(kcm / 2, nk2 - c2 * (CH_BYTES / 32));
-            for (int ks = 0; ks < ks_here; ++ks)
-              for (int pr = 0; pr < NPROD; ++pr) {
-                const unsigned char* a = a2 + (pr == 2 ? lbytes / S::NS : 0);
-                const unsigned char* bb = sB2 + (pr == 1 ? S::B2 : 0) + c2 * S::CB2 + bt;
-                const uint32_t acc = (d2 || ks > 0 || pr > 0) ? 1u : 0u;
-                mma<TF32>(tD2, sdesc(smem_u32(a) + ks * 256, rowb), sdesc(smem_u32(bb) + ks * 256, SBO_FULL), id,
-                          acc);
-              }
+            const uint64_t da = sdesc(smem_u32(sL + b * lbytes), kcm * 128);
+            const uint64_t db = sdesc(smem_u32(sB2 + c2 * S::CB2 + bt), SBO_FULL);
+            const uint32_t lo = (uint32_t)(lbytes / S::NS / 16);
+#pragma unroll
+            for (int ks = 0; ks < CH_BYTES / 32; ++ks) {
+              if (ks >= ks_here) break;
+#pragma unroll
+              for (int pr = 0; pr < NPROD; ++pr)
+                mma<TF32>(tD2, da + (pr == 2 ? lo : 0) + ks * 16, db + (pr == 1 ? S::B2 / 16 : 0) + ks * 16, id,
+                          (d2 || ks > 0 || pr > 0) ? 1u : 0u);
+            }
             commit(&mbar2[b]);
           }
+          com ^= 1u << b;
+          used |= 1u << b;
           d2 = true;
-          m2_out |= 1u << b;
+          if (++c2 == nch2) {
+            c2 = 0;
+            ++t;
+          }
         }
       }
+      if (wid == 1)  // the slices beyond the buffers, each once its buffer's MMAs are done
+        for (int st = 1 << lsh; st < nsteps && !fail; ++st) {
+          drain(mbar2, st & ((1 << lsh) - 1), pm2, m2_out, 5, wait_ns);
+          if (!fail) issue2(c, m0, st, nch2);
+        }
       __syncthreads();
     }
   }
-  // every copy and MMA of this CTA done (bounded) before TMEM is read or released
-  if (ctl) {
+  // every copy and MMA of this CTA done (bounded) before TMEM is read or
+  // released: warp 0 GEMM1's copies and all its own MMAs, warp 1 its L copies
+  if (wid == 0) {
     for (int b = 0; b < 2; ++b) {
       drain(lbar1, b, pl1, l1_out, 1, TC_WAIT_NS);
       drain(mbar1, b, pm1, m1_out, 2, TC_WAIT_NS);
     }
-    for (int b = 0; b < TC_LB; ++b) {
-      drain(lbar2, b, pl2, l2_out, 3, TC_WAIT_NS);
-      drain(mbar2, b, pm2, m2_out, 5, TC_WAIT_NS);
-    }
+    com = ~com;  // the phase of the last commit
+    for (int b = 0; b < TC_LB; ++b) drain(mbar2, b, com, used, 5, TC_WAIT_NS);
+  }
+  if (wid == 1) {
+    pl2 = ~pl2;
+    for (int b = 0; b < TC_LB; ++b) drain(lbar2, b, pl2, l2_out, 3, TC_WAIT_NS);
   }
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
