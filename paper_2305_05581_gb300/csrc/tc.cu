@@ -202,6 +202,18 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
                : "memory");
 }
 
+// true in one lane of the (converged) warp, always the same one.  Bulk copies,
+// MMAs and commits take their operands from uniform registers: under a test of
+// the lane number they are issued in a loop over the lanes that may be active,
+// some 30 instructions each; the compiler knows an elected lane to be alone
+// (split-BF16: 24 orbitals, D = 512, 9 sectors 3.56 -> 3.13 ms, all sectors
+// 3.12 -> 2.50 ms; 13 orbitals TF32 133 -> 120 us).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t one;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.b32 %0, 1, 0, p;\n}" : "=r"(one));
+  return one != 0;
+}
+
 __device__ __forceinline__ unsigned long long gtimer() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
@@ -415,15 +427,16 @@ __global__ void __launch_bounds__(TC_NT, TC_CTAS)
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tD1 = tbase, tD2 = tbase + 64;
   // Roles, each a warp whose lanes walk the same state (phases and outstanding
-  // completions of the barriers, as bit masks) and whose lane 0 issues: warp 0
+  // completions of the barriers, as bit masks) and one of which issues: warp 0
   // the MMAs and GEMM1's chunks beyond the second, warp 1 the L slices, all
   // warps a share of the next step's first GEMM1 chunks.  A bulk copy or an MMA
-  // takes its thread 60 to 150 clocks to issue (lanes of one warp take turns),
+  // took its thread 60 to 150 clocks to issue (lanes of one warp take turns),
   // so one thread that issued all of them, and waited for copies where they
   // were needed, took 15.7 thousand clocks a step (24 orbitals, D = 512 in 9
   // sectors, 5.37 ms a product; copies a phase ahead, still one warp: 4.61 ms;
-  // the roles split as here: 3.56 ms, and 16 orbitals, D = 256, 4 vectors
-  // 1955 / 1753 / 1283 us, 13 orbitals TF32 148 / 146 / 133 us).
+  // the roles split as here: 3.56 ms; an elected lane instead of lane 0:
+  // 3.13 ms; 16 orbitals, D = 333, 4 vectors 1955 / 1753 / 1283 / 1159 us, 13
+  // orbitals TF32 148 / 146 / 133 / 120 us).
   const int lane = tid & 31, wid = tid >> 5;
   uint32_t pl1 = 0, pm1 = 0, pl2 = 0, pm2 = 0;      // phase bit of barrier b
   uint32_t l1_out = 0, m1_out = 0, l2_out = 0, m2_out = 0;
@@ -480,13 +493,12 @@ __global__ void __launch_bounds__(TC_NT, TC_CTAS)
     const XBlock& XB = M.xb;
     const int pc = M.pc, mc16 = (min(TC_MC, XB.m - m0) + 15) & ~15;
     const int xng = max(0, min(mc16 / 8, XB.img.rg - m0 / 8));
-    if (w == 0) {  // a copy that completes before its barrier is armed only counts ahead
-      for (int kc = kc0; kc < kc0 + nk; ++kc) {
-        if (lane == 0) expect_tx(&lbar1[kc & 1], (uint32_t)(pc * ng + xng) * (chunk_w(XB.img, kc) / 16) * 128 * S::NS);
-        l1_out |= 1u << (kc & 1);
-      }
-    }
-    if (lane == 0)
+    if (w == 0)
+      for (int kc = kc0; kc < kc0 + nk; ++kc) l1_out |= 1u << (kc & 1);
+    if (elect_one()) {
+      if (w == 0)  // a copy that completes before its barrier is armed only counts ahead
+        for (int kc = kc0; kc < kc0 + nk; ++kc)
+          expect_tx(&lbar1[kc & 1], (uint32_t)(pc * ng + xng) * (chunk_w(XB.img, kc) / 16) * 128 * S::NS);
       for (int i = w; i < (pc + 1) * nk * S::NS; i += nw) {
         const int p = i & (S::NS - 1), q = S::NS == 2 ? i >> 1 : i, kc = kc0 + (nk == 2 ? q & 1 : 0), t = nk == 2 ? q >> 1 : q;
         const int b = kc & 1;
@@ -501,6 +513,7 @@ __global__ void __launch_bounds__(TC_NT, TC_CTAS)
                    &lbar1[b]);
         }
       }
+    }
   };
   // the first (up to) two GEMM1 chunks of a step, into free G1 buffers (all warps)
   auto prefetch1 = [&](int c, int m0) {
@@ -519,7 +532,7 @@ __global__ void __launch_bounds__(TC_NT, TC_CTAS)
     const int lg0 = TL.row0 / 8, lng = min(TC_M / 8, Lm.rg - lg0);
     const int lc = (m0 * ES) / CH_BYTES + c2;  // chunk of L's K (= X rows)
     const uint32_t rowb = (chunk_w(Lm, lc) / 16) * 128, bytes = (uint32_t)lng * rowb;
-    if (lane == 0) {
+    if (elect_one()) {
       expect_tx(&lbar2[b], bytes * S::NS);
       for (int p = 0; p < S::NS; ++p)
         bulk_g2s(sL + b * lbytes + p * (lbytes / S::NS), (p ? ops_lo : ops_hi) + chunk_off(Lm, lc) + (long long)lg0 * rowb,
@@ -583,7 +596,7 @@ __global__ void __launch_bounds__(TC_NT, TC_CTAS)
           drain(lbar1, b, pl1, l1_out, 1, wait_ns);
           if (fail) break;
           asm volatile("tcgen05.fence::after_thread_sync;");
-          if (lane == 0) {
+          if (elect_one()) {
             const int kcm = chunk_w(XB.img, kc) / 16;
             const uint64_t da = sdesc(smem_u32(sA1(b)), kcm * 128), db = sdesc(smem_u32(sB1(b)), kcm * 128);
 #pragma unroll
@@ -667,7 +680,7 @@ __global__ void __launch_bounds__(TC_NT, TC_CTAS)
           drain(lbar2, b, pl2, wait_it, 3, wait_ns);
           if (fail) break;
           asm volatile("tcgen05.fence::after_thread_sync;");
-          if (lane == 0) {
+          if (elect_one()) {
             const int kcm = chunk_w(M.t[t].L, (m0 * ES) / CH_BYTES + c2) / 16;
             const uint32_t bt = (uint32_t)(t * rp / 8) * SBO_FULL;  // product t's rows inside a B2 chunk
             const int ks_here = min(kcm / 2, nk2 - c2 * (CH_BYTES / 32));
@@ -862,7 +875,7 @@ __global__ void __launch_bounds__(WS_NT, 1)
 
   if (warp == 0) {
     // ------------------------------ copies ------------------------------
-    if (lane == 0) {
+    if (elect_one()) {
       long long i1 = 0, i2 = 0;  // running slot counters of the two rings
       int armed1[WS_S1], armed2[S::S2];
       for (int i = 0; i < WS_S1; ++i) armed1[i] = 0;
@@ -960,7 +973,7 @@ __global__ void __launch_bounds__(WS_NT, 1)
     }
   } else if (warp == 1) {
     // ------------------------------- MMAs -------------------------------
-    if (lane == 0) {
+    if (elect_one()) {
       long long i1 = 0, i2 = 0, s = 0;
       int piece = 0;  // pieces with work of this CTA so far (D2 buffer and its phase)
       bool go = true;
