@@ -21,8 +21,9 @@
 // pipe stays out of the product loop.
 //
 // One CTA (256 threads) per output tile piece (128 rows x <= 64 columns);
-// warp 0 issues copies (its lanes share them out) and MMAs from the chunk's
-// product metadata, which all threads stage in shared memory one chunk ahead;
+// warp 0 issues the MMAs, warp 1 copies the L slices and all warps share the
+// first copies of the next step, from the chunk's product metadata, which all
+// threads stage in shared memory one chunk ahead;
 // GEMM1's copies run under the previous step's T pass and GEMM2, GEMM2's under
 // GEMM1; all threads do the T pass and the epilogue.  Steps of 32 X rows and
 // an L region of 18 KB keep a CTA at 75 KB of shared memory, three per SM.
@@ -383,8 +384,8 @@ __global__ void __launch_bounds__(TC_NT, TC_CTAS)
   __shared__ uint32_t tbase;
   __shared__ volatile int bad;
   // metadata of the products of a chunk (at most TC_M / 16 share one X
-  // block), double-buffered by chunk parity: thread 0's copy and MMA issue
-  // reads it from here instead of from global memory
+  // block), double-buffered by chunk parity: the issuing warps
+  // read it from here instead of from global memory
   struct MetaT {
     Img L, R;
     float alpha;
@@ -737,7 +738,7 @@ __global__ void __launch_bounds__(TC_NT, TC_CTAS)
     for (int j0 = 8 * wg; j0 < rp; j0 += 16) {
       uint32_t r[8] = {0, 0, 0, 0, 0, 0, 0, 0};
       // warp-collective load: the condition must be uniform over the CTA (d2 is
-      // thread 0's own bookkeeping; a tile with chunks always issued GEMM2)
+      // warp 0's own bookkeeping; a tile with chunks always issued GEMM2)
       if (has_work && !bad) {
         const uint32_t addr = tD2 + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)j0;
         asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"

@@ -123,6 +123,33 @@ def test_adjoint_matches_dfma(system):
         assert _close(a, b)
 
 
+@pytest.mark.parametrize("system", [CASES[1], CASES[3]])
+def test_adjoint_lists_kept_for_the_step(system):
+    """The adjoint's lists outlive a call: other vectors, a subset of the
+    gradients and an arena changed before build_env give what a context that
+    never ran it before gives (both FP64, so within the bound above)."""
+    ctx, k, (desc, length) = _ctx(None, system)
+    ref, _, _ = _ctx("dfma", system)
+    arenas = [arena_tensor(c, k, 0) for c in (ctx, ref)]
+
+    def grads(c, x, yb, which):
+        res = [torch.zeros(length, device="cuda", dtype=torch.float64)]
+        res += [torch.zeros_like(arena_tensor(c, k, side)) for side in (0, 1)]
+        c.heff_adjoint_ptr(k, x.data_ptr(), yb.data_ptr(), *(r.data_ptr() if w else 0 for r, w in zip(res, which)))
+        torch.cuda.synchronize()
+        return res
+
+    a, b = _vector("normal", desc, length, 2)
+    for x, yb, which in ((a, b, (1, 1, 1)), (b, a, (1, 1, 1)), (a + b, b, (0, 1, 0)), (a, a - b, (1, 0, 1))):
+        for g, w in zip(grads(ctx, x, yb, which), grads(ref, x, yb, which)):
+            assert _close(g, w)
+    for arena, c in zip(arenas, (ctx, ref)):
+        arena.mul_(0.5)
+        c.build_env(k)
+    for g, w in zip(grads(ctx, a, b, (1, 1, 1)), grads(ref, a, b, (1, 1, 1))):
+        assert _close(g, w)
+
+
 @pytest.mark.parametrize("bad", [float("nan"), float("inf"), -float("inf")])
 def test_non_finite_entries_reach_the_same_outputs(bad):
     system = CASES[3]
