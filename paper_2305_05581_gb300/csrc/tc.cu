@@ -1849,8 +1849,8 @@ bool prepare_tasks_tc(CudaBackend& be, const TaskList& tl, DevList& d, int nvec,
     const std::vector<double>& cc = plan->ccost_h;
     auto cost = [&](const TcChunk& C, const TcTile&) { return cc[&C - ch.data()]; };
     split_plan(tiles, plan->chunks_h, reds, psize, (double)TC_CTAS * plan->sms, kRounds[variant], cost);
-    const double wunits[2] = {(double)SwCfg<16>::UNITS * plan->sms,
-                              (double)SwCfg<32>::UNITS * plan->sms};
+    const double wunits[2] = {(double)SwCfg<16>::WARPS * SwCfg<16>::CTAS * plan->sms,
+                              (double)SwCfg<32>::WARPS * SwCfg<32>::CTAS * plan->sms};
     for (int w = 0; w < 2; ++w) {
       // one partial-tile arena: each kernel's partial tiles after the previous ones
       std::vector<SplitRed> wreds;
