@@ -206,7 +206,7 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
 // true in one lane of the (converged) warp, always the same one.  Bulk copies,
 // MMAs and commits take their operands from uniform registers: under a test of
 // the lane number they are issued in a loop over the lanes that may be active,
-// some 30 instructions each; the compiler knows an elected lane to be alone
+// some 25 instructions more each by the counters; an elected lane is known to be alone
 // (split-BF16: 24 orbitals, D = 512, 9 sectors 3.56 -> 3.13 ms, all sectors
 // 3.12 -> 2.50 ms; 13 orbitals TF32 133 -> 120 us).
 __device__ __forceinline__ bool elect_one() {
