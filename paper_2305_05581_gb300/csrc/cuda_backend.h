@@ -38,10 +38,10 @@ struct Tile {  // an output tile of a group: rows [row0, row0+nrows), cols [col0
 // classes of the FP64 digit kernel (fp64_digits.cu): most rows of the a side
 // and columns of the b side of a tile, l and k staged at a time, CTAs per SM
 struct DgClass {
-  int a, b, lk, km, ctas;
+  int a, b, km, ctas;
 };
 constexpr int kDgClasses = 3;
-constexpr DgClass kDgClass[kDgClasses] = {{16, 16, 16, 16, 12}, {32, 32, 32, 32, 4}, {64, 64, 64, 32, 2}};
+constexpr DgClass kDgClass[kDgClasses] = {{16, 16, 16, 12}, {32, 32, 32, 4}, {64, 64, 32, 2}};
 cudaError_t fp64_digits_init();
 class CudaBackend;
 struct DevList;
@@ -147,8 +147,8 @@ class CudaBackend : public Backend {
   CudaBackend(int device, cudaStream_t s, bool own);
   // FP64 product kernel of every list: 0 DFMA tile classes, 1 DMMA (mma.sync
   // m8n8k4 f64), 2 exact digit products on the f16 tensor cores
-  // (fp64_digits.cu); -1 (default): digits where the list allows them, else
-  // DFMA; environment TNS_FP64_KERNEL=dfma|dmma|digits
+  // (fp64_digits.cu) where a list has images; -1 (default): digits where the
+  // list allows them, else DFMA; environment TNS_FP64_KERNEL=dfma|dmma|digits
   int fp64_kernel = -1;
   // bound of one wait inside the tensor-core product loop (ns); the
   // environment variable TNS_TC_WAIT_NS overrides the default 0.2 s when the

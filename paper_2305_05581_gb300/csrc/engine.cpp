@@ -2362,7 +2362,7 @@ int Engine::adjoint_plan(const bool want[3], std::string& err) {
   };
   auto list = [](TaskList& tl, const std::vector<Blk>& blocks, auto&& products) {
     tl.clear();
-    tl.persistent = tl.digits = true;
+    tl.persistent = true;
     for (const Blk& b : blocks) {
       Group g;
       g.yoff = b.off;
@@ -2430,7 +2430,6 @@ int Engine::adjoint_plan(const bool want[3], std::string& err) {
       }
     }
     list(A.sum, cb, [&](long long off) -> const std::vector<Task>* { return &add[off]; });
-    A.sum.digits = false;  // sums of blocks
     P.have[1 + s] = true;
   }
   return 0;

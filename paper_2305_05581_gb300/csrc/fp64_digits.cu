@@ -25,24 +25,21 @@
 //     GEMM2  Y[a][b] += alpha sum_k T[a][k] B[b][k]
 // Each warp owns 16 rows a.  GEMM1's accumulators are fragments whose layout
 // is that of GEMM2's A operand, so T is normalised per row, cut into digits
-// again and used from registers.  The row scales of X (one per k) go to the
-// columns of B before B is cut.  Y is kept in FP64 registers: one DFMA per
-// output and 32 terms of k, where the DFMA kernel needs 32.
+// again and used from registers.
 //
-// Two kernels: k_tasks_dg cuts its operands where it uses them, from the FP64
-// blocks into shared-memory planes of 8 x 8 f16 core matrices (ldmatrix) --
-// for lists that run once, and where there is no memory for images;
-// k_tasks_im, further down, reads digits cut beforehand, for lists that are
-// kept.  Both are bound by the integer work around the MMAs (joining the
-// weight sums, cutting T) and by the 8 to 12 warps that registers and shared
-// memory leave an SM to hide its latencies (MMA pipe 30 % busy, issue slots
-// 27 to 49 %).  One H_eff*psi, DFMA tile classes -> here (time, useful rate):
+// The digits are cut beforehand (images, below), so the kernel is for lists that
+// are kept; lists that run once or have no room for images, and the adjoint,
+// whose operands change between calls, stay with the FMA kernel.  The kernel is
+// bound by the integer work around the MMAs (joining the weight sums, cutting T)
+// and by the 8 to 12 warps that registers and shared memory leave an SM to hide
+// its latencies (MMA pipe 30 % busy, issue slots 27 to 49 %).  One H_eff*psi,
+// DFMA tile classes -> here (time, useful rate):
 //   24 orbitals, D = 512, all sectors (blocks <= 26):  36.4 -> 14.9 ms, 1.15 TFLOP/s
 //   24 orbitals, D = 512, 9 sectors (blocks <= 68):     153 -> 47.4 ms, 2.45 TFLOP/s
 //   13 orbitals, D = 260, 3 sectors (blocks <= 99):    3.03 -> 0.78 ms, 2.81 TFLOP/s
 // (cuBLAS DGEMM: 1.10 TFLOP/s).
 //
-// Values that the fixed-point form cannot hold: a chunk in which an operand
+// Values that the fixed-point form cannot hold: a product in which an operand
 // has an infinity, a NaN or a magnitude of 2^330 or more is evaluated with
 // plain FP64 FMAs instead; rows whose largest magnitude is below 2^-700 are
 // taken relative to 2^-700.
@@ -58,27 +55,10 @@ namespace tns {
 namespace {
 
 constexpr int DG_N = 7;                        // digits of an operand
-constexpr int DG_T = 8;                        // digits of T: its rows may be graded
 constexpr int DG_S = 8;                        // weights s = i + j kept: 0 .. 7
 constexpr unsigned DG_MAGIC = 0x4B400000u;     // bits of 1.5 * 2^23
 constexpr int DG_EMIN = 322;                   // smallest biased exponent of a row scale (2^-700)
 constexpr int DG_EMAX = (1023 + 330) << 20;    // high word from which on a value leaves the fixed-point form
-
-template <int W_, int NBT_, int LK_, int KM_, int CTAS_>
-struct DgCfg {
-  static constexpr int CTAS = CTAS_;  // resident CTAs per SM
-  static constexpr int W = W_;        // warps: 16 rows of the a side each
-  static constexpr int NBT = NBT_;    // 8-column tiles of the b side
-  static constexpr int LK = LK_;      // l staged at a time
-  static constexpr int KM = KM_;      // k staged at a time (at most 32: exactness)
-  static constexpr int NT = 32 * W, AR = 16 * W, BR = 8 * NBT;
-  static constexpr int PA = AR * LK * 2, PX = KM * LK * 2, PB = BR * KM * 2;  // bytes of one digit plane
-  static constexpr int off_xb = DG_N * PA;                                    // X, then B, in one region
-  static constexpr int off_e = off_xb + DG_N * (PX > PB ? PX : PB);           // row scales of A, X, B
-  static constexpr int total = off_e + 4 * (AR + KM + BR + 4);
-  static_assert(KM <= 32 && LK % 16 == 0 && KM % 16 == 0, "chunk sizes");
-  static_assert(DG_N * PA >= AR * BR * 8, "the A region holds a tile of FP64 values");
-};
 
 __device__ __forceinline__ uint32_t sm_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -114,110 +94,6 @@ __device__ __forceinline__ uint32_t digit2(uint32_t h0, uint32_t l0, uint32_t h1
   return *(const uint32_t*)&d;
 }
 
-// An operand view: element (r, k) = p[r * sr + k * sk] for r < nr and k < nk, else 0
-struct View {
-  const double* p;
-  int sr, sk, nr, nk;
-};
-
-// Rows [0, rpad) x columns [0, KC) of an operand view into digit planes.  A
-// thread takes 8 columns of a row; the KC / 8 threads of a row are adjacent
-// lanes and agree on its scale (ef: biased exponent, the row below 2^(ef -
-// 1022)), unless it was found before (have).  With dk, column k carries a
-// factor 2^(dk[k] - 1022).  Core matrix (row group, octet o) holds row r at
-// slot r ^ o, so that neither these stores nor ldmatrix meet a bank twice.
-// One copy of this code per kernel: inlined at its six uses it is what the
-// instruction cache misses on.
-template <int NT, int KC>
-__device__ __noinline__ void dg_slice(const View vw, int rpad, uint32_t dst, int plane, int* ef, bool have,
-                                      const int* dk, int* bad) {
-  constexpr int OC = KC / 8;
-  const int units = rpad * OC;
-  for (int u0 = 0; u0 < units; u0 += NT) {
-    const int u = u0 + threadIdx.x;
-    const int row = u / OC, o = u % OC;
-    const double* q = vw.p + (long long)row * vw.sr + (long long)(8 * o) * vw.sk;
-    uint32_t hi[8], lo[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const double x = (row < vw.nr && 8 * o + e < vw.nk) ? __ldg(q + (long long)e * vw.sk) : 0.0;
-      hi[e] = (uint32_t)__double2hiint(x);
-      lo[e] = (uint32_t)__double2loint(x);
-    }
-    int uu[8], mx = INT32_MIN, raw = 0;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      uu[e] = (int)(hi[e] & 0x7fffffffu);
-      raw = max(raw, uu[e]);
-    }
-    if (dk) {
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        uu[e] = uu[e] ? uu[e] + ((dk[8 * o + e] - 1022) << 20) : -(1 << 30);
-        mx = max(mx, uu[e]);
-      }
-    } else {
-      mx = raw;
-    }
-    if (raw >= DG_EMAX) *bad = 1;
-    int E;
-    if (have) {
-      E = ef[min(row, rpad - 1)];
-    } else {
-#pragma unroll
-      for (int s = 1; s < OC; s <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, s));
-      E = max((mx + 0x2100) >> 20, DG_EMIN);  // within 0.8% of a power of two counts as that power: no carry out of digit 0
-      if (o == 0 && u < units) ef[row] = E;
-    }
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      // v = (mantissa << 10) >> (E - exponent), sign by complement, + 0x80 in every byte
-      const int sh = min(E - (uu[e] >> 20), 63);
-      const unsigned long long m =
-          ((unsigned long long)((hi[e] & 0xfffffu) | 0x100000u) << 32 | lo[e]) << 10;
-      const unsigned long long v = m >> sh;
-      const uint32_t sg = (uint32_t)((int)hi[e] >> 31);
-      const unsigned long long b =
-          ((unsigned long long)((uint32_t)(v >> 32) ^ sg) << 32 | ((uint32_t)v ^ sg)) + 0x8080808080808080ull;
-      hi[e] = (uint32_t)(b >> 32);
-      lo[e] = (uint32_t)b;
-    }
-    if (u < units) {
-      const uint32_t at = dst + (uint32_t)(((row >> 3) * OC + o) * 128 + (((row & 7) ^ (o & 7)) << 4));
-#define DG_PUT(P)                                                                                                  \
-  asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(at + (P) * (uint32_t)plane),                          \
-               "r"(digit2<P>(hi[0], lo[0], hi[1], lo[1])), "r"(digit2<P>(hi[2], lo[2], hi[3], lo[3])),             \
-               "r"(digit2<P>(hi[4], lo[4], hi[5], lo[5])), "r"(digit2<P>(hi[6], lo[6], hi[7], lo[7]))              \
-               : "memory")
-      DG_PUT(0);
-      DG_PUT(1);
-      DG_PUT(2);
-      DG_PUT(3);
-      DG_PUT(4);
-      DG_PUT(5);
-      DG_PUT(6);
-#undef DG_PUT
-    }
-  }
-}
-
-// the scale of whole rows longer than one staged chunk
-template <int NT, int KC>
-__device__ __noinline__ void dg_rowmax(const View v, int rpad, int* ef, int* bad) {
-  constexpr int OC = KC / 8;
-  for (int u0 = 0; u0 < rpad * OC; u0 += NT) {
-    const int u = u0 + threadIdx.x, row = u / OC, o = u % OC;
-    int mx = 0;
-    if (row < v.nr)
-      for (int k = o; k < v.nk; k += OC)
-        mx = max(mx, __double2hiint(__ldg(v.p + (long long)row * v.sr + (long long)k * v.sk)) & 0x7fffffff);
-    if (mx >= DG_EMAX) *bad = 1;
-#pragma unroll
-    for (int s = 1; s < OC; s <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, s));
-    if (o == 0 && u < rpad * OC) ef[row] = max((mx + 0x2100) >> 20, DG_EMIN);
-  }
-}
-
 // the weight sums of one output as an integer, sum_s i_s 2^(43 - 8 s), below
 // 2^62.1.  T rounds to the nearest; Y (floor) meets the complement that
 // dg_double takes of negative numbers, so that it errs towards zero alike on
@@ -251,309 +127,15 @@ __device__ __forceinline__ double dg_double(long long v, int e) {
   return __hiloint2double((int)dh, (int)dl);
 }
 
-template <class C>
-__global__ void __launch_bounds__(C::NT, C::CTAS)
-    k_tasks_dg(const Task* __restrict__ tasks, const Group* __restrict__ groups, const Tile* __restrict__ tiles,
-               int tile0, const double* xv, double* yv, long long xs, long long ys, double* part, long long psize,
-               int nv) {
-  constexpr int W = C::W, NBT = C::NBT, LK = C::LK, KM = C::KM, NT = C::NT;
-  constexpr int KT = KM / 8;  // 8-wide tiles of k
-  extern __shared__ __align__(128) unsigned char sm[];
-  int* const eA = (int*)(sm + C::off_e);
-  int* const eX = eA + C::AR;
-  int* const eB = eX + KM;
-  int* const bad = eB + C::BR;
-  const uint32_t sA = sm_u32(sm), sXB = sm_u32(sm + C::off_xb);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
-  const int mj = lane >> 3, mr = lane & 7;  // ldmatrix: the matrix and row this lane addresses
-  const Tile TL = tiles[tile0 + blockIdx.x / nv];
-  const Group G = groups[TL.g];
-  const int vec = blockIdx.x % nv;
-  const double* X0 = xv ? xv + (long long)vec * xs : nullptr;
-  const bool bl = TL.aside != 0;  // the a side is op(L) and the rows of Y
-  const int na = bl ? TL.nrows : TL.ncols, nb = bl ? TL.ncols : TL.nrows;
-  const int a0 = bl ? TL.row0 : TL.col0, b0 = bl ? TL.col0 : TL.row0;
-  const int nbt = (nb + 7) >> 3, apad = (na + 15) & ~15, bpad = nbt * 8;
-  const bool mine = 16 * warp < na;  // warp-uniform: this warp has rows
-  double y[NBT][4];
-#pragma unroll
-  for (int b = 0; b < NBT; ++b)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) y[b][e] = 0.0;
-  auto sync = [&]() {
-    if (W == 1) __syncwarp();
-    else __syncthreads();
-  };
-  if (tid == 0) *bad = 0;
-  sync();
-
-  uint32_t tf[KT / 2][DG_T][4];  // T's digits over a staged chunk of k: GEMM2's A operand
-  auto scale = [](double alpha, int n) { return alpha * __hiloint2double((n + 1023) << 20, 0); };  // alpha 2^n
-
-  for (int ti = TL.t0; ti < TL.t1; ++ti) {
-    const Task tk = tasks[ti];
-    const int f = tk.flags;
-    const double* pX = (f & TF_XV) ? X0 + (long long)(size_t)tk.X : tk.X;
-    const int sXi = (f & TF_XT) ? 1 : tk.n, sXj = (f & TF_XT) ? tk.m : 1;
-    const int sLi = (f & TF_LT) ? 1 : tk.m, sLk = (f & TF_LT) ? tk.q : 1;
-    const int sRj = (f & TF_RT) ? 1 : tk.n, sRk = (f & TF_RT) ? tk.r : 1;
-    const int sXk = bl ? sXj : sXi, sXl = bl ? sXi : sXj;
-    const int K3 = bl ? tk.n : tk.m, L = bl ? tk.m : tk.n;
-    const bool ai = (f & (bl ? TF_LI : TF_RI)) != 0, bi = (f & (bl ? TF_RI : TF_LI)) != 0;
-    if (ai && bi) {  // Y += alpha X
-      if (mine)
-#pragma unroll
-        for (int b = 0; b < NBT; ++b)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int a = 16 * warp + g + 8 * (e >> 1), c = 8 * b + 2 * t + (e & 1);
-            if (a < na && c < nb)
-              y[b][e] = fma(tk.alpha, __ldg(pX + (long long)(b0 + c) * sXk + (long long)(a0 + a) * sXl), y[b][e]);
-          }
-      continue;
-    }
-    // views A (a, l), X (k, l), B (b, k); with one identity factor two views
-    // are left: Y[a][b] += alpha sum_k P[a][k] Q[b][k], P in A's place, Q in B's
-    const bool two = ai || bi || (f & TF_XI);
-    View A{(bl ? tk.L : tk.R), bl ? sLi : sRj, bl ? sLk : sRk, na, L};
-    View B{(bl ? tk.R : tk.L), bl ? sRj : sLi, bl ? sRk : sLk, nb, K3};
-    A.p += ai ? 0 : (long long)a0 * A.sr;
-    B.p += bi ? 0 : (long long)b0 * B.sr;
-    if (ai) A = View{pX + (long long)a0 * sXl, sXl, sXk, na, K3};
-    if (bi) B = View{pX + (long long)b0 * sXk, sXk, sXl, nb, L};
-    const int K = two ? A.nk : K3;
-    const bool long_l = !two && L > LK;
-    int hsh = 0;  // head room of T beyond one sum of 32
-    while ((32 << hsh) < L) ++hsh;
-    bool slow = false;
-    sync();
-    if (!two) {
-      if (long_l) dg_rowmax<NT, LK>(A, apad, eA, bad);
-      else dg_slice<NT, LK>(A, apad, sA, C::PA, eA, false, nullptr, bad);
-    }
-    for (int k0 = 0; k0 < K; k0 += KM) {
-      const int kc = min(KM, K - k0), kpad = (kc + 15) & ~15;
-      const View Bk{B.p + (long long)k0 * B.sk, B.sr, B.sk, nb, kc};
-      double s0 = 0.0, s1 = 0.0;
-      if (two && !slow) {
-        sync();
-        dg_slice<NT, KM>(View{A.p + (long long)k0 * A.sk, A.sr, A.sk, na, kc}, apad, sA, C::PA, eA, false, nullptr, bad);
-      } else if (!slow) {
-        const View X{pX + (long long)k0 * sXk, sXk, sXl, kc, L};
-        long long T[KT][4];
-        sync();
-        if (long_l) {
-          dg_rowmax<NT, LK>(X, kpad, eX, bad);
-          sync();
-        }
-#pragma unroll
-        for (int b = 0; b < KT; ++b)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) T[b][e] = 0;
-        for (int l0 = 0; l0 < L; l0 += LK) {
-          const int lc = min(LK, L - l0);
-          if (l0) sync();
-          if (long_l)
-            dg_slice<NT, LK>(View{A.p + (long long)l0 * A.sk, A.sr, A.sk, na, lc}, apad, sA, C::PA, eA, true, nullptr, bad);
-          dg_slice<NT, LK>(View{X.p + (long long)l0 * sXl, sXk, sXl, kc, lc}, kpad, sXB, C::PX, eX, long_l, nullptr, bad);
-          sync();
-          if (*bad) slow = true;
-          if (slow) break;
-          if (!mine) continue;
-#pragma unroll
-          for (int kp = 0; kp < KT / 2; ++kp) {
-            if (16 * kp >= kc) break;
-            for (int l32 = 0; l32 < lc; l32 += 32) {
-              float acc[2][DG_S][4];
-#pragma unroll
-              for (int h = 0; h < 2; ++h) {
-                if (h == 1 && l32 + 16 >= lc) break;
-                const int ob = l32 / 8 + 2 * h;
-                uint32_t xf[DG_N][4];
-                {
-                  const int o = ob + (mj & 1);
-                  const uint32_t xa =
-                      sXB + (uint32_t)(((2 * kp + (mj >> 1)) * (LK / 8) + o) * 128 + ((mr ^ (o & 7)) << 4));
-#pragma unroll
-                  for (int j = 0; j < DG_N; ++j) ldsm4(xf[j], xa + j * C::PX);
-                }
-                const int o = ob + (mj >> 1);
-                const uint32_t aa =
-                    sA + (uint32_t)(((2 * warp + (mj & 1)) * (LK / 8) + o) * 128 + ((mr ^ (o & 7)) << 4));
-#pragma unroll
-                for (int i = 0; i < DG_N; ++i) {
-                  uint32_t af[4];
-                  ldsm4(af, aa + i * C::PA);
-#pragma unroll
-                  for (int j = 0; j < DG_N && i + j < DG_S; ++j) {
-                    if (h == 0 && (i == 0 || (i == 1 && j == DG_N - 1))) {
-                      mma_first(acc[0][i + j], af, xf[j][0], xf[j][1]);
-                      mma_first(acc[1][i + j], af, xf[j][2], xf[j][3]);
-                    } else {
-                      mma_acc(acc[0][i + j], af, xf[j][0], xf[j][1]);
-                      mma_acc(acc[1][i + j], af, xf[j][2], xf[j][3]);
-                    }
-                  }
-                }
-              }
-#pragma unroll
-              for (int c = 0; c < 2; ++c)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                  const long long v = dg_join<true>(acc[c][0][e], acc[c][1][e], acc[c][2][e], acc[c][3][e], acc[c][4][e],
-                                              acc[c][5][e], acc[c][6][e], acc[c][7][e]);
-                  T[2 * kp + c][e] += hsh ? v >> hsh : v;
-                }
-            }
-          }
-        }
-        if (mine && !slow) {
-          // normalise T per row over the chunk and cut it again
-          int m0 = 0, m1 = 0;
-#pragma unroll
-          for (int b = 0; b < KT; ++b)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const int h = (int)(T[b][e] >> 32), ah = h ^ (h >> 31);
-              if (e < 2) m0 = max(m0, ah);
-              else m1 = max(m1, ah);
-            }
-#pragma unroll
-          for (int s = 1; s < 4; s <<= 1) {
-            m0 = max(m0, __shfl_xor_sync(0xffffffffu, m0, s));
-            m1 = max(m1, __shfl_xor_sync(0xffffffffu, m1, s));
-          }
-          const int z0 = __clz(m0 + (m0 >> 7) + 1) - 1, z1 = __clz(m1 + (m1 >> 7) + 1) - 1;
-#pragma unroll
-          for (int kk = 0; kk < KT / 2; ++kk)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {  // q: rows g, g + 8 of the first 8 k, then of the second
-              const int b = 2 * kk + (q >> 1), e = 2 * (q & 1), z = q & 1 ? z1 : z0;
-              const unsigned long long v0 = ((unsigned long long)T[b][e] << z) + 0x8080808080808080ull;
-              const unsigned long long v1 = ((unsigned long long)T[b][e + 1] << z) + 0x8080808080808080ull;
-              const uint32_t h0 = (uint32_t)(v0 >> 32), l0 = (uint32_t)v0, h1 = (uint32_t)(v1 >> 32), l1 = (uint32_t)v1;
-              tf[kk][0][q] = digit2<0>(h0, l0, h1, l1);
-              tf[kk][1][q] = digit2<1>(h0, l0, h1, l1);
-              tf[kk][2][q] = digit2<2>(h0, l0, h1, l1);
-              tf[kk][3][q] = digit2<3>(h0, l0, h1, l1);
-              tf[kk][4][q] = digit2<4>(h0, l0, h1, l1);
-              tf[kk][5][q] = digit2<5>(h0, l0, h1, l1);
-              tf[kk][6][q] = digit2<6>(h0, l0, h1, l1);
-              tf[kk][7][q] = digit2<7>(h0, l0, h1, l1);
-            }
-          s0 = scale(tk.alpha, eA[16 * warp + g] - 1022 + 6 + hsh - z0 - 57);
-          s1 = scale(tk.alpha, eA[16 * warp + g + 8] - 1022 + 6 + hsh - z1 - 57);
-        }
-        sync();
-      }
-      if (!slow) {
-        dg_slice<NT, KM>(Bk, bpad, sXB, C::PB, eB, false, two ? nullptr : eX, bad);
-        sync();
-        if (*bad) slow = true;
-      }
-      if (slow) {  // uniform: this and the remaining chunks of the product in plain FP64
-        double* D = (double*)sm;
-        sync();
-        for (int e = tid; e < na * nb; e += NT) {
-          const int a = e / nb, b = e % nb;
-          double s = 0.0;
-          for (int k = k0; k < k0 + kc; ++k) {
-            double x = 0.0;
-            if (two)
-              x = __ldg(A.p + (long long)a * A.sr + (long long)k * A.sk);
-            else
-              for (int l = 0; l < L; ++l)
-                x = fma(__ldg(pX + (long long)k * sXk + (long long)l * sXl), __ldg(A.p + (long long)a * A.sr + (long long)l * A.sk), x);
-            s = fma(__ldg(B.p + (long long)b * B.sr + (long long)k * B.sk), x, s);
-          }
-          D[e] = s;
-        }
-        if (tid == 0) *bad = 0;
-        sync();
-        if (mine)
-#pragma unroll
-          for (int b = 0; b < NBT; ++b)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const int a = 16 * warp + g + 8 * (e >> 1), c = 8 * b + 2 * t + (e & 1);
-              if (a < na && c < nb) y[b][e] = fma(tk.alpha, D[a * nb + c], y[b][e]);
-            }
-        continue;
-      }
-      if (!mine) continue;
-      if (two) {
-#pragma unroll
-        for (int kk = 0; kk < KT / 2; ++kk)
-#pragma unroll
-          for (int i = 0; i < DG_T; ++i) {
-            const int o = 2 * kk + (mj >> 1);
-            if (i == DG_N) tf[kk][i][0] = tf[kk][i][1] = tf[kk][i][2] = tf[kk][i][3] = 0u;
-            else ldsm4(tf[kk][i], sA + i * C::PA + (uint32_t)(((2 * warp + (mj & 1)) * KT + o) * 128 + ((mr ^ o) << 4)));
-          }
-        s0 = scale(tk.alpha, eA[16 * warp + g] - 1022 - 57);
-        s1 = scale(tk.alpha, eA[16 * warp + g + 8] - 1022 - 57);
-      }
-      // GEMM2: the planes of B against T's digits, joined into Y
-#pragma unroll
-      for (int b = 0; b < NBT; ++b) {
-        if (b >= nbt) break;
-        float acc[DG_S][4];
-        uint32_t bf[DG_N][4];
-        const int o = KT == 4 ? mj : (mj & 1);
-        const uint32_t ba = sXB + (uint32_t)((b * KT + o) * 128 + ((mr ^ o) << 4));
-#pragma unroll
-        for (int j = 0; j < DG_N; ++j) ldsm4(bf[j], ba + j * C::PB);
-#pragma unroll
-        for (int i = 0; i < DG_T; ++i)
-#pragma unroll
-          for (int j = 0; j < DG_N && i + j < DG_S; ++j) {
-            if (i == 0 || (i == 1 && j == DG_N - 1)) mma_first(acc[i + j], tf[0][i], bf[j][0], bf[j][1]);
-            else mma_acc(acc[i + j], tf[0][i], bf[j][0], bf[j][1]);
-          }
-        if (KT == 4 && kc > 16) {
-#pragma unroll
-          for (int i = 0; i < DG_T; ++i)
-#pragma unroll
-            for (int j = 0; j < DG_N && i + j < DG_S; ++j) mma_acc(acc[i + j], tf[KT / 2 - 1][i], bf[j][2], bf[j][3]);
-        }
-        const int e0 = eB[8 * b + 2 * t] + 63, e1 = eB[8 * b + 2 * t + 1] + 63;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const long long v = dg_join<false>(acc[0][e], acc[1][e], acc[2][e], acc[3][e], acc[4][e], acc[5][e], acc[6][e], acc[7][e]);
-          y[b][e] = fma(dg_double(v, e & 1 ? e1 : e0), e < 2 ? s0 : s1, y[b][e]);
-        }
-      }
-    }
-  }
-
-  double* Y = yv + (long long)vec * ys + G.yoff;
-  double* P = TL.poff >= 0 ? part + (long long)vec * psize + TL.poff : nullptr;  // split piece
-  if (mine)
-#pragma unroll
-    for (int b = 0; b < NBT; ++b)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int a = 16 * warp + g + 8 * (e >> 1), c = 8 * b + 2 * t + (e & 1);
-        if (a >= na || c >= nb) continue;
-        const int i = bl ? a : c, j = bl ? c : a;
-        if (P) P[i * TL.ncols + j] = y[b][e];
-        else Y[(long long)(TL.row0 + i) * G.r + TL.col0 + j] = y[b][e];
-      }
-}
-
 // ---------------------------------------------------------------------------
-// The same products from prepared digits (lists that are run many times).
-//
 // Every distinct operand of the list has an image: its digits, cut once, in
 // units of 8 rows x 8 columns x 7 planes of f16 core matrices (896 bytes; row
 // groups outermost, columns padded to 16), after the scales of its rows.  The
 // vectors are cut once per call, each block in the orientation its products
 // read, into 8 digits (all 64 bits of v; the pair (0, 7) joins the others).
-// Here the scales of X cannot go to the columns of B, so T is brought to a
-// common scale over k as it is normalised: a shift per element by the distance
-// of its row of X from the block's largest.  Against cutting operands where
-// they are used this takes 40% of the instructions off the product loop (24
-// orbitals: 36.5 -> 14.9 ms, 9 sectors 64 -> 47 ms).
+// The scales of X cannot go to the columns of B, which are cut before X is
+// known, so T is brought to a common scale over k as it is normalised: a shift
+// per element by the distance of its row of X from the block's largest.
 // ---------------------------------------------------------------------------
 constexpr int IM_UNIT = DG_N * 128;  // bytes of one 8 x 8 unit of an operator
 constexpr int IM_NX = 8;             // digits of the vector and of T
@@ -1163,22 +745,11 @@ using ImS = ImCfg<1, 2, 16, 16, 12>;
 using ImM = ImCfg<2, 4, 32, 32, 4>;
 using ImL = ImCfg<4, 8, 32, 32, 2>;
 
-using DgS = DgCfg<1, 2, 16, 16, 12>;
-using DgM = DgCfg<2, 4, 32, 32, 4>;
-using DgL = DgCfg<4, 8, 64, 32, 2>;
-static_assert(DgS::CTAS == kDgClass[0].ctas && DgM::CTAS == kDgClass[1].ctas && DgL::CTAS == kDgClass[2].ctas &&
-                  DgS::AR == kDgClass[0].a && DgM::AR == kDgClass[1].a && DgL::AR == kDgClass[2].a &&
-                  DgS::BR == kDgClass[0].b && DgM::BR == kDgClass[1].b && DgL::BR == kDgClass[2].b &&
-                  DgS::LK == kDgClass[0].lk && DgM::LK == kDgClass[1].lk && DgL::LK == kDgClass[2].lk &&
-                  DgS::KM == kDgClass[0].km && DgM::KM == kDgClass[1].km && DgL::KM == kDgClass[2].km,
+static_assert(ImS::CTAS == kDgClass[0].ctas && ImM::CTAS == kDgClass[1].ctas && ImL::CTAS == kDgClass[2].ctas &&
+                  ImS::AR == kDgClass[0].a && ImM::AR == kDgClass[1].a && ImL::AR == kDgClass[2].a &&
+                  ImS::BR == kDgClass[0].b && ImM::BR == kDgClass[1].b && ImL::BR == kDgClass[2].b &&
+                  ImS::KM == kDgClass[0].km && ImM::KM == kDgClass[1].km && ImL::KM == kDgClass[2].km,
               "the classes the host plans with");
-
-template <class C>
-void launch_one(unsigned grid, cudaStream_t s, const Task* tasks, const Group* groups, const Tile* tiles, int tile0,
-                const double* xv, double* yv, long long xs, long long ys, double* part, long long psize, int nv) {
-  k_tasks_dg<C><<<grid, C::NT, C::total, s>>>(tasks, groups, tiles, tile0, xv, yv, xs, ys, part, psize, nv);
-}
-
 
 template <class C>
 void launch_im(unsigned grid, cudaStream_t s, const DgRec* recs, const Task* tasks, const Group* groups,
@@ -1221,7 +792,7 @@ void release_digit_plan(void* p) {
 // The plan of a list that is kept on the device: its images and records, made
 // on the device in three launches.  Images are made only where they leave at
 // least half of the memory that neither the step's own plan nor anything else
-// has a claim to; without them the kernel above cuts its operands itself.
+// has a claim to; without them the list stays with the FMA kernel.
 bool prepare_digits(CudaBackend& be, const TaskList& tl, DevList& d, int nvec, long long length) {
   if (d.dg_none || !be.ok()) return false;
   DgPlan* P = (DgPlan*)d.dg;
@@ -1336,24 +907,19 @@ cudaError_t fp64_digits_init() {
   auto set = [](const void* f, int bytes) {
     return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   };
-  cudaError_t e = set((const void*)k_tasks_dg<DgL>, DgL::total);
-  if (e == cudaSuccess) e = set((const void*)k_tasks_im<ImM>, ImM::total);
+  cudaError_t e = set((const void*)k_tasks_im<ImM>, ImM::total);
   if (e == cudaSuccess) e = set((const void*)k_tasks_im<ImL>, ImL::total);
   return e;
 }
 
-// one class of tiles: from the list's images if it has a plan, else from its operands
+// one class of tiles
 void launch_fp64_digits(int cls, unsigned grid, cudaStream_t s, const void* plan, const Task* tasks,
                         const Group* groups, const Tile* tiles, int tile0, const double* xv, double* yv, long long xs,
                         long long ys, double* part, long long psize, int nv) {
-  if (const DgPlan* P = (const DgPlan*)plan) {
-    auto f = cls == 0 ? launch_im<ImS> : cls == 1 ? launch_im<ImM> : launch_im<ImL>;
-    f(grid, s, P->recs, tasks, groups, tiles, tile0, P->ops, P->x, P->xbytes, P->xscale, P->nx, xv, yv, xs, ys, part,
-      psize, nv);
-  } else {
-    auto f = cls == 0 ? launch_one<DgS> : cls == 1 ? launch_one<DgM> : launch_one<DgL>;
-    f(grid, s, tasks, groups, tiles, tile0, xv, yv, xs, ys, part, psize, nv);
-  }
+  const DgPlan* P = (const DgPlan*)plan;
+  auto f = cls == 0 ? launch_im<ImS> : cls == 1 ? launch_im<ImM> : launch_im<ImL>;
+  f(grid, s, P->recs, tasks, groups, tiles, tile0, P->ops, P->x, P->xbytes, P->xscale, P->nx, xv, yv, xs, ys, part,
+    psize, nv);
 }
 
 }  // namespace tns

@@ -1272,27 +1272,25 @@ static void dfma_tiles(const TaskList& tl, DevList& d) {
 
 // Estimated time of one product on an a x b tile of a digit-kernel class, in
 // clocks of one SM whose resident CTAs share it: its MMAs (34 digit pairs, 8
-// clocks each on one of four tensor cores), the cutting of T (and, without
-// images, of the operands), the joining of sums into Y, and a fixed part per
-// staged chunk.  Only ratios matter: they decide classes, sides and splits.
-static double dg_cost(int cls, const Task& t, int aside, int a, int b, bool images) {
+// clocks each on one of four tensor cores), the cutting of T, the joining of
+// sums into Y, and a fixed part per staged chunk.  Only ratios matter: they
+// decide classes, sides and splits.
+static double dg_cost(int cls, const Task& t, int aside, int a, int b) {
   const DgClass& c = kDgClass[cls];
   const int K = aside ? t.n : t.m, L = aside ? t.m : t.n;
   auto up = [](int x, int m) { return (double)((x + m - 1) / m * m); };
   const double ap = up(a, 16), bp = up(b, 8);
-  const double ovh0[kDgClasses] = {300.0, 700.0, 1300.0}, ovh1[kDgClasses] = {150.0, 400.0, 800.0};
-  const double ovh = images ? ovh1[cls] : ovh0[cls], mm = 34.0 * 8.0 / 2048.0, cut = images ? 0.0 : 1.7;
-  const int lk = images ? c.km : c.lk;
+  const double fixed[kDgClasses] = {150.0, 400.0, 800.0};
+  const double ovh = fixed[cls], mm = 34.0 * 8.0 / 2048.0;
   const bool ai = (t.flags & (aside ? TF_LI : TF_RI)) != 0, bi = (t.flags & (aside ? TF_RI : TF_LI)) != 0;
   if (ai && bi) return ovh + a * b / 4.0;
   if (ai || bi || (t.flags & TF_XI)) {
     const double kk = up(ai ? K : L, 16), ch = std::ceil(kk / c.km);
-    return ovh * ch + 0.25 * (ap * bp * kk * mm + cut * kk * (ap + bp) + 4.0 * ap * bp * ch);
+    return ovh * ch + 0.25 * (ap * bp * kk * mm + 4.0 * ap * bp * ch);
   }
-  const double kp = up(K, 16), lp = up(L, 16), ch = std::ceil(kp / c.km), lch = std::ceil((double)L / lk);
+  const double kp = up(K, 16), lp = up(L, 16), ch = std::ceil(kp / c.km), lch = std::ceil((double)L / c.km);
   return ovh * ch * (1.0 + 0.5 * (lch - 1)) +
-         0.25 * (mm * ap * kp * (lp + bp) + cut * (kp * lp + bp * kp + ap * lp * (lch > 1 ? ch : 1.0)) +
-                 2.4 * ap * kp * lch + 4.0 * ap * bp * ch);
+         0.25 * (mm * ap * kp * (lp + bp) + 2.4 * ap * kp * lch + 4.0 * ap * bp * ch);
 }
 
 // cut an extent into near-equal parts of at most mx, at multiples of 8 (the row groups of images)
@@ -1302,7 +1300,7 @@ static std::vector<std::pair<int, int>> cut8(int len, int mx) {
   return out;
 }
 
-// lists of products on vectors that are kept get digit images
+// the digit kernel reads images, which lists of products on vectors that are kept have
 static bool digit_images(const TaskList& tl) {
   return tl.persistent && !tl.tasks.empty() && (tl.tasks[0].flags & TF_XV);
 }
@@ -1311,7 +1309,6 @@ static bool digit_images(const TaskList& tl) {
 // contracted with X first, whichever costs least over the group's products
 // (summed over their distinct shapes)
 static void dg_tiles(const TaskList& tl, DevList& d) {
-  const bool images = digit_images(tl);
   d.dg_aside.assign(tl.groups.size(), 0);
   struct Shape {
     int m, n, f, count;
@@ -1341,7 +1338,7 @@ static void dg_tiles(const TaskList& tl, DevList& d) {
         const int ea = s ? G.q : G.r, eb = s ? G.r : G.q;
         const int na = (ea + kDgClass[c].a - 1) / kDgClass[c].a, nb = (eb + kDgClass[c].b - 1) / kDgClass[c].b;
         double w = 0;
-        for (const Shape& x : sh) w += x.count * dg_cost(c, *x.t, s, (ea + na - 1) / na, (eb + nb - 1) / nb, images);
+        for (const Shape& x : sh) w += x.count * dg_cost(c, *x.t, s, (ea + na - 1) / na, (eb + nb - 1) / nb);
         w *= (double)na * nb;
         if (best < 0 || w < best) {
           best = w;
@@ -1365,7 +1362,7 @@ static void dg_tiles(const TaskList& tl, DevList& d) {
         t.aside = pa;
         t.poff = -1;
         double w = 0;
-        for (const Shape& x : sh) w += x.count * dg_cost(pc, *x.t, pa, aa.second, bb.second, images);
+        for (const Shape& x : sh) w += x.count * dg_cost(pc, *x.t, pa, aa.second, bb.second);
         d.fp_tiles[1][pc].push_back(t);
         d.fp_cost[1][pc].push_back(w);
       }
@@ -1387,7 +1384,7 @@ void CudaBackend::plan_variant(const TaskList& tl, DevList& d, int dig, int v) {
     note(cudaFuncSetAttribute(k_tasks_fp64<C3_NT, C3_ACC, C3_TR, C3_TC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               fp64_smem(C3_TR, C3_TC)),
          "k_tasks_fp64 shared memory");
-    note(fp64_digits_init(), "k_tasks_dg shared memory");
+    note(fp64_digits_init(), "k_tasks_im shared memory");
     attr = true;
   }
   const bool digits = dig != 0;
@@ -1433,7 +1430,7 @@ void CudaBackend::plan_variant(const TaskList& tl, DevList& d, int dig, int v) {
       double tot = 0;
       for (int k = t.t0; k < t.t1; ++k)
         tot += kc[k - t.t0] =
-            digits ? dg_cost(c, tl.tasks[k], t.aside, t.aside ? t.nrows : t.ncols, t.aside ? t.ncols : t.nrows, digit_images(tl))
+            digits ? dg_cost(c, tl.tasks[k], t.aside, t.aside ? t.nrows : t.ncols, t.aside ? t.ncols : t.nrows)
                    : (double)tile_fmas(tl.tasks[k], t.nrows, t.ncols, nullptr) + kTaskOverhead;
       SplitRed R;
       R.g = t.g;
@@ -1536,8 +1533,7 @@ void CudaBackend::enqueue_fp64(const DevList& d, int dig, int v, const double* x
   // (they fill its tail), joined before the split reduction
   int order[kFpClasses] = {0, 1, 2, 3};
   std::stable_sort(order, order + kFpClasses, [&](int a, int b) { return f.ccost[a] > f.ccost[b]; });
-  const void* plan = dig && !d.dg_none ? d.dg : nullptr;
-  if (plan) enqueue_digit_vectors(*this, d, xv, xs, nvec);
+  if (dig) enqueue_digit_vectors(*this, d, xv, xs, nvec);
   const int nact = (f.ncls[0] > 0) + (f.ncls[1] > 0) + (f.ncls[2] > 0) + (f.ncls[3] > 0);
   const bool fork = nact > 1 && fork_ready();
   if (fork) {
@@ -1559,7 +1555,7 @@ void CudaBackend::enqueue_fp64(const DevList& d, int dig, int v, const double* x
     if (fork && oi > 0) s = fstream_[side++];
     const int t0 = tbeg[c];
     if (dig)
-      launch_fp64_digits(c, grid, s, plan, d.tasks, d.groups, f.tiles, t0, xv, yv, xs, ys, f.part, f.psize, nvec);
+      launch_fp64_digits(c, grid, s, d.dg, d.tasks, d.groups, f.tiles, t0, xv, yv, xs, ys, f.part, f.psize, nvec);
     else if (c == 0)
       k_tasks_fp64<C0_NT, C0_ACC, C0_TR, C0_TC><<<grid, C0_NT, fp64_smem(C0_TR, C0_TC), s>>>(
           d.tasks, d.groups, f.tiles, t0, xv, yv, xs, ys, f.part, f.psize, nvec);
@@ -1573,7 +1569,7 @@ void CudaBackend::enqueue_fp64(const DevList& d, int dig, int v, const double* x
       k_tasks_fp64<C3_NT, C3_ACC, C3_TR, C3_TC><<<grid, C3_NT, fp64_smem(C3_TR, C3_TC), s>>>(
           d.tasks, d.groups, f.tiles, t0, xv, yv, xs, ys, f.part, f.psize, nvec);
     launches++;
-    note(cudaGetLastError(), dig ? "k_tasks_dg" : "k_tasks_fp64");
+    note(cudaGetLastError(), dig ? "k_tasks_im" : "k_tasks_fp64");
   }
   if (fork) {
     for (int i = 0; i < 3; ++i) {
@@ -1664,7 +1660,6 @@ void CudaBackend::run(const TaskList& tl, const double* xv, double* yv, int nvec
   }
   // the FP64 kernel: the one asked for, else digits where the list and the call allow them
   const int fk = fp64_kernel >= 0 ? fp64_kernel : (precision == 0 && tl.digits) ? 2 : 0;
-  const int dig = fk == 2 ? 1 : 0;
   const int code = precision;  // tuned schedules and graphs are kept per code and vector count
   if (precision == kFp64Fma) precision = 0;
   if (!tl.persistent) {
@@ -1685,9 +1680,9 @@ void CudaBackend::run(const TaskList& tl, const double* xv, double* yv, int nvec
         note(cudaGetLastError(), "k_tasks_dmma");
       }
     } else {
-      plan_variant(tl, tmp, dig, 1);
-      if (ok() && tmp.tasks && tmp.groups && ensure_part(tmp, tmp.fv[dig][1], nvec))
-        enqueue_fp64(tmp, dig, 1, xv, yv, nvec, xs, ys);
+      plan_variant(tl, tmp, 0, 1);
+      if (ok() && tmp.tasks && tmp.groups && ensure_part(tmp, tmp.fv[0][1], nvec))
+        enqueue_fp64(tmp, 0, 1, xv, yv, nvec, xs, ys);
     }
     free_list(tmp);
     return;
@@ -1722,12 +1717,16 @@ void CudaBackend::run(const TaskList& tl, const double* xv, double* yv, int nvec
   const bool tuning = tu.best < 0;
   const bool timing = tuning && tu.step > 0;
   const int v = !tuning ? tu.best : timing ? (tu.step - 1) % nvar : 1;
+  int dig = 0;
   if (precision != 0) {
     if (!prepare_tasks_tc(*this, tl, d, nvec, v, precision)) return;
   } else {
+    if (fk == 2 && digit_images(tl)) {
+      if (!d.fp_tiled[1]) dg_tiles(tl, d);
+      dig = prepare_digits(*this, tl, d, nvec, xs) ? 1 : 0;
+    }
     plan_variant(tl, d, dig, v);
     if (!ok() || !ensure_part(d, d.fv[dig][v], nvec)) return;
-    if (dig && digit_images(tl)) prepare_digits(*this, tl, d, nvec, xs);
   }
   auto enqueue = [&](const double* x, double* y) {
     if (precision != 0)

@@ -1,0 +1,192 @@
+"""FP64 products hold entry by entry and for every magnitude, as an FMA chain does.
+
+H_eff*psi and its adjoint on vectors whose states carry weights over many
+decades, and on vectors and operators near the small end of the FP64 range.
+
+Entries: on a basis of determinants and with density-density integrals alone
+(h_ii and (ii|jj)) every operator that counts is diagonal, so that weakly weighted
+states get their result from weakly weighted entries and nothing larger hides its
+error; with all integrals their sums have larger terms too.  Each entry is held
+against its own sum S = sum |L| |X| |R|^T (the oracle's heff_apply_abs).  A sum
+of n terms by FMAs is within n 2^-53 S, and its roundings add up like random
+ones; the lists here have at most some 4,000 products, sqrt(4000) 2^-53 = 2^-47,
+so two such evaluations are within 2^-45 S.
+
+Magnitudes: without an underflow every FP64 operation commutes with powers of
+two, so the product of 2^-p x is compared with 2^-p times the product of x.
+"""
+import os
+
+import numpy as np
+import pytest
+
+import synth
+from oracle import dmrg as O3
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2305_05581_gb300 import Context, DEFAULT_LIB, TNS_FP64, blocks_to_vector, vector_to_blocks  # noqa: E402
+from paper_2305_05581_gb300.autograd import arena_tensor  # noqa: E402
+
+TOL_ENTRY = 2.0 ** -45
+TOL = 1e-13  # of the result's norm: two FP64 evaluations of a few thousand products of up to 100 x 100 terms
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    if not os.path.exists(DEFAULT_LIB):
+        from paper_2305_05581_gb300 import build as b
+        b.build()
+
+
+def _ctx(kernel, N, n, s2, D, k, h, v, bonds, sites):
+    if kernel:
+        os.environ["TNS_FP64_KERNEL"] = kernel
+    try:
+        ctx = Context(device=0, stream=torch.cuda.current_stream().cuda_stream)
+    finally:
+        os.environ.pop("TNS_FP64_KERNEL", None)
+    ctx.load_integrals(h, v)
+    ctx.mps_import(N, n, s2, D, bonds, sites)
+    ctx.build_env(k)
+    return ctx
+
+
+def _determinants(N, n, s2, k):
+    """A random MPS with the blocks beside the step replaced by 0/1 isometries: every left and right state is one
+    determinant."""
+    bonds, sites = synth.random_mps(N, n, s2, 10 ** 6, center=k, seed=1)
+    for b in range(N):
+        left, right = dict(bonds[b]), dict(bonds[b + 1])
+        if b < k:
+            for qr, dr in bonds[b + 1]:
+                keys = [((qr[0] - a, qr[1] - c), s) for s, (a, c) in enumerate(synth.SITE_QN)]
+                at = 0
+                for key in keys:
+                    if key[0] in left:
+                        sites[b][key] = np.ascontiguousarray(np.eye(dr)[at:at + left[key[0]]])
+                        at += left[key[0]]
+                assert at == dr
+        elif b > k + 1:
+            for ql, dl in bonds[b]:
+                at = 0
+                for s, (a, c) in enumerate(synth.SITE_QN):
+                    qr = (ql[0] + a, ql[1] + c)
+                    if qr in right:
+                        sites[b][(ql, s)] = np.ascontiguousarray(np.eye(dl)[:, at:at + right[qr]])
+                        at += right[qr]
+                assert at == dl
+    return bonds, sites
+
+
+@pytest.fixture(scope="module", params=[(8, 8, 0, 3, True), (10, 9, 1, 4, True), (8, 8, 0, 3, False)],
+                ids=["N8_density", "N10_density", "N8"])
+def determinants(request):
+    N, n, s2, k, density = request.param
+    h, v = synth.integrals(N, 3.0, 5)
+    if density:
+        i = np.arange(N)
+        keep = np.zeros_like(v)
+        keep[i[:, None], i[:, None], i[None], i[None]] = 1.0
+        h, v = np.diag(np.diag(h)), v * keep
+    bonds, sites = _determinants(N, n, s2, k)
+    heff = O3.DenseHeff(O3.Integrals(h, v), bonds, sites, k, n, s2)
+    yield (N, n, s2, 10 ** 6, k, h, v, bonds, sites), heff, synth.psi_keys(bonds, N, n, s2, k)
+
+
+def _graded(keys, decades):
+    """Gaussian blocks whose left and right states carry weights over that many decades each."""
+    rng = np.random.default_rng(11)
+    wl, wr, out = {}, {}, {}
+    for key, (m, n) in keys:
+        wl.setdefault(key[0], 10.0 ** (-decades * rng.random(m)))
+        wr.setdefault(key[3], 10.0 ** (-decades * rng.random(n)))
+        out[key] = rng.standard_normal((m, n)) * wl[key[0]][:, None] * wr[key[3]][None]
+    return out
+
+
+def _apply(ctx, k, x):
+    y = torch.empty_like(x)
+    ctx.heff_apply_ptr(k, x.data_ptr(), y.data_ptr(), x.shape[0], TNS_FP64)
+    torch.cuda.synchronize()
+    return y
+
+
+def _entries_hold(desc, got, want, bound):
+    got, want = vector_to_blocks(desc, got), vector_to_blocks(desc, want)
+    for q in bound:
+        err = np.abs(got[q] - want[q])
+        assert np.all(err <= TOL_ENTRY * bound[q]), (q, float(np.max(err / np.maximum(bound[q], 1e-300))))
+
+
+@pytest.mark.parametrize("decades", [4, 9])
+def test_entries_of_the_adjoint(determinants, decades):
+    """Xbar = H_eff Ybar for a symmetric H_eff, so the same sums bound it."""
+    system, heff, keys = determinants
+    k = system[4]
+    Y = _graded(keys, decades)
+    ctx, ref = _ctx(None, *system), _ctx("dfma", *system)
+    desc, length = ctx.psi_layout(k)
+    x = torch.tensor(blocks_to_vector(desc, length, _graded(keys, 0)), device="cuda")
+    yb = torch.tensor(blocks_to_vector(desc, length, Y), device="cuda")
+    out = []
+    for c in (ctx, ref):
+        xb = torch.zeros_like(x)
+        c.heff_adjoint_ptr(k, x.data_ptr(), yb.data_ptr(), xb.data_ptr(), 0, 0)
+        torch.cuda.synchronize()
+        out.append(xb.cpu().numpy())
+    _entries_hold(desc, out[0], out[1], heff.apply_abs(Y))
+
+
+SYSTEMS = [(8, 8, 0, 256, 3, 0), (13, 13, 1, 260, 6, 3)]
+
+
+def _random(system):
+    N, n, s2, D, k, ms = system
+    h, v = synth.integrals(N, 3.0, 60 + N)
+    bonds, sites = synth.random_mps(N, n, s2, D, center=k, seed=k, max_sectors=ms)
+    return (N, n, s2, D, k, h, v, bonds, sites)
+
+
+def _close(a, b):
+    return float(torch.linalg.norm(a - b)) <= TOL * float(torch.linalg.norm(b))
+
+
+UP = 2.0 ** 400  # brings results back where their norms do not underflow
+
+
+def _small(desc, x, p, part):
+    """2^-p x; with part > 1 only one block in `part`, and the others at 2^-(p - 40)."""
+    x = x.clone()
+    for i, row in enumerate(desc):
+        m, n, off = (int(v) for v in row[6:9])
+        x[:, off:off + m * n] *= 2.0 ** -(p if i % part == 0 else p - 40)
+    return x
+
+
+MAGNITUDES = pytest.mark.parametrize("p,part", [(430, 1), (714, 1), (764, 1), (960, 1), (764, 4), (960, 4)])
+
+
+@pytest.mark.parametrize("system", SYSTEMS)
+@MAGNITUDES
+def test_small_vectors_in_the_adjoint(system, p, part):
+    args = _random(system)
+    k = args[4]
+    grads = []
+    for kernel in (None, "dfma"):
+        c = _ctx(kernel, *args)
+        desc, length = c.psi_layout(k)
+        g = torch.Generator(device="cuda").manual_seed(7)
+        x = torch.randn(1, length, device="cuda", dtype=torch.float64, generator=g)
+        small = _small(desc, x, p, part)
+        res = [torch.zeros(length, device="cuda", dtype=torch.float64)]
+        res += [torch.zeros_like(arena_tensor(c, k, side)) for side in (0, 1)]
+        c.heff_adjoint_ptr(k, x.data_ptr(), small.data_ptr(), *(r.data_ptr() for r in res))
+        torch.cuda.synchronize()
+        assert all(float(r.abs().max()) > 0 for r in res)
+        grads.append(res)
+    for u, w in zip(*grads):
+        assert _close(u * UP, w * UP)
