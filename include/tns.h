@@ -43,7 +43,8 @@ extern "C" {
 #define TNS_ERR_CUDA (-6)           /* a CUDA runtime call failed */
 
 /* arithmetic of the sector GEMMs in tns_heff_apply */
-#define TNS_FP64 0    /* FP64: exact digit products on the f16 tensor cores where a list's rounding is free, else DFMA */
+#define TNS_FP64 0    /* FP64: every entry of Y within the rounding error bound of FP64 FMA chains, n 2^-53 sum |L||X||R|^T;
+                         by digit products on the f16 tensor cores where each piece is checked to hold it, else DFMA */
 #define TNS_TF32 1    /* TF32 operands, FP32 accumulation (tcgen05 kind::tf32; mma.sync m16n8k8 for blocks <= 32) */
 #define TNS_BF16X3 2  /* split-BF16 hi/lo, 3 products, FP32 accumulation (tcgen05 kind::f16; mma.sync m16n8k16) */
 

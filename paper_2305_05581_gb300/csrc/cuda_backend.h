@@ -41,17 +41,17 @@ struct DgClass {
   int a, b, km, ctas;
 };
 constexpr int kDgClasses = 3;
-constexpr DgClass kDgClass[kDgClasses] = {{16, 16, 16, 12}, {32, 32, 32, 4}, {64, 64, 32, 2}};
+constexpr DgClass kDgClass[kDgClasses] = {{16, 16, 16, 12}, {32, 32, 32, 4}, {64, 56, 32, 2}};
 cudaError_t fp64_digits_init();
 class CudaBackend;
 struct DevList;
 struct Tile;
 bool prepare_digits(CudaBackend& be, const TaskList& tl, DevList& d, int nvec, long long length);
-void enqueue_digit_vectors(CudaBackend& be, const DevList& d, const double* xv, long long xs, int nvec);
+void enqueue_digit_vectors(CudaBackend& be, const DevList& d, const double* xv, long long xs, int nvec, int* failed);
 void release_digit_plan(void* plan);
 void launch_fp64_digits(int cls, unsigned grid, cudaStream_t s, const void* plan, const Task* tasks,
                         const Group* groups, const Tile* tiles, int tile0, const double* xv, double* yv, long long xs,
-                        long long ys, double* part, long long psize, int nv);
+                        long long ys, double* part, long long psize, int nv, int* nfailed, int* failed);
 
 struct SplitRed {  // a split tile: sum of nsplit partial tiles (fixed order) -> output
   int g;
@@ -84,6 +84,8 @@ struct FpVariant {
   long long psize = 0;       // partial-tile elements per vector
   double* part = nullptr;    // partial tiles (psize * part_nvec)
   int part_nvec = 0;
+  int* failed = nullptr;     // digit classes: how many pieces have no certificate (4 ints), then which
+  int failed_nvec = 0;
 };
 
 // online autotuner state of one (precision, nvec) use of a work list: the
@@ -103,6 +105,10 @@ constexpr int kTuneRounds = 2;
 // stays unless another needs less than kSteady of its time, so that a few
 // per cent of timing noise do not decide where an unconverged solve ends.
 constexpr double kSteady = 0.8;
+// A digit product takes 0.3 to 0.7 of the FMA kernel's time, and what has no
+// certificate is done again by that kernel: beyond a third the sum is no gain
+// (24 orbitals, D = 512, all sectors: 21 ms and a tenth of 36.5 ms again).
+constexpr double kFailedShare = 0.2;
 constexpr int kSteadyKey = 1 << 16;  // schedules and graphs of such products are kept apart
 
 // captured launch sequence of one (precision, nvec) use: replayed with the
@@ -134,6 +140,7 @@ struct DevList {
   // digit images of the list (fp64_digits.cu); dg_none: they cannot be had
   void* dg = nullptr;
   bool dg_none = false;
+  bool dg_kept = false;  // the first product's certificates held (kFailedShare)
   std::vector<unsigned char> dg_aside;  // per group: the tiles' a side
   // tensor-core form (precision != FP64)
   void* tc = nullptr;
@@ -237,6 +244,7 @@ class CudaBackend : public Backend {
 
  private:
   int device_;
+  int sms_ = 152;
   cudaStream_t stream_;
   bool own_;
   std::string err_;
@@ -251,9 +259,10 @@ class CudaBackend : public Backend {
   cudaStream_t fstream_[3] = {nullptr, nullptr, nullptr};
   cudaEvent_t fev_[4] = {nullptr, nullptr, nullptr, nullptr};
   bool fork_ready();
+  double failed_share(const FpVariant& f, int nvec);
   void upload_list(const TaskList& tl, DevList& d);
   void plan_variant(const TaskList& tl, DevList& d, int dig, int v);
-  bool ensure_part(DevList& d, FpVariant& f, int nvec);
+  bool ensure_part(DevList& d, FpVariant& f, int dig, int nvec);
   void free_list(DevList& d);
   template <class F>
   void launch_graphed(DevList& d, int key, const double* xv, double* yv, int nvec, long long xs, long long ys,

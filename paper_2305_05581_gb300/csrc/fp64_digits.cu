@@ -11,11 +11,29 @@
 // digits are at most 2^14; a sum over K = 32 of the pairs of equal weight
 // s = i + j (at most 7 of them) stays below 2^22, so it is an exact integer in
 // an FP32 accumulator that starts at 1.5 * 2^23, read off its mantissa without
-// a conversion.  The pairs with s <= 7 are kept (34 of them).  On Gaussian,
-// diagonal-dominant and graded operands the result is closer to the exact one
-// than a chain of FP64 FMAs (0.3 to 0.9 of its error; without the pairs of
-// s = 7 it can be twice as far).
+// a conversion.  The pairs with s <= 7 are kept (34 of them).
 // The eight integers of an output are put together in a 64-bit integer.
+//
+// Digits hold an entry to 2^-56 of its row's largest, an FMA chain to 2^-53 of
+// itself: norms come out as exact as the chain's, but an output that hangs on
+// small entries alone (a weakly weighted state behind a diagonal operator) would
+// not.  So every piece of a tile carries a certificate: for each output a lower
+// bound S of sum |alpha||L||X||R| and an upper bound E of what the digits left
+// out, both kept with the sums.  Where E exceeds the rounding errors that an FMA
+// chain may make in the same products, sum (K + L) 2^-53 S (K and L the lengths
+// of the two contractions), the piece is given to the FMA kernel, which runs
+// behind this one (k_tasks_fp64_failed).  S comes from one more digit pair: the
+// leading digits' magnitudes less a half.  E is, in units of 2^-56 of the
+// scales of A's and B's rows and X's block,
+//     sum_k |b_k| (sum_l |x_kl| + 0.033 L + rounding of T's sums)    A's last digit, dropped pairs
+//   + sum_k |t_k| + max |t| (0.05 K + 0.6)                           B's last digit, T's last bits, dropped pairs
+// with |a|, |b|, |x| < 1 after scaling (magnitudes of rows of X are summed where
+// they are cut).  On dense operators S (K + L) 8 is 5 to 50 times E; with
+// states weighted over three decades 1 of 400 pieces fails (24 orbitals, D = 512
+// in 9 sectors), where blocks have few states one of ten (the same, all sectors).
+// Magnitudes that the fixed-point form cannot hold (infinities, NaN, vector
+// entries of 2^330 and more or blocks below 2^-700, operators of 2^50 and more,
+// rows or products far below the rest) are failures like any other.
 //
 // One CTA owns one output tile of one block and walks the block's products in
 // a fixed order, as the DFMA classes do.  With A the operand of the tile's
@@ -28,21 +46,17 @@
 // again and used from registers.
 //
 // The digits are cut beforehand (images, below), so the kernel is for lists that
-// are kept; lists that run once or have no room for images, and the adjoint,
-// whose operands change between calls, stay with the FMA kernel.  The kernel is
-// bound by the integer work around the MMAs (joining the weight sums, cutting T)
-// and by the 8 to 12 warps that registers and shared memory leave an SM to hide
-// its latencies (MMA pipe 30 % busy, issue slots 27 to 49 %).  One H_eff*psi,
-// DFMA tile classes -> here (time, useful rate):
-//   24 orbitals, D = 512, all sectors (blocks <= 26):  36.4 -> 14.9 ms, 1.15 TFLOP/s
-//   24 orbitals, D = 512, 9 sectors (blocks <= 68):     153 -> 47.4 ms, 2.45 TFLOP/s
-//   13 orbitals, D = 260, 3 sectors (blocks <= 99):    3.03 -> 0.78 ms, 2.81 TFLOP/s
+// are kept; lists that run once or have no room for images, lists whose first
+// product fails in more than a fifth of its work, and the adjoint, whose operands
+// change between calls, stay with the FMA kernel.  The kernel is bound by the
+// integer work around the MMAs (joining the weight sums, cutting T) and by the 8
+// to 12 warps that registers and shared memory leave an SM to hide its latencies.
+// One H_eff*psi, DFMA tile classes -> here (time, useful rate; in brackets
+// without certificates):
+//   24 orbitals, D = 512, all sectors (blocks <= 26):  36.4 -> 23.9 ms, 0.72 TFLOP/s [15.9]
+//   24 orbitals, D = 512, 9 sectors (blocks <= 68):     153 -> 51 ms, 2.3 TFLOP/s    [47]
+//   13 orbitals, D = 260, 3 sectors (blocks <= 99):    3.03 -> 0.90 ms, 2.4 TFLOP/s  [0.78]
 // (cuBLAS DGEMM: 1.10 TFLOP/s).
-//
-// Values that the fixed-point form cannot hold: a product in which an operand
-// has an infinity, a NaN or a magnitude of 2^330 or more is evaluated with
-// plain FP64 FMAs instead; rows whose largest magnitude is below 2^-700 are
-// taken relative to 2^-700.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -57,8 +71,11 @@ namespace {
 constexpr int DG_N = 7;                        // digits of an operand
 constexpr int DG_S = 8;                        // weights s = i + j kept: 0 .. 7
 constexpr unsigned DG_MAGIC = 0x4B400000u;     // bits of 1.5 * 2^23
-constexpr int DG_EMIN = 322;                   // smallest biased exponent of a row scale (2^-700)
-constexpr int DG_EMAX = (1023 + 330) << 20;    // high word from which on a value leaves the fixed-point form
+constexpr float DG_LIMIT = 0.96f * 8.f;        // 2^-53 in units of 2^-56, less the roundings of the certificate itself
+constexpr int DG_EMIN = 322;                   // smallest scale of a vector block (2^-700)
+constexpr int DG_DEPTH = 60;                   // rows' scales are at most this far below 1 (operators) or their block's (vectors)
+constexpr int DG_EMAX = (1023 + 330) << 20;    // high word from which on a vector entry leaves the fixed-point form
+constexpr int DG_OPMAX = (1023 + 50) << 20;    // the same for an operator entry (ranges of the certificate)
 
 __device__ __forceinline__ uint32_t sm_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -141,6 +158,7 @@ constexpr int IM_UNIT = DG_N * 128;  // bytes of one 8 x 8 unit of an operator
 constexpr int IM_NX = 8;             // digits of the vector and of T
 constexpr int IM_XUNIT = IM_NX * 128;
 constexpr int IM_SLOW = 0x7fffffff;  // scale of a block that the fixed-point form cannot hold
+constexpr int IM_ZERO = 0;           // scale of a block of zeros
 
 __host__ __device__ inline int im_oct(int cols) { return (cols + 15) / 16 * 2; }
 __host__ __device__ inline int im_head(int rows) { return ((rows + 7) / 8 * 8 * 4 + 127) / 128 * 128; }
@@ -148,11 +166,15 @@ __host__ __device__ inline long long im_bytes(int rows, int cols) {
   return im_head(rows) + (long long)((rows + 7) / 8) * im_oct(cols) * IM_UNIT;
 }
 
+// an image of a vector block has the sums of its rows' magnitudes (floats, in
+// units of the rows' scales) between the scales and the digits
+__host__ __device__ inline int im_xhead(int rows) { return 2 * im_head(rows); }
+
 struct DgRec {  // a product in the orientation of its tile
   uint32_t a, b, x;  // images of A (rows a) and B (rows b) in the operator arena, of X in the vector arena; 128-byte units
   int xb;            // scale index of X
   double alpha;
-  int K, L, f, pad;  // f: 1 A is the identity, 2 B is, 4 an operand does not fit the fixed-point form
+  int K, L, f, pad;  // f: 1 A is the identity, 2 B is, 4 an operator does not fit the fixed-point form
 };
 struct DgImage {  // an operand to cut: op(M) is rows x cols, element (r, c) = src[r * sr + c * sc]
   const double* src;
@@ -196,34 +218,56 @@ __device__ __forceinline__ void im_cut(const double (&x)[8], int E, unsigned cha
 #undef IM_PUT
 }
 
-__device__ __forceinline__ int im_scale(int mx) { return max((mx + 0x2100) >> 20, DG_EMIN); }
+__device__ __forceinline__ int im_scale(int mx, int least) { return max((mx + 0x2100) >> 20, least); }
+// the scale of a row of zeros where the largest is top: 2^(it - top), as the bits of a float, is 0
+__device__ __forceinline__ int im_none(int top) { return top - 127; }
+__device__ __forceinline__ float im_pow2(int e) { return __uint_as_float((uint32_t)(e + 127) << 23); }  // -127 <= e <= 127
+constexpr int IM_ONE = 1022;  // the scale of magnitudes below 1
+
+// high word of a magnitude, at least 1 where the value is not zero
+__device__ __forceinline__ int im_high(double x) {
+  return (__double2hiint(x) & 0x7fffffff) | (__double2loint(x) != 0 ? 1 : 0);
+}
 
 // the image of a matrix by a CTA of 4 warps, a warp per group of 8 rows: the
-// rows' scales, then their digits; returns the largest high word seen
+// rows' scales (and sums, for a vector block), then their digits; returns the
+// largest high word seen
 template <int N>
 __device__ __forceinline__ int im_rows(const double* __restrict__ src, int rows, int cols, int sr, int sc, int groups,
-                                       unsigned char* img) {
+                                       int top_scale, int least, unsigned char* img) {
   const int oc = im_oct(cols), lane = threadIdx.x & 31, warp = threadIdx.x >> 5, r7 = lane & 7, q = lane >> 3;
   int* scale = (int*)img;
-  unsigned char* units = img + im_head(8 * groups);
+  unsigned char* units = img + (N == IM_NX ? im_xhead(8 * groups) : im_head(8 * groups));
   int top = 0;
   for (int rg = warp; rg < groups; rg += 4) {
     const int row = 8 * rg + r7;
     int mx = 0;
     if (row < rows)
       for (int c = q; c < cols; c += 4)
-        mx = max(mx, __double2hiint(__ldg(src + (long long)row * sr + (long long)c * sc)) & 0x7fffffff);
+        mx = max(mx, im_high(__ldg(src + (long long)row * sr + (long long)c * sc)));
     mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
     mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
     top = max(top, mx);
-    const int E = im_scale(mx);
-    if (q == 0) scale[row] = E;
+    const int E = im_scale(mx, least);
+    if (q == 0) scale[row] = mx ? E : im_none(top_scale);
+    float sum = 0.f;
     for (int o = q; o < oc; o += 4) {
       double x[8];
 #pragma unroll
       for (int e = 0; e < 8; ++e)
         x[e] = (row < rows && 8 * o + e < cols) ? __ldg(src + (long long)row * sr + (long long)(8 * o + e) * sc) : 0.0;
       im_cut<N>(x, E, units + ((long long)rg * oc + o) * (N * 128) + r7 * 16);
+      if (N == IM_NX)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {  // 1.m 2^(exponent - E), rounded up
+          const int h = im_high(x[e]);
+          if (h) sum += __uint_as_float((uint32_t)max((h >> 20) - E + 126, 1) << 23 | (uint32_t)(h & 0xfffff) << 3 | 7u);
+        }
+    }
+    if (N == IM_NX) {
+      sum += __shfl_xor_sync(0xffffffffu, sum, 8);
+      sum += __shfl_xor_sync(0xffffffffu, sum, 16);
+      if (q == 0) ((float*)(img + im_head(8 * groups)))[row] = sum;
     }
   }
   return top;
@@ -231,26 +275,32 @@ __device__ __forceinline__ int im_rows(const double* __restrict__ src, int rows,
 
 __global__ void __launch_bounds__(128) k_dg_ops(DgImage* __restrict__ jobs, unsigned char* arena) {
   DgImage& J = jobs[blockIdx.x];
-  if (im_rows<DG_N>(J.src, J.rows, J.cols, J.sr, J.sc, (J.rows + 7) / 8, arena + (long long)J.off * 128) >= DG_EMAX)
+  if (im_rows<DG_N>(J.src, J.rows, J.cols, J.sr, J.sc, (J.rows + 7) / 8, IM_ONE, IM_ONE - DG_DEPTH,
+                    arena + (long long)J.off * 128) >= DG_OPMAX)
     J.slow = 1;
 }
 
-// vector images: one CTA per block, orientation and vector
+// vector images: one CTA per block, orientation and vector.  The first one
+// clears the counts of pieces without a certificate, whose kernels come later.
 __global__ void __launch_bounds__(128) k_dg_x(const DgXBlock* __restrict__ blocks, int nblk, const double* xv,
-                                              long long xs, unsigned char* arena, long long xbytes, int* scales) {
+                                              long long xs, unsigned char* arena, long long xbytes, int* scales,
+                                              int* failed) {
   const DgXBlock B = blocks[blockIdx.x];
   const double* X = xv + (long long)blockIdx.y * xs + B.src;
   unsigned char* img = arena + (long long)blockIdx.y * xbytes + (long long)B.off * 128;
   const int n = B.rows * B.cols;
   __shared__ int red[4];
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kDgClasses) failed[threadIdx.x] = 0;
   int mx = 0;
-  for (int e = threadIdx.x; e < n; e += 128) mx = max(mx, __double2hiint(X[e]) & 0x7fffffff);
+  for (int e = threadIdx.x; e < n; e += 128) mx = max(mx, im_high(X[e]));
   mx = __reduce_max_sync(0xffffffffu, mx);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
   __syncthreads();
   mx = max(max(red[0], red[1]), max(red[2], red[3]));
-  if (threadIdx.x == 0) scales[(long long)blockIdx.y * nblk + blockIdx.x] = mx >= DG_EMAX ? IM_SLOW : im_scale(mx);
-  im_rows<IM_NX>(X, B.rows, B.cols, B.sr, B.sc, (B.rows + 15) / 16 * 2, img);  // GEMM1 takes X in pairs of row groups
+  const int ex = im_scale(mx, DG_EMIN);
+  if (threadIdx.x == 0) scales[(long long)blockIdx.y * nblk + blockIdx.x] = mx == 0 ? IM_ZERO : mx >= DG_EMAX ? IM_SLOW : ex;
+  // GEMM1 takes X in pairs of row groups
+  im_rows<IM_NX>(X, B.rows, B.cols, B.sr, B.sc, (B.rows + 15) / 16 * 2, ex, max(ex - DG_DEPTH, DG_EMIN), img);
 }
 
 // ---- planning on the device: distinct operands by a hash table of (address,
@@ -336,7 +386,7 @@ __global__ void k_dg_find(const Task* __restrict__ tasks, const Group* __restric
       B.cols = o ? t.m : t.n;
       B.sr = o ? 1 : t.n;
       B.sc = o ? t.n : 1;
-      B.off = (uint32_t)atomicAdd(&st->xunits, (unsigned long long)((im_head((B.rows + 15) / 16 * 16) + (B.rows + 15) / 16 * 2 * im_oct(B.cols) * IM_XUNIT) / 128));
+      B.off = (uint32_t)atomicAdd(&st->xunits, (unsigned long long)((im_xhead((B.rows + 15) / 16 * 16) + (B.rows + 15) / 16 * 2 * im_oct(B.cols) * IM_XUNIT) / 128));
       B.pad = 0;
       xblocks[j] = B;
       *slot = j + 1;
@@ -392,18 +442,46 @@ __global__ void k_dg_records(const Task* __restrict__ tasks, const Group* __rest
   }
 }
 
-template <int W_, int NBT_, int LK_, int KM_, int CTAS_>
+// lower bounds of the magnitudes of two entries from their leading digits: the
+// digits below it make up less than half of one
+__device__ __forceinline__ uint32_t dg_low(uint32_t d) {
+  const __half2 v = __hmax2(__hsub2(__habs2(*(const __half2*)&d), __floats2half2_rn(0.5f, 0.5f)), __floats2half2_rn(0.f, 0.f));
+  return *(const uint32_t*)&v;
+}
+// their magnitudes, and upper bounds of them
+__device__ __forceinline__ uint32_t dg_abs(uint32_t d) { return d & 0x7fff7fffu; }
+__device__ __forceinline__ uint32_t dg_high(uint32_t d) {
+  const __half2 v = __hadd2(__habs2(*(const __half2*)&d), __floats2half2_rn(0.51f, 0.51f));
+  return *(const uint32_t*)&v;
+}
+__device__ __forceinline__ uint32_t dg_pack(float x, float y) {
+  const __half2 v = __floats2half2_rn(x, y);
+  return *(const uint32_t*)&v;
+}
+__device__ __forceinline__ uint32_t dg_mul(uint32_t x, uint32_t y) {
+  const __half2 v = __hmul2(*(const __half2*)&x, *(const __half2*)&y);
+  return *(const uint32_t*)&v;
+}
+// s plus two floats, at most 2^15
+__device__ __forceinline__ uint32_t dg_more(uint32_t s, float x, float y) {
+  const __half2 m = __floats2half2_rn(32768.f, 32768.f);
+  const __half2 v = __hmin2(__hadd2(*(const __half2*)&s, __floats2half2_rn(fminf(x, 32768.f), fminf(y, 32768.f))), m);
+  return *(const uint32_t*)&v;
+}
+
+template <int W_, int NBT_, int DBT_, int LK_, int KM_, int CTAS_>
 struct ImCfg {
-  static constexpr int W = W_, NBT = NBT_, LK = LK_, KM = KM_, CTAS = CTAS_;
+  static constexpr int W = W_, NBT = NBT_, DBT = DBT_, LK = LK_, KM = KM_, CTAS = CTAS_;
   static constexpr int NT = 32 * W, AR = 16 * W, BR = 8 * NBT;
   static constexpr int LO = LK / 8, KO = KM / 8;              // octets staged
-  static constexpr int off_x = (AR / 8) * LO * IM_XUNIT;      // X after A (or the vector in its place) in the first slot
+  static constexpr int off_x = (AR / 8) * LO * IM_UNIT;       // X after A in the first slot; a vector in A's place takes both
   static constexpr int off_b = off_x + (KM / 8) * LO * IM_XUNIT;
   static constexpr int off_y = off_b + NBT * KO * IM_UNIT;    // the tile's sums
-  static constexpr int off_e = off_y + AR * BR * 8;           // row scales of A, B and X
-  static constexpr int total = off_e + 4 * (AR + BR + KM);
+  static constexpr int off_d = off_y + AR * BR * 8;           // their certificates; beyond DBT tiles one per two columns
+  static constexpr int off_e = off_d + AR * (8 * DBT * 4 + 8 * (NBT - DBT) * 2);           // row scales of A, B and X, row sums of X
+  static constexpr int total = off_e + 4 * (AR + BR + 2 * KM);
   static_assert(CTAS * (total + 1024) <= 228 * 1024, "resident CTAs");
-  static_assert(KM == LK && off_b >= AR * BR * 8, "chunks; the first slot holds a tile of FP64 values");
+  static_assert(KM == LK && off_b >= (AR / 8) * LO * IM_XUNIT, "chunks; the first slot holds the vector in A's place");
 };
 
 __device__ __forceinline__ void cp16(uint32_t dst, const void* src) {
@@ -412,11 +490,12 @@ __device__ __forceinline__ void cp16(uint32_t dst, const void* src) {
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
-// `rows` runs of n 16-byte pieces, a warp per run.  Out of line: the kernel has
-// ten such copies, and inlined they are a third of the code that its warps
-// fetch again for every product.
+// `rows` runs of n 16-byte pieces, a warp per run.  Out of line in the CTAs of
+// several warps: the kernel has ten such copies, and inlined they are a third of
+// the code that its warps fetch again for every product.  The one-warp class has
+// no registers to spare for what a call leaves to its caller.
 template <int W>
-__device__ __noinline__ void im_copy(uint32_t dst, const unsigned char* src, int n, int rows, int sstride, int dstride) {
+__device__ __forceinline__ void im_copy_body(uint32_t dst, const unsigned char* src, int n, int rows, int sstride, int dstride) {
   const int warp = W == 1 ? 0 : threadIdx.x >> 5, lane = threadIdx.x & 31;
   src += (long long)warp * sstride + lane * 16;
   dst += (uint32_t)(warp * dstride + lane * 16);
@@ -426,13 +505,23 @@ __device__ __noinline__ void im_copy(uint32_t dst, const unsigned char* src, int
     dst += W * dstride;
   }
 }
+template <int W>
+__device__ __noinline__ void im_copy_call(uint32_t dst, const unsigned char* src, int n, int rows, int sstride, int dstride) {
+  im_copy_body<W>(dst, src, n, rows, sstride, dstride);
+}
+template <int W>
+__device__ __forceinline__ void im_copy(uint32_t dst, const unsigned char* src, int n, int rows, int sstride, int dstride) {
+  if constexpr (W == 1) im_copy_body<W>(dst, src, n, rows, sstride, dstride);
+  else im_copy_call<W>(dst, src, n, rows, sstride, dstride);
+}
 
 template <class C>
 __global__ void __launch_bounds__(C::NT, C::CTAS)
     k_tasks_im(const DgRec* __restrict__ recs, const Task* __restrict__ tasks, const Group* __restrict__ groups,
                const Tile* __restrict__ tiles, int tile0, const unsigned char* __restrict__ ops,
                const unsigned char* __restrict__ xin, long long xbytes, const int* __restrict__ xscale, int nxb,
-               const double* xv, double* yv, long long xs, long long ys, double* part, long long psize, int nv) {
+               const double* xv, double* yv, long long xs, long long ys, double* part, long long psize, int nv,
+               int* nfailed, int* failed) {
   constexpr int W = C::W, NBT = C::NBT, LK = C::LK, KM = C::KM, NT = C::NT, LO = C::LO, KO = C::KO;
   constexpr int KT = KM / 8;
   extern __shared__ __align__(128) unsigned char sm[];
@@ -440,7 +529,8 @@ __global__ void __launch_bounds__(C::NT, C::CTAS)
   const int* const eA = (const int*)(sm + C::off_e);
   const int* const eB = eA + C::AR;
   const int* const eX = eB + C::BR;
-  const uint32_t sEA = sm_u32(eA), sEB = sm_u32(eB), sEX = sm_u32(eX);
+  const float* const xsum = (const float*)(eX + KM);
+  const uint32_t sEA = sm_u32(eA), sEB = sm_u32(eB), sEX = sm_u32(eX), sXS = sm_u32(xsum);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
   const int mj = lane >> 3, mr16 = (lane & 7) * 16;
   const Tile TL = tiles[tile0 + blockIdx.x / nv];
@@ -459,21 +549,23 @@ __global__ void __launch_bounds__(C::NT, C::CTAS)
   // tiles rolled (unrolled over registers its code missed the instruction
   // cache) and 8 NBT registers free
   double2* const Ys = (double2*)(sm + C::off_y) + warp * (NBT * 64) + lane;
+  constexpr int DBT = C::DBT;
+  float2* const Ds = (float2*)(sm + C::off_d) + warp * (DBT * 64) + lane;
+  float* const Dp = (float*)(sm + C::off_d + W * DBT * 64 * 8) + (warp * (NBT - DBT) - DBT) * 64 + lane;
   auto sync = [&]() {
     if (W == 1) __syncwarp();
     else __syncthreads();
   };
-  // alpha 2^n; below 2^-1000 only rows of zeros meet rows of zeros
-  auto scale = [](double alpha, int n) { return alpha * __hiloint2double((max(n, -1000) + 1023) << 20, 0); };
+  auto scale = [](double alpha, int n) { return alpha * __hiloint2double((n + 1023) << 20, 0); };  // alpha 2^n
   // the row groups this CTA never copies (a tile of fewer rows than the slot
   // has) are read by ldmatrix as absent rows: zero once
   for (int i = tid; i < C::total / 16; i += NT) ((uint4*)sm)[i] = make_uint4(0, 0, 0, 0);
   sync();
 
   // row groups rg0 .. rg0 + nrg, octets from o0 (at most mo) of an image with U-byte units
-  auto rows = [&](uint32_t dst, int doct, const unsigned char* img, int img_rows, int cols, int U, int rg0, int nrg, int o0) {
+  auto rows = [&](uint32_t dst, int doct, const unsigned char* img, int head, int cols, int U, int rg0, int nrg, int o0) {
     const int oc = im_oct(cols), no = min(doct, oc - o0);
-    im_copy<W>(dst, img + im_head(img_rows) + ((long long)rg0 * oc + o0) * U, no * (U / 16), nrg, oc * U, doct * U);
+    im_copy<W>(dst, img + head + ((long long)rg0 * oc + o0) * U, no * (U / 16), nrg, oc * U, doct * U);
   };
   auto scales = [&](uint32_t dst, const unsigned char* img, int row, int groups) {
     for (int i = tid; i < 2 * groups; i += NT) cp16(dst + i * 16, img + (row + 4 * i) * 4);
@@ -484,13 +576,15 @@ __global__ void __launch_bounds__(C::NT, C::CTAS)
     if (f == 3) return;
     const unsigned char* ix = xi + (long long)r.x * 128;
     const unsigned char* ia = f == 1 ? ix : ops + (long long)r.a * 128;  // f == 1: P[a][k] = X^T, rows a of the vector image
-    rows(sA, LO, ia, f == 1 ? (arows + 15) / 16 * 16 : arows, f == 1 ? r.K : r.L, f == 1 ? IM_XUNIT : IM_UNIT, a0 >> 3, arg,
+    rows(sA, LO, ia, f == 1 ? im_xhead((arows + 15) / 16 * 16) : im_head(arows), f == 1 ? r.K : r.L, f == 1 ? IM_XUNIT : IM_UNIT, a0 >> 3, arg,
          (f ? k0 : l0) >> 3);
     scales(sEA, ia, a0, arg);
     if (f == 0) {
       const int kg = ((min(KM, r.K - k0) + 15) >> 4) * 2;
-      rows(sX, LO, ix, (r.K + 15) / 16 * 16, r.L, IM_XUNIT, k0 >> 3, kg, l0 >> 3);
+      const int kr = (r.K + 15) / 16 * 16;
+      rows(sX, LO, ix, im_xhead(kr), r.L, IM_XUNIT, k0 >> 3, kg, l0 >> 3);
       scales(sEX, ix, k0, kg);
+      scales(sXS, ix + im_head(kr), k0, kg);
     }
   };
   // second-slot copy: B (or the vector block in its place, without its last digit), columns from k0
@@ -499,74 +593,101 @@ __global__ void __launch_bounds__(C::NT, C::CTAS)
     const unsigned char* ib = v ? xi + (long long)r.x * 128 : ops + (long long)r.b * 128;
     if (v) {
       const int oc = im_oct(r.L), no = min(KO, oc - (k0 >> 3));
-      const unsigned char* u = ib + im_head((brows + 15) / 16 * 16) + ((long long)(b0 >> 3) * oc + (k0 >> 3)) * IM_XUNIT;
+      const unsigned char* u = ib + im_xhead((brows + 15) / 16 * 16) + ((long long)(b0 >> 3) * oc + (k0 >> 3)) * IM_XUNIT;
       for (int g = 0; g < nbt; ++g)
         im_copy<W>(sB + g * KO * IM_UNIT, u + (long long)g * oc * IM_XUNIT, IM_UNIT / 16, no, IM_XUNIT, IM_UNIT);
     } else {
-      rows(sB, KO, ib, brows, r.K, IM_UNIT, b0 >> 3, nbt, k0 >> 3);
+      rows(sB, KO, ib, im_head(brows), r.K, IM_UNIT, b0 >> 3, nbt, k0 >> 3);
     }
     scales(sEB, ib, b0, nbt);
   };
 
-  DgRec rec, nxt;
+  DgRec rec;
+  bool bad = false;      // an operand or a scale that this form cannot hold (alike in all threads of the CTA, or a lane's own)
+  int ref = INT32_MIN;   // exponent that the certificate is kept relative to: of the first product that is not zero
   if (TL.t0 < TL.t1) {
-    nxt = recs[TL.t0];
-    load1(nxt, 0, 0);
+    load1(recs[TL.t0], 0, 0);
     cp_commit();
   }
   for (int ti = TL.t0; ti < TL.t1; ++ti) {
-    rec = nxt;
+    rec = recs[ti];
     const int ex = xsc[rec.xb];
     const bool more = ti + 1 < TL.t1;
-    if (more) nxt = recs[ti + 1];
+    // the next record waits in L1 (in registers it would cost this product spills)
+    if (more) asm volatile("prefetch.global.L1 [%0];" ::"l"(recs + ti + 1));
     const int f = rec.f & 3;
-    if (f == 3 || (rec.f & 4) || ex == IM_SLOW) {
-      // Y += alpha X, or plain FP64 for what the fixed-point form cannot hold
-      const Task tk = tasks[ti];
-      const double* pX = xv + (long long)vec * xs + (long long)(size_t)tk.X;
-      double* D = (double*)sm;
-      cp_wait();
-      sync();
-      for (int e = tid; e < na * nb; e += NT) {
-        const int a = a0 + e / nb, b = b0 + e % nb, i = bl ? a : b, j = bl ? b : a;
-        double s = 0.0;
-        for (int k = (tk.flags & TF_LI) ? i : 0; k < ((tk.flags & TF_LI) ? i + 1 : tk.m); ++k) {
-          double x = 0.0;
-          if (tk.flags & TF_RI) {
-            x = pX[(long long)k * tk.n + j];
-          } else {
-            for (int l = 0; l < tk.n; ++l)
-              x = fma(pX[(long long)k * tk.n + l], (tk.flags & TF_RT) ? tk.R[(long long)l * tk.r + j] : tk.R[(long long)j * tk.n + l], x);
-          }
-          s = (tk.flags & TF_LI) ? x : fma((tk.flags & TF_LT) ? tk.L[(long long)k * tk.q + i] : tk.L[(long long)i * tk.m + k], x, s);
-        }
-        D[e] = s;
-      }
-      sync();
-      if (mine)
+    const int ea = __double2hiint(rec.alpha) >> 20 & 0x7ff;
+    if ((rec.f & 4) || ex == IM_SLOW || ea == 0x7ff || (ea == 0 && rec.alpha != 0.0)) {
+      bad = true;
+      break;
+    }
+    if (f == 3 || ex == IM_ZERO || ea == 0) {
+      if (mine && ex != IM_ZERO && ea != 0) {  // Y += alpha X, as the FMA kernel does it
+        const Task tk = tasks[ti];
+        const double* pX = xv + (long long)vec * xs + (long long)(size_t)tk.X;
+        const long long sa = bl ? tk.n : 1, sb = bl ? 1 : tk.n;
         for (int b = 0; b < nbt; ++b)
           for (int h = 0; h < 2; ++h) {
             const int a = 16 * warp + g + 8 * h, c = 8 * b + 2 * t;
+            const double* x = pX + (a0 + a) * sa + (b0 + c) * sb;
             double2 v = Ys[(2 * b + h) * 32];
-            if (a < na && c < nb) v.x = fma(rec.alpha, D[a * nb + c], v.x);
-            if (a < na && c + 1 < nb) v.y = fma(rec.alpha, D[a * nb + c + 1], v.y);
+            if (a < na && c < nb) v.x = fma(rec.alpha, x[0], v.x);
+            if (a < na && c + 1 < nb) v.y = fma(rec.alpha, x[sb], v.y);
             Ys[(2 * b + h) * 32] = v;
           }
+      }
+      cp_wait();
       sync();
-      // D lay over the first slot: clear what it held, the images leave absent row groups alone
-      for (int i = tid; i < C::off_b / 16; i += NT) ((uint4*)sm)[i] = make_uint4(0, 0, 0, 0);
-      sync();
-      if (more) load1(nxt, 0, 0);
+      if (more) load1(recs[ti + 1], 0, 0);
       cp_commit();
       continue;
     }
+    if (ref == INT32_MIN) ref = ea + ex;
+    // the certificate's weight of a row with scale e: 2^n times alpha's mantissa, n relative to ref; what lies too far
+    // below counts with its errors alone
+    const float am = __uint_as_float(0x3f800000u | (uint32_t)(__double2hiint(rec.alpha) & 0xfffff) << 3);
+    const int atop = f == 1 ? ex : IM_ONE, btop = f == 2 ? ex : IM_ONE;
+    auto weight = [&](int e) {
+      const int n = ea + ex - ref + e - atop;
+      if (e == im_none(atop)) return 0.f;
+      if (n > 50) bad = true;
+      return am * im_pow2(max(min(n, 50), -60));
+    };
+    auto far = [&](int e) { return e != 0 && e != im_none(atop) && ea + ex - ref + e - atop < -60; };  // 0: no such row
+    // alpha 2^n, the scale of a row of sums; one that underflows (while its sums may not) is for the FMA kernel
+    auto row_scale = [&](int e, int n) {
+      if (e != 0 && ea - 1023 + n < -1000) bad = true;
+      return scale(rec.alpha, n);
+    };
     const int K = f == 2 ? rec.L : rec.K, L = rec.L;
     int hsh = 0;
     while ((32 << hsh) < L) ++hsh;
+    // errors of a T entry beside A's last digits (1 per unit of X's row sum), in
+    // units of 2^-56 of the scales: dropped pairs, X's last bit, the joined sums' roundings
+    const float el = 0.01f + 0.033f * L + (float)((L + LK - 1) / LK) * (hsh ? 0.3f + 0.51f * (float)(1 << hsh) : 0.26f);
+    // a sum may err by K + L units of 2^-53 of its magnitudes
+    const float lim = fminf(DG_LIMIT * (float)(f == 0 ? K + L : K + 1), 4096.f);
+    const float lim14 = lim * 0x1p-14f;
     for (int k0 = 0; k0 < K; k0 += KM) {
       const int kc = min(KM, K - k0);
-      uint32_t tf[KT / 2][IM_NX][4];
+      // T's digits; as f16, in units of 2^-59 of X's scale, what T may err by (lower bounds of sum |A||X|) and what it
+      // errs by (upper bounds)
+      uint32_t tf[KT / 2][IM_NX][4], mt[KT / 2][4], et[KT / 2][2];
+      auto hide = [&](int e0, int e1) {  // no lower bounds for rows too far below
+#pragma unroll
+        for (int kk = 0; kk < KT / 2; ++kk)
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (far(q & 1 ? e1 : e0)) mt[kk][q] = 0u;
+      };
       double s0 = 0.0, s1 = 0.0;
+      float ws0 = 0.f, ws1 = 0.f, wt0 = 0.f, wt1 = 0.f;
+#pragma unroll
+      for (int kk = 0; kk < KT / 2; ++kk) {
+        et[kk][0] = et[kk][1] = 0u;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) mt[kk][q] = 0u;
+      }
       cp_wait();
       sync();  // the first slot is in, the second is free
       load2(rec, k0);
@@ -587,42 +708,59 @@ __global__ void __launch_bounds__(C::NT, C::CTAS)
             sync();
           }
           if (!mine) continue;
+          uint32_t alow[LK / 16][4];
+#pragma unroll
+          for (int h = 0; h < LK / 16; ++h) {
+            ldsm4(alow[h], sA + (uint32_t)(((2 * warp + (mj & 1)) * LO + 2 * h + (mj >> 1)) * IM_UNIT + mr16));
+#pragma unroll
+            for (int q = 0; q < 4; ++q) alow[h][q] = dg_low(alow[h][q]);
+          }
 #pragma unroll
           for (int kp = 0; kp < KT / 2; ++kp) {
             if (16 * kp >= kc) break;
-            float acc[2][DG_S][4];
 #pragma unroll
-            for (int h = 0; h < LK / 16; ++h) {
-              if (h > 0 && 16 * h >= lc) break;
-              uint32_t xf[IM_NX][4];
-              const uint32_t xa = sX + (uint32_t)(((2 * kp + (mj >> 1)) * LO + 2 * h + (mj & 1)) * IM_XUNIT + mr16);
+            for (int c = 0; c < 2; ++c) {  // 8 rows of X at a time: both would take the registers of another warp
+              float acc[DG_S][4], sa[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-              for (int j = 0; j < IM_NX; ++j) ldsm4(xf[j], xa + j * 128);
-              const uint32_t aa = sA + (uint32_t)(((2 * warp + (mj & 1)) * LO + 2 * h + (mj >> 1)) * IM_UNIT + mr16);
+              for (int h = 0; h < LK / 16; ++h) {
+                if (h > 0 && 16 * h >= lc) break;
+                uint32_t xf[IM_NX / 2][4];  // two digits each, in halves
+                const uint32_t xa = sX + (uint32_t)(((2 * kp + c) * LO + 2 * h + (mj & 1)) * IM_XUNIT + (mj >> 1) * 128 + mr16);
 #pragma unroll
-              for (int i = 0; i < DG_N; ++i) {
-                uint32_t af[4];
-                ldsm4(af, aa + i * 128);
+                for (int j = 0; j < IM_NX / 2; ++j) ldsm4(xf[j], xa + j * 256);
+                const uint32_t aa = sA + (uint32_t)(((2 * warp + (mj & 1)) * LO + 2 * h + (mj >> 1)) * IM_UNIT + mr16);
 #pragma unroll
-                for (int j = 0; i + j < DG_S; ++j) {
-                  if (h == 0 && i == 0) {
-                    mma_first(acc[0][i + j], af, xf[j][0], xf[j][1]);
-                    mma_first(acc[1][i + j], af, xf[j][2], xf[j][3]);
-                  } else {
-                    mma_acc(acc[0][i + j], af, xf[j][0], xf[j][1]);
-                    mma_acc(acc[1][i + j], af, xf[j][2], xf[j][3]);
+                for (int i = 0; i < DG_N; ++i) {
+                  uint32_t af[4];
+                  ldsm4(af, aa + i * 128);
+#pragma unroll
+                  for (int j = 0; i + j < DG_S; ++j) {
+                    const uint32_t x0 = xf[j / 2][2 * (j & 1)], x1 = xf[j / 2][2 * (j & 1) + 1];
+                    if (h == 0 && i == 0) mma_first(acc[i + j], af, x0, x1);
+                    else mma_acc(acc[i + j], af, x0, x1);
                   }
                 }
+                mma_acc(sa, alow[h], dg_low(xf[0][0]), dg_low(xf[0][1]));  // the same sums of lower bounds
               }
-            }
-#pragma unroll
-            for (int c = 0; c < 2; ++c)
 #pragma unroll
               for (int e = 0; e < 4; ++e) {
-                const long long v = dg_join<true>(acc[c][0][e], acc[c][1][e], acc[c][2][e], acc[c][3][e], acc[c][4][e],
-                                            acc[c][5][e], acc[c][6][e], acc[c][7][e]);
+                const long long v = dg_join<true>(acc[0][e], acc[1][e], acc[2][e], acc[3][e], acc[4][e], acc[5][e], acc[6][e], acc[7][e]);
                 T[2 * kp + c][e] += hsh ? v >> hsh : v;
               }
+              const int k = 16 * kp + 8 * c + 2 * t;
+              const int2 ek = *(const int2*)(eX + k);
+              const float2 sk = *(const float2*)(xsum + k);
+              auto down = [&](int e) { return __uint_as_float((uint32_t)max(124 - ex + e, 0) << 23); };  // 2^(-3 - distance)
+              const float f0 = down(ek.x), f1 = down(ek.y), m0 = f0 * lim14, m1 = f1 * lim14;
+              if (l0 == 0) {
+                mt[kp][2 * c] = dg_pack(sa[0] * m0, sa[1] * m1);
+                mt[kp][2 * c + 1] = dg_pack(sa[2] * m0, sa[3] * m1);
+                et[kp][c] = dg_pack(fmaf(sk.x, -1.015f, -el) * f0, fmaf(sk.y, -1.015f, -el) * f1);
+              } else {
+                mt[kp][2 * c] = dg_more(mt[kp][2 * c], sa[0] * m0, sa[1] * m1);
+                mt[kp][2 * c + 1] = dg_more(mt[kp][2 * c + 1], sa[2] * m0, sa[3] * m1);
+              }
+            }
           }
         }
         if (mine) {
@@ -665,8 +803,16 @@ __global__ void __launch_bounds__(C::NT, C::CTAS)
               tf[kk][7][q] = digit2<7>(h0, l0_, h1, l1_);
             }
           const int base = ex - 1022 - 1022 - 57 + 63 - 57 + hsh;  // scales of X and A, of T's sums, of Y's
-          s0 = scale(rec.alpha, eA[16 * warp + g] + base - z0);
-          s1 = scale(rec.alpha, eA[16 * warp + g + 8] + base - z1);
+          const int e0 = eA[16 * warp + g], e1 = eA[16 * warp + g + 8];
+          s0 = row_scale(e0, e0 + base - z0);
+          s1 = row_scale(e1, e1 + base - z1);
+          ws0 = weight(e0);
+          ws1 = weight(e1);
+          wt0 = ws0 * im_pow2(6 + hsh - z0);  // T's scale after normalising
+          wt1 = ws1 * im_pow2(6 + hsh - z1);
+          if (far(e0) || far(e1)) hide(e0, e1);
+          ws0 *= 0x1p-4f;  // 2^3 of down, 2^-7 of B's digit
+          ws1 *= 0x1p-4f;
         }
       } else if (mine) {
 #pragma unroll
@@ -677,22 +823,62 @@ __global__ void __launch_bounds__(C::NT, C::CTAS)
             if (i < DG_N || f == 1) ldsm4(tf[kk][i], sA + at);
             else tf[kk][i][0] = tf[kk][i][1] = tf[kk][i][2] = tf[kk][i][3] = 0u;
           }
-        s0 = scale(rec.alpha, eA[16 * warp + g] - 1022 - 57);
-        s1 = scale(rec.alpha, eA[16 * warp + g + 8] - 1022 - 57);
+        const uint32_t lim7 = dg_pack(lim * 0x1p-7f, lim * 0x1p-7f);
+#pragma unroll
+        for (int kk = 0; kk < KT / 2; ++kk) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) mt[kk][q] = dg_mul(dg_low(tf[kk][0][q]), lim7);
+          et[kk][0] = et[kk][1] = f == 2 ? dg_pack(-1.02f, -1.02f) : 0u;  // A's last digits against the magnitudes of B
+        }
+        const int e0 = eA[16 * warp + g], e1 = eA[16 * warp + g + 8];
+        s0 = row_scale(e0, e0 - 1022 - 57);
+        s1 = row_scale(e1, e1 - 1022 - 57);
+        wt0 = weight(e0);
+        wt1 = weight(e1);
+        if (far(e0) || far(e1)) hide(e0, e1);
+        ws0 = wt0 * 0x1p-7f;
+        ws1 = wt1 * 0x1p-7f;
+      }
+      if (mine) {
+        // B's last digits against T's magnitudes (its leading digits and the rest, at most half of one), T's last
+        // bits, the dropped pairs and the joined sum's last bit
+        float st[4] = {0.f, 0.f, 0.f, 0.f};
+        const uint32_t one = dg_pack(1.f, 1.f);
+        uint32_t a[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) a[q] = dg_abs(tf[0][0][q]);
+        mma_acc(st, a, one, one);
+        if (KT == 4 && kc > 16) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) a[q] = dg_abs(tf[KT / 2 - 1][0][q]);
+          mma_acc(st, a, one, one);
+        }
+        const float rest = 0.05f * kc + 0.6f;
+        wt0 *= -fmaf(st[0], 1.02f * 0x1p-7f, rest);
+        wt1 *= -fmaf(st[2], 1.02f * 0x1p-7f, rest);
       }
       cp_wait();
       sync();  // the second slot is in, the first is free
       if (k0 + KM < K) load1(rec, k0 + KM, 0);
-      else if (more) load1(nxt, 0, 0);
+      else if (more) load1(recs[ti + 1], 0, 0);
       cp_commit();
       if (!mine) continue;
 #pragma unroll 1
       for (int b = 0; b < nbt; ++b) {
         float acc[DG_S][4];
-        uint32_t bf[DG_N][4];
+        uint32_t bf[DG_N][KT];
         const uint32_t ba = sB + (uint32_t)((b * KO + (KT == 4 ? mj : (mj & 1))) * IM_UNIT + mr16);
 #pragma unroll
-        for (int j = 0; j < DG_N; ++j) ldsm4(bf[j], ba + j * 128);
+        for (int j = 0; j < DG_N; j += KT == 4 ? 1 : 2) {
+          uint32_t r[4];  // four octets of a digit, or two of two digits
+          ldsm4(r, ba + (KT == 4 ? j : min(j + (mj >> 1), DG_N - 1)) * 128);
+          bf[j][0] = r[0];
+          bf[j][1] = r[1];
+          if (KT == 4 || j + 1 < DG_N) {
+            bf[KT == 4 ? j : j + 1][KT - 2] = r[2];
+            bf[KT == 4 ? j : j + 1][KT - 1] = r[3];
+          }
+        }
 #pragma unroll
         for (int i = 0; i < IM_NX; ++i)
 #pragma unroll
@@ -704,11 +890,32 @@ __global__ void __launch_bounds__(C::NT, C::CTAS)
 #pragma unroll
           for (int i = 0; i < IM_NX; ++i)
 #pragma unroll
-            for (int j = 0; j < DG_N && i + j < DG_S; ++j) mma_acc(acc[i + j], tf[KT / 2 - 1][i], bf[j][2], bf[j][3]);
+            for (int j = 0; j < DG_N && i + j < DG_S; ++j) mma_acc(acc[i + j], tf[KT / 2 - 1][i], bf[j][KT - 2], bf[j][KT - 1]);
         }
         const int2 eb = *(const int2*)(eB + 8 * b + 2 * t);
+        float sa[4] = {0.f, 0.f, 0.f, 0.f};  // what the sums may err by, less what they do
+        {
+          const uint32_t ea0[4] = {et[0][0], et[0][0], et[0][1], et[0][1]};
+          mma_acc(sa, mt[0], dg_low(bf[0][0]), dg_low(bf[0][1]));
+          mma_acc(sa, ea0, dg_high(bf[0][0]), dg_high(bf[0][1]));
+          if (KT == 4 && kc > 16) {
+            const uint32_t ea1[4] = {et[KT / 2 - 1][0], et[KT / 2 - 1][0], et[KT / 2 - 1][1], et[KT / 2 - 1][1]};
+            mma_acc(sa, mt[KT / 2 - 1], dg_low(bf[0][KT - 2]), dg_low(bf[0][KT - 1]));
+            mma_acc(sa, ea1, dg_high(bf[0][KT - 2]), dg_high(bf[0][KT - 1]));
+          }
+        }
+        const float c0 = im_pow2(eb.x - btop), c1 = im_pow2(eb.y - btop);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
+          const float d0 = fmaf(h ? ws1 : ws0, sa[2 * h], h ? wt1 : wt0), d1 = fmaf(h ? ws1 : ws0, sa[2 * h + 1], h ? wt1 : wt0);
+          if (DBT == NBT || b < DBT) {
+            float2 v = Ds[(2 * b + h) * 32];
+            v.x = fmaf(c0, d0, v.x);
+            v.y = fmaf(c1, d1, v.y);
+            Ds[(2 * b + h) * 32] = v;
+          } else {  // the sum of the smaller of two is at most either's sum
+            Dp[(2 * b + h) * 32] += 8 * b + 2 * t + 1 < nb ? fminf(c0 * d0, c1 * d1) : c0 * d0;
+          }
           double2 v = Ys[(2 * b + h) * 32];
 #pragma unroll
           for (int c = 0; c < 2; ++c) {
@@ -724,6 +931,18 @@ __global__ void __launch_bounds__(C::NT, C::CTAS)
   }
   cp_wait();
 
+  // without a certificate the piece goes to the FMA kernel, which runs after this one
+  if (mine && !bad)
+    for (int b = 0; b < nbt; ++b)
+      for (int h = 0; h < 2; ++h)
+        if (16 * warp + g + 8 * h < na && 8 * b + 2 * t < nb) {
+          const float2 d = DBT == NBT || b < DBT ? Ds[(2 * b + h) * 32] : make_float2(Dp[(2 * b + h) * 32], 0.f);
+          if (!(d.x >= 0.f) || (8 * b + 2 * t + 1 < nb && !(d.y >= 0.f))) bad = true;
+        }
+  if (W == 1 ? __any_sync(0xffffffffu, bad) : __syncthreads_or(bad)) {
+    if (tid == 0) failed[atomicAdd(nfailed, 1)] = blockIdx.x;
+    return;
+  }
   double* Y = yv + (long long)vec * ys + G.yoff;
   double* P = TL.poff >= 0 ? part + (long long)vec * psize + TL.poff : nullptr;  // split piece
   if (mine)
@@ -741,24 +960,15 @@ __global__ void __launch_bounds__(C::NT, C::CTAS)
 
 // residency: 12 CTAs of one warp (168 registers), 4 of two and 2 of four (shared
 // memory: digits of both operands' chunks and the sums)
-using ImS = ImCfg<1, 2, 16, 16, 12>;
-using ImM = ImCfg<2, 4, 32, 32, 4>;
-using ImL = ImCfg<4, 8, 32, 32, 2>;
+using ImS = ImCfg<1, 2, 2, 16, 16, 12>;
+using ImM = ImCfg<2, 4, 3, 32, 32, 4>;
+using ImL = ImCfg<4, 7, 7, 32, 32, 2>;
 
 static_assert(ImS::CTAS == kDgClass[0].ctas && ImM::CTAS == kDgClass[1].ctas && ImL::CTAS == kDgClass[2].ctas &&
                   ImS::AR == kDgClass[0].a && ImM::AR == kDgClass[1].a && ImL::AR == kDgClass[2].a &&
                   ImS::BR == kDgClass[0].b && ImM::BR == kDgClass[1].b && ImL::BR == kDgClass[2].b &&
                   ImS::KM == kDgClass[0].km && ImM::KM == kDgClass[1].km && ImL::KM == kDgClass[2].km,
               "the classes the host plans with");
-
-template <class C>
-void launch_im(unsigned grid, cudaStream_t s, const DgRec* recs, const Task* tasks, const Group* groups,
-               const Tile* tiles, int tile0, const unsigned char* ops, const unsigned char* x, long long xbytes,
-               const int* xscale, int nx, const double* xv, double* yv, long long xs, long long ys, double* part,
-               long long psize, int nv) {
-  k_tasks_im<C><<<grid, C::NT, C::total, s>>>(recs, tasks, groups, tiles, tile0, ops, x, xbytes, xscale, nx, xv, yv, xs,
-                                               ys, part, psize, nv);
-}
 
 struct DgPlan {
   void* mem = nullptr;  // records, operator images and vector blocks
@@ -893,11 +1103,10 @@ bool prepare_digits(CudaBackend& be, const TaskList& tl, DevList& d, int nvec, l
   return true;
 }
 
-// the vectors' digits, ahead of the product kernels
-void enqueue_digit_vectors(CudaBackend& be, const DevList& d, const double* xv, long long xs, int nvec) {
+// the vectors' digits, ahead of the product kernels; clears the counts of failed pieces
+void enqueue_digit_vectors(CudaBackend& be, const DevList& d, const double* xv, long long xs, int nvec, int* failed) {
   const DgPlan* P = (const DgPlan*)d.dg;
-  if (!P || P->nx == 0) return;
-  k_dg_x<<<dim3(P->nx, nvec), 128, 0, be.stream()>>>(P->xblocks, P->nx, xv, xs, P->x, P->xbytes, P->xscale);
+  k_dg_x<<<dim3(P->nx, nvec), 128, 0, be.stream()>>>(P->xblocks, P->nx, xv, xs, P->x, P->xbytes, P->xscale, failed);
   be.launches++;
   be.note(cudaGetLastError(), "k_dg_x");
 }
@@ -912,14 +1121,18 @@ cudaError_t fp64_digits_init() {
   return e;
 }
 
-// one class of tiles
+// one class of tiles; pieces without a certificate are listed in failed, their number in nfailed
 void launch_fp64_digits(int cls, unsigned grid, cudaStream_t s, const void* plan, const Task* tasks,
                         const Group* groups, const Tile* tiles, int tile0, const double* xv, double* yv, long long xs,
-                        long long ys, double* part, long long psize, int nv) {
+                        long long ys, double* part, long long psize, int nv, int* nfailed, int* failed) {
   const DgPlan* P = (const DgPlan*)plan;
-  auto f = cls == 0 ? launch_im<ImS> : cls == 1 ? launch_im<ImM> : launch_im<ImL>;
-  f(grid, s, P->recs, tasks, groups, tiles, tile0, P->ops, P->x, P->xbytes, P->xscale, P->nx, xv, yv, xs, ys, part,
-    psize, nv);
+  auto go = [&](auto kernel, int nt, int smem) {
+    kernel<<<grid, nt, smem, s>>>(P->recs, tasks, groups, tiles, tile0, P->ops, P->x, P->xbytes, P->xscale, P->nx, xv, yv,
+                                  xs, ys, part, psize, nv, nfailed, failed);
+  };
+  if (cls == 0) go(k_tasks_im<ImS>, ImS::NT, ImS::total);
+  else if (cls == 1) go(k_tasks_im<ImM>, ImM::NT, ImM::total);
+  else go(k_tasks_im<ImL>, ImL::NT, ImL::total);
 }
 
 }  // namespace tns

@@ -53,6 +53,7 @@ constexpr int C1_NT = 128, C1_ACC = 8, C1_TR = 32, C1_TC = 32;
 constexpr int C2_NT = 256, C2_ACC = 16, C2_TR = 128, C2_TC = 32;  // tall
 constexpr int C3_NT = 256, C3_ACC = 16, C3_TR = 32, C3_TC = 128;  // wide
 constexpr int kFpClasses = 4;
+constexpr int CD_NT = 256, CD_ACC = 16, CD_TR = 64, CD_TC = 64;  // pieces of the largest digit class
 constexpr int kTallR = 128, kTallC = 32, kWideR = 32, kWideC = 128;
 
 // dynamic shared memory of a class: max(SA, SB) + SR doubles (see the kernel)
@@ -76,20 +77,20 @@ __host__ __device__ inline long long tile_fmas(const Task& t, int nr, int nc, bo
   return cb < ca ? cb : ca;
 }
 
+static_assert(8 * C0_TR * C0_TC <= fp64_smem(C0_TR, C0_TC) && 8 * C1_TR * C1_TC <= fp64_smem(C1_TR, C1_TC) &&
+                  8 * CD_TR * CD_TC <= fp64_smem(CD_TR, CD_TC),
+              "the staging region holds a tile of sums");
+
 template <int NT, int ACC, int TR, int TC>
-__global__ void __launch_bounds__(NT, NT >= 256 ? 2 : NT >= 128 ? 4 : 16) k_tasks_fp64(const Task* __restrict__ tasks, const Group* __restrict__ groups,
-                                                   const Tile* __restrict__ tiles, int tile0, const double* xv,
-                                                   double* yv, long long xs, long long ys, double* part,
-                                                   long long psize, int nv) {
+__device__ __forceinline__ void fp64_tile(const Task* __restrict__ tasks, const Group* __restrict__ groups,
+                                          const Tile& T, int vec, const double* xv, double* yv, long long xs,
+                                          long long ys, double* part, long long psize) {
   constexpr int SA = CH * (TC + 1);  // L (X R^T): CH rows of X R^T, TC columns
   constexpr int SB = TR * (CH + 1);  // (L X) R^T: TR rows of L X, CH columns
   constexpr int TE = CH * TC / NT;   // elements of X R^T per thread and chunk (upper bound)
   extern __shared__ double S[];      // max(SA, SB) + SR doubles, SR = CH * (TC + 1)
   double* const Rt = S + (SA > SB ? SA : SB);  // L (X R^T): a K slice of the tile's R rows, transposed
-  // the vectors of one tile piece are adjacent CTAs (they read the same operator blocks)
-  const Tile T = tiles[tile0 + blockIdx.x / nv];
   const Group G = groups[T.g];
-  const int vec = blockIdx.x % nv;
   const double* X0 = xv ? xv + (long long)vec * xs : nullptr;
   double* Y = yv + (long long)vec * ys + G.yoff;
   const int nc = T.ncols, nr = T.nrows;
@@ -238,6 +239,66 @@ __global__ void __launch_bounds__(NT, NT >= 256 ? 2 : NT >= 128 ? 4 : 16) k_task
       if (P) P[ri[u] * nc + cj[u]] = acc[u];
       else Y[(long long)(T.row0 + ri[u]) * G.r + T.col0 + cj[u]] = acc[u];
     }
+}
+
+// the vectors of one tile piece are adjacent CTAs (they read the same operator blocks)
+template <int NT, int ACC, int TR, int TC>
+__global__ void __launch_bounds__(NT, NT >= 256 ? 2 : NT >= 128 ? 4 : 16)
+    k_tasks_fp64(const Task* __restrict__ tasks, const Group* __restrict__ groups, const Tile* __restrict__ tiles,
+                 int tile0, const double* xv, double* yv, long long xs, long long ys, double* part, long long psize,
+                 int nv) {
+  const Tile T = tiles[tile0 + blockIdx.x / nv];
+  fp64_tile<NT, ACC, TR, TC>(tasks, groups, T, blockIdx.x % nv, xv, yv, xs, ys, part, psize);
+}
+
+// The pieces of one class that the digit kernel left without a certificate
+// (fp64_digits.cu).  They are few and their task lists long (one CTA each: 44 ms
+// after a digit kernel of 56 ms, 24 orbitals, D = 512 in 9 sectors), so a
+// cluster takes a piece: each CTA a fixed share of its products, whose sums are
+// added up in CTA order through distributed shared memory.  The grid walks the
+// list, whose order does not matter since every piece has its own output.
+constexpr int kRedoCluster = 16;
+
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+template <int NT, int ACC, int TR, int TC>
+__global__ void __launch_bounds__(NT, NT >= 256 ? 2 : NT >= 128 ? 4 : 16)
+    k_tasks_fp64_failed(const Task* __restrict__ tasks, const Group* __restrict__ groups,
+                        const Tile* __restrict__ tiles, int tile0, const double* xv, double* yv, long long xs,
+                        long long ys, double* part, long long psize, int nv, const int* __restrict__ nfailed,
+                        const int* __restrict__ failed) {
+  extern __shared__ double S[];
+  const uint32_t sums = (uint32_t)__cvta_generic_to_shared(S);
+  const int n = *nfailed, rank = blockIdx.x % kRedoCluster;
+  for (int i = blockIdx.x / kRedoCluster; i < n; i += gridDim.x / kRedoCluster) {
+    const int vec = failed[i] % nv;
+    const Tile F = tiles[tile0 + failed[i] / nv];
+    Tile T = F;
+    const int len = F.t1 - F.t0;
+    T.t0 = F.t0 + (int)((long long)len * rank / kRedoCluster);
+    T.t1 = F.t0 + (int)((long long)len * (rank + 1) / kRedoCluster);
+    T.poff = 0;
+    fp64_tile<NT, ACC, TR, TC>(tasks, groups, T, vec, xv, yv, xs, ys, S, 0);  // its last product's operands have been read
+    cluster_sync();
+    double* P = F.poff >= 0 ? part + (long long)vec * psize + F.poff : nullptr;
+    double* Y = yv + (long long)vec * ys + groups[F.g].yoff;
+    const int ld = groups[F.g].r;
+    for (int e = rank * NT + threadIdx.x; e < F.nrows * F.ncols; e += kRedoCluster * NT) {
+      double s = 0.0;
+      for (int q = 0; q < kRedoCluster; ++q) {
+        uint32_t at;
+        double v;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(sums + 8u * e), "r"(q));
+        asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(at) : "memory");
+        s += v;
+      }
+      if (P) P[e] = s;
+      else Y[(long long)(F.row0 + e / F.ncols) * ld + F.col0 + e % F.ncols] = s;
+    }
+    cluster_sync();  // the sums have been read
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -935,6 +996,7 @@ void launch_gather(CudaBackend& be, const double* src, const long long* so, cons
 // backend
 // ---------------------------------------------------------------------------
 CudaBackend::CudaBackend(int device, cudaStream_t s, bool own) : device_(device), stream_(s), own_(own) {
+  if (cudaDeviceGetAttribute(&sms_, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) cudaGetLastError();
   const char* gr = std::getenv("TNS_GRAPHS");
   if (gr && std::strcmp(gr, "0") == 0) use_graphs = false;
   const char* at = std::getenv("TNS_AUTOTUNE");
@@ -1149,6 +1211,7 @@ void CudaBackend::free_list(DevList& d) {
       if (f.tiles) dfree(f.tiles);
       if (f.reds) dfree(f.reds);
       if (f.part) dfree(f.part);
+      if (f.failed) dfree(f.failed);
     }
   if (d.tc) release_tc_plan(d.tc);
   if (d.dg) release_digit_plan(d.dg);
@@ -1385,6 +1448,12 @@ void CudaBackend::plan_variant(const TaskList& tl, DevList& d, int dig, int v) {
                               fp64_smem(C3_TR, C3_TC)),
          "k_tasks_fp64 shared memory");
     note(fp64_digits_init(), "k_tasks_im shared memory");
+    auto wide = [&](const void* f) {
+      note(cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1), "k_tasks_fp64_failed cluster size");
+    };
+    wide((const void*)k_tasks_fp64_failed<C0_NT, C0_ACC, C0_TR, C0_TC>);
+    wide((const void*)k_tasks_fp64_failed<C1_NT, C1_ACC, C1_TR, C1_TC>);
+    wide((const void*)k_tasks_fp64_failed<CD_NT, CD_ACC, CD_TR, CD_TC>);
     attr = true;
   }
   const bool digits = dig != 0;
@@ -1398,8 +1467,7 @@ void CudaBackend::plan_variant(const TaskList& tl, DevList& d, int dig, int v) {
   for (int c = 0; c < kFpClasses; ++c)
     for (double w : ccost[c]) ctot[c] += w;
   // resident CTAs per SM of each class (registers) x SMs x rounds
-  int sms = 152;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device_);
+  const int sms = sms_;
   const double rounds = kRounds[v];
   const double ctas[kFpClasses] = {digits ? (double)kDgClass[0].ctas : 16.0, digits ? (double)kDgClass[1].ctas : 4.0,
                                    digits ? (double)kDgClass[2].ctas : 2.0, 2.0};
@@ -1489,7 +1557,23 @@ void CudaBackend::plan_variant(const TaskList& tl, DevList& d, int dig, int v) {
   note(cudaStreamSynchronize(stream_), "schedule upload");
 }
 
-bool CudaBackend::ensure_part(DevList& d, FpVariant& f, int nvec) {
+bool CudaBackend::ensure_part(DevList& d, FpVariant& f, int dig, int nvec) {
+  if (dig && f.failed_nvec < nvec) {
+    if (f.failed) {
+      free_graphs(d);
+      cudaStreamSynchronize(stream_);
+      dfree(f.failed);
+    }
+    f.failed = nullptr;
+    f.failed_nvec = 0;
+    if (dmalloc(&f.failed, sizeof(int) * (4 + (long long)f.ntiles * nvec)) != cudaSuccess) {
+      cudaGetLastError();
+      note(cudaErrorMemoryAllocation, "failed pieces");
+      f.failed = nullptr;
+      return false;
+    }
+    f.failed_nvec = nvec;
+  }
   if (f.psize == 0 || f.part_nvec >= nvec) return true;
   if (f.part) {
     // graphs captured with the smaller buffer would write through a freed pointer
@@ -1533,7 +1617,7 @@ void CudaBackend::enqueue_fp64(const DevList& d, int dig, int v, const double* x
   // (they fill its tail), joined before the split reduction
   int order[kFpClasses] = {0, 1, 2, 3};
   std::stable_sort(order, order + kFpClasses, [&](int a, int b) { return f.ccost[a] > f.ccost[b]; });
-  if (dig) enqueue_digit_vectors(*this, d, xv, xs, nvec);
+  if (dig) enqueue_digit_vectors(*this, d, xv, xs, nvec, f.failed);
   const int nact = (f.ncls[0] > 0) + (f.ncls[1] > 0) + (f.ncls[2] > 0) + (f.ncls[3] > 0);
   const bool fork = nact > 1 && fork_ready();
   if (fork) {
@@ -1554,9 +1638,31 @@ void CudaBackend::enqueue_fp64(const DevList& d, int dig, int v, const double* x
     cudaStream_t s = stream_;
     if (fork && oi > 0) s = fstream_[side++];
     const int t0 = tbeg[c];
-    if (dig)
-      launch_fp64_digits(c, grid, s, d.dg, d.tasks, d.groups, f.tiles, t0, xv, yv, xs, ys, f.part, f.psize, nvec);
-    else if (c == 0)
+    if (dig) {
+      int* const list = f.failed + 4 + (long long)t0 * nvec;
+      launch_fp64_digits(c, grid, s, d.dg, d.tasks, d.groups, f.tiles, t0, xv, yv, xs, ys, f.part, f.psize, nvec,
+                         f.failed + c, list);
+      auto rest = [&](auto kernel, int nt, int per_sm, int smem) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = kRedoCluster;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3(std::min(grid, (unsigned)(sms_ * per_sm / kRedoCluster)) * kRedoCluster);
+        cfg.blockDim = dim3(nt);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = s;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        note(cudaLaunchKernelEx(&cfg, kernel, (const Task*)d.tasks, (const Group*)d.groups, (const Tile*)f.tiles, t0, xv, yv,
+                                xs, ys, f.part, f.psize, nvec, (const int*)(f.failed + c), (const int*)list),
+             "k_tasks_fp64_failed");
+      };
+      if (c == 0) rest(k_tasks_fp64_failed<C0_NT, C0_ACC, C0_TR, C0_TC>, C0_NT, 16, fp64_smem(C0_TR, C0_TC));
+      else if (c == 1) rest(k_tasks_fp64_failed<C1_NT, C1_ACC, C1_TR, C1_TC>, C1_NT, 4, fp64_smem(C1_TR, C1_TC));
+      else rest(k_tasks_fp64_failed<CD_NT, CD_ACC, CD_TR, CD_TC>, CD_NT, 2, fp64_smem(CD_TR, CD_TC));
+      launches++;
+    } else if (c == 0)
       k_tasks_fp64<C0_NT, C0_ACC, C0_TR, C0_TC><<<grid, C0_NT, fp64_smem(C0_TR, C0_TC), s>>>(
           d.tasks, d.groups, f.tiles, t0, xv, yv, xs, ys, f.part, f.psize, nvec);
     else if (c == 1)
@@ -1578,6 +1684,20 @@ void CudaBackend::enqueue_fp64(const DevList& d, int dig, int v, const double* x
     }
   }
   launch_reduce_splits(*this, f.reds, f.nreds, f.red_el, d.groups, f.part, f.psize, yv, ys, nvec);
+}
+
+// the part of a digit product, by estimated cost, that was done again by the
+// FMA kernel (synchronises)
+double CudaBackend::failed_share(const FpVariant& f, int nvec) {
+  int n[kDgClasses] = {0, 0, 0};
+  note(cudaMemcpyAsync(n, f.failed, sizeof(n), cudaMemcpyDeviceToHost, stream_), "failed pieces");
+  note(cudaStreamSynchronize(stream_), "failed pieces");
+  double all = 0, again = 0;
+  for (int c = 0; c < kDgClasses; ++c) {
+    all += f.ccost[c];
+    if (f.ncls[c] > 0) again += f.ccost[c] * n[c] / ((double)f.ncls[c] * nvec);
+  }
+  return all > 0 ? again / all : 0.0;
 }
 
 // Replay (capturing it first if needed) the launch sequence `enqueue` of one
@@ -1681,7 +1801,7 @@ void CudaBackend::run(const TaskList& tl, const double* xv, double* yv, int nvec
       }
     } else {
       plan_variant(tl, tmp, 0, 1);
-      if (ok() && tmp.tasks && tmp.groups && ensure_part(tmp, tmp.fv[0][1], nvec))
+      if (ok() && tmp.tasks && tmp.groups && ensure_part(tmp, tmp.fv[0][1], 0, nvec))
         enqueue_fp64(tmp, 0, 1, xv, yv, nvec, xs, ys);
     }
     free_list(tmp);
@@ -1726,7 +1846,23 @@ void CudaBackend::run(const TaskList& tl, const double* xv, double* yv, int nvec
       dig = prepare_digits(*this, tl, d, nvec, xs) ? 1 : 0;
     }
     plan_variant(tl, d, dig, v);
-    if (!ok() || !ensure_part(d, d.fv[dig][v], nvec)) return;
+    if (!ok() || !ensure_part(d, d.fv[dig][v], dig, nvec)) return;
+    if (dig && !d.dg_kept && fp64_kernel != 2) {
+      // the list's first product: where too much of it has no certificate, the
+      // list is for the FMA kernel, this product included
+      enqueue_fp64(d, 1, v, xv, yv, nvec, xs, ys);
+      if (failed_share(d.fv[1][v], nvec) <= kFailedShare) {
+        d.dg_kept = true;
+        if (tuning && !timing) ++tu.step;
+        return;
+      }
+      release_digit_plan(d.dg);
+      d.dg = nullptr;
+      d.dg_none = true;
+      dig = 0;
+      plan_variant(tl, d, 0, v);
+      if (!ok() || !ensure_part(d, d.fv[0][v], 0, nvec)) return;
+    }
   }
   auto enqueue = [&](const double* x, double* y) {
     if (precision != 0)

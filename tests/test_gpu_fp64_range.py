@@ -122,6 +122,26 @@ def _entries_hold(desc, got, want, bound):
         assert np.all(err <= TOL_ENTRY * bound[q]), (q, float(np.max(err / np.maximum(bound[q], 1e-300))))
 
 
+# the FP64 kernels by the library's rule, and digits wherever a list has images: pieces without a certificate, all of
+# them in some of these systems, are then done again by the FMA kernel
+KERNELS = pytest.mark.parametrize("kernel", [None, "digits"])
+
+
+@KERNELS
+@pytest.mark.parametrize("decades", [0, 4, 9])
+def test_entries_of_weak_states(determinants, decades, kernel):
+    system, heff, keys = determinants
+    k = system[4]
+    X = _graded(keys, decades)
+    bound = heff.apply_abs(X)
+    ctx, ref = _ctx(kernel, *system), _ctx("dfma", *system)
+    desc, length = ctx.psi_layout(k)
+    x = torch.tensor(blocks_to_vector(desc, length, X), device="cuda")[None]
+    got, want = _apply(ctx, k, x), _apply(ref, k, x)
+    _entries_hold(desc, got[0].cpu().numpy(), want[0].cpu().numpy(), bound)
+    _entries_hold(desc, want[0].cpu().numpy(), blocks_to_vector(desc, length, heff.apply(X)), bound)
+
+
 @pytest.mark.parametrize("decades", [4, 9])
 def test_entries_of_the_adjoint(determinants, decades):
     """Xbar = H_eff Ybar for a symmetric H_eff, so the same sums bound it."""
@@ -190,3 +210,45 @@ def test_small_vectors_in_the_adjoint(system, p, part):
         grads.append(res)
     for u, w in zip(*grads):
         assert _close(u * UP, w * UP)
+
+
+@KERNELS
+@pytest.mark.parametrize("system", SYSTEMS)
+@MAGNITUDES
+def test_small_vectors(system, p, part, kernel):
+    args = _random(system)
+    k = args[4]
+    ctx, ref = _ctx(kernel, *args), _ctx("dfma", *args)
+    desc, length = ctx.psi_layout(k)
+    g = torch.Generator(device="cuda").manual_seed(7)
+    x = torch.randn(1, length, device="cuda", dtype=torch.float64, generator=g)
+    small = _small(desc, x, p, part)
+    got = _apply(ctx, k, small)
+    assert _close(got * UP, _apply(ref, k, small) * UP)
+    if part == 1:  # powers of two pass through
+        assert _close(got * UP, _apply(ref, k, x) * 2.0 ** (400 - p))
+
+
+@KERNELS
+def test_small_operators_and_small_vector(kernel):
+    """Left operators and a vector whose products are near 1e-286: one block of X, and the output blocks of other left
+    sectors, which only an operator of the left block reaches."""
+    args = _random(SYSTEMS[1])
+    k = args[4]
+    out = []
+    for name in (kernel, "dfma"):
+        ctx = _ctx(name, *args)
+        desc, length = ctx.psi_layout(k)
+        rows = [[int(v) for v in r] for r in desc]
+        big = max(rows, key=lambda r: r[6] * r[7])
+        g = torch.Generator(device="cuda").manual_seed(7)
+        x = torch.zeros(1, length, device="cuda", dtype=torch.float64)
+        x[:, big[8]:big[8] + big[6] * big[7]] = 2.0 ** -470 * torch.randn(
+            big[6] * big[7], device="cuda", dtype=torch.float64, generator=g)
+        arena_tensor(ctx, k, 0).mul_(2.0 ** -480)
+        torch.cuda.synchronize()
+        ctx.build_env(k)
+        y = _apply(ctx, k, x)[0] * 2.0 ** 900
+        out.append(torch.cat([y[r[8]:r[8] + r[6] * r[7]] for r in rows if r[:2] != big[:2]]))
+    assert float(out[1].abs().max()) > 0
+    assert _close(*out)
