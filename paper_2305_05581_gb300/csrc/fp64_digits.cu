@@ -111,35 +111,37 @@ __device__ __forceinline__ uint32_t digit2(uint32_t h0, uint32_t l0, uint32_t h1
   return *(const uint32_t*)&d;
 }
 
-// the weight sums of one output as an integer, sum_s i_s 2^(43 - 8 s), below
-// 2^62.1.  T rounds to the nearest; Y (floor) meets the complement that
-// dg_double takes of negative numbers, so that it errs towards zero alike on
-// both sides: a common sign of the error would add up over the products.
-template <bool ROUND>
+// the weight sums of one output as an integer, sum_s i_s 2^(43 - 8 s) to the
+// nearest, below 2^62.1
 __device__ __forceinline__ long long dg_join(float f0, float f1, float f2, float f3, float f4, float f5, float f6,
                                              float f7) {
   constexpr unsigned c = DG_MAGIC * 257u;
   auto two = [](float hi, float lo, unsigned off) {
     return (int)((unsigned)__float_as_int(hi) * 256u + (unsigned)__float_as_int(lo) - off);
   };
-  const int P = two(f0, f1, c), Q = two(f2, f3, c), R = two(f4, f5, c), U = two(f6, f7, ROUND ? c - (1u << 12) : c);
+  const int P = two(f0, f1, c), Q = two(f2, f3, c), R = two(f4, f5, c), U = two(f6, f7, c - (1u << 12));
   const int V = R + (U >> 16);
   const unsigned long long hi = (unsigned long long)((unsigned)P * 8u + (unsigned)(Q >> 13)) << 32 | ((unsigned)Q << 19);
   const unsigned long long lo = (unsigned long long)(unsigned)(V >> 29) << 32 | ((unsigned)V << 3 | ((unsigned)U >> 13 & 7u));
   return (long long)(hi + lo);
 }
 
-// v 2^(e - 1085) as a double (towards zero)
+// v 2^(e - 1085) as the nearest double: the leading one goes to bit 62, so that
+// rounding may carry into bit 63 and from there into the exponent
 __device__ __forceinline__ double dg_double(long long v, int e) {
-  const uint32_t sg = (uint32_t)((int)(v >> 32) >> 31);
-  uint32_t h = (uint32_t)(v >> 32) ^ sg, l = (uint32_t)v ^ sg;
+  const long long sg = v >> 63;
+  const unsigned long long m = (unsigned long long)((v ^ sg) - sg);
+  uint32_t h = (uint32_t)(m >> 32), l = (uint32_t)m;
   const bool low = h == 0;
   h = low ? l : h;
   l = low ? 0u : l;
   const int z = __clz((int)h);
   const uint32_t hs = __funnelshift_lc(l, h, z), ls = l << (z & 31);
-  uint32_t dh = (sg & 0x80000000u) | ((uint32_t)((e - z - (low ? 32 : 0)) << 20) + (hs >> 11));
-  uint32_t dl = __funnelshift_r(ls, hs, 11);
+  const uint32_t half = __funnelshift_r(ls, hs, 1);  // sums have few bits more than a double: ties are common, and go to even
+  const unsigned long long r = ((unsigned long long)(hs >> 1) << 32 | half) + (0x1ffu + (half >> 10 & 1u));
+  const uint32_t rh = (uint32_t)(r >> 32), rl = (uint32_t)r;
+  uint32_t dh = ((uint32_t)sg & 0x80000000u) | ((uint32_t)((e - z - (low ? 32 : 0)) << 20) + (rh >> 10));
+  uint32_t dl = __funnelshift_r(rl, rh, 10);
   if (h == 0) dh = dl = 0u;
   return __hiloint2double((int)dh, (int)dl);
 }
@@ -744,7 +746,7 @@ __global__ void __launch_bounds__(C::NT, C::CTAS)
               }
 #pragma unroll
               for (int e = 0; e < 4; ++e) {
-                const long long v = dg_join<true>(acc[0][e], acc[1][e], acc[2][e], acc[3][e], acc[4][e], acc[5][e], acc[6][e], acc[7][e]);
+                const long long v = dg_join(acc[0][e], acc[1][e], acc[2][e], acc[3][e], acc[4][e], acc[5][e], acc[6][e], acc[7][e]);
                 T[2 * kp + c][e] += hsh ? v >> hsh : v;
               }
               const int k = 16 * kp + 8 * c + 2 * t;
@@ -920,7 +922,7 @@ __global__ void __launch_bounds__(C::NT, C::CTAS)
 #pragma unroll
           for (int c = 0; c < 2; ++c) {
             const int e = 2 * h + c;
-            const long long j = dg_join<false>(acc[0][e], acc[1][e], acc[2][e], acc[3][e], acc[4][e], acc[5][e], acc[6][e], acc[7][e]);
+            const long long j = dg_join(acc[0][e], acc[1][e], acc[2][e], acc[3][e], acc[4][e], acc[5][e], acc[6][e], acc[7][e]);
             double& o = c ? v.y : v.x;
             o = fma(dg_double(j, (c ? eb.y : eb.x) + 63), h ? s1 : s0, o);
           }

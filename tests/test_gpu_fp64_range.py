@@ -252,3 +252,24 @@ def test_small_operators_and_small_vector(kernel):
         out.append(torch.cat([y[r[8]:r[8] + r[6] * r[7]] for r in rows if r[:2] != big[:2]]))
     assert float(out[1].abs().max()) > 0
     assert _close(*out)
+
+
+@pytest.mark.parametrize("system", SYSTEMS + [(11, 11, 1, 130, 5, 5)])
+def test_rounding_has_no_direction(system):
+    """Both kernels round to the nearest, so the difference of their results has no component along the result.  The
+    entries' errors are a few units of 2^-53 of their typical magnitude and independent, so over n entries the
+    component is a few 2^-53 / sqrt(n): 0.05 units at the 5,000 entries of the smallest system.  Dropping the bits
+    below the last makes every contribution too small, which shows as 2 to 3.5 units (contributions are larger than
+    the results they cancel to), and ties away from zero as 0.17."""
+    args = _random(system)
+    k = args[4]
+    ctx, ref = _ctx("digits", *args), _ctx("dfma", *args)
+    _, length = ctx.psi_layout(k)
+    assert length > 4000
+    g = torch.Generator(device="cuda").manual_seed(3)
+    along = []
+    for _ in range(8):
+        x = torch.randn(1, length, device="cuda", dtype=torch.float64, generator=g)
+        got, want = _apply(ctx, k, x), _apply(ref, k, x)
+        along.append(float(((got - want) * want).sum() / (want * want).sum()) * 2.0 ** 53)
+    assert abs(np.mean(along)) < 0.15, along
