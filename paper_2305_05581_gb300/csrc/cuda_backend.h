@@ -109,6 +109,11 @@ constexpr double kSteady = 0.8;
 // certificate is done again by that kernel: beyond a third the sum is no gain
 // (24 orbitals, D = 512, all sectors: 21 ms and a tenth of 36.5 ms again).
 constexpr double kFailedShare = 0.2;
+// Lists below these flops stay with the FMA kernel: making the images takes
+// their first product 0.16 ms, and what a later one gains is 0.04 ms at 2.6e7
+// flops (8 orbitals: 0.236 -> 0.193 ms), nothing at 8e6, but 0.33 ms at 9.4e7
+// (10 orbitals, D = 96: 0.705 -> 0.371 ms).
+constexpr double kDigitFlops = 5e7;
 constexpr int kSteadyKey = 1 << 16;  // schedules and graphs of such products are kept apart
 
 // captured launch sequence of one (precision, nvec) use: replayed with the
@@ -140,6 +145,7 @@ struct DevList {
   // digit images of the list (fp64_digits.cu); dg_none: they cannot be had
   void* dg = nullptr;
   bool dg_none = false;
+  double flops = -1;     // of the list's products, once asked for
   bool dg_kept = false;  // the first product's certificates held (kFailedShare)
   std::vector<unsigned char> dg_aside;  // per group: the tiles' a side
   // tensor-core form (precision != FP64)

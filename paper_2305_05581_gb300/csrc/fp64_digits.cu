@@ -973,7 +973,7 @@ static_assert(ImS::CTAS == kDgClass[0].ctas && ImM::CTAS == kDgClass[1].ctas && 
               "the classes the host plans with");
 
 struct DgPlan {
-  void* mem = nullptr;  // records, operator images and vector blocks
+  void* mem = nullptr;  // records, operator images, vector blocks and the images of the first call's vectors
   DgRec* recs = nullptr;
   unsigned char* ops = nullptr;
   DgXBlock* xblocks = nullptr;
@@ -982,6 +982,13 @@ struct DgPlan {
   long long xbytes = 0;
   int* xscale = nullptr;  // nx a vector
   int x_nvec = 0;
+  void* xmem = nullptr;   // images of more vectors
+  long long vectors(int nvec) const { return (xbytes + 4LL * nx + 512) * nvec; }
+  void set_vectors(unsigned char* p, int nvec) {
+    x = p;
+    xscale = (int*)(p + xbytes * nvec);
+    x_nvec = nvec;
+  }
 };
 
 template <class T>
@@ -997,7 +1004,7 @@ void release_digit_plan(void* p) {
   DgPlan* P = (DgPlan*)p;
   if (!P) return;
   if (P->mem) dfree(P->mem);
-  if (P->x) dfree(P->x);
+  if (P->xmem) dfree(P->xmem);
   delete P;
 }
 
@@ -1017,9 +1024,10 @@ bool prepare_digits(CudaBackend& be, const TaskList& tl, DevList& d, int nvec, l
     P = new DgPlan();
     const int max_x = (int)(4 * ng + 4096);
     bool made = false;
-    // a table of a quarter of the products' count holds the operators of a
-    // long list many times over; a larger one is tried if it does not
-    for (long long want = std::max(nt / 4, 4096LL); !made; want *= 8) {
+    // a short list may have as many operators as products, in the table half as
+    // many as slots; of a long one a quarter of the products' count holds them
+    // many times over, and a larger table is tried if it does not
+    for (long long want = nt <= (1 << 16) ? std::max(2 * nt, 4096LL) : nt / 4; !made; want *= 8) {
       unsigned cap = 4096;
       while (cap < want && cap < (1u << 30)) cap <<= 1;
       const int max_jobs = (int)(cap / 2);
@@ -1027,9 +1035,10 @@ bool prepare_digits(CudaBackend& be, const TaskList& tl, DevList& d, int nvec, l
                               (long long)sizeof(DgXBlock) * max_x + ng + 8192;
       if (bytes + nt * (long long)sizeof(DgRec) > avail / 2) break;
       // small tables stay for the next list, large ones go back
-      const bool keep = bytes <= (16LL << 20);
+      const long long room = (bytes + (4LL << 20) - 1) >> 22 << 22;
+      const bool keep = bytes <= (16LL << 20) && room <= avail / 2;
       unsigned char* tmp = nullptr;
-      if (keep) tmp = (unsigned char*)be.scratch(16 << 20, 4);
+      if (keep) tmp = (unsigned char*)be.scratch(room, 4);
       else if (dmalloc(&tmp, bytes) != cudaSuccess) cudaGetLastError();
       if (!tmp) break;
       unsigned char* p = tmp;
@@ -1057,13 +1066,17 @@ bool prepare_digits(CudaBackend& be, const TaskList& tl, DevList& d, int nvec, l
       if (!state()) {
         again = be.ok() && want < 4 * nt;
       } else {
+        // with the vectors of this call: an allocation takes a short list's product half as long as it runs
+        P->nx = h.nx;
+        P->xbytes = (long long)h.xunits * 128;
         const long long total = (long long)h.units * 128 + (long long)sizeof(DgRec) * nt +
-                                (long long)sizeof(DgXBlock) * h.nx + 1024;
+                                (long long)sizeof(DgXBlock) * h.nx + P->vectors(nvec) + 1280;
         if (total <= avail / 2 && dmalloc(&P->mem, total) == cudaSuccess) {
           unsigned char* q = (unsigned char*)P->mem;
           P->ops = carve<unsigned char>(q, (long long)h.units * 128);
           P->recs = carve<DgRec>(q, nt);
           P->xblocks = carve<DgXBlock>(q, h.nx);
+          P->set_vectors(carve<unsigned char>(q, P->vectors(nvec)), nvec);
           if (h.njobs > 0) k_dg_ops<<<(unsigned)h.njobs, 128, 0, be.stream()>>>(jobs, P->ops);
           k_dg_records<<<(unsigned)ng, 128, 0, be.stream()>>>(d.tasks, d.groups, aside, keys, slot, cap - 1, jobs, xtab, xb,
                                                               P->recs, st);
@@ -1071,8 +1084,6 @@ bool prepare_digits(CudaBackend& be, const TaskList& tl, DevList& d, int nvec, l
           be.note(cudaGetLastError(), "digit images");
           be.note(cudaMemcpyAsync(P->xblocks, xb, sizeof(DgXBlock) * h.nx, cudaMemcpyDeviceToDevice, be.stream()), "digit plan");
           made = state();
-          P->nx = h.nx;
-          P->xbytes = (long long)h.xunits * 128;
         } else {
           cudaGetLastError();
         }
@@ -1087,21 +1098,19 @@ bool prepare_digits(CudaBackend& be, const TaskList& tl, DevList& d, int nvec, l
     d.dg = P;
     d.dg_none = false;
   }
-  if (P->x) {
-    be.free_graphs(d);  // graphs captured with the smaller images would write through freed pointers
-    cudaStreamSynchronize(be.stream());
-    dfree(P->x);
-  }
-  P->x = nullptr;
+  if (P->x_nvec >= nvec) return true;
+  be.free_graphs(d);  // graphs captured with the smaller images would write through freed pointers
+  cudaStreamSynchronize(be.stream());
+  if (P->xmem) dfree(P->xmem);
+  P->xmem = nullptr;
   P->x_nvec = 0;
-  const long long bytes = (P->xbytes + 4LL * P->nx + 512) * nvec;
-  if (bytes > avail / 2 || dmalloc(&P->x, bytes) != cudaSuccess) {
+  const long long bytes = P->vectors(nvec);
+  if (bytes > avail / 2 || dmalloc(&P->xmem, bytes) != cudaSuccess) {
     cudaGetLastError();
     d.dg_none = true;
     return false;
   }
-  P->xscale = (int*)(P->x + P->xbytes * nvec);
-  P->x_nvec = nvec;
+  P->set_vectors((unsigned char*)P->xmem, nvec);
   return true;
 }
 

@@ -1333,28 +1333,41 @@ static void dfma_tiles(const TaskList& tl, DevList& d) {
   d.fp_tiled[0] = true;
 }
 
-// Estimated time of one product on an a x b tile of a digit-kernel class, in
-// clocks of one SM whose resident CTAs share it: its MMAs (34 digit pairs, 8
+// Estimated time of products on an a x b tile of a digit-kernel class, in
+// clocks of one SM whose resident CTAs share it: their MMAs (34 digit pairs, 8
 // clocks each on one of four tensor cores), the cutting of T, the joining of
 // sums into Y, and a fixed part per staged chunk.  Only ratios matter: they
-// decide classes, sides and splits.
-static double dg_cost(int cls, const Task& t, int aside, int a, int b) {
-  const DgClass& c = kDgClass[cls];
-  const int K = aside ? t.n : t.m, L = aside ? t.m : t.n;
-  auto up = [](int x, int m) { return (double)((x + m - 1) / m * m); };
-  const double ap = up(a, 16), bp = up(b, 8);
-  const double fixed[kDgClasses] = {150.0, 400.0, 800.0};
-  const double ovh = fixed[cls], mm = 34.0 * 8.0 / 2048.0;
-  const bool ai = (t.flags & (aside ? TF_LI : TF_RI)) != 0, bi = (t.flags & (aside ? TF_RI : TF_LI)) != 0;
-  if (ai && bi) return ovh + a * b / 4.0;
-  if (ai || bi || (t.flags & TF_XI)) {
-    const double kk = up(ai ? K : L, 16), ch = std::ceil(kk / c.km);
-    return ovh * ch + 0.25 * (ap * bp * kk * mm + 4.0 * ap * bp * ch);
+// decide classes, sides and splits.  What the products' inner sizes contribute
+// is summed once (add) for every side and tile (at); a list's planning is part
+// of its first product.
+struct DgCost {
+  double both = 0, two_ch = 0, two_k = 0;                 // products with two, one identity factor: count, chunks, k
+  double steps = 0, kl = 0, k = 0, klch = 0, ch = 0;      // others: steps, k l, k, k times l chunks, chunks
+  void add(const Task& t, int aside, int km, double count) {
+    const int K = aside ? t.n : t.m, L = aside ? t.m : t.n;
+    const bool ai = (t.flags & (aside ? TF_LI : TF_RI)) != 0, bi = (t.flags & (aside ? TF_RI : TF_LI)) != 0;
+    if (ai && bi) {
+      both += count;
+    } else if (ai || bi || (t.flags & TF_XI)) {
+      const int kk = ((ai ? K : L) + 15) & ~15;
+      two_ch += count * ((kk + km - 1) / km);
+      two_k += count * kk;
+    } else {
+      const int kp = (K + 15) & ~15, lp = (L + 15) & ~15, c = (kp + km - 1) / km, lc = (L + km - 1) / km;
+      steps += count * c * (0.5 + 0.5 * lc);
+      kl += count * kp * lp;
+      k += count * kp;
+      klch += count * kp * lc;
+      ch += count * c;
+    }
   }
-  const double kp = up(K, 16), lp = up(L, 16), ch = std::ceil(kp / c.km), lch = std::ceil((double)L / c.km);
-  return ovh * ch * (1.0 + 0.5 * (lch - 1)) +
-         0.25 * (mm * ap * kp * (lp + bp) + 2.4 * ap * kp * lch + 4.0 * ap * bp * ch);
-}
+  double at(int cls, int a, int b) const {
+    const double fixed[kDgClasses] = {150.0, 400.0, 800.0}, mm = 34.0 * 8.0 / 2048.0;
+    const double ap = (a + 15) & ~15, bp = (b + 7) & ~7;
+    return fixed[cls] * (both + two_ch + steps) + both * a * b / 4.0 +
+           0.25 * ap * (bp * (mm * (two_k + k) + 4.0 * (two_ch + ch)) + mm * kl + 2.4 * klch);
+  }
+};
 
 // cut an extent into near-equal parts of at most mx, at multiples of 8 (the row groups of images)
 static std::vector<std::pair<int, int>> cut8(int len, int mx) {
@@ -1368,6 +1381,15 @@ static bool digit_images(const TaskList& tl) {
   return tl.persistent && !tl.tasks.empty() && (tl.tasks[0].flags & TF_XV);
 }
 
+static double list_flops(const TaskList& tl, DevList& d) {
+  if (d.flops < 0) {
+    d.flops = tl.flops;
+    if (d.flops <= 0)
+      for (const Task& t : tl.tasks) d.flops += 2.0 * (double)tile_fmas(t, t.q, t.r, nullptr);
+  }
+  return d.flops;
+}
+
 // digit-kernel tiles of every group: the class and the side that is
 // contracted with X first, whichever costs least over the group's products
 // (summed over their distinct shapes)
@@ -1375,34 +1397,57 @@ static void dg_tiles(const TaskList& tl, DevList& d) {
   d.dg_aside.assign(tl.groups.size(), 0);
   struct Shape {
     int m, n, f, count;
+    unsigned at;  // its place in the table
     const Task* t;
   };
   std::vector<Shape> sh;
+  std::vector<int> slot(256, 0);  // open addressing: 1 + the shape's index
+  auto hash = [](int m, int n, int f) { return (unsigned)m * 37u + (unsigned)n * 5u + (unsigned)f; };
   for (int g = 0; g < (int)tl.groups.size(); ++g) {
     const Group& G = tl.groups[g];
     if (G.q <= 0 || G.r <= 0) continue;
+    for (const Shape& x : sh) slot[x.at] = 0;
     sh.clear();
-    size_t last = 0;
     for (int i = G.t0; i < G.t1; ++i) {
       const Task& t = tl.tasks[i];
       const int f = t.flags & (TF_LI | TF_RI | TF_XI);
-      auto same = [&](const Shape& s) { return s.m == t.m && s.n == t.n && s.f == f; };
-      if (last >= sh.size() || !same(sh[last])) {
-        for (last = 0; last < sh.size() && !same(sh[last]); ++last) {
+      if (4 * sh.size() > slot.size()) {
+        slot.assign(2 * slot.size(), 0);
+        for (size_t j = 0; j < sh.size(); ++j) {
+          unsigned at = hash(sh[j].m, sh[j].n, sh[j].f);
+          while (slot[at &= slot.size() - 1]) ++at;
+          slot[sh[j].at = at] = (int)j + 1;
         }
-        if (last == sh.size()) sh.push_back({t.m, t.n, f, 0, &t});
       }
-      ++sh[last].count;
+      unsigned at = hash(t.m, t.n, f);
+      for (;; ++at) {
+        int& s = slot[at &= slot.size() - 1];
+        if (s == 0) {
+          sh.push_back({t.m, t.n, f, 1, at, &t});
+          s = (int)sh.size();
+          break;
+        }
+        Shape& x = sh[s - 1];
+        if (x.m == t.m && x.n == t.n && x.f == f) {
+          ++x.count;
+          break;
+        }
+      }
     }
+    DgCost cost[kDgClasses][2];
+    for (int c = 0; c < kDgClasses; ++c)
+      for (int s = 0; s < 2; ++s) {
+        if (c > 0 && kDgClass[c].km == kDgClass[c - 1].km) cost[c][s] = cost[c - 1][s];
+        else
+          for (const Shape& x : sh) cost[c][s].add(*x.t, s, kDgClass[c].km, x.count);
+      }
     double best = -1;
     int pc = 0, pa = 0;
     for (int c = 0; c < kDgClasses; ++c)
       for (int s = 0; s < 2; ++s) {
         const int ea = s ? G.q : G.r, eb = s ? G.r : G.q;
         const int na = (ea + kDgClass[c].a - 1) / kDgClass[c].a, nb = (eb + kDgClass[c].b - 1) / kDgClass[c].b;
-        double w = 0;
-        for (const Shape& x : sh) w += x.count * dg_cost(c, *x.t, s, (ea + na - 1) / na, (eb + nb - 1) / nb);
-        w *= (double)na * nb;
+        const double w = cost[c][s].at(c, (ea + na - 1) / na, (eb + nb - 1) / nb) * na * nb;
         if (best < 0 || w < best) {
           best = w;
           pc = c;
@@ -1424,10 +1469,8 @@ static void dg_tiles(const TaskList& tl, DevList& d) {
         t.t1 = G.t1;
         t.aside = pa;
         t.poff = -1;
-        double w = 0;
-        for (const Shape& x : sh) w += x.count * dg_cost(pc, *x.t, pa, aa.second, bb.second);
         d.fp_tiles[1][pc].push_back(t);
-        d.fp_cost[1][pc].push_back(w);
+        d.fp_cost[1][pc].push_back(cost[pc][pa].at(pc, aa.second, bb.second));
       }
   }
   d.fp_tiled[1] = true;
@@ -1475,6 +1518,7 @@ void CudaBackend::plan_variant(const TaskList& tl, DevList& d, int dig, int v) {
   for (int c = 0; c < kFpClasses; ++c) slots[c] = ctas[c] * sms * rounds;
   std::vector<Tile> all;
   std::vector<SplitRed> reds;
+  std::vector<double> kc;
   long long poff = 0;
   for (int c = 0; c < kFpClasses; ++c) {
     const double target = std::max(ctot[c] / slots[c], 1.0);
@@ -1494,12 +1538,23 @@ void CudaBackend::plan_variant(const TaskList& tl, DevList& d, int dig, int v) {
         continue;
       }
       // cut the task range at equal shares of its cost on this tile
-      std::vector<double> kc(ntask);
+      kc.resize(ntask);
       double tot = 0;
-      for (int k = t.t0; k < t.t1; ++k)
-        tot += kc[k - t.t0] =
-            digits ? dg_cost(c, tl.tasks[k], t.aside, t.aside ? t.nrows : t.ncols, t.aside ? t.ncols : t.nrows)
-                   : (double)tile_fmas(tl.tasks[k], t.nrows, t.ncols, nullptr) + kTaskOverhead;
+      const Task* seen = nullptr;  // neighbours mostly have one shape
+      for (int k = t.t0; k < t.t1; ++k) {
+        const Task& x = tl.tasks[k];
+        if (!digits) {
+          kc[k - t.t0] = (double)tile_fmas(x, t.nrows, t.ncols, nullptr) + kTaskOverhead;
+        } else if (seen && seen->m == x.m && seen->n == x.n && seen->flags == x.flags) {
+          kc[k - t.t0] = kc[k - 1 - t.t0];
+        } else {
+          DgCost one;
+          one.add(x, t.aside, kDgClass[c].km, 1.0);
+          kc[k - t.t0] = one.at(c, t.aside ? t.nrows : t.ncols, t.aside ? t.ncols : t.nrows);
+        }
+        seen = &x;
+        tot += kc[k - t.t0];
+      }
       SplitRed R;
       R.g = t.g;
       R.row0 = t.row0;
@@ -1508,10 +1563,10 @@ void CudaBackend::plan_variant(const TaskList& tl, DevList& d, int dig, int v) {
       R.ncols = t.ncols;
       R.poff = poff;
       int start = t.t0, made = 0;
-      double acc = 0, last = 0;
+      double acc = 0, last = 0, cut = tot * 1 / ns;
       for (int k = t.t0; k < t.t1 && made < ns - 1; ++k) {
         acc += kc[k - t.t0];
-        if (acc >= tot * (made + 1) / ns) {
+        if (acc >= cut) {
           Tile p = t;
           p.t0 = start;
           p.t1 = k + 1;
@@ -1521,6 +1576,7 @@ void CudaBackend::plan_variant(const TaskList& tl, DevList& d, int dig, int v) {
           pcost.push_back(acc - last);
           last = acc;
           ++made;
+          cut = tot * (made + 1) / ns;
           ++count;
           start = k + 1;
         }
@@ -1536,13 +1592,14 @@ void CudaBackend::plan_variant(const TaskList& tl, DevList& d, int dig, int v) {
       R.nsplit = made + 1;
       reds.push_back(R);
     }
-    // costliest pieces first: CTAs are dispatched in index order, so the long
-    // pieces start in the first wave and the short ones fill in behind them
-    std::vector<int> ord(pcost.size());
-    for (size_t i = 0; i < ord.size(); ++i) ord[i] = (int)i;
-    std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) { return pcost[a] > pcost[b]; });
+    // costliest pieces first (of equal ones the earlier): CTAs are dispatched in
+    // index order, so the long pieces start in the first wave and the short ones
+    // fill in behind them
+    std::vector<std::pair<double, int>> ord(pcost.size());
+    for (size_t i = 0; i < ord.size(); ++i) ord[i] = {-pcost[i], (int)i};
+    std::sort(ord.begin(), ord.end());
     std::vector<Tile> sorted(ord.size());
-    for (size_t i = 0; i < ord.size(); ++i) sorted[i] = all[first + ord[i]];
+    for (size_t i = 0; i < ord.size(); ++i) sorted[i] = all[first + ord[i].second];
     std::copy(sorted.begin(), sorted.end(), all.begin() + first);
     f.ncls[c] = count;
     f.ccost[c] = ctot[c];
@@ -1841,7 +1898,7 @@ void CudaBackend::run(const TaskList& tl, const double* xv, double* yv, int nvec
   if (precision != 0) {
     if (!prepare_tasks_tc(*this, tl, d, nvec, v, precision)) return;
   } else {
-    if (fk == 2 && digit_images(tl)) {
+    if (fk == 2 && digit_images(tl) && (fp64_kernel == 2 || list_flops(tl, d) >= kDigitFlops)) {
       if (!d.fp_tiled[1]) dg_tiles(tl, d);
       dig = prepare_digits(*this, tl, d, nvec, xs) ? 1 : 0;
     }

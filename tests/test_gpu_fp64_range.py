@@ -21,6 +21,7 @@ import numpy as np
 import pytest
 
 import synth
+import test_gpu_fp64_digits
 from oracle import dmrg as O3
 
 torch = pytest.importorskip("torch")
@@ -252,6 +253,36 @@ def test_small_operators_and_small_vector(kernel):
         out.append(torch.cat([y[r[8]:r[8] + r[6] * r[7]] for r in rows if r[:2] != big[:2]]))
     assert float(out[1].abs().max()) > 0
     assert _close(*out)
+
+
+@pytest.mark.parametrize("system", test_gpu_fp64_digits.CASES)
+@pytest.mark.parametrize("kind", ["normal", "graded", "sparse", "huge"])
+def test_digits_of_small_lists(system, kind):
+    """Lists that the library leaves to the FMA kernel for their size, on the digit kernel."""
+    args = _random(system)
+    k = args[4]
+    ctx, ref = _ctx("digits", *args), _ctx("dfma", *args)
+    desc, length = ctx.psi_layout(k)
+    for nvec in (1, 3):
+        x = test_gpu_fp64_digits._vector(kind, desc, length, nvec)
+        assert _close(_apply(ctx, k, x), _apply(ref, k, x))
+    assert torch.equal(_apply(ctx, k, x[:1]), _apply(ctx, k, x)[:1])
+
+
+def test_first_product_of_a_small_list_allocates_no_images():
+    """Below the line by size the first product costs what it costs with the FMA kernel alone."""
+    args = _random(SYSTEMS[0])
+    k = args[4]
+    used = []
+    for kernel in (None, "dfma"):
+        ctx = _ctx(kernel, *args)
+        _, length = ctx.psi_layout(k)
+        x = torch.ones(1, length, device="cuda", dtype=torch.float64)
+        before = ctx.memory_stats()["device_used"]
+        _apply(ctx, k, x)
+        used.append(ctx.memory_stats()["device_used"] - before)
+        ctx.close()
+    assert used[0] == used[1]
 
 
 @pytest.mark.parametrize("system", SYSTEMS + [(11, 11, 1, 130, 5, 5)])
