@@ -47,6 +47,7 @@ class CudaBackend;
 struct DevList;
 struct Tile;
 bool prepare_digits(CudaBackend& be, const TaskList& tl, DevList& d, int nvec, long long length);
+int digit_vectors(const DevList& d);  // how many vectors the list's images are for
 void enqueue_digit_vectors(CudaBackend& be, const DevList& d, const double* xv, long long xs, int nvec, int* failed);
 void release_digit_plan(void* plan);
 void launch_fp64_digits(int cls, unsigned grid, cudaStream_t s, const void* plan, const Task* tasks,
@@ -234,6 +235,8 @@ class CudaBackend : public Backend {
   // launches of the FP64 product kernels of variant v (no allocation, no
   // synchronisation: capturable)
   void enqueue_fp64(const DevList& d, int dig, int v, const double* xv, double* yv, int nvec, long long xs, long long ys);
+  void enqueue_fp64_vectors(const DevList& d, int dig, const FpVariant& f, const double* xv, double* yv, int nvec,
+                            long long xs, long long ys, double* part);
   // room for `bytes` of the backend's own allocations (the engine's hook)
   void need(long long bytes) {
     if (room && bytes > (64LL << 20)) room(bytes);

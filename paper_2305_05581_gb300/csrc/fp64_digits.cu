@@ -1099,20 +1099,22 @@ bool prepare_digits(CudaBackend& be, const TaskList& tl, DevList& d, int nvec, l
     d.dg_none = false;
   }
   if (P->x_nvec >= nvec) return true;
+  // images of more vectors, where they leave half of what is free; otherwise
+  // the call runs on as many at a time as there are
+  void* more = nullptr;
+  if (P->vectors(nvec) > avail / 2 || dmalloc(&more, P->vectors(nvec)) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
   be.free_graphs(d);  // graphs captured with the smaller images would write through freed pointers
   cudaStreamSynchronize(be.stream());
   if (P->xmem) dfree(P->xmem);
-  P->xmem = nullptr;
-  P->x_nvec = 0;
-  const long long bytes = P->vectors(nvec);
-  if (bytes > avail / 2 || dmalloc(&P->xmem, bytes) != cudaSuccess) {
-    cudaGetLastError();
-    d.dg_none = true;
-    return false;
-  }
-  P->set_vectors((unsigned char*)P->xmem, nvec);
+  P->xmem = more;
+  P->set_vectors((unsigned char*)more, nvec);
   return true;
 }
+
+int digit_vectors(const DevList& d) { return ((const DgPlan*)d.dg)->x_nvec; }
 
 // the vectors' digits, ahead of the product kernels; clears the counts of failed pieces
 void enqueue_digit_vectors(CudaBackend& be, const DevList& d, const double* xv, long long xs, int nvec, int* failed) {

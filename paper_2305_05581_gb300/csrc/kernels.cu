@@ -1669,6 +1669,19 @@ void CudaBackend::enqueue_fp64(const DevList& d, int dig, int v, const double* x
                                long long ys) {
   if (!ok()) return;
   const FpVariant& f = d.fv[dig][v];
+  double* part = f.part;
+  const int most = dig ? digit_vectors(d) : nvec;
+  for (; nvec > most; nvec -= most) {
+    enqueue_fp64_vectors(d, dig, f, xv, yv, most, xs, ys, part);
+    xv += (long long)most * xs;
+    yv += (long long)most * ys;
+    part += (long long)most * f.psize;
+  }
+  enqueue_fp64_vectors(d, dig, f, xv, yv, nvec, xs, ys, part);
+}
+
+void CudaBackend::enqueue_fp64_vectors(const DevList& d, int dig, const FpVariant& f, const double* xv, double* yv,
+                                       int nvec, long long xs, long long ys, double* part) {
   // the classes write disjoint tiles and partial tiles: the costliest class
   // runs on the launching stream and the others on forked streams beside it
   // (they fill its tail), joined before the split reduction
@@ -1697,7 +1710,7 @@ void CudaBackend::enqueue_fp64(const DevList& d, int dig, int v, const double* x
     const int t0 = tbeg[c];
     if (dig) {
       int* const list = f.failed + 4 + (long long)t0 * nvec;
-      launch_fp64_digits(c, grid, s, d.dg, d.tasks, d.groups, f.tiles, t0, xv, yv, xs, ys, f.part, f.psize, nvec,
+      launch_fp64_digits(c, grid, s, d.dg, d.tasks, d.groups, f.tiles, t0, xv, yv, xs, ys, part, f.psize, nvec,
                          f.failed + c, list);
       auto rest = [&](auto kernel, int nt, int per_sm, int smem) {
         cudaLaunchConfig_t cfg = {};
@@ -1712,7 +1725,7 @@ void CudaBackend::enqueue_fp64(const DevList& d, int dig, int v, const double* x
         cfg.attrs = at;
         cfg.numAttrs = 1;
         note(cudaLaunchKernelEx(&cfg, kernel, (const Task*)d.tasks, (const Group*)d.groups, (const Tile*)f.tiles, t0, xv, yv,
-                                xs, ys, f.part, f.psize, nvec, (const int*)(f.failed + c), (const int*)list),
+                                xs, ys, part, f.psize, nvec, (const int*)(f.failed + c), (const int*)list),
              "k_tasks_fp64_failed");
       };
       if (c == 0) rest(k_tasks_fp64_failed<C0_NT, C0_ACC, C0_TR, C0_TC>, C0_NT, 16, fp64_smem(C0_TR, C0_TC));
@@ -1721,16 +1734,16 @@ void CudaBackend::enqueue_fp64(const DevList& d, int dig, int v, const double* x
       launches++;
     } else if (c == 0)
       k_tasks_fp64<C0_NT, C0_ACC, C0_TR, C0_TC><<<grid, C0_NT, fp64_smem(C0_TR, C0_TC), s>>>(
-          d.tasks, d.groups, f.tiles, t0, xv, yv, xs, ys, f.part, f.psize, nvec);
+          d.tasks, d.groups, f.tiles, t0, xv, yv, xs, ys, part, f.psize, nvec);
     else if (c == 1)
       k_tasks_fp64<C1_NT, C1_ACC, C1_TR, C1_TC><<<grid, C1_NT, fp64_smem(C1_TR, C1_TC), s>>>(
-          d.tasks, d.groups, f.tiles, t0, xv, yv, xs, ys, f.part, f.psize, nvec);
+          d.tasks, d.groups, f.tiles, t0, xv, yv, xs, ys, part, f.psize, nvec);
     else if (c == 2)
       k_tasks_fp64<C2_NT, C2_ACC, C2_TR, C2_TC><<<grid, C2_NT, fp64_smem(C2_TR, C2_TC), s>>>(
-          d.tasks, d.groups, f.tiles, t0, xv, yv, xs, ys, f.part, f.psize, nvec);
+          d.tasks, d.groups, f.tiles, t0, xv, yv, xs, ys, part, f.psize, nvec);
     else
       k_tasks_fp64<C3_NT, C3_ACC, C3_TR, C3_TC><<<grid, C3_NT, fp64_smem(C3_TR, C3_TC), s>>>(
-          d.tasks, d.groups, f.tiles, t0, xv, yv, xs, ys, f.part, f.psize, nvec);
+          d.tasks, d.groups, f.tiles, t0, xv, yv, xs, ys, part, f.psize, nvec);
     launches++;
     note(cudaGetLastError(), dig ? "k_tasks_im" : "k_tasks_fp64");
   }
@@ -1740,7 +1753,7 @@ void CudaBackend::enqueue_fp64(const DevList& d, int dig, int v, const double* x
       note(cudaStreamWaitEvent(stream_, fev_[1 + i], 0), "join");
     }
   }
-  launch_reduce_splits(*this, f.reds, f.nreds, f.red_el, d.groups, f.part, f.psize, yv, ys, nvec);
+  launch_reduce_splits(*this, f.reds, f.nreds, f.red_el, d.groups, part, f.psize, yv, ys, nvec);
 }
 
 // the part of a digit product, by estimated cost, that was done again by the

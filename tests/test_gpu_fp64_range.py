@@ -269,6 +269,34 @@ def test_digits_of_small_lists(system, kind):
     assert torch.equal(_apply(ctx, k, x[:1]), _apply(ctx, k, x)[:1])
 
 
+@pytest.mark.parametrize("graphs", ["0", "1"])
+def test_vectors_beyond_the_images(graphs):
+    """No memory for the images of more vectors: the call runs on the images there are, with the same results, and the
+    one-vector products before and after, by replayed graphs too, stay as they were."""
+    args = _random(SYSTEMS[1])
+    k = args[4]
+    os.environ.update(TNS_GRAPHS=graphs, TNS_AUTOTUNE="0")
+    try:
+        ctx, free = _ctx(None, *args), _ctx(None, *args)
+    finally:
+        os.environ.pop("TNS_GRAPHS")
+        os.environ.pop("TNS_AUTOTUNE")
+    _, length = ctx.psi_layout(k)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    x = torch.randn(3, length, device="cuda", dtype=torch.float64, generator=g)
+    want = _apply(free, k, x)
+    one = [_apply(ctx, k, x[:1]) for _ in range(3)]
+    ctx.set_memory_budget(ctx.memory_stats()["device_used"] + (1 << 26))
+    try:
+        assert torch.equal(_apply(ctx, k, x), want)
+        one += [_apply(ctx, k, x[:1]) for _ in range(2)]
+    finally:
+        ctx.set_memory_budget(0)
+    assert torch.equal(_apply(ctx, k, x), want)
+    one += [_apply(ctx, k, x[:1]) for _ in range(2)]
+    assert all(torch.equal(y, want[:1]) for y in one)
+
+
 def test_first_product_of_a_small_list_allocates_no_images():
     """Below the line by size the first product costs what it costs with the FMA kernel alone."""
     args = _random(SYSTEMS[0])
