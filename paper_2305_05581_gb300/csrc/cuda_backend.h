@@ -191,6 +191,7 @@ class CudaBackend : public Backend {
   void download(double* dst, const double* src, long long n) override;
   void zero(double* p, long long n) override;
   void copy(double* dst, const double* src, long long n) override;
+  bool trim() override;
   void lincomb(const LCList& l) override;
   void run(const TaskList& tl, const double* xv, double* yv, int nvec, long long xs, long long ys,
            int precision) override;
@@ -258,6 +259,7 @@ class CudaBackend : public Backend {
   bool own_;
   std::string err_;
   std::map<const TaskList*, DevList> lists_;
+  const DevList* running_ = nullptr;  // the list of the current run()
   // best schedule variant per (precision, nvec, shape signature): work lists
   // of later steps with the same shape take it without tuning again
   std::map<std::pair<int, unsigned long long>, int> tune_cache_;

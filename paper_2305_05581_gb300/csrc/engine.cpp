@@ -221,6 +221,8 @@ int Engine::make_room(long long bytes, std::string& err) {
     const long long fr = be_->mem_free() - reserve;
     if (fr < avail) avail = fr;
     if (bytes <= avail) return 0;
+    // what is kept for speed alone goes first
+    if (be_->spare() || be_->trim()) continue;
     // the movable catalogue farthest from the current step (L_j is read at
     // step j, R_j at step j-2)
     Catalogue* victim = nullptr;
@@ -2293,6 +2295,7 @@ void Engine::drop_adjoint() {
     *p = nullptr;
   }
   P.gen = -1;
+  P.bytes = 0;
   P.have[0] = P.have[1] = P.have[2] = false;
 }
 
@@ -2441,6 +2444,12 @@ int Engine::heff_adjoint(const double* X, const double* Yb, double* Xb, double* 
     return -2;
   }
   const bool want[3] = {Xb != nullptr, Lb != nullptr, Rb != nullptr};
+  struct Running {
+    bool& r;
+    explicit Running(bool& r) : r(r) { r = true; }
+    ~Running() { r = false; }
+  } in_use(adj_running_);
+  const long long base = be_->mem_used() - adj_.bytes;
   int rc = adjoint_plan(want, err);
   if (rc) return rc;
   AdjointPlan& P = adj_;
@@ -2457,17 +2466,12 @@ int Engine::heff_adjoint(const double* X, const double* Yb, double* Xb, double* 
   }
   be_->sync();
   std::string e = be_->error();
-  // the lists and buffers stay for the step's next call where they take little
-  // of the memory that is left, and go back at once otherwise
-  long long bytes = 8 * (2 * step_.length);
-  for (int s = 0; s < 2; ++s) {
-    if (P.side[s].G) bytes += 8 * (s ? Rcat_[step_.k + 2].size : Lcat_[step_.k].size);
-    if (P.side[s].M) bytes += 8 * (s ? step_.R.size : step_.L.size);
-    bytes += (long long)sizeof(Task) * 3 / 2 * (long long)(P.side[s].direct.tasks.size() + P.side[s].partial.tasks.size() + P.side[s].sum.tasks.size());
-  }
-  bytes += (long long)sizeof(Task) * 3 / 2 * (long long)P.xbar.tasks.size();
+  // the lists and buffers stay for the step's next call where all that the call
+  // added to the device takes little of the memory that is left, and go back at
+  // once otherwise, or when something else needs the room
+  P.bytes = std::max(be_->mem_used() - base, 0LL);
   const long long limit = be_->mem_limit();
-  if (!e.empty() || (limit > 0 && bytes * 16 > std::min(limit - be_->mem_used(), be_->mem_free()))) drop_adjoint();
+  if (!e.empty() || (limit > 0 && P.bytes * 16 > std::min(limit - be_->mem_used(), be_->mem_free()))) drop_adjoint();
   if (!e.empty()) {
     err = e;
     return -6;

@@ -333,6 +333,9 @@ struct Backend {
   virtual void upload(double* dst, const double* src, long long n) = 0;
   virtual void download(double* dst, const double* src, long long n) = 0;
   virtual void zero(double* p, long long n) = 0;
+  // give back what the backend keeps of lists only to run them faster (not of a
+  // list that is running); true if that freed anything
+  virtual bool trim() { return false; }
   virtual void copy(double* dst, const double* src, long long n) {  // within backend memory
     std::vector<double> h((size_t)n);
     download(h.data(), src, n);
@@ -368,6 +371,8 @@ struct Backend {
   // called by the backend before a large allocation of its own: the engine
   // moves catalogues it does not need off the device to make room
   std::function<int(long long)> room;
+  // set by the engine: gives back what it keeps of a step only to run it faster; true if that freed anything
+  std::function<bool()> spare;
   virtual void sync() = 0;
   virtual std::string error() = 0;  // "" if fine
 };
@@ -440,6 +445,7 @@ struct AdjointSide {
 };
 struct AdjointPlan {
   long long gen = -1;
+  long long bytes = 0;  // device memory that the lists, their schedules and the buffers took
   bool have[3] = {false, false, false};  // Xbar, left, right
   double *x = nullptr, *yb = nullptr;    // copies of X and Ybar that the lists read
   TaskList xbar;
@@ -461,6 +467,11 @@ struct MemStats {
 class Engine {
  public:
   explicit Engine(Backend* be) : be_(be) {
+    be_->spare = [this]() {
+      if (adj_.gen < 0 || adj_running_) return false;
+      drop_adjoint();
+      return true;
+    };
     be_->room = [this](long long bytes) {
       std::string e;
       return make_room(bytes, e);
@@ -559,6 +570,7 @@ class Engine {
   std::vector<Catalogue> Rcat_;  // Rcat_[k]: orbitals k..N-1
   Step step_;
   AdjointPlan adj_;
+  bool adj_running_ = false;
   void drop_adjoint();
   int adjoint_plan(const bool want[3], std::string& err);
   // catalogue staging: the position of the current work (eviction order is

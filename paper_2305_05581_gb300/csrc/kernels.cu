@@ -1063,9 +1063,9 @@ std::string CudaBackend::error() {
 
 double* CudaBackend::alloc(long long n) {
   void* p = nullptr;
-  if (dmalloc(&p, (size_t)n * sizeof(double)) != cudaSuccess) {
+  while (dmalloc(&p, (size_t)n * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();
-    return nullptr;
+    if (!(spare && spare()) && !trim()) return nullptr;
   }
   return (double*)p;
 }
@@ -1665,6 +1665,22 @@ void CudaBackend::drop(const TaskList& tl) {
   }
 }
 
+// the digit images of every list but the running one; a list makes them again
+// with its next product if there is room by then
+bool CudaBackend::trim() {
+  bool any = false;
+  for (auto& kv : lists_) {
+    DevList& d = kv.second;
+    if (!d.dg || &d == running_) continue;
+    free_graphs(d);
+    cudaStreamSynchronize(stream_);
+    release_digit_plan(d.dg);
+    d.dg = nullptr;
+    any = true;
+  }
+  return any;
+}
+
 void CudaBackend::enqueue_fp64(const DevList& d, int dig, int v, const double* xv, double* yv, int nvec, long long xs,
                                long long ys) {
   if (!ok()) return;
@@ -1778,8 +1794,9 @@ double CudaBackend::failed_share(const FpVariant& f, int nvec) {
 template <class F>
 void CudaBackend::launch_graphed(DevList& d, int key, const double* xv, double* yv, int nvec, long long xs,
                                  long long ys, F&& enqueue) {
+  if (!d.graphs[key].exec && !d.graphs[key].failed)
+    need(2LL * (long long)sizeof(double) * nvec * std::max(xs, ys));  // may free graphs of the list
   GraphSlot& gs = d.graphs[key];
-  if (!gs.exec && !gs.failed) need(2LL * (long long)sizeof(double) * nvec * std::max(xs, ys));
   const long long elems = (long long)nvec * xs;
   if (!use_graphs || gs.failed || xs != ys || xs == 0) {  // xs == 0: a list on fixed operands
     enqueue(xv, yv);
@@ -1879,6 +1896,12 @@ void CudaBackend::run(const TaskList& tl, const double* xv, double* yv, int nvec
   }
   DevList& d = dev(tl);
   if (!ok() || !d.tasks || !d.groups) return;
+  struct Running {
+    const DevList*& r;
+    const DevList* was;
+    Running(const DevList*& r, const DevList* d) : r(r), was(r) { r = d; }
+    ~Running() { r = was; }
+  } in_use(running_, precision == 0 ? &d : nullptr);
   if (precision == 0 && fk == 1) {
     if (d.nwtiles > 0) {
       dim3 grid((d.nwtiles + DM_WARPS - 1) / DM_WARPS, nvec);
