@@ -2299,11 +2299,12 @@ void Engine::drop_adjoint() {
   P.have[0] = P.have[1] = P.have[2] = false;
 }
 
-// The work lists of the adjoint for the wanted outputs, on fixed copies of X
-// and Ybar, so that they hold for every call of the step: making them (one
-// product per product of the step and output) takes the host several times
-// as long as running them (13 orbitals, D = 160: 9 of 12 ms).
-int Engine::adjoint_plan(const bool want[3], std::string& err) {
+// The work lists of the adjoint for the wanted outputs: on fixed copies of X
+// and Ybar (X, Yb null), so that they hold for every call of the step -- making
+// them (one product per product of the step and output) takes the host several
+// times as long as running them (13 orbitals, D = 160: 9 of 12 ms) -- or, where
+// the memory is short, on the call's own vectors
+int Engine::adjoint_plan(const bool want[3], const double* X, const double* Yb, std::string& err) {
   Step& st = step_;
   AdjointPlan& P = adj_;
   const TaskList& fw = st.heff_full;
@@ -2315,7 +2316,7 @@ int Engine::adjoint_plan(const bool want[3], std::string& err) {
     if (!p) p = be_->alloc(std::max(n, 1LL));
     return p != nullptr;
   };
-  bool good = get(P.x, st.length) && get(P.yb, st.length);
+  bool good = X || (get(P.x, st.length) && get(P.yb, st.length));
   for (int s = 0; s < 2; ++s)
     if (want[1 + s]) good = good && get(P.side[s].G, cats[s]->size) && (sides[s]->size == 0 || get(P.side[s].M, sides[s]->size));
   if (!good) {
@@ -2326,14 +2327,16 @@ int Engine::adjoint_plan(const bool want[3], std::string& err) {
   bool make[3];
   for (int i = 0; i < 3; ++i) make[i] = want[i] && !P.have[i];
   if (!make[0] && !make[1] && !make[2]) return 0;
+  const double* const px = X ? X : P.x;
+  const double* const pyb = X ? Yb : P.yb;
   // products by the block they contribute to
   std::unordered_map<const double*, std::vector<Task>> tx, ts[2];
   for (size_t g = 0; g < fw.groups.size(); ++g) {
     const Group& G = fw.groups[g];
-    const double* yb = P.yb + G.yoff;
+    const double* yb = pyb + G.yoff;
     for (int i = G.t0; i < G.t1; ++i) {
       const Task& t = fw.tasks[i];
-      const double* xblk = P.x + st.psi[t.pad].off;
+      const double* xblk = px + st.psi[t.pad].off;
       const int lf = t.flags & (TF_LI | TF_LT), rf = t.flags & (TF_RI | TF_RT);
       const int q = t.q, m = t.m, n = t.n, r = t.r;
       if (make[0])  // Xb (m x n) += a op(L)^T Yb op(R)
@@ -2387,7 +2390,7 @@ int Engine::adjoint_plan(const bool want[3], std::string& err) {
   if (make[0]) {
     std::vector<Blk> v;
     for (auto& p : st.psi) v.push_back({p.off, p.m, p.n});
-    list(P.xbar, v, of(tx, P.x));
+    list(P.xbar, v, of(tx, px));
     P.have[0] = true;
   }
   for (int s = 0; s < 2; ++s) {
@@ -2449,29 +2452,60 @@ int Engine::heff_adjoint(const double* X, const double* Yb, double* Xb, double* 
     explicit Running(bool& r) : r(r) { r = true; }
     ~Running() { r = false; }
   } in_use(adj_running_);
-  const long long base = be_->mem_used() - adj_.bytes;
-  int rc = adjoint_plan(want, err);
-  if (rc) return rc;
+  const long long limit = be_->mem_limit();
+  auto room = [&]() { return std::min(limit - be_->mem_used(), be_->mem_free()); };
   AdjointPlan& P = adj_;
-  be_->copy(P.x, X, step_.length);
-  be_->copy(P.yb, Yb, step_.length);
-  if (Xb) be_->run(P.xbar, nullptr, Xb, 1, 0, 0, 0);
-  double* const out[2] = {Lb, Rb};
-  for (int s = 0; s < 2; ++s) {
-    if (!out[s]) continue;
-    AdjointSide& A = P.side[s];
+  double* const out[3] = {Xb, Lb, Rb};
+  auto run = [&](int i) {
+    if (i == 0) {
+      be_->run(P.xbar, nullptr, Xb, 1, 0, 0, 0);
+      return;
+    }
+    AdjointSide& A = P.side[i - 1];
     be_->run(A.direct, nullptr, A.G, 1, 0, 0, 0);
     if (A.M) be_->run(A.partial, nullptr, A.M, 1, 0, 0, 0);
-    be_->run(A.sum, nullptr, out[s], 1, 0, 0, 0);
+    be_->run(A.sum, nullptr, out[i], 1, 0, 0, 0);
+  };
+  // lists that would not stay anyway are made, run and given back one output at a time
+  if (adj_.gen < 0 && limit > 0) {
+    long long bytes = 16 * step_.length;
+    for (int i = 0; i < 3; ++i)
+      if (want[i]) bytes += (long long)sizeof(Task) * 3 / 2 * (long long)step_.heff_full.tasks.size();
+    if (Lb) bytes += 8 * (Lcat_[step_.k].size + step_.L.size);
+    if (Rb) bytes += 8 * (Rcat_[step_.k + 2].size + step_.R.size);
+    if (bytes * 16 > room()) {
+      int rc = 0;
+      for (int i = 0; i < 3 && !rc; ++i) {
+        if (!want[i]) continue;
+        const bool one[3] = {i == 0, i == 1, i == 2};
+        rc = adjoint_plan(one, X, Yb, err);
+        if (!rc) run(i);
+        be_->sync();
+        drop_adjoint();
+      }
+      const std::string e = be_->error();
+      if (rc) return rc;
+      if (!e.empty()) {
+        err = e;
+        return -6;
+      }
+      return 0;
+    }
   }
+  const long long base = be_->mem_used() - adj_.bytes;
+  int rc = adjoint_plan(want, nullptr, nullptr, err);
+  if (rc) return rc;
+  be_->copy(P.x, X, step_.length);
+  be_->copy(P.yb, Yb, step_.length);
+  for (int i = 0; i < 3; ++i)
+    if (want[i]) run(i);
   be_->sync();
   std::string e = be_->error();
   // the lists and buffers stay for the step's next call where all that the call
   // added to the device takes little of the memory that is left, and go back at
   // once otherwise, or when something else needs the room
   P.bytes = std::max(be_->mem_used() - base, 0LL);
-  const long long limit = be_->mem_limit();
-  if (!e.empty() || (limit > 0 && P.bytes * 16 > std::min(limit - be_->mem_used(), be_->mem_free()))) drop_adjoint();
+  if (!e.empty() || (limit > 0 && P.bytes * 16 > room())) drop_adjoint();
   if (!e.empty()) {
     err = e;
     return -6;

@@ -572,7 +572,7 @@ class Engine {
   AdjointPlan adj_;
   bool adj_running_ = false;
   void drop_adjoint();
-  int adjoint_plan(const bool want[3], std::string& err);
+  int adjoint_plan(const bool want[3], const double* X, const double* Yb, std::string& err);
   // catalogue staging: the position of the current work (eviction order is
   // the distance from it: the catalogue needed last leaves first), the
   // catalogues in use (never moved), pinned host memory in use and budget

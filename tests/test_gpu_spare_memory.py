@@ -117,3 +117,23 @@ def test_adjoint_lists_make_room(state):
     for a, b in zip(_adjoint(ctx, x, want), grads):
         assert torch.equal(a, b)
     ctx.close()
+
+
+def test_adjoint_where_memory_is_short(state):
+    """Made, run and given back one output at a time, the lists give the same gradients."""
+    ctx, length = _ctx(state)
+    x = _vector(length)
+    yb = x.flip(0)
+    before = ctx.memory_stats()["device_used"]
+    want = _adjoint(ctx, x, yb)
+    kept = ctx.memory_stats()["device_used"] - before
+    ctx.build_env(K)
+    used = ctx.memory_stats()["device_used"]
+    ctx.set_memory_budget(used + kept)
+    try:
+        for a, b in zip(_adjoint(ctx, x, yb), want):
+            assert torch.equal(a, b)
+        assert ctx.memory_stats()["device_used"] == used
+    finally:
+        ctx.set_memory_budget(0)
+    ctx.close()
