@@ -314,6 +314,7 @@ struct DgPlanState {
   int njobs, nx, fail, pad;
 };
 
+// the first half of MurmurHash3's 64-bit finaliser (Appleby, public domain)
 __device__ __forceinline__ unsigned im_hash(unsigned long long k) {
   k ^= k >> 33;
   k *= 0xff51afd7ed558ccdull;

@@ -1337,9 +1337,13 @@ static void dfma_tiles(const TaskList& tl, DevList& d) {
 // clocks of one SM whose resident CTAs share it: their MMAs (34 digit pairs, 8
 // clocks each on one of four tensor cores), the cutting of T, the joining of
 // sums into Y, and a fixed part per staged chunk.  Only ratios matter: they
-// decide classes, sides and splits.  What the products' inner sizes contribute
-// is summed once (add) for every side and tile (at); a list's planning is part
-// of its first product.
+// decide classes, sides and splits.  Kernel times over these estimates, of seven
+// lists (13 to 24 orbitals): 1.8 to 2.0 in the 16-class, 2.5 to 2.8 in the
+// 32-class (1.7 where its blocks fill it), 1.7 to 2.7 in the 64-class; raising
+// the two larger classes by 1.2 and 1.1, or 1.4 and 1.15, made nine lists up to
+// 10 % slower and none faster by more than 1 %, so they stand as they are.  What
+// the products' inner sizes contribute is summed once (add) for every side and
+// tile (at); a list's planning is part of its first product.
 struct DgCost {
   double both = 0, two_ch = 0, two_k = 0;                 // products with two, one identity factor: count, chunks, k
   double steps = 0, kl = 0, k = 0, klch = 0, ch = 0;      // others: steps, k l, k, k times l chunks, chunks
