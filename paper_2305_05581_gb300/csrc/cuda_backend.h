@@ -101,14 +101,24 @@ struct Tune {
 // such as cold caches land there), then kTuneRounds timed samples of every
 // variant, the fastest sample of each compared
 constexpr int kTuneRounds = 2;
-// Inside an eigensolver the reduced-precision products feed the next vectors,
-// and a schedule shows in their FP32 partial sums: there the default variant
-// stays unless another needs less than kSteady of its time, so that a few
-// per cent of timing noise do not decide where an unconverged solve ends.
-constexpr double kSteady = 0.8;
+// Inside an eigensolver the products feed the next vectors, and a schedule shows
+// in the last bits of their partial sums: there the default variant stays unless
+// another needs less than this part of its time, so that timing noise does not
+// decide where an unconverged solve ends.  FP64 schedules differ by up to 13 %
+// and their samples by 1 to 2 %; of the reduced precisions the split reduction's
+// speed alone reorders schedules that lie within 20 %.
+constexpr double kSteady = 0.8, kSteadyFp64 = 0.97;
+constexpr int kDefaultVariant = 1;
+inline int pick_variant(const float* ms, int n, double steady) {
+  int best = 0;
+  for (int i = 1; i < n; ++i)
+    if (ms[i] < ms[best]) best = i;
+  return ms[best] > steady * ms[kDefaultVariant] ? kDefaultVariant : best;
+}
 // A digit product takes 0.3 to 0.7 of the FMA kernel's time, and what has no
-// certificate is done again by that kernel: beyond a third the sum is no gain
-// (24 orbitals, D = 512, all sectors: 21 ms and a tenth of 36.5 ms again).
+// certificate is done again by that kernel, in clusters: beyond a fifth the sum
+// is no gain.  24 orbitals, D = 512, all sectors: a tenth, 25 against 36 ms; a
+// swept step of 16 orbitals with more than a fifth: 17 against 13 ms.
 constexpr double kFailedShare = 0.2;
 // Lists below these flops stay with the FMA kernel: making the images takes
 // their first product 0.16 ms, and what a later one gains is 0.04 ms at 2.6e7

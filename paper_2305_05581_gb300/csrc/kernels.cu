@@ -1984,10 +1984,7 @@ void CudaBackend::run(const TaskList& tl, const double* xv, double* yv, int nvec
     cudaEventDestroy(b);
     tu.ms[v] = std::min(tu.ms[v], ms);
     if (++tu.step == 1 + kTuneRounds * nvar) {
-      tu.best = 0;
-      for (int i = 1; i < nvar; ++i)
-        if (tu.ms[i] < tu.ms[tu.best]) tu.best = i;
-      if (iterating && precision != 0 && tu.ms[tu.best] > kSteady * tu.ms[1]) tu.best = 1;
+      tu.best = pick_variant(tu.ms, nvar, !iterating ? 1.0 : precision != 0 ? kSteady : kSteadyFp64);
       tune_cache_[ckey] = tu.best;
       ++tuned;
     }
