@@ -117,13 +117,13 @@ inline int pick_variant(const float* ms, int n, double steady) {
 }
 // A digit product takes 0.3 to 0.7 of the FMA kernel's time, and what has no
 // certificate is done again by that kernel, in clusters: beyond a fifth the sum
-// is no gain.  24 orbitals, D = 512, all sectors: a tenth, 25 against 36 ms; a
+// is no gain.  24 orbitals, D = 512, all sectors: a tenth, 19 against 36 ms; a
 // swept step of 16 orbitals with more than a fifth: 17 against 13 ms.
 constexpr double kFailedShare = 0.2;
 // Lists below these flops stay with the FMA kernel: making the images takes
-// their first product 0.16 ms, and what a later one gains is 0.04 ms at 2.6e7
-// flops (8 orbitals: 0.236 -> 0.193 ms), nothing at 8e6, but 0.33 ms at 9.4e7
-// (10 orbitals, D = 96: 0.705 -> 0.371 ms).
+// their first product 0.2 ms, and what a later one gains is 0.06 ms at 2.6e7
+// flops (8 orbitals: 0.235 -> 0.177 ms), nothing at 8e6, but 0.38 ms at 9.4e7
+// (10 orbitals, D = 96: 0.706 -> 0.330 ms).
 constexpr double kDigitFlops = 5e7;
 constexpr int kSteadyKey = 1 << 16;  // schedules and graphs of such products are kept apart
 

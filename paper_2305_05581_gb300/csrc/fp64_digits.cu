@@ -53,9 +53,9 @@
 // to 12 warps that registers and shared memory leave an SM to hide its latencies.
 // One H_eff*psi, DFMA tile classes -> here (time, useful rate; in brackets
 // without certificates):
-//   24 orbitals, D = 512, all sectors (blocks <= 26):  36.4 -> 23.9 ms, 0.72 TFLOP/s [15.9]
-//   24 orbitals, D = 512, 9 sectors (blocks <= 68):     153 -> 51 ms, 2.3 TFLOP/s    [47]
-//   13 orbitals, D = 260, 3 sectors (blocks <= 99):    3.03 -> 0.90 ms, 2.4 TFLOP/s  [0.78]
+//   24 orbitals, D = 512, all sectors (blocks <= 26):  36.5 -> 19.3 ms, 0.89 TFLOP/s [15.9]
+//   24 orbitals, D = 512, 9 sectors (blocks <= 68):     153 -> 52 ms, 2.2 TFLOP/s    [47]
+//   13 orbitals, D = 260, 3 sectors (blocks <= 99):    3.03 -> 0.83 ms, 2.6 TFLOP/s  [0.78]
 // (cuBLAS DGEMM: 1.10 TFLOP/s).
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -476,6 +476,7 @@ template <int W_, int NBT_, int DBT_, int LK_, int KM_, int CTAS_>
 struct ImCfg {
   static constexpr int W = W_, NBT = NBT_, DBT = DBT_, LK = LK_, KM = KM_, CTAS = CTAS_;
   static constexpr int NT = 32 * W, AR = 16 * W, BR = 8 * NBT;
+  static constexpr int GU = W == 4 ? KM / 8 : 1;  // bodies of GEMM1, eight rows of X each
   static constexpr int LO = LK / 8, KO = KM / 8;              // octets staged
   static constexpr int off_x = (AR / 8) * LO * IM_UNIT;       // X after A in the first slot; a vector in A's place takes both
   static constexpr int off_b = off_x + (KM / 8) * LO * IM_XUNIT;
@@ -493,31 +494,30 @@ __device__ __forceinline__ void cp16(uint32_t dst, const void* src) {
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
-// `rows` runs of n 16-byte pieces, a warp per run.  Out of line in the CTAs of
-// several warps: the kernel has ten such copies, and inlined they are a third of
-// the code that its warps fetch again for every product.  The one-warp class has
-// no registers to spare for what a call leaves to its caller.
+// `rows` runs of n 16-byte pieces, a warp per run.  Out of line: inlined, the
+// kernel's copies are a third of the code that its warps fetch again for every
+// product.
 template <int W>
-__device__ __forceinline__ void im_copy_body(uint32_t dst, const unsigned char* src, int n, int rows, int sstride, int dstride) {
+__device__ __noinline__ void im_copy(uint32_t dst, const unsigned char* src, int n, int rows, int sstride, int dstride) {
   const int warp = W == 1 ? 0 : threadIdx.x >> 5, lane = threadIdx.x & 31;
   src += (long long)warp * sstride + lane * 16;
   dst += (uint32_t)(warp * dstride + lane * 16);
+#pragma unroll 1
   for (int r = warp; r < rows; r += W) {
+#pragma unroll 1
     for (int i = lane; i < n; i += 32) cp16(dst + (uint32_t)(i - lane) * 16, src + (i - lane) * 16);
     src += (long long)W * sstride;
     dst += W * dstride;
   }
 }
-template <int W>
-__device__ __noinline__ void im_copy_call(uint32_t dst, const unsigned char* src, int n, int rows, int sstride, int dstride) {
-  im_copy_body<W>(dst, src, n, rows, sstride, dstride);
-}
-template <int W>
-__device__ __forceinline__ void im_copy(uint32_t dst, const unsigned char* src, int n, int rows, int sstride, int dstride) {
-  if constexpr (W == 1) im_copy_body<W>(dst, src, n, rows, sstride, dstride);
-  else im_copy_call<W>(dst, src, n, rows, sstride, dstride);
-}
 
+// The kernel's size counts: its warps run through all of it for every product,
+// and with every loop over a tile unrolled it was 80 KB of code, a quarter of
+// the time fetches of it (24 orbitals, D = 512, all sectors 27.2 ms, 9 sectors
+// 53.4).  Loops that are not held in registers stay rolled (22.7 and 50.9 ms),
+// the two places that copy the next operands are one, and the two smaller
+// classes run GEMM1 in one body over X's rows (20.8 ms; the 64-class is slower
+// with it, 51.8).
 template <class C>
 __global__ void __launch_bounds__(C::NT, C::CTAS)
     k_tasks_im(const DgRec* __restrict__ recs, const Task* __restrict__ tasks, const Group* __restrict__ groups,
@@ -562,6 +562,7 @@ __global__ void __launch_bounds__(C::NT, C::CTAS)
   auto scale = [](double alpha, int n) { return alpha * __hiloint2double((n + 1023) << 20, 0); };  // alpha 2^n
   // the row groups this CTA never copies (a tile of fewer rows than the slot
   // has) are read by ldmatrix as absent rows: zero once
+#pragma unroll 1
   for (int i = tid; i < C::total / 16; i += NT) ((uint4*)sm)[i] = make_uint4(0, 0, 0, 0);
   sync();
 
@@ -571,6 +572,7 @@ __global__ void __launch_bounds__(C::NT, C::CTAS)
     im_copy<W>(dst, img + head + ((long long)rg0 * oc + o0) * U, no * (U / 16), nrg, oc * U, doct * U);
   };
   auto scales = [&](uint32_t dst, const unsigned char* img, int row, int groups) {
+#pragma unroll 1
     for (int i = tid; i < 2 * groups; i += NT) cp16(dst + i * 16, img + (row + 4 * i) * 4);
   };
   // first-slot copy: A (or what stands in its place) and X for chunk (k0, l0)
@@ -597,6 +599,7 @@ __global__ void __launch_bounds__(C::NT, C::CTAS)
     if (v) {
       const int oc = im_oct(r.L), no = min(KO, oc - (k0 >> 3));
       const unsigned char* u = ib + im_xhead((brows + 15) / 16 * 16) + ((long long)(b0 >> 3) * oc + (k0 >> 3)) * IM_XUNIT;
+#pragma unroll 1
       for (int g = 0; g < nbt; ++g)
         im_copy<W>(sB + g * KO * IM_UNIT, u + (long long)g * oc * IM_XUNIT, IM_UNIT / 16, no, IM_XUNIT, IM_UNIT);
     } else {
@@ -629,7 +632,9 @@ __global__ void __launch_bounds__(C::NT, C::CTAS)
         const Task tk = tasks[ti];
         const double* pX = xv + (long long)vec * xs + (long long)(size_t)tk.X;
         const long long sa = bl ? tk.n : 1, sb = bl ? 1 : tk.n;
+#pragma unroll 1
         for (int b = 0; b < nbt; ++b)
+#pragma unroll 1
           for (int h = 0; h < 2; ++h) {
             const int a = 16 * warp + g + 8 * h, c = 8 * b + 2 * t;
             const double* x = pX + (a0 + a) * sa + (b0 + c) * sb;
@@ -664,6 +669,7 @@ __global__ void __launch_bounds__(C::NT, C::CTAS)
     };
     const int K = f == 2 ? rec.L : rec.K, L = rec.L;
     int hsh = 0;
+#pragma unroll 1
     while ((32 << hsh) < L) ++hsh;
     // errors of a T entry beside A's last digits (1 per unit of X's row sum), in
     // units of 2^-56 of the scales: dropped pairs, X's last bit, the joined sums' roundings
@@ -718,52 +724,61 @@ __global__ void __launch_bounds__(C::NT, C::CTAS)
 #pragma unroll
             for (int q = 0; q < 4; ++q) alow[h][q] = dg_low(alow[h][q]);
           }
+          // 8 rows of X at a time: 16 would take the registers of another warp
+#pragma unroll(C::GU)
+          for (int q8 = 0; q8 < KT; ++q8) {
+            if (8 * q8 >= ((kc + 15) & ~15)) break;
+            float acc[DG_S][4], sa[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-          for (int kp = 0; kp < KT / 2; ++kp) {
-            if (16 * kp >= kc) break;
+            for (int h = 0; h < LK / 16; ++h) {
+              if (h > 0 && 16 * h >= lc) break;
+              uint32_t xf[IM_NX / 2][4];  // two digits each, in halves
+              const uint32_t xa = sX + (uint32_t)((q8 * LO + 2 * h + (mj & 1)) * IM_XUNIT + (mj >> 1) * 128 + mr16);
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {  // 8 rows of X at a time: both would take the registers of another warp
-              float acc[DG_S][4], sa[4] = {0.f, 0.f, 0.f, 0.f};
+              for (int j = 0; j < IM_NX / 2; ++j) ldsm4(xf[j], xa + j * 256);
+              const uint32_t aa = sA + (uint32_t)(((2 * warp + (mj & 1)) * LO + 2 * h + (mj >> 1)) * IM_UNIT + mr16);
 #pragma unroll
-              for (int h = 0; h < LK / 16; ++h) {
-                if (h > 0 && 16 * h >= lc) break;
-                uint32_t xf[IM_NX / 2][4];  // two digits each, in halves
-                const uint32_t xa = sX + (uint32_t)(((2 * kp + c) * LO + 2 * h + (mj & 1)) * IM_XUNIT + (mj >> 1) * 128 + mr16);
+              for (int i = 0; i < DG_N; ++i) {
+                uint32_t af[4];
+                ldsm4(af, aa + i * 128);
 #pragma unroll
-                for (int j = 0; j < IM_NX / 2; ++j) ldsm4(xf[j], xa + j * 256);
-                const uint32_t aa = sA + (uint32_t)(((2 * warp + (mj & 1)) * LO + 2 * h + (mj >> 1)) * IM_UNIT + mr16);
-#pragma unroll
-                for (int i = 0; i < DG_N; ++i) {
-                  uint32_t af[4];
-                  ldsm4(af, aa + i * 128);
-#pragma unroll
-                  for (int j = 0; i + j < DG_S; ++j) {
-                    const uint32_t x0 = xf[j / 2][2 * (j & 1)], x1 = xf[j / 2][2 * (j & 1) + 1];
-                    if (h == 0 && i == 0) mma_first(acc[i + j], af, x0, x1);
-                    else mma_acc(acc[i + j], af, x0, x1);
-                  }
+                for (int j = 0; i + j < DG_S; ++j) {
+                  const uint32_t x0 = xf[j / 2][2 * (j & 1)], x1 = xf[j / 2][2 * (j & 1) + 1];
+                  if (h == 0 && i == 0) mma_first(acc[i + j], af, x0, x1);
+                  else mma_acc(acc[i + j], af, x0, x1);
                 }
-                mma_acc(sa, alow[h], dg_low(xf[0][0]), dg_low(xf[0][1]));  // the same sums of lower bounds
               }
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                const long long v = dg_join(acc[0][e], acc[1][e], acc[2][e], acc[3][e], acc[4][e], acc[5][e], acc[6][e], acc[7][e]);
-                T[2 * kp + c][e] += hsh ? v >> hsh : v;
-              }
-              const int k = 16 * kp + 8 * c + 2 * t;
-              const int2 ek = *(const int2*)(eX + k);
-              const float2 sk = *(const float2*)(xsum + k);
-              auto down = [&](int e) { return __uint_as_float((uint32_t)max(124 - ex + e, 0) << 23); };  // 2^(-3 - distance)
-              const float f0 = down(ek.x), f1 = down(ek.y), m0 = f0 * lim14, m1 = f1 * lim14;
-              if (l0 == 0) {
-                mt[kp][2 * c] = dg_pack(sa[0] * m0, sa[1] * m1);
-                mt[kp][2 * c + 1] = dg_pack(sa[2] * m0, sa[3] * m1);
-                et[kp][c] = dg_pack(fmaf(sk.x, -1.015f, -el) * f0, fmaf(sk.y, -1.015f, -el) * f1);
-              } else {
-                mt[kp][2 * c] = dg_more(mt[kp][2 * c], sa[0] * m0, sa[1] * m1);
-                mt[kp][2 * c + 1] = dg_more(mt[kp][2 * c + 1], sa[2] * m0, sa[3] * m1);
-              }
+              mma_acc(sa, alow[h], dg_low(xf[0][0]), dg_low(xf[0][1]));  // the same sums of lower bounds
             }
+            long long v[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              v[e] = dg_join(acc[0][e], acc[1][e], acc[2][e], acc[3][e], acc[4][e], acc[5][e], acc[6][e], acc[7][e]);
+              if (hsh) v[e] >>= hsh;
+            }
+            const int k = 8 * q8 + 2 * t;
+            const int2 ek = *(const int2*)(eX + k);
+            const float2 sk = *(const float2*)(xsum + k);
+            auto down = [&](int e) { return __uint_as_float((uint32_t)max(124 - ex + e, 0) << 23); };  // 2^(-3 - distance)
+            const float f0 = down(ek.x), f1 = down(ek.y), m0 = f0 * lim14, m1 = f1 * lim14;
+            const uint32_t e2 = dg_pack(fmaf(sk.x, -1.015f, -el) * f0, fmaf(sk.y, -1.015f, -el) * f1);
+            auto keep = [&](int b) {
+#pragma unroll
+              for (int e = 0; e < 4; ++e) T[b][e] += v[e];
+              uint32_t &u0 = mt[b / 2][2 * (b & 1)], &u1 = mt[b / 2][2 * (b & 1) + 1];
+              if (l0 == 0) {
+                u0 = dg_pack(sa[0] * m0, sa[1] * m1);
+                u1 = dg_pack(sa[2] * m0, sa[3] * m1);
+                et[b / 2][b & 1] = e2;
+              } else {
+                u0 = dg_more(u0, sa[0] * m0, sa[1] * m1);
+                u1 = dg_more(u1, sa[2] * m0, sa[3] * m1);
+              }
+            };
+            if (q8 == 0) keep(0);
+            else if (q8 == 1) keep(1);
+            else if (KT == 4 && q8 == 2) keep(KT - 2);
+            else if (KT == 4) keep(KT - 1);
           }
         }
         if (mine) {
@@ -862,8 +877,10 @@ __global__ void __launch_bounds__(C::NT, C::CTAS)
       }
       cp_wait();
       sync();  // the second slot is in, the first is free
-      if (k0 + KM < K) load1(rec, k0 + KM, 0);
-      else if (more) load1(recs[ti + 1], 0, 0);
+      const bool on = k0 + KM < K;
+      DgRec nx = rec;
+      if (!on && more) nx = recs[ti + 1];
+      if (on || more) load1(nx, on ? k0 + KM : 0, 0);
       cp_commit();
       if (!mine) continue;
 #pragma unroll 1
@@ -936,7 +953,9 @@ __global__ void __launch_bounds__(C::NT, C::CTAS)
 
   // without a certificate the piece goes to the FMA kernel, which runs after this one
   if (mine && !bad)
+#pragma unroll 1
     for (int b = 0; b < nbt; ++b)
+#pragma unroll 1
       for (int h = 0; h < 2; ++h)
         if (16 * warp + g + 8 * h < na && 8 * b + 2 * t < nb) {
           const float2 d = DBT == NBT || b < DBT ? Ds[(2 * b + h) * 32] : make_float2(Dp[(2 * b + h) * 32], 0.f);
@@ -949,6 +968,7 @@ __global__ void __launch_bounds__(C::NT, C::CTAS)
   double* Y = yv + (long long)vec * ys + G.yoff;
   double* P = TL.poff >= 0 ? part + (long long)vec * psize + TL.poff : nullptr;  // split piece
   if (mine)
+#pragma unroll 1
     for (int b = 0; b < nbt; ++b)
 #pragma unroll
       for (int e = 0; e < 4; ++e) {

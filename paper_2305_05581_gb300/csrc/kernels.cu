@@ -1338,12 +1338,13 @@ static void dfma_tiles(const TaskList& tl, DevList& d) {
 // clocks each on one of four tensor cores), the cutting of T, the joining of
 // sums into Y, and a fixed part per staged chunk.  Only ratios matter: they
 // decide classes, sides and splits.  Kernel times over these estimates, of seven
-// lists (13 to 24 orbitals): 1.8 to 2.0 in the 16-class, 2.5 to 2.8 in the
-// 32-class (1.7 where its blocks fill it), 1.7 to 2.7 in the 64-class; raising
-// the two larger classes by 1.2 and 1.1, or 1.4 and 1.15, made nine lists up to
-// 10 % slower and none faster by more than 1 %, so they stand as they are.  What
-// the products' inner sizes contribute is summed once (add) for every side and
-// tile (at); a list's planning is part of its first product.
+// lists (13 to 24 orbitals): 1.4 to 1.5 in the 16-class, 1.7 to 2.4 in the
+// 32-class, 1.5 to 2.2 in the 64-class.  Of factors 0.85 to 1.4 on the two larger
+// classes 1.15 on the largest is the only one that made one of nine lists faster
+// (13 orbitals, 0.88 -> 0.83 ms) and none slower; 1.15 on the 32-class, or less
+// than 1 on either, cost up to 22 %.  What the products' inner sizes contribute
+// is summed once (add) for every side and tile (at); a list's planning is part
+// of its first product.
 struct DgCost {
   double both = 0, two_ch = 0, two_k = 0;                 // products with two, one identity factor: count, chunks, k
   double steps = 0, kl = 0, k = 0, klch = 0, ch = 0;      // others: steps, k l, k, k times l chunks, chunks
@@ -1368,8 +1369,9 @@ struct DgCost {
   double at(int cls, int a, int b) const {
     const double fixed[kDgClasses] = {150.0, 400.0, 800.0}, mm = 34.0 * 8.0 / 2048.0;
     const double ap = (a + 15) & ~15, bp = (b + 7) & ~7;
-    return fixed[cls] * (both + two_ch + steps) + both * a * b / 4.0 +
-           0.25 * ap * (bp * (mm * (two_k + k) + 4.0 * (two_ch + ch)) + mm * kl + 2.4 * klch);
+    return (cls == 2 ? 1.15 : 1.0) *
+           (fixed[cls] * (both + two_ch + steps) + both * a * b / 4.0 +
+            0.25 * ap * (bp * (mm * (two_k + k) + 4.0 * (two_ch + ch)) + mm * kl + 2.4 * klch));
   }
 };
 
