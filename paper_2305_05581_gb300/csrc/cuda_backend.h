@@ -118,13 +118,15 @@ inline int pick_variant(const float* ms, int n, double steady) {
 // A digit product takes 0.3 to 0.7 of the FMA kernel's time, and what has no
 // certificate is done again by that kernel, in clusters: beyond a fifth the sum
 // is no gain.  24 orbitals, D = 512, all sectors: a tenth, 19 against 36 ms; a
-// swept step of 16 orbitals with more than a fifth: 17 against 13 ms.
+// swept step of 16 orbitals with more than a fifth: 14.2 against 13.2 ms.
 constexpr double kFailedShare = 0.2;
-// Lists below these flops stay with the FMA kernel: making the images takes
-// their first product 0.2 ms, and what a later one gains is 0.06 ms at 2.6e7
-// flops (8 orbitals: 0.235 -> 0.177 ms), nothing at 8e6, but 0.38 ms at 9.4e7
-// (10 orbitals, D = 96: 0.706 -> 0.330 ms).
-constexpr double kDigitFlops = 5e7;
+// Lists below kDigitFlops stay with the FMA kernel: at 8e6 flops digits are no
+// faster (12 orbitals, D = 130, 2 sectors: 0.066 and 0.075 ms), at 2.6e7 they are
+// (8 orbitals: 0.235 and 0.177 ms).  Making the images takes a product 0.2 ms,
+// more than the first product gains below kDigitsAtOnce (8 orbitals 1.36 -> 1.60
+// ms, 10 orbitals at 9.4e7 flops 2.40 -> 2.62; at 4.4e8 and above the same or
+// less): there they are made with the second one.
+constexpr double kDigitFlops = 2e7, kDigitsAtOnce = 4e8;
 constexpr int kSteadyKey = 1 << 16;  // schedules and graphs of such products are kept apart
 
 // captured launch sequence of one (precision, nvec) use: replayed with the

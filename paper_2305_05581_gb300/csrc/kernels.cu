@@ -1940,27 +1940,33 @@ void CudaBackend::run(const TaskList& tl, const double* xv, double* yv, int nvec
   if (precision != 0) {
     if (!prepare_tasks_tc(*this, tl, d, nvec, v, precision)) return;
   } else {
-    if (fk == 2 && digit_images(tl) && (fp64_kernel == 2 || list_flops(tl, d) >= kDigitFlops)) {
+    // a list's untimed first product of a schedule yet to be tuned is the FMA kernel's where making the images
+    // would take longer than it
+    const bool later = tuning && !timing && !d.dg && list_flops(tl, d) < kDigitsAtOnce;
+    if (fk == 2 && digit_images(tl) && (fp64_kernel == 2 || (list_flops(tl, d) >= kDigitFlops && !later))) {
       if (!d.fp_tiled[1]) dg_tiles(tl, d);
       dig = prepare_digits(*this, tl, d, nvec, xs) ? 1 : 0;
     }
     plan_variant(tl, d, dig, v);
     if (!ok() || !ensure_part(d, d.fv[dig][v], dig, nvec)) return;
     if (dig && !d.dg_kept && fp64_kernel != 2) {
-      // the list's first product: where too much of it has no certificate, the
-      // list is for the FMA kernel, this product included
+      // the first product on digits: where too much of it has no certificate,
+      // the list is for the FMA kernel, this product included
       enqueue_fp64(d, 1, v, xv, yv, nvec, xs, ys);
       if (failed_share(d.fv[1][v], nvec) <= kFailedShare) {
         d.dg_kept = true;
-        if (tuning && !timing) ++tu.step;
-        return;
+        if (!timing) {
+          if (tuning) ++tu.step;
+          return;
+        }
+      } else {
+        release_digit_plan(d.dg);
+        d.dg = nullptr;
+        d.dg_none = true;
+        dig = 0;
+        plan_variant(tl, d, 0, v);
+        if (!ok() || !ensure_part(d, d.fv[0][v], 0, nvec)) return;
       }
-      release_digit_plan(d.dg);
-      d.dg = nullptr;
-      d.dg_none = true;
-      dig = 0;
-      plan_variant(tl, d, 0, v);
-      if (!ok() || !ensure_part(d, d.fv[0][v], 0, nvec)) return;
     }
   }
   auto enqueue = [&](const double* x, double* y) {
